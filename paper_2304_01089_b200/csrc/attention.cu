@@ -18,82 +18,16 @@
 // shared memory in the same order. Pass 2 holds the sums of up to eight V units (a whole head) in
 // registers. The packed codes of the next key tile are copied into a staging buffer (cp.async) while
 // the current tile is multiplied.
-#include <cuda_fp16.h>
-
-#include "rptq_internal.h"
-#include "unpack.cuh"
+#include "attn_common.cuh"
 
 namespace rptq {
 namespace attn {
 
 constexpr int BM = 64, BN = 64, THREADS = 128;
-constexpr int MAX_UNITS = 8;                 // units of 32 positions per head
 constexpr int QK_PITCH_MAX = 32 * MAX_UNITS + 16;
 constexpr int V_CHUNK_UNITS = 8;
 constexpr int VT_PITCH = BN + 16;
-constexpr float NEG_BIG = -1.0e30f;
 
-struct Params {
-    const uint8_t *q, *k, *v;
-    int64_t q_row_bytes, k_row_bytes, v_row_bytes;
-    int bits_q, bits_k, bits_v;
-    int Tq, Tk, H, gh_qk, gh_v, causal;     // Tq queries and Tk keys per sequence; blockIdx.z is the sequence
-    int n_used_qk, n_used_v;                 // units that belong to a cluster
-    const int32_t *unit_cluster_qk, *unit_cluster_v;
-    const float2 *unit_sz_q, *unit_sz_k, *unit_sz_v;
-    const uint16_t* src_v;                   // channel at each padded position of V's layout
-    const int32_t* jidx_v;                   // -1 at pad positions
-    float inv_sP, s_P, qk_scale_log2e;
-    __half* out;
-    int64_t ldo;
-    uint8_t* p_dbg;
-    int raw_pitch;                           // bytes per key row of the staging buffers for packed codes
-};
-
-__device__ __forceinline__ void load_unit(const uint8_t* row, int unit, int bits, uint32_t (&o)[8])
-{
-    if (bits == 4) {
-        const uint4 t = __ldg(reinterpret_cast<const uint4*>(row) + unit);
-        const uint32_t p[4] = {t.x, t.y, t.z, t.w};
-        unpack_act32<4>(p, o);
-    } else if (bits == 3) {
-        const uint32_t* w = reinterpret_cast<const uint32_t*>(row) + unit * 3;
-        const uint32_t p[3] = {__ldg(w), __ldg(w + 1), __ldg(w + 2)};
-        unpack_act32<3>(p, o);
-    } else {
-        const uint4* w = reinterpret_cast<const uint4*>(row) + unit * 2;
-        const uint4 a = __ldg(w), b = __ldg(w + 1);
-        o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
-    }
-}
-
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-// The same from a staged copy of the packed row in shared memory (`row` points at the head's first unit;
-// 4-byte aligned for 3-bit codes, 16-byte aligned otherwise).
-__device__ __forceinline__ void load_unit_smem(const uint8_t* row, int unit, int bits, uint32_t (&o)[8])
-{
-    if (bits == 4) {
-        const uint4 t = *(reinterpret_cast<const uint4*>(row) + unit);
-        const uint32_t p[4] = {t.x, t.y, t.z, t.w};
-        unpack_act32<4>(p, o);
-    } else if (bits == 3) {
-        const uint32_t* w = reinterpret_cast<const uint32_t*>(row) + unit * 3;
-        const uint32_t p[3] = {w[0], w[1], w[2]};
-        unpack_act32<3>(p, o);
-    } else {
-        const uint4* w = reinterpret_cast<const uint4*>(row) + unit * 2;
-        const uint4 a = w[0], b = w[1];
-        o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
-    }
-}
-// 16 bytes global -> shared without passing through registers; src_bytes = 0 writes zeros
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int src_bytes)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 __device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t (&r)[4])
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -105,24 +39,6 @@ __device__ __forceinline__ void mma_u8(int (&d)[4], const uint32_t (&a)[4], uint
                  : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ float ex2(float x)
-{
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
-// first unit whose cluster is >= c among the first n units (their clusters do not decrease)
-__device__ __forceinline__ int first_unit_of(const int32_t* unit_cluster, int n, int c)
-{
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(unit_cluster + mid) < c) lo = mid + 1; else hi = mid;
-    }
-    return lo;
-}
-
 // Key of the tile that sits in slot s (0..63) of the second product's contraction: slots 4t..4t+3 of a
 // 16-slot half hold keys 2t, 2t+1, 8+2t, 8+2t+1 of the half's 16 keys.
 __device__ __forceinline__ int key_of_slot(int s)
@@ -132,10 +48,9 @@ __device__ __forceinline__ int key_of_slot(int s)
 }
 
 __global__ void __launch_bounds__(THREADS)
-attention_kernel(const Params p)
+attention_kernel(const AttnParams p, const int raw_pitch)
 {
     extern __shared__ __align__(16) uint8_t smem[];
-    __shared__ int s_rng[4];
     __shared__ float s_coef[MAX_UNITS], s_czq[MAX_UNITS], s_col[BN];
     __shared__ uint8_t s_last[MAX_UNITS];
 
@@ -145,20 +60,14 @@ attention_kernel(const Params p)
     const int qt = (int)gridDim.x - 1 - (int)blockIdx.x;      // the tiles with the most visible keys first
     const int i0 = qt * BM;
 
-    if (tid == 0) {
-        s_rng[0] = first_unit_of(p.unit_cluster_qk, p.n_used_qk, h * p.gh_qk);
-        s_rng[1] = first_unit_of(p.unit_cluster_qk, p.n_used_qk, (h + 1) * p.gh_qk);
-        s_rng[2] = first_unit_of(p.unit_cluster_v, p.n_used_v, h * p.gh_v);
-        s_rng[3] = first_unit_of(p.unit_cluster_v, p.n_used_v, (h + 1) * p.gh_v);
-    }
-    __syncthreads();
-    const int uq0 = s_rng[0], nuq = s_rng[1] - s_rng[0], uv0 = s_rng[2], nuv = s_rng[3] - s_rng[2];
+    const int uq0 = __ldg(p.cl_unit0_k + h * p.gh_k), nuq = __ldg(p.cl_unit0_k + (h + 1) * p.gh_k) - uq0;
+    const int uv0 = __ldg(p.cl_unit0_v + h * p.gh_v), nuv = __ldg(p.cl_unit0_v + (h + 1) * p.gh_v) - uv0;
     const int pitch = 32 * nuq + 16;
     uint8_t* Qs = smem;
     uint8_t* Ks = Qs + BM * QK_PITCH_MAX;
     uint8_t* Vt = Ks + BN * QK_PITCH_MAX;
     uint8_t* rawK = Vt + 32 * V_CHUNK_UNITS * VT_PITCH;         // [2][BN][raw_pitch] packed K codes of a tile, as they lie in memory
-    uint8_t* rawV = rawK + 2 * BN * p.raw_pitch;
+    uint8_t* rawV = rawK + 2 * BN * raw_pitch;
     // a head's packed codes are a contiguous piece of a row; the staged window starts at the 16-byte boundary below it
     const int bytesK = 4 * p.bits_k, bytesV = 4 * p.bits_v;
     const int winK = (bytesK * uq0) & ~15, offK = bytesK * uq0 - winK, nK16 = (offK + bytesK * nuq + 15) >> 4;
@@ -169,7 +78,7 @@ attention_kernel(const Params p)
         const float c = q.x * k.x * p.qk_scale_log2e;
         s_coef[tid] = c;
         s_czq[tid] = -c * q.y;
-        s_last[tid] = (tid == nuq - 1) || (__ldg(p.unit_cluster_qk + uq0 + tid + 1) != __ldg(p.unit_cluster_qk + uq0 + tid));
+        s_last[tid] = (tid == nuq - 1) || (__ldg(p.unit_cluster_k + uq0 + tid + 1) != __ldg(p.unit_cluster_k + uq0 + tid));
     }
     // the queries' codes, as bytes
     for (int it = tid; it < BM * nuq; it += THREADS) {
@@ -194,24 +103,24 @@ attention_kernel(const Params p)
         const int buf = kt & 1;
         for (int it = tid; it < BN * nK16; it += THREADS) {
             const int r = it / nK16, c = it - r * nK16, j = kt * BN + r;
-            cp_async16(smem_u32(rawK + (buf * BN + r) * p.raw_pitch + 16 * c),
+            cp_async16(smem_u32(rawK + (buf * BN + r) * raw_pitch + 16 * c),
                        p.k + (k_row0 + min(j, p.Tk - 1)) * p.k_row_bytes + winK + 16 * c, j < p.Tk ? 16 : 0);
         }
         if (with_v)
             for (int it = tid; it < BN * nV16; it += THREADS) {
                 const int r = it / nV16, c = it - r * nV16, j = kt * BN + r;
-                cp_async16(smem_u32(rawV + (buf * BN + r) * p.raw_pitch + 16 * c),
+                cp_async16(smem_u32(rawV + (buf * BN + r) * raw_pitch + 16 * c),
                            p.v + (k_row0 + min(j, p.Tk - 1)) * p.v_row_bytes + winV + 16 * c, j < p.Tk ? 16 : 0);
             }
         cp_async_commit();
     };
     // Tile kt has been staged and a block-wide barrier passed since: unpack it to bytes
     auto load_k_tile = [&](int kt) {
-        const uint8_t* raw = rawK + (kt & 1) * BN * p.raw_pitch + offK;
+        const uint8_t* raw = rawK + (kt & 1) * BN * raw_pitch + offK;
         for (int it = tid; it < BN * nuq; it += THREADS) {
             const int r = it / nuq, u = it - r * nuq;
             uint32_t o[8];
-            load_unit_smem(raw + r * p.raw_pitch, u, p.bits_k, o);
+            load_unit_smem(raw + r * raw_pitch, u, p.bits_k, o);
             uint4* d = reinterpret_cast<uint4*>(Ks + r * pitch + 32 * u);
             d[0] = make_uint4(o[0], o[1], o[2], o[3]);
             d[1] = make_uint4(o[4], o[5], o[6], o[7]);
@@ -319,13 +228,13 @@ attention_kernel(const Params p)
             __syncthreads();                 // everyone's copies of tile kt have landed
             load_k_tile(kt);
             // V tile, transposed: Vt[position][slot] = code of key key_of_slot(slot)
-            const uint8_t* rawv = rawV + (kt & 1) * BN * p.raw_pitch + offV;
+            const uint8_t* rawv = rawV + (kt & 1) * BN * raw_pitch + offV;
             for (int it = tid; it < cu * 16; it += THREADS) {
                 const int u = it >> 4, w = it & 15;
                 uint32_t o[4][8];
 #pragma unroll
                 for (int b = 0; b < 4; ++b)
-                    load_unit_smem(rawv + key_of_slot(4 * w + b) * p.raw_pitch, c0 + u, p.bits_v, o[b]);
+                    load_unit_smem(rawv + key_of_slot(4 * w + b) * raw_pitch, c0 + u, p.bits_v, o[b]);
 #pragma unroll
                 for (int e = 0; e < 8; ++e) {        // positions 4e..4e+3 of the unit: a 4 x 4 byte transpose
                     const uint32_t x01l = __byte_perm(o[0][e], o[1][e], 0x5140), x01h = __byte_perm(o[0][e], o[1][e], 0x7362);
@@ -403,30 +312,6 @@ attention_kernel(const Params p)
 }  // namespace attn
 }  // namespace rptq
 
-static bool units_in_cluster_order(const rptq_layout_t* L, int* n_used)
-{
-    int prev = 0, n = 0;
-    for (int u = 0; u < L->n_units; ++u) {
-        const int c = L->unit_cluster[u];
-        if (c < 0) { for (int v = u; v < L->n_units; ++v) if (L->unit_cluster[v] >= 0) return false; break; }
-        if (c < prev) return false;
-        prev = c;
-        ++n;
-    }
-    *n_used = n;
-    return true;
-}
-
-static int max_units_per_head(const rptq_layout_t* L, int n_used, int H)
-{
-    const int gh = L->g / H;
-    std::vector<int> cnt((size_t)H, 0);
-    for (int u = 0; u < n_used; ++u) ++cnt[(size_t)(L->unit_cluster[u] / gh)];
-    int m = 0;
-    for (int c : cnt) m = c > m ? c : m;
-    return m;
-}
-
 extern "C" int rptq_attention(const rptq_layout_t* LQ, const rptq_layout_t* LK, const rptq_layout_t* LV, int n_heads,
                               const void* q_codes, int Tq, const void* k_codes, const void* v_codes, int Tk, int n_seq,
                               float s_P, int z_P, float qk_scale, int causal,
@@ -438,36 +323,39 @@ extern "C" int rptq_attention(const rptq_layout_t* LQ, const rptq_layout_t* LK, 
     if (n_heads < 1 || Tq < 0 || Tk < Tq || n_seq < 0 || !(s_P > 0.f) || !(qk_scale >= 0.f)) return RPTQ_ERR_INVALID_ARG;
     if (LQ->g % n_heads || LK->g != LQ->g || LV->g % n_heads || ldo < LV->C) return RPTQ_ERR_INVALID_ARG;
     if (!aligned16(q_codes) || !aligned16(k_codes) || !aligned16(v_codes) || (reinterpret_cast<uintptr_t>(out_f16) & 1u)) return RPTQ_ERR_INVALID_ARG;
-    // Q and K pair equal positions: same reorder index, same cluster sizes, same placement
-    if (LQ->C != LK->C || LQ->size != LK->size || LQ->perm != LK->perm || LQ->pos != LK->pos || LQ->unit_cluster != LK->unit_cluster)
-        return RPTQ_ERR_INVALID_ARG;
+    // Q and K pair equal positions: same reorder index, same cluster sizes (the placement follows from them and the unit order)
+    if (LQ->C != LK->C || LQ->in_cluster_order != LK->in_cluster_order || LQ->size != LK->size || LQ->perm != LK->perm) return RPTQ_ERR_INVALID_ARG;
     if (z_P != 0 || n_heads > 65535 || n_seq > 65535) return RPTQ_ERR_UNSUPPORTED;
-    int n_used_qk = 0, n_used_v = 0;
-    if (!units_in_cluster_order(LQ, &n_used_qk) || !units_in_cluster_order(LV, &n_used_v)) return RPTQ_ERR_UNSUPPORTED;
-    if (max_units_per_head(LQ, n_used_qk, n_heads) > MAX_UNITS || max_units_per_head(LV, n_used_v, n_heads) > MAX_UNITS) return RPTQ_ERR_UNSUPPORTED;
+    if (!LQ->in_cluster_order || !LV->in_cluster_order) return RPTQ_ERR_UNSUPPORTED;
+    const int units_k = max_units_per_head(LQ, n_heads), units_v = max_units_per_head(LV, n_heads);
+    if (units_k > MAX_UNITS || units_v > MAX_UNITS) return RPTQ_ERR_UNSUPPORTED;
     if ((int64_t)Tk * 255 * 255 > 2147483647ll) return RPTQ_ERR_UNSUPPORTED;      // the int32 sums of the second product
     if (Tq == 0 || n_seq == 0) return RPTQ_OK;
     int dev = -1;
     if (LQ->device < 0 || cudaGetDevice(&dev) != cudaSuccess) return RPTQ_ERR_CUDA;
     if (dev != LQ->device || dev != LK->device || dev != LV->device) return RPTQ_ERR_INVALID_ARG;
 
-    Params p{};
+    AttnParams p{};
     p.q = static_cast<const uint8_t*>(q_codes); p.k = static_cast<const uint8_t*>(k_codes); p.v = static_cast<const uint8_t*>(v_codes);
     p.q_row_bytes = LQ->row_bytes; p.k_row_bytes = LK->row_bytes; p.v_row_bytes = LV->row_bytes;
     p.bits_q = LQ->bits; p.bits_k = LK->bits; p.bits_v = LV->bits;
-    p.Tq = Tq; p.Tk = Tk; p.H = n_heads; p.gh_qk = LQ->g / n_heads; p.gh_v = LV->g / n_heads; p.causal = causal ? 1 : 0;
-    p.n_used_qk = n_used_qk; p.n_used_v = n_used_v;
-    p.unit_cluster_qk = LQ->d_unit_cluster; p.unit_cluster_v = LV->d_unit_cluster;
+    p.Tq = Tq; p.Tk = Tk; p.H = n_heads; p.gh_k = LQ->g / n_heads; p.gh_v = LV->g / n_heads; p.causal = causal ? 1 : 0;
+    p.cl_unit0_k = LQ->d_cl_unit0; p.cl_unit0_v = LV->d_cl_unit0; p.unit_cluster_k = LQ->d_unit_cluster;
     p.unit_sz_q = LQ->d_unit_sz; p.unit_sz_k = LK->d_unit_sz; p.unit_sz_v = LV->d_unit_sz;
     p.src_v = LV->d_src; p.jidx_v = LV->d_jidx;
     p.inv_sP = 1.0f / s_P; p.s_P = s_P; p.qk_scale_log2e = qk_scale * 1.4426950408889634f;
     p.out = static_cast<__half*>(out_f16); p.ldo = ldo; p.p_dbg = p_codes_out;
 
+    auto st = static_cast<cudaStream_t>(stream);
+    int n_sm = 0;
+    if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return RPTQ_ERR_CUDA;
+    if (attn_decode::fits(p, false)) return attn_decode::launch(p, false, units_k, units_v, n_seq, n_sm, st);
+
     const int max_bits = LK->bits > LV->bits ? LK->bits : LV->bits;
-    p.raw_pitch = 4 * max_bits * MAX_UNITS + 32;          // a head's packed codes plus the alignment slack, a multiple of 16
-    const int smem = (BM + BN) * QK_PITCH_MAX + 32 * V_CHUNK_UNITS * VT_PITCH + 4 * BN * p.raw_pitch;
+    const int raw_pitch = 4 * max_bits * MAX_UNITS + 32;          // a head's packed codes plus the alignment slack, a multiple of 16
+    const int smem = (BM + BN) * QK_PITCH_MAX + 32 * V_CHUNK_UNITS * VT_PITCH + 4 * BN * raw_pitch;
     if (cudaFuncSetAttribute(attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return RPTQ_ERR_CUDA;
     const dim3 grid((unsigned)((Tq + BM - 1) / BM), (unsigned)n_heads, (unsigned)n_seq);
-    attention_kernel<<<grid, THREADS, smem, static_cast<cudaStream_t>(stream)>>>(p);
+    attention_kernel<<<grid, THREADS, smem, st>>>(p, raw_pitch);
     return cudaGetLastError() == cudaSuccess ? RPTQ_OK : RPTQ_ERR_CUDA;
 }

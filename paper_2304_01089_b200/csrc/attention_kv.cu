@@ -12,50 +12,16 @@
 //     -z^K_c sum_p Q[i][p] is the same for every key of a row and cancels in the softmax.
 //   - Online softmax (running row maximum and sum, fp32), probabilities rounded to fp16 for the second
 //     product, V read with ldmatrix.trans; O = s^V_c (sum_j P V_q / sum_j P - z^V_c), fp16 out.
-#include <cuda_fp16.h>
-
-#include "rptq_internal.h"
-#include "unpack.cuh"
+#include "attn_common.cuh"
 
 namespace rptq {
 namespace attnkv {
 
+using namespace attn;
+
 constexpr int BM = 128, BN = 64, THREADS = 256;
-constexpr int MAX_UNITS = 8;                         // units of 32 positions per head
 constexpr int PITCH = 32 * MAX_UNITS * 2 + 16;       // bytes per row of the fp16 tiles: an odd number of 16-byte chunks
-constexpr float NEG_BIG = -1.0e30f;
 
-struct Params {
-    const __half* q; int64_t ldq;
-    const uint8_t *k, *v;
-    int64_t k_row_bytes, v_row_bytes;
-    int bits_k, bits_v;
-    int Tq, Tk, H, hd, gh_k, gh_v, causal;
-    int n_used_k, n_used_v;
-    const int32_t *unit_cluster_k, *unit_cluster_v;
-    const float2 *unit_sz_k, *unit_sz_v;
-    const uint16_t *src_k, *src_v;                   // channel at each padded position
-    const int32_t *jidx_k, *jidx_v;                  // -1 at pad positions
-    float qk_scale_log2e;
-    __half* out; int64_t ldo;
-};
-
-__device__ __forceinline__ void load_unit(const uint8_t* row, int unit, int bits, uint32_t (&o)[8])
-{
-    if (bits == 4) {
-        const uint4 t = __ldg(reinterpret_cast<const uint4*>(row) + unit);
-        const uint32_t p[4] = {t.x, t.y, t.z, t.w};
-        unpack_act32<4>(p, o);
-    } else if (bits == 3) {
-        const uint32_t* w = reinterpret_cast<const uint32_t*>(row) + unit * 3;
-        const uint32_t p[3] = {__ldg(w), __ldg(w + 1), __ldg(w + 2)};
-        unpack_act32<3>(p, o);
-    } else {
-        const uint4* w = reinterpret_cast<const uint4*>(row) + unit * 2;
-        const uint4 a = __ldg(w), b = __ldg(w + 1);
-        o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
-    }
-}
 // four code bytes -> four fp16 integers (two words)
 __device__ __forceinline__ void bytes_to_half4(uint32_t w, uint32_t& lo, uint32_t& hi)
 {
@@ -77,7 +43,6 @@ __device__ __forceinline__ void store_unit_half(uint8_t* dst, const uint32_t (&o
     }
 }
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 __device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t (&r)[4])
 {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
@@ -94,32 +59,10 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], const uint32_t (&a)[4], u
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
-__device__ __forceinline__ float ex2(float x)
-{
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ uint32_t pack_half2(float a, float b)
-{
-    const __half2 h = __floats2half2_rn(a, b);
-    return *reinterpret_cast<const uint32_t*>(&h);
-}
-__device__ __forceinline__ int first_unit_of(const int32_t* unit_cluster, int n, int c)
-{
-    int lo = 0, hi = n;
-    while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (__ldg(unit_cluster + mid) < c) lo = mid + 1; else hi = mid;
-    }
-    return lo;
-}
-
 __global__ void __launch_bounds__(THREADS)
-attention_kv_kernel(const Params p)
+attention_kv_kernel(const AttnParams p)
 {
     extern __shared__ __align__(16) uint8_t smem[];
-    __shared__ int s_rng[4];
     __shared__ float s_coef[MAX_UNITS];
     __shared__ uint8_t s_last[MAX_UNITS];
 
@@ -129,14 +72,8 @@ attention_kv_kernel(const Params p)
     const int qt = (int)gridDim.x - 1 - (int)blockIdx.x;      // the tiles with the most visible keys first
     const int i0 = qt * BM;
 
-    if (tid == 0) {
-        s_rng[0] = first_unit_of(p.unit_cluster_k, p.n_used_k, h * p.gh_k);
-        s_rng[1] = first_unit_of(p.unit_cluster_k, p.n_used_k, (h + 1) * p.gh_k);
-        s_rng[2] = first_unit_of(p.unit_cluster_v, p.n_used_v, h * p.gh_v);
-        s_rng[3] = first_unit_of(p.unit_cluster_v, p.n_used_v, (h + 1) * p.gh_v);
-    }
-    __syncthreads();
-    const int uk0 = s_rng[0], nuk = s_rng[1] - s_rng[0], uv0 = s_rng[2], nuv = s_rng[3] - s_rng[2];
+    const int uk0 = __ldg(p.cl_unit0_k + h * p.gh_k), nuk = __ldg(p.cl_unit0_k + (h + 1) * p.gh_k) - uk0;
+    const int uv0 = __ldg(p.cl_unit0_v + h * p.gh_v), nuv = __ldg(p.cl_unit0_v + (h + 1) * p.gh_v) - uv0;
     uint8_t* Qs = smem;                       // [BM][PITCH] fp16, K's position order
     uint8_t* Ks = Qs + BM * PITCH;            // [BN][PITCH] fp16 integers
     uint8_t* Vs = Ks + BN * PITCH;            // [BN][PITCH] fp16 integers, V's position order
@@ -155,7 +92,7 @@ attention_kv_kernel(const Params p)
     for (int it = tid; it < BM * p.hd; it += THREADS) {
         const int r = it / p.hd, c = it - r * p.hd;
         __half v = __float2half_rn(0.f);
-        if (i0 + r < p.Tq) v = p.q[(q_row0 + i0 + r) * p.ldq + h * p.hd + c];
+        if (i0 + r < p.Tq) v = p.q_f16[(q_row0 + i0 + r) * p.ldq + h * p.hd + c];
         *reinterpret_cast<__half*>(Ks + r * PITCH + 2 * c) = v;
     }
     __syncthreads();
@@ -301,39 +238,15 @@ attention_kv_kernel(const Params p)
 }  // namespace attnkv
 }  // namespace rptq
 
-static bool kv_units_in_cluster_order(const rptq_layout_t* L, int* n_used)
-{
-    int prev = 0, n = 0;
-    for (int u = 0; u < L->n_units; ++u) {
-        const int c = L->unit_cluster[u];
-        if (c < 0) { for (int v = u; v < L->n_units; ++v) if (L->unit_cluster[v] >= 0) return false; break; }
-        if (c < prev) return false;
-        prev = c;
-        ++n;
-    }
-    *n_used = n;
-    return true;
-}
-
 // head h's clusters hold exactly the channels h * hd .. (h + 1) * hd - 1 (the kernel reads a head's query slice by that rule)
 static bool kv_heads_own_their_channels(const rptq_layout_t* L, int H)
 {
     const int gh = L->g / H, hd = L->C / H;
-    size_t j = 0;
-    for (int c = 0; c < L->g; ++c)
-        for (int i = 0; i < L->size[(size_t)c]; ++i, ++j)
-            if (L->perm[j] / hd != c / gh) return false;
+    for (int c = 0; c < L->g; ++c) {
+        const size_t i = (size_t)c;
+        if (L->cl_ch_hi[i] >= 0 && (L->cl_ch_lo[i] / hd != c / gh || L->cl_ch_hi[i] / hd != c / gh)) return false;
+    }
     return true;
-}
-
-static int kv_max_units_per_head(const rptq_layout_t* L, int n_used, int H)
-{
-    const int gh = L->g / H;
-    std::vector<int> cnt((size_t)H, 0);
-    for (int u = 0; u < n_used; ++u) ++cnt[(size_t)(L->unit_cluster[u] / gh)];
-    int m = 0;
-    for (int c : cnt) m = c > m ? c : m;
-    return m;
 }
 
 extern "C" int rptq_attention_kv(const rptq_layout_t* LK, const rptq_layout_t* LV, int n_heads,
@@ -348,30 +261,34 @@ extern "C" int rptq_attention_kv(const rptq_layout_t* LK, const rptq_layout_t* L
     if (!aligned16(k_codes) || !aligned16(v_codes) || (reinterpret_cast<uintptr_t>(q_f16) & 1u) || (reinterpret_cast<uintptr_t>(out_f16) & 1u))
         return RPTQ_ERR_INVALID_ARG;
     if (n_heads > 65535 || n_seq > 65535) return RPTQ_ERR_UNSUPPORTED;
-    int n_used_k = 0, n_used_v = 0;
-    if (!kv_units_in_cluster_order(LK, &n_used_k) || !kv_units_in_cluster_order(LV, &n_used_v)) return RPTQ_ERR_UNSUPPORTED;
-    if (kv_max_units_per_head(LK, n_used_k, n_heads) > MAX_UNITS || kv_max_units_per_head(LV, n_used_v, n_heads) > MAX_UNITS) return RPTQ_ERR_UNSUPPORTED;
+    if (!LK->in_cluster_order || !LV->in_cluster_order) return RPTQ_ERR_UNSUPPORTED;
+    const int units_k = max_units_per_head(LK, n_heads), units_v = max_units_per_head(LV, n_heads);
+    if (units_k > MAX_UNITS || units_v > MAX_UNITS) return RPTQ_ERR_UNSUPPORTED;
     if (!kv_heads_own_their_channels(LK, n_heads)) return RPTQ_ERR_INVALID_ARG;
     if (Tq == 0 || n_seq == 0) return RPTQ_OK;
     int dev = -1;
     if (LK->device < 0 || cudaGetDevice(&dev) != cudaSuccess) return RPTQ_ERR_CUDA;
     if (dev != LK->device || dev != LV->device) return RPTQ_ERR_INVALID_ARG;
 
-    Params p{};
-    p.q = static_cast<const __half*>(q_f16); p.ldq = ldq;
+    AttnParams p{};
+    p.q_f16 = static_cast<const __half*>(q_f16); p.ldq = ldq;
     p.k = static_cast<const uint8_t*>(k_codes); p.v = static_cast<const uint8_t*>(v_codes);
     p.k_row_bytes = LK->row_bytes; p.v_row_bytes = LV->row_bytes; p.bits_k = LK->bits; p.bits_v = LV->bits;
     p.Tq = Tq; p.Tk = Tk; p.H = n_heads; p.hd = LK->C / n_heads; p.gh_k = LK->g / n_heads; p.gh_v = LV->g / n_heads; p.causal = causal ? 1 : 0;
-    p.n_used_k = n_used_k; p.n_used_v = n_used_v;
-    p.unit_cluster_k = LK->d_unit_cluster; p.unit_cluster_v = LV->d_unit_cluster;
+    p.cl_unit0_k = LK->d_cl_unit0; p.cl_unit0_v = LV->d_cl_unit0; p.unit_cluster_k = LK->d_unit_cluster;
     p.unit_sz_k = LK->d_unit_sz; p.unit_sz_v = LV->d_unit_sz;
     p.src_k = LK->d_src; p.src_v = LV->d_src; p.jidx_k = LK->d_jidx; p.jidx_v = LV->d_jidx;
     p.qk_scale_log2e = qk_scale * 1.4426950408889634f;
     p.out = static_cast<__half*>(out_f16); p.ldo = ldo;
 
+    auto st = static_cast<cudaStream_t>(stream);
+    int n_sm = 0;
+    if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return RPTQ_ERR_CUDA;
+    if (attn_decode::fits(p, true)) return attn_decode::launch(p, true, units_k, units_v, n_seq, n_sm, st);
+
     const int smem = (BM + 2 * BN) * PITCH;
     if (cudaFuncSetAttribute(attention_kv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return RPTQ_ERR_CUDA;
     const dim3 grid((unsigned)((Tq + BM - 1) / BM), (unsigned)n_heads, (unsigned)n_seq);
-    attention_kv_kernel<<<grid, THREADS, smem, static_cast<cudaStream_t>(stream)>>>(p);
+    attention_kv_kernel<<<grid, THREADS, smem, st>>>(p);
     return cudaGetLastError() == cudaSuccess ? RPTQ_OK : RPTQ_ERR_CUDA;
 }

@@ -1,0 +1,109 @@
+// Shared by the attention kernels: launch parameters, packed-row readers, small PTX wrappers, and the
+// host-side checks of per-head layouts.
+#pragma once
+#include <cuda_fp16.h>
+
+#include "rptq_internal.h"
+#include "unpack.cuh"
+
+namespace rptq {
+namespace attn {
+
+constexpr int MAX_UNITS = 8;                 // units of 32 positions per head
+constexpr float NEG_BIG = -1.0e30f;
+
+// One attention call. KV-only calls (rptq_attention_kv) have q_f16 and no q codes.
+struct AttnParams {
+    const uint8_t *q, *k, *v;
+    const __half* q_f16; int64_t ldq;
+    int64_t q_row_bytes, k_row_bytes, v_row_bytes;
+    int bits_q, bits_k, bits_v;
+    int Tq, Tk, H, hd, gh_k, gh_v, causal;   // Tq queries and Tk keys per sequence; hd channels per head (KV-only)
+    const int32_t *cl_unit0_k, *cl_unit0_v;  // first unit of every cluster, one past the last one's end
+    const int32_t *unit_cluster_k;
+    const float2 *unit_sz_q, *unit_sz_k, *unit_sz_v;
+    const uint16_t *src_k, *src_v;           // channel at each padded position
+    const int32_t *jidx_k, *jidx_v;          // -1 at pad positions
+    float inv_sP, s_P, qk_scale_log2e;
+    __half* out;
+    int64_t ldo;
+    uint8_t* p_dbg;
+};
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// 16 bytes global -> shared without passing through registers; src_bytes = 0 writes zeros
+__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int src_bytes)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
+__device__ __forceinline__ float ex2(float x)
+{
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ uint32_t pack_half2(float a, float b)
+{
+    const __half2 h = __floats2half2_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// Unit `unit` of a packed row in global memory as 32 bytes.
+__device__ __forceinline__ void load_unit(const uint8_t* row, int unit, int bits, uint32_t (&o)[8])
+{
+    if (bits == 4) {
+        const uint4 t = __ldg(reinterpret_cast<const uint4*>(row) + unit);
+        const uint32_t p[4] = {t.x, t.y, t.z, t.w};
+        unpack_act32<4>(p, o);
+    } else if (bits == 3) {
+        const uint32_t* w = reinterpret_cast<const uint32_t*>(row) + unit * 3;
+        const uint32_t p[3] = {__ldg(w), __ldg(w + 1), __ldg(w + 2)};
+        unpack_act32<3>(p, o);
+    } else {
+        const uint4* w = reinterpret_cast<const uint4*>(row) + unit * 2;
+        const uint4 a = __ldg(w), b = __ldg(w + 1);
+        o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
+    }
+}
+// The same from a staged copy of the packed row in shared memory (`row` points at the head's first unit;
+// 4-byte aligned for 3-bit codes, 16-byte aligned otherwise).
+__device__ __forceinline__ void load_unit_smem(const uint8_t* row, int unit, int bits, uint32_t (&o)[8])
+{
+    if (bits == 4) {
+        const uint4 t = *(reinterpret_cast<const uint4*>(row) + unit);
+        const uint32_t p[4] = {t.x, t.y, t.z, t.w};
+        unpack_act32<4>(p, o);
+    } else if (bits == 3) {
+        const uint32_t* w = reinterpret_cast<const uint32_t*>(row) + unit * 3;
+        const uint32_t p[3] = {w[0], w[1], w[2]};
+        unpack_act32<3>(p, o);
+    } else {
+        const uint4* w = reinterpret_cast<const uint4*>(row) + unit * 2;
+        const uint4 a = w[0], b = w[1];
+        o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
+    }
+}
+
+// Largest number of units a head takes in the layout (whose g clusters are n_heads equal groups).
+inline int max_units_per_head(const rptq_layout_t* L, int n_heads)
+{
+    const int gh = L->g / n_heads;
+    int m = 0;
+    for (int h = 0; h < n_heads; ++h) {
+        const int n = L->cl_unit0[(size_t)((h + 1) * gh)] - L->cl_unit0[(size_t)(h * gh)];
+        m = n > m ? n : m;
+    }
+    return m;
+}
+
+}  // namespace attn
+
+// The decode kernel (attention_decode.cu): few queries per sequence, the keys split over a cluster of blocks.
+namespace attn_decode {
+bool fits(const attn::AttnParams& p, bool kv);     // false: the prefill kernel takes the call
+int launch(const attn::AttnParams& p, bool kv, int units_k, int units_v, int n_seq, int n_sm, cudaStream_t st);
+}
+}  // namespace rptq

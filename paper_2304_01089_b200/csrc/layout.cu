@@ -253,6 +253,22 @@ int rptq_layout_create(rptq_layout_t** out, int C, int g, int bits, const int32_
             ui.nvalid = (n - 32 * uc) < 32 ? (n - 32 * uc) : 32;
         }
     }
+    // ---- what the attention entry points ask about per-head layouts on every call
+    L->in_cluster_order = true;
+    for (int u = 1; u < cur; ++u)
+        if (L->unit_cluster[u] < L->unit_cluster[u - 1]) { L->in_cluster_order = false; break; }
+    L->cl_unit0.assign((size_t)g + 1, 0);
+    L->cl_ch_lo.assign((size_t)g, C);
+    L->cl_ch_hi.assign((size_t)g, -1);
+    for (int c = 0; c < g; ++c) {
+        L->cl_unit0[c + 1] = L->cl_unit0[c] + n_units_of[c];
+        for (int i = 0; i < cluster_size[c]; ++i) {
+            const int ch = perm_host[j_start[c] + i];
+            L->cl_ch_lo[c] = std::min(L->cl_ch_lo[c], ch);
+            L->cl_ch_hi[c] = std::max(L->cl_ch_hi[c], ch);
+        }
+    }
+
     // ---- which channel of a cluster goes to which of the cluster's positions. All channels of a
     // cluster share (s_c, z_c), so any assignment is the same quantisation. rptq_ln_reorder_quant
     // gives every unit to one thread, and the 32 threads of a warp (32 consecutive units) read
@@ -312,6 +328,7 @@ int rptq_layout_create(rptq_layout_t** out, int C, int g, int bits, const int32_
         if (L->unit_cluster[u] >= 0) unit_sz[u] = make_float2(scale_host[L->unit_cluster[u]], (float)zero_host[L->unit_cluster[u]]);
     if (rc == RPTQ_OK) rc = upload(&L->d_unit_sz, unit_sz.data(), unit_sz.size());
     if (rc == RPTQ_OK) rc = upload(&L->d_unit_cluster, L->unit_cluster.data(), L->unit_cluster.size());
+    if (rc == RPTQ_OK) rc = upload(&L->d_cl_unit0, L->cl_unit0.data(), L->cl_unit0.size());
     if (rc != RPTQ_OK) { rptq_layout_destroy(L); return rc; }
     *out = L;
     return RPTQ_OK;
@@ -348,6 +365,7 @@ int rptq_layout_destroy(rptq_layout_t* L)
     cudaFree(L->d_seg_cluster);
     cudaFree(L->d_unit_sz);
     cudaFree(L->d_unit_cluster);
+    cudaFree(L->d_cl_unit0);
     delete L;
     return RPTQ_OK;
 }

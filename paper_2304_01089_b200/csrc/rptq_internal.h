@@ -40,6 +40,9 @@ struct rptq_layout {
     std::vector<int32_t> pos;            // [C]       padded position of reordered channel j
     std::vector<int32_t> unit_cluster;   // [n_units] owning cluster, -1 past the last cluster
     std::vector<float> scale;
+    bool in_cluster_order = false;       // the units' clusters never decrease along the row
+    std::vector<int32_t> cl_unit0;       // [g + 1] with in_cluster_order: first unit of each cluster, then the number of used units
+    std::vector<int32_t> cl_ch_lo, cl_ch_hi;   // [g] smallest and largest channel of each cluster (C, -1 when empty)
     // device tables
     uint16_t* d_src = nullptr;          // [K_pad] channel read for each padded position (at pads: some channel, the code is masked)
     int32_t* d_jidx = nullptr;          // [K_pad] reordered index at each padded position, -1 at pads
@@ -52,6 +55,7 @@ struct rptq_layout {
     int32_t* d_seg_cluster = nullptr;   // [n_seg]  the cluster of each entry of d_seg_scale
     float2* d_unit_sz = nullptr;        // [n_units] {s_c, (float) z_c} of the unit's cluster ({1, 0} where there is none)
     int32_t* d_unit_cluster = nullptr;  // [n_units]
+    int32_t* d_cl_unit0 = nullptr;      // [g + 1] cl_unit0
 };
 
 namespace rptq {

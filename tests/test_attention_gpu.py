@@ -288,3 +288,16 @@ def test_empty_and_oversized_calls():
     with pytest.raises(binding.RptqError) as e:      # more keys than the int32 sums of the second product can take
         binding.attention(c.LQ, c.LK, c.LV, 2, c.dq, c.dk, c.dv, out, c.s_P, c.qk_scale, True, Tq=8, Tk=40000)
     assert e.value.status == binding.ERR_UNSUPPORTED
+
+
+# The kernel for at most seven queries splits the keys over warps (tiles of 32 keys) and a cluster of blocks: sizes around a
+# tile, around four warps' tiles, an empty last block, eight blocks per head, every pair of code widths.
+@pytest.mark.parametrize("bits", [(4, 4, 4), (3, 3, 3), (8, 8, 8), (4, 8, 3), (8, 3, 8)])
+@pytest.mark.parametrize("Tq,Tk,causal", [(1, 31, True), (7, 33, True), (2, 128, False), (7, 1000, True), (1, 2500, True)])
+def test_few_queries(Tq, Tk, causal, bits):
+    Case(900 + Tk + 10 * bits[0] + bits[1], H=2, hd=72, gh=4, Tq=Tq, Tk=Tk, bits=bits).check(causal)
+
+
+def test_few_queries_of_many_heads_take_one_block_per_head():
+    """300 heads: no split of the keys."""
+    Case(950, H=300, hd=16, gh=4, Tq=3, Tk=40, bits=(4, 4, 4)).check(True)

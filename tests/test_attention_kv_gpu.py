@@ -156,3 +156,11 @@ def test_opt66b_heads_sampled_rows():
         got, w = o[i, chans[real]], want[0, :vs.stop - vs.start][real]
         vmax = float(c.sV[cl].max()) * 15
         assert np.all(np.abs(got - w) <= 2.0 ** -10 * vmax + 2.0 ** -11 * np.abs(w) + 1e-5 * vmax)
+
+
+# The kernel for at most eight queries: see test_attention_gpu.py::test_few_queries.
+@pytest.mark.parametrize("bits", [(4, 4, 4), (4, 3, 3), (4, 8, 8), (4, 8, 3), (4, 4, 8)])
+@pytest.mark.parametrize("Tq,Tk,n_seq,causal", [(1, 31, 1, True), (8, 33, 3, True), (2, 128, 1, False), (8, 1000, 1, True), (1, 2500, 2, True)])
+def test_few_queries(Tq, Tk, n_seq, causal, bits):
+    c = Case(900 + Tk + 10 * bits[1] + bits[2], H=2, hd=72, gh=4, Tq=Tq * n_seq, Tk=Tk * n_seq, bits=bits)
+    _check(c, _query(np.random.default_rng(3), Tq * n_seq, 144), causal, n_seq=n_seq)
