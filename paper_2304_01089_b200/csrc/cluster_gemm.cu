@@ -26,6 +26,10 @@
 //               interleaved unit order a small cluster's step sits between those of a large one,
 //               which keeps its buffer, so the small cluster's drain runs under the large
 //               cluster's remaining products
+//   warps 2-3   column tables: zero-point correction, s_w and bias of the columns of the tile to come, and
+//               with per-cluster weight parameters the coefficients of each cluster's drain (they are
+//               the same for every token row: formed once per block instead of in every epilogue thread.
+//               1024 x 4096 x 16384, 16 clusters: MEASURED_ASYM)
 //   warps 8-15  epilogue: drain a finished cluster's accumulator (tcgen05.ld), add s_c * acc into
 //               fp32 running sums held in registers while the next cluster's MMAs run; after the
 //               last cluster apply the zero-point correction, s_w, bias, activation, and store
@@ -44,6 +48,7 @@ namespace gemm {
 
 constexpr int TILE_M = 128, TILE_N = 256, KBLK = 128;   // TILE_M is per CTA
 constexpr int THREADS = 512;
+constexpr int TABLE_WARP0 = 2, N_TABLE_WARPS = 2;
 constexpr int UNPACK_WARP0 = 4, N_UNPACK_WARPS = 4;
 constexpr int EPI_WARP0 = 8, N_EPI_WARPS = 8;
 // registers per thread after the in-kernel re-partition (the block is launched with 128 each): the
@@ -65,9 +70,10 @@ __host__ __device__ constexpr int a_slot_pitch(int bits) { return bits == 3 ? 48
 __host__ __device__ constexpr int n_a_stages(int bits) { return bits == 8 ? 2 : 4; }
 
 struct SmemLayout {
-    int u_stage, p_stage, a_stage, off_p, off_a, off_flags, off_seg_scale, off_seg_buf, off_cl_sz, off_tab, off_bar, total;
+    int u_stage, p_stage, a_stage, off_p, off_a, off_flags, off_seg_scale, off_seg_buf, off_cl_sz, off_tab, off_seg_tab, off_seg_cl, off_bar, total;
 };
-__host__ __device__ constexpr SmemLayout smem_layout(int ncta, int bits, bool a8)
+constexpr int SEG_SLOTS = 2;                             // ASYM: clusters whose column tables are held at a time
+__host__ __device__ constexpr SmemLayout smem_layout(int ncta, int bits, bool a8, bool asym)
 {
     SmemLayout s{};
     s.u_stage = A8_BYTES + w_rows(ncta) * KBLK;
@@ -80,8 +86,10 @@ __host__ __device__ constexpr SmemLayout smem_layout(int ncta, int bits, bool a8
     s.off_seg_buf = s.off_seg_scale + kMaxGemmSegments * 4;
     s.off_cl_sz = s.off_seg_buf + kMaxGemmSegments;
     s.off_tab = s.off_cl_sz + kMaxGemmSegments * 4;
-    s.off_bar = s.off_tab + 2 * 3 * TILE_N * 4;
-    s.total = s.off_bar + 256;
+    s.off_seg_tab = s.off_tab + 2 * 3 * TILE_N * 4;
+    s.off_seg_cl = s.off_seg_tab + (asym ? SEG_SLOTS * 2 * TILE_N * 4 : 0);
+    s.off_bar = s.off_seg_cl + (asym ? kMaxGemmSegments * 2 : 0);
+    s.total = s.off_bar + 320;
     return s;
 }
 
@@ -390,7 +398,7 @@ cluster_gemm_kernel(const Params p)
     constexpr bool ASYM = MODE == MODE_ASYM, DEQ = MODE == MODE_DEQ;
     static_assert(!(DEQ && A8), "the de-quantising variant unpacks every bit width");
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    constexpr SmemLayout SL = smem_layout(NCTA, BITS, A8);
+    constexpr SmemLayout SL = smem_layout(NCTA, BITS, A8, ASYM);
     constexpr int W_ROWS = w_rows(NCTA);                 // weight rows this CTA stages and unpacks
     constexpr int N_P = n_p_stages(NCTA, BITS), N_U = n_u_stages(NCTA, A8);
     constexpr uint32_t kInstrDesc = DEQ ? instr_desc_bf16(NCTA) : instr_desc(NCTA);
@@ -404,12 +412,14 @@ cluster_gemm_kernel(const Params p)
     uint8_t* s_seg_buf = smem + SL.off_seg_buf;
     float* s_cl_sz = reinterpret_cast<float*>(smem + SL.off_cl_sz);
     float* s_tab = reinterpret_cast<float*>(smem + SL.off_tab);           // [2][3][TILE_N]
+    float4* s_seg_tab = reinterpret_cast<float4*>(smem + SL.off_seg_tab); // ASYM: [SEG_SLOTS][TILE_N / 2]
+    uint16_t* s_seg_cl = reinterpret_cast<uint16_t*>(smem + SL.off_seg_cl);   // ASYM: the cluster of each segment
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SL.off_bar);
     // barrier indices
     constexpr int B_PFULL = 0, B_PEMPTY = B_PFULL + N_P, B_UFULL = B_PEMPTY + N_P, B_UEMPTY = B_UFULL + N_U,
-                  B_ACCFULL = B_UEMPTY + N_U, B_ACCEMPTY = B_ACCFULL + 2, B_TAB = B_ACCEMPTY + 2, B_DRAIN = B_TAB + 2,
-                  N_BARS = B_DRAIN + 1;
-    static_assert(N_BARS * 8 + 16 <= 256, "barrier block too small");
+                  B_ACCFULL = B_UEMPTY + N_U, B_ACCEMPTY = B_ACCFULL + 2, B_TAB = B_ACCEMPTY + 2, B_TABEMPTY = B_TAB + 2,
+                  B_SEGFULL = B_TABEMPTY + 2, B_SEGEMPTY = B_SEGFULL + SEG_SLOTS, B_DRAIN = B_SEGEMPTY + SEG_SLOTS, N_BARS = B_DRAIN + 1;
+    static_assert(N_BARS * 8 + 16 <= 320, "barrier block too small");
     uint32_t* s_tmem_ptr = reinterpret_cast<uint32_t*>(bars + N_BARS);
     volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem_ptr + 1);
     const uint32_t bar0 = smem_u32(bars);
@@ -426,8 +436,10 @@ cluster_gemm_kernel(const Params p)
         for (int i = 0; i < N_P; ++i) { mbar_init(bar(B_PFULL + i), 1); mbar_init(bar(B_PEMPTY + i), N_UNPACK_WARPS); }
         for (int i = 0; i < N_U; ++i) { mbar_init(bar(B_UFULL + i), N_UNPACK_WARPS * NCTA); mbar_init(bar(B_UEMPTY + i), 1); }
         for (int i = 0; i < 2; ++i) {
-            mbar_init(bar(B_ACCFULL + i), 1); mbar_init(bar(B_ACCEMPTY + i), N_EPI_WARPS * NCTA); mbar_init(bar(B_TAB + i), N_EPI_WARPS);
+            mbar_init(bar(B_ACCFULL + i), 1); mbar_init(bar(B_ACCEMPTY + i), N_EPI_WARPS * NCTA); mbar_init(bar(B_TAB + i), N_TABLE_WARPS);
+            mbar_init(bar(B_TABEMPTY + i), N_EPI_WARPS);
         }
+        for (int i = 0; i < SEG_SLOTS; ++i) { mbar_init(bar(B_SEGFULL + i), N_TABLE_WARPS); mbar_init(bar(B_SEGEMPTY + i), N_EPI_WARPS); }
         mbar_init(bar(B_DRAIN), 1);
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -435,6 +447,7 @@ cluster_gemm_kernel(const Params p)
     for (int i = tid; i < n_steps; i += THREADS) s_flags[i] = p.step_flags[i];
     for (int i = tid; i < p.n_seg; i += THREADS) { s_seg_scale[i] = p.seg_scale[i] * 0.0625f; s_seg_buf[i] = p.seg_buf[i]; }   // operands were 16 * w
     for (int i = tid; i < p.g; i += THREADS) s_cl_sz[i] = p.cl_sz[i];
+    if constexpr (ASYM) for (int i = tid; i < p.n_seg; i += THREADS) s_seg_cl[i] = (uint16_t)p.seg_cluster[i];
     if (warp == 1) {
         if constexpr (NCTA == 1) {
             asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(s_tmem_ptr)) : "memory");
@@ -575,7 +588,79 @@ cluster_gemm_kernel(const Params p)
                 mbar_wait(bar(B_DRAIN), 0, s_abort, false);
             }
         }
-      }   // warps 2 and 3 only fill the first warpgroup
+      } else {
+        // ------------------------------------------------------------ column tables
+        // Thread tt prepares columns 4 tt .. 4 tt + 3 of the tile ahead of the epilogue: the zero-point
+        // correction, s_w and the bias of every tile, and with ASYM for every cluster of the tile the two
+        // coefficients its drain needs per column.
+        const int tt = tid - TABLE_WARP0 * 32;
+        uint32_t n_tile = 0, n_seg_done = 0;
+        bool ok = true;
+        for (int t = pair_id; t < p.n_tiles && ok; t += n_pairs, ++n_tile) {
+            const int n = (t / p.tiles_m) * TILE_N + 4 * tt;
+            const bool vec = (p.ld_w & 3) == 0 && n + 4 <= p.ld_w;
+            float corr[4] = {0.f, 0.f, 0.f, 0.f};
+            if constexpr (ASYM) {
+                // y += s^X_c s^W_c[n] / 16 * (acc' + Z xsum), Z = -16 (z^W_c[n] - 8); the tile constant is
+                // sum_c s^X_c z^X_c s^W_c[n] (Wsum_c[n] - n_c z^W_c[n])
+                for (int sgi = 0; sgi < p.n_seg; ++sgi, ++n_seg_done) {
+                    const int cid = s_seg_cl[sgi];
+                    const int64_t i = (int64_t)cid * p.ld_w + n;
+                    float4 sw4 = make_float4(0.f, 0.f, 0.f, 0.f);
+                    int4 zw4 = make_int4(8, 8, 8, 8), ws4 = make_int4(0, 0, 0, 0);
+                    if (vec) {
+                        sw4 = __ldg(reinterpret_cast<const float4*>(p.sw_c + i));
+                        zw4 = __ldg(reinterpret_cast<const int4*>(p.zw_c + i));
+                        ws4 = __ldg(reinterpret_cast<const int4*>(p.wsum + i));
+                    }
+                    const float sz = s_cl_sz[cid], nc = __ldg(p.cl_n + cid), sc = s_seg_scale[sgi];
+                    corr[0] = __fmaf_rn(sz * sw4.x, (float)ws4.x - nc * (float)zw4.x, corr[0]);
+                    corr[1] = __fmaf_rn(sz * sw4.y, (float)ws4.y - nc * (float)zw4.y, corr[1]);
+                    corr[2] = __fmaf_rn(sz * sw4.z, (float)ws4.z - nc * (float)zw4.z, corr[2]);
+                    corr[3] = __fmaf_rn(sz * sw4.w, (float)ws4.w - nc * (float)zw4.w, corr[3]);
+                    const uint32_t sl = n_seg_done % SEG_SLOTS;
+                    if (!mbar_wait(bar(B_SEGEMPTY + sl), ((n_seg_done / SEG_SLOTS) & 1) ^ 1, s_abort)) { ok = false; break; }
+                    float4* d = s_seg_tab + sl * (TILE_N / 2) + 2 * tt;
+                    d[0] = make_float4(sc * sw4.x, sc * sw4.y, (float)(128 - 16 * zw4.x), (float)(128 - 16 * zw4.y));
+                    d[1] = make_float4(sc * sw4.z, sc * sw4.w, (float)(128 - 16 * zw4.z), (float)(128 - 16 * zw4.w));
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(B_SEGFULL + sl));
+                }
+                if (!ok) break;
+            } else if constexpr (!DEQ) {
+                if (p.corr) {
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) if (n + e < p.N) corr[e] = __ldg(p.corr + n + e);
+                } else if (vec) {
+#pragma unroll 4
+                    for (int c = 0; c < p.g; ++c) {
+                        const int4 ws = __ldg(reinterpret_cast<const int4*>(p.wsum + (int64_t)c * p.ld_w + n));
+                        const float sz = s_cl_sz[c];
+                        corr[0] = __fmaf_rn(sz, (float)ws.x, corr[0]); corr[1] = __fmaf_rn(sz, (float)ws.y, corr[1]);
+                        corr[2] = __fmaf_rn(sz, (float)ws.z, corr[2]); corr[3] = __fmaf_rn(sz, (float)ws.w, corr[3]);
+                    }
+                } else {
+                    for (int c = 0; c < p.g; ++c) {
+                        const float sz = s_cl_sz[c];
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) if (n + e < p.N) corr[e] = __fmaf_rn(sz, (float)__ldg(p.wsum + (int64_t)c * p.ld_w + n + e), corr[e]);
+                    }
+                }
+            }
+            const uint32_t b = n_tile & 1;
+            if (!mbar_wait(bar(B_TABEMPTY + b), ((n_tile >> 1) & 1) ^ 1, s_abort)) break;
+            float* tab = s_tab + b * 3 * TILE_N + 4 * tt;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                const bool in = n + e < p.N;
+                // ASYM: the column's scale is applied per cluster; DEQ: the weight operands were 16 w, zero points are in X^
+                const float sw = !in ? 0.f : ASYM ? 1.f : DEQ ? __ldg(p.s_w + n + e) * 0.0625f : __ldg(p.s_w + n + e);
+                tab[e] = corr[e]; tab[TILE_N + e] = sw; tab[2 * TILE_N + e] = in && p.bias ? __ldg(p.bias + n + e) : 0.f;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(B_TAB + b));
+        }
+      }
     } else if (warp < EPI_WARP0) {
         // ------------------------------------------------------------ unpack warps
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_UNPACK));
@@ -813,10 +898,10 @@ cluster_gemm_kernel(const Params p)
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_EPI));
         const int ew = warp - EPI_WARP0;
         const int q = ew & 3, h = ew >> 2;           // TMEM lane quarter (= warp % 4), column half
-        const int et = ew * 32 + lane;               // 0..255: the column whose tile constants I prepare
         uint32_t n_tile_done = 0;
         uint32_t par = 0;                    // bit b: parity of how many clusters of accumulator b I have drained
         bool ok = true;
+        uint32_t n_seg_done = 0;                     // ASYM: clusters drained so far, over all tiles
         float2 R[64];                                // running sums of columns 2 i, 2 i + 1
         for (int t = pair_id; t < p.n_tiles && ok; t += n_pairs, ++n_tile_done) {
             const int m0 = (t % p.tiles_m) * (TILE_M * NCTA) + (int)cta_rank * TILE_M, n0 = (t / p.tiles_m) * TILE_N;
@@ -824,33 +909,14 @@ cluster_gemm_kernel(const Params p)
             // a warp whose 32 accumulator lanes all lie beyond the last token row keeps the barriers'
             // protocol but reads and accumulates nothing (few-token calls: most of the tile is empty)
             const bool live = m0 + 32 * q < p.M;
-            {   // per-tile column constants: zero-point correction sum_c s_c z_c Wsum_c[n], s_w[n], bias[n]
-                const int n = n0 + et;
-                float corr = 0.f, sw = 0.f, bs = 0.f;
-                if (n < p.N) {
-                    if constexpr (ASYM) {
-                        // sum_c s^X_c z^X_c s^W_c[n] (Wsum_c[n] - n_c z^W_c[n]); the column's scale is applied per cluster
-                        for (int c = 0; c < p.g; ++c) {
-                            const int64_t i = (int64_t)c * p.ld_w + n;
-                            const float t = (float)__ldg(p.wsum + i) - __ldg(p.cl_n + c) * (float)__ldg(p.zw_c + i);
-                            corr = __fmaf_rn(s_cl_sz[c] * __ldg(p.sw_c + i), t, corr);
-                        }
-                        sw = 1.0f;
-                    } else if constexpr (DEQ) {
-                        sw = __ldg(p.s_w + n) * 0.0625f;             // the weight operands were 16 w; zero points are in X^
-                    } else {
-                        if (p.corr) corr = __ldg(p.corr + n);
-                        else for (int c = 0; c < p.g; ++c) corr = __fmaf_rn(s_cl_sz[c], (float)__ldg(p.wsum + (int64_t)c * p.ld_w + n), corr);
-                        sw = __ldg(p.s_w + n);
-                    }
-                    bs = p.bias ? __ldg(p.bias + n) : 0.f;
-                }
-                tab[et] = corr; tab[TILE_N + et] = sw; tab[2 * TILE_N + et] = bs;
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar(B_TAB + (n_tile_done & 1)));
-            }
 #pragma unroll
             for (int i = 0; i < 64; ++i) R[i] = make_float2(0.f, 0.f);
+            // ASYM: my token's code sum of the cluster to come
+            const int32_t* xs_row = nullptr;
+            int xs_next = 0;
+            if constexpr (ASYM) {
+                if (m0 + 32 * q + lane < p.M) { xs_row = p.xsum + (int64_t)(m0 + 32 * q + lane) * p.g; xs_next = __ldg(xs_row + s_seg_cl[0]); }
+            }
             for (int sgi = 0; sgi < (DEQ ? 1 : p.n_seg); ++sgi) {
                 const uint32_t buf = DEQ ? (n_tile_done & 1u) : (uint32_t)s_seg_buf[sgi];
                 if (!mbar_wait(bar(B_ACCFULL + buf), (par >> buf) & 1u, s_abort)) { ok = false; break; }
@@ -858,42 +924,29 @@ cluster_gemm_kernel(const Params p)
                 tc_fence_after();
                 const float sc = s_seg_scale[sgi];
                 const float2 sc2 = make_float2(sc, sc);
+                const uint32_t seg_slot = n_seg_done % SEG_SLOTS;
+                const float4* seg_tab = s_seg_tab + seg_slot * (TILE_N / 2) + h * 64;
+                float2 xs2 = make_float2(0.f, 0.f);
+                if constexpr (ASYM) {
+                    if (!mbar_wait(bar(B_SEGFULL + seg_slot), (n_seg_done / SEG_SLOTS) & 1, s_abort)) { ok = false; break; }
+                    ++n_seg_done;
+                    const float x = (float)xs_next;
+                    xs2 = make_float2(x, x);
+                    if (xs_row && sgi + 1 < p.n_seg) xs_next = __ldg(xs_row + s_seg_cl[sgi + 1]);
+                }
                 const uint32_t taddr = tmem_base + ((uint32_t)(32 * q) << 16) + buf * TILE_N + h * 128;
                 if (live) {
                 uint32_t va[16], vb[16];
                 tc_ld16(taddr, va);
-                // ASYM: this cluster's row of the weight tables and my token's code sum
-                int64_t tab_row = 0;
-                float xs = 0.f, sx = 0.f;
-                if constexpr (ASYM) {
-                    const int cid = __ldg(p.seg_cluster + sgi);
-                    const int m_row = m0 + 32 * q + lane;
-                    tab_row = (int64_t)cid * p.ld_w + n0 + h * 128;
-                    xs = m_row < p.M ? (float)__ldg(p.xsum + (int64_t)m_row * p.g + cid) : 0.f;
-                    sx = sc * 16.0f;                 // s^X_c itself (s_seg_scale carries the 1/16 of the operands)
-                }
                 // R += s_c * acc, two columns per packed fused multiply-add
                 auto accumulate = [&](const uint32_t (&v)[16], int c0) {
                     if constexpr (ASYM) {
-                        // R += s^X_c s^W_c[n] (acc' - (z^W_c[n] - 8) xsum): 16 columns, the tables four at a time
-                        const int col = 2 * c0;                      // first of these columns within my 128
+                        // R += s^X_c s^W_c[n] / 16 (acc' - 16 (z^W_c[n] - 8) xsum), coefficients of two columns per load
 #pragma unroll
-                        for (int i4 = 0; i4 < 4; ++i4) {
-                            float sw4[4] = {0.f, 0.f, 0.f, 0.f};
-                            int zw4[4] = {8, 8, 8, 8};
-                            if (n0 + h * 128 + col + 4 * i4 + 4 <= p.ld_w) {
-                                const float4 a = __ldg(reinterpret_cast<const float4*>(p.sw_c + tab_row + col + 4 * i4));
-                                const int4 b = __ldg(reinterpret_cast<const int4*>(p.zw_c + tab_row + col + 4 * i4));
-                                sw4[0] = a.x; sw4[1] = a.y; sw4[2] = a.z; sw4[3] = a.w;
-                                zw4[0] = b.x; zw4[1] = b.y; zw4[2] = b.z; zw4[3] = b.w;
-                            }
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                const int i = 4 * i4 + e;
-                                const float t = __fmaf_rn((float)(int)v[i], 0.0625f, -(float)(zw4[e] - 8) * xs);
-                                float& r = (i & 1) ? R[c0 + (i >> 1)].y : R[c0 + (i >> 1)].x;
-                                r = __fmaf_rn(sx * sw4[e], t, r);
-                            }
+                        for (int i = 0; i < 8; ++i) {
+                            const float4 k = seg_tab[c0 + i];
+                            const float2 t = fma2(make_float2(k.z, k.w), xs2, make_float2((float)(int)v[2 * i], (float)(int)v[2 * i + 1]));
+                            R[c0 + i] = fma2(make_float2(k.x, k.y), t, R[c0 + i]);
                         }
                     } else if constexpr (DEQ) {
 #pragma unroll
@@ -916,7 +969,10 @@ cluster_gemm_kernel(const Params p)
                 }
                 tc_fence_before();
                 __syncwarp();
-                if (lane == 0) arrive_leader(bar(B_ACCEMPTY + buf));
+                if (lane == 0) {
+                    if constexpr (ASYM) mbar_arrive(bar(B_SEGEMPTY + seg_slot));
+                    arrive_leader(bar(B_ACCEMPTY + buf));
+                }
             }
             if (!ok) break;
             if (!mbar_wait(bar(B_TAB + (n_tile_done & 1)), (n_tile_done >> 1) & 1, s_abort)) { ok = false; break; }
@@ -935,6 +991,8 @@ cluster_gemm_kernel(const Params p)
                     Rf(i) = v;
                 }
             }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(bar(B_TABEMPTY + (n_tile_done & 1)));
             if (m < p.M) {
                 if (p.y_dtype == RPTQ_OUT_F32) {
                     float* dst = static_cast<float*>(p.y) + (int64_t)m * p.ldy + nb;
@@ -1009,7 +1067,7 @@ cluster_gemm_kernel(const Params p)
 template <int BITS, int NCTA, bool A8, int MODE>
 static int launch(const Params& p, int n_sm, cudaStream_t st)
 {
-    constexpr SmemLayout SL = smem_layout(NCTA, BITS, A8);
+    constexpr SmemLayout SL = smem_layout(NCTA, BITS, A8, MODE == MODE_ASYM);
     const int smem = SL.total + 1024;     // slack for the in-kernel 1024-byte alignment
     const void* fn = reinterpret_cast<const void*>(cluster_gemm_kernel<BITS, NCTA, A8, MODE>);
     cudaFuncAttributes attr;
