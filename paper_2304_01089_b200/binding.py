@@ -108,10 +108,21 @@ def _dev_ptr(t) -> Optional[int]:
     return t.data_ptr()
 
 
+_current_raw_stream = None       # () -> cudaStream_t of the calling thread's current stream
+
+
 def _stream_ptr(stream) -> Optional[int]:
+    global _current_raw_stream
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        if _current_raw_stream is None:
+            import torch
+            raw, device = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+            if raw is not None and device is not None:
+                torch.cuda.init()
+                _current_raw_stream = lambda: raw(device())     # without the Stream object: 4 us less per call
+            else:
+                _current_raw_stream = lambda: torch.cuda.current_stream().cuda_stream
+        return _current_raw_stream()
     return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
 
 

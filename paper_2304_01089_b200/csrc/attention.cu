@@ -56,6 +56,8 @@ attention_kernel(const AttnParams p, const int raw_pitch)
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g8 = lane >> 2, t4 = lane & 3;
     const int h = blockIdx.y;
+    pdl_trigger();
+    pdl_wait();
     const int64_t q_row0 = (int64_t)blockIdx.z * p.Tq, k_row0 = (int64_t)blockIdx.z * p.Tk;      // this sequence's first rows
     const int qt = (int)gridDim.x - 1 - (int)blockIdx.x;      // the tiles with the most visible keys first
     const int i0 = qt * BM;
@@ -347,15 +349,15 @@ extern "C" int rptq_attention(const rptq_layout_t* LQ, const rptq_layout_t* LK, 
     p.out = static_cast<__half*>(out_f16); p.ldo = ldo; p.p_dbg = p_codes_out;
 
     auto st = static_cast<cudaStream_t>(stream);
-    int n_sm = 0;
-    if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return RPTQ_ERR_CUDA;
-    if (attn_decode::fits(p, false)) return attn_decode::launch(p, false, units_k, units_v, n_seq, n_sm, st);
+    const int n_sm = sm_count(dev);
+    if (n_sm == 0) return RPTQ_ERR_CUDA;
+    if (attn_decode::fits(p, false)) return attn_decode::launch(p, false, units_k, units_v, n_seq, dev, n_sm, st);
 
     const int max_bits = LK->bits > LV->bits ? LK->bits : LV->bits;
     const int raw_pitch = 4 * max_bits * MAX_UNITS + 32;          // a head's packed codes plus the alignment slack, a multiple of 16
     const int smem = (BM + BN) * QK_PITCH_MAX + 32 * V_CHUNK_UNITS * VT_PITCH + 4 * BN * raw_pitch;
-    if (cudaFuncSetAttribute(attention_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return RPTQ_ERR_CUDA;
+    static std::atomic<uint64_t> done{0};
+    if (allow_smem(reinterpret_cast<const void*>(attention_kernel), dev, 220 * 1024, done) != RPTQ_OK) return RPTQ_ERR_CUDA;
     const dim3 grid((unsigned)((Tq + BM - 1) / BM), (unsigned)n_heads, (unsigned)n_seq);
-    attention_kernel<<<grid, THREADS, smem, st>>>(p, raw_pitch);
-    return cudaGetLastError() == cudaSuccess ? RPTQ_OK : RPTQ_ERR_CUDA;
+    return launch_kernel(attention_kernel, grid, THREADS, (size_t)smem, 0, st, p, raw_pitch);
 }

@@ -209,6 +209,8 @@ decode_kernel(const AttnParams p, int keys_block, int units_k_max, int units_v_m
         __syncwarp();
     };
 
+    pdl_trigger();
+    pdl_wait();
     const int pk = raw_pitch(p.bits_k, units_k_max), pv = raw_pitch(p.bits_v, units_v_max);
 #pragma unroll 1
     for (int i = 0; i < STAGES - 1; ++i) stage_tile(i, p.k, p.k_row_bytes, p.bits_k, uk0, nuk, pk);
@@ -702,31 +704,23 @@ bool fits(const AttnParams& p, bool kv)
 }
 
 template <int MODE, int BK, int BV>
-static int launch_one(const AttnParams& p, int units_k, int units_v, int n_seq, int n_sm, cudaStream_t st)
+static int launch_one(const AttnParams& p, int units_k, int units_v, int n_seq, int dev, int n_sm, cudaStream_t st)
 {
     int n_ranks = 1, keys_block = 0, smem = 0;
     if (!plan(p, MODE == HALF, units_k, units_v, n_seq, n_sm, &n_ranks, &keys_block, &smem)) return RPTQ_ERR_UNSUPPORTED;
-    if (cudaFuncSetAttribute(decode_kernel<MODE, BK, BV>, cudaFuncAttributeMaxDynamicSharedMemorySize, 212 * 1024) != cudaSuccess) return RPTQ_ERR_CUDA;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)n_ranks, (unsigned)p.H, (unsigned)n_seq);
-    cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)n_ranks; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, decode_kernel<MODE, BK, BV>, p, keys_block, units_k, units_v) == cudaSuccess ? RPTQ_OK : RPTQ_ERR_CUDA;
+    static std::atomic<uint64_t> done{0};
+    if (allow_smem(reinterpret_cast<const void*>(decode_kernel<MODE, BK, BV>), dev, 212 * 1024, done) != RPTQ_OK) return RPTQ_ERR_CUDA;
+    return launch_kernel(decode_kernel<MODE, BK, BV>, dim3((unsigned)n_ranks, (unsigned)p.H, (unsigned)n_seq), THREADS, (size_t)smem, (unsigned)n_ranks, st,
+                         p, keys_block, units_k, units_v);
 }
 
-int launch(const AttnParams& p, bool kv, int units_k, int units_v, int n_seq, int n_sm, cudaStream_t st)
+int launch(const AttnParams& p, bool kv, int units_k, int units_v, int n_seq, int dev, int n_sm, cudaStream_t st)
 {
     const bool k8 = p.bits_k == 8, v8 = p.bits_v == 8;
     auto pick = [&](auto mode) {
         constexpr int MODE = decltype(mode)::value;
-        if (k8) return v8 ? launch_one<MODE, 8, 8>(p, units_k, units_v, n_seq, n_sm, st) : launch_one<MODE, 8, 4>(p, units_k, units_v, n_seq, n_sm, st);
-        return v8 ? launch_one<MODE, 4, 8>(p, units_k, units_v, n_seq, n_sm, st) : launch_one<MODE, 4, 4>(p, units_k, units_v, n_seq, n_sm, st);
+        if (k8) return v8 ? launch_one<MODE, 8, 8>(p, units_k, units_v, n_seq, dev, n_sm, st) : launch_one<MODE, 8, 4>(p, units_k, units_v, n_seq, dev, n_sm, st);
+        return v8 ? launch_one<MODE, 4, 8>(p, units_k, units_v, n_seq, dev, n_sm, st) : launch_one<MODE, 4, 4>(p, units_k, units_v, n_seq, dev, n_sm, st);
     };
     if (!kv) return pick(std::integral_constant<int, INT>());
     return p.Tq <= LIMB_Q ? pick(std::integral_constant<int, LIMB>()) : pick(std::integral_constant<int, HALF>());

@@ -68,6 +68,8 @@ attention_kv_kernel(const AttnParams p)
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g8 = lane >> 2, t4 = lane & 3;
     const int h = blockIdx.y;
+    pdl_trigger();
+    pdl_wait();
     const int64_t q_row0 = (int64_t)blockIdx.z * p.Tq, k_row0 = (int64_t)blockIdx.z * p.Tk;
     const int qt = (int)gridDim.x - 1 - (int)blockIdx.x;      // the tiles with the most visible keys first
     const int i0 = qt * BM;
@@ -282,13 +284,13 @@ extern "C" int rptq_attention_kv(const rptq_layout_t* LK, const rptq_layout_t* L
     p.out = static_cast<__half*>(out_f16); p.ldo = ldo;
 
     auto st = static_cast<cudaStream_t>(stream);
-    int n_sm = 0;
-    if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return RPTQ_ERR_CUDA;
-    if (attn_decode::fits(p, true)) return attn_decode::launch(p, true, units_k, units_v, n_seq, n_sm, st);
+    const int n_sm = sm_count(dev);
+    if (n_sm == 0) return RPTQ_ERR_CUDA;
+    if (attn_decode::fits(p, true)) return attn_decode::launch(p, true, units_k, units_v, n_seq, dev, n_sm, st);
 
     const int smem = (BM + 2 * BN) * PITCH;
-    if (cudaFuncSetAttribute(attention_kv_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return RPTQ_ERR_CUDA;
+    static std::atomic<uint64_t> done{0};
+    if (allow_smem(reinterpret_cast<const void*>(attention_kv_kernel), dev, 220 * 1024, done) != RPTQ_OK) return RPTQ_ERR_CUDA;
     const dim3 grid((unsigned)((Tq + BM - 1) / BM), (unsigned)n_heads, (unsigned)n_seq);
-    attention_kv_kernel<<<grid, THREADS, smem, st>>>(p);
-    return cudaGetLastError() == cudaSuccess ? RPTQ_OK : RPTQ_ERR_CUDA;
+    return launch_kernel(attention_kv_kernel, grid, THREADS, (size_t)smem, 0, st, p);
 }

@@ -104,6 +104,6 @@ inline int max_units_per_head(const rptq_layout_t* L, int n_heads)
 // The decode kernel (attention_decode.cu): few queries per sequence, the keys split over a cluster of blocks.
 namespace attn_decode {
 bool fits(const attn::AttnParams& p, bool kv);     // false: the prefill kernel takes the call
-int launch(const attn::AttnParams& p, bool kv, int units_k, int units_v, int n_seq, int n_sm, cudaStream_t st);
+int launch(const attn::AttnParams& p, bool kv, int units_k, int units_v, int n_seq, int dev, int n_sm, cudaStream_t st);
 }
 }  // namespace rptq

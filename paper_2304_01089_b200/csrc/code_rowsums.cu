@@ -15,6 +15,8 @@ code_rowsums_kernel(const uint8_t* __restrict__ codes, int64_t row_bytes, int n_
 {
     extern __shared__ int32_t s_sum[];
     for (int c = threadIdx.x; c < g; c += blockDim.x) s_sum[c] = 0;
+    pdl_trigger();
+    pdl_wait();
     __syncthreads();
     const uint32_t* row = reinterpret_cast<const uint32_t*>(codes + (int64_t)blockIdx.x * row_bytes);
     for (int u = threadIdx.x; u < n_units; u += blockDim.x) {
@@ -48,8 +50,7 @@ extern "C" int rptq_code_rowsums(const rptq_layout_t* L, const void* codes, int 
     auto st = static_cast<cudaStream_t>(stream);
     const size_t smem = sizeof(int32_t) * (size_t)L->g;
     const uint8_t* c = static_cast<const uint8_t*>(codes);
-    if (L->bits == 3) code_rowsums_kernel<3><<<M, 128, smem, st>>>(c, L->row_bytes, L->n_units, L->d_unit_cluster, L->g, xsum);
-    else if (L->bits == 4) code_rowsums_kernel<4><<<M, 128, smem, st>>>(c, L->row_bytes, L->n_units, L->d_unit_cluster, L->g, xsum);
-    else code_rowsums_kernel<8><<<M, 128, smem, st>>>(c, L->row_bytes, L->n_units, L->d_unit_cluster, L->g, xsum);
-    return cudaGetLastError() == cudaSuccess ? RPTQ_OK : RPTQ_ERR_CUDA;
+    if (L->bits == 3) return launch_kernel(code_rowsums_kernel<3>, dim3((unsigned)M), 128, smem, 0, st, c, L->row_bytes, L->n_units, (const int32_t*)L->d_unit_cluster, L->g, xsum);
+    if (L->bits == 4) return launch_kernel(code_rowsums_kernel<4>, dim3((unsigned)M), 128, smem, 0, st, c, L->row_bytes, L->n_units, (const int32_t*)L->d_unit_cluster, L->g, xsum);
+    return launch_kernel(code_rowsums_kernel<8>, dim3((unsigned)M), 128, smem, 0, st, c, L->row_bytes, L->n_units, (const int32_t*)L->d_unit_cluster, L->g, xsum);
 }

@@ -16,20 +16,33 @@ namespace rptq {
 // up a wait writes to the word of the device it runs on.
 constexpr int kMaxDevices = 64;
 static std::mutex g_status_mutex;
-static int* g_status_word[kMaxDevices] = {};
+static std::atomic<int*> g_status_word[kMaxDevices] = {};
 
 int* device_status_word()
 {
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
+    if (int* p = g_status_word[dev].load(std::memory_order_acquire)) return p;
     std::lock_guard<std::mutex> lock(g_status_mutex);
-    if (g_status_word[dev] == nullptr) {
-        int* p = nullptr;
+    int* p = g_status_word[dev].load(std::memory_order_acquire);
+    if (p == nullptr) {
         if (cudaMalloc(&p, 256) != cudaSuccess) return nullptr;
         if (cudaMemset(p, 0, 256) != cudaSuccess) { cudaFree(p); return nullptr; }
-        g_status_word[dev] = p;
+        g_status_word[dev].store(p, std::memory_order_release);
     }
-    return g_status_word[dev];
+    return p;
+}
+
+int sm_count(int device)
+{
+    static std::atomic<int> count[kMaxDevices] = {};
+    if (device < 0 || device >= kMaxDevices) return 0;
+    int n = count[device].load(std::memory_order_relaxed);
+    if (n == 0) {
+        if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return 0;
+        count[device].store(n, std::memory_order_relaxed);
+    }
+    return n;
 }
 
 template <class T>

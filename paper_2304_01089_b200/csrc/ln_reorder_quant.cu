@@ -170,6 +170,8 @@ ln_reorder_quant_kernel(const LnParams p)
         *reinterpret_cast<uint4*>(zero16) = make_uint4(0u, 0u, 0u, 0u);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    pdl_trigger();
+    pdl_wait();
     // Gains and biases pass through the last two ring slots (coalesced loads) so that the gather
     // threads can pick their own channels' values from shared memory; scattered 2-byte global loads
     // for 64 values per thread would cost more than a few hundred rows of the kernel proper. The
@@ -498,8 +500,7 @@ static int launch_ln(const rptq_layout_t* L, const void* x, int64_t ldx, const v
         if (cudaMemcpyToSymbol(c_selftest_wait_budget, &wait_budget, sizeof(wait_budget)) != cudaSuccess ||
             cudaMemcpyToSymbol(c_selftest_tx_extra, &tx_extra, sizeof(tx_extra)) != cudaSuccess) return RPTQ_ERR_CUDA;
     }
-    fn<<<M < blocks ? M : blocks, T, smem, static_cast<cudaStream_t>(stream)>>>(p);
-    return cudaGetLastError() == cudaSuccess ? RPTQ_OK : RPTQ_ERR_CUDA;
+    return launch_kernel(fn, dim3((unsigned)(M < blocks ? M : blocks)), (unsigned)T, smem, 0, static_cast<cudaStream_t>(stream), p);
 }
 
 extern "C" int rptq_ln_reorder_quant(const rptq_layout_t* L, const void* x, int64_t ldx, const void* gamma,

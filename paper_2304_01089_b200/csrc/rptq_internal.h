@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <vector>
 
 #include "rptq.h"
@@ -70,8 +71,47 @@ struct SmallMParams {
 };
 namespace smallm {
 bool fits(int M, int bits, int K_pad);
-int launch(const SmallMParams& p, int bits, cudaStream_t st);
+int launch(const SmallMParams& p, int bits, int device, cudaStream_t st);
 }
+
+// Programmatic dependent launch: every kernel of the library is launched so that its blocks may become resident, and
+// run their set-up, while the kernel before it in the stream drains. pdl_wait() returns when that kernel has
+// completed and its writes are visible; nothing but the layout's own tables (uploaded before rptq_layout_create
+// returned) is touched before it. pdl_trigger() lets the next kernel's blocks come in. A LayerNorm + GEMM pair of one token:
+// 10.9 -> 10.0 us on the device, a LayerNorm launch 3.8 -> 2.7 us.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class... P, class... A>
+inline int launch_kernel(void (*fn)(P...), dim3 grid, unsigned threads, size_t smem, unsigned cluster, cudaStream_t st, A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = cluster; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cluster > 0 ? 2 : 1;
+    return cudaLaunchKernelEx(&cfg, fn, args...) == cudaSuccess ? RPTQ_OK : RPTQ_ERR_CUDA;
+}
+
+// The dynamic shared memory a kernel may ask for, raised once per kernel and device to the most that any launch of it
+// asks for (the runtime call costs about a microsecond of host time). `done`: one bit per device, a static of the caller.
+inline int allow_smem(const void* fn, int device, int bytes, std::atomic<uint64_t>& done)
+{
+    const uint64_t bit = uint64_t(1) << (device & 63);
+    if (done.load(std::memory_order_acquire) & bit) return RPTQ_OK;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return RPTQ_ERR_CUDA;
+    if (device >= 0 && device < 64) done.fetch_or(bit, std::memory_order_release);
+    return RPTQ_OK;
+}
+
+int sm_count(int device);    // of the device, asked for once; 0 on failure
 
 int* device_status_word();   // lazily allocated device int, RPTQ_OK when clear; nullptr on failure
 

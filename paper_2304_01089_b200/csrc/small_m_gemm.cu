@@ -104,6 +104,8 @@ small_m_kernel(const SmallMParams p)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
+    pdl_trigger();
+    pdl_wait();
 
     const int tileA = 2 * (int)blockIdx.x;
     const bool haveB = tileA + 1 < p.n_wtiles;
@@ -299,13 +301,13 @@ static int smem_bytes(int nt, int K_pad)
 }
 
 template <int BITS, int NT>
-static int launch_one(const SmallMParams& p, cudaStream_t st)
+static int launch_one(const SmallMParams& p, int device, cudaStream_t st)
 {
     const int smem = smem_bytes(NT, p.K_pad);
-    if (cudaFuncSetAttribute(small_m_kernel<BITS, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess) return RPTQ_ERR_CUDA;
+    static std::atomic<uint64_t> done{0};
+    if (allow_smem(reinterpret_cast<const void*>(small_m_kernel<BITS, NT>), device, 226 * 1024, done) != RPTQ_OK) return RPTQ_ERR_CUDA;
     const int blocks = (p.n_wtiles + 1) / 2;
-    small_m_kernel<BITS, NT><<<blocks, THREADS, smem, st>>>(p);
-    return cudaGetLastError() == cudaSuccess ? RPTQ_OK : RPTQ_ERR_CUDA;
+    return launch_kernel(small_m_kernel<BITS, NT>, dim3((unsigned)blocks), THREADS, (size_t)smem, 0, st, p);
 }
 
 bool fits(int M, int bits, int K_pad)
@@ -313,10 +315,10 @@ bool fits(int M, int bits, int K_pad)
     return M <= 16 && (bits == 3 || bits == 4) && smem_bytes(M <= 8 ? 1 : 2, K_pad) <= 226 * 1024;
 }
 
-int launch(const SmallMParams& p, int bits, cudaStream_t st)
+int launch(const SmallMParams& p, int bits, int device, cudaStream_t st)
 {
-    if (p.M <= 8) return bits == 3 ? launch_one<3, 1>(p, st) : launch_one<4, 1>(p, st);
-    return bits == 3 ? launch_one<3, 2>(p, st) : launch_one<4, 2>(p, st);
+    if (p.M <= 8) return bits == 3 ? launch_one<3, 1>(p, device, st) : launch_one<4, 1>(p, device, st);
+    return bits == 3 ? launch_one<3, 2>(p, device, st) : launch_one<4, 2>(p, device, st);
 }
 
 }  // namespace smallm
