@@ -341,7 +341,7 @@ extern "C" int rptq_attention(const rptq_layout_t* LQ, const rptq_layout_t* LK, 
     p.q = static_cast<const uint8_t*>(q_codes); p.k = static_cast<const uint8_t*>(k_codes); p.v = static_cast<const uint8_t*>(v_codes);
     p.q_row_bytes = LQ->row_bytes; p.k_row_bytes = LK->row_bytes; p.v_row_bytes = LV->row_bytes;
     p.bits_q = LQ->bits; p.bits_k = LK->bits; p.bits_v = LV->bits;
-    p.Tq = Tq; p.Tk = Tk; p.H = n_heads; p.gh_k = LQ->g / n_heads; p.gh_v = LV->g / n_heads; p.causal = causal ? 1 : 0;
+    p.Tq = Tq; p.Tk = Tk; p.H = n_heads; p.hd = LV->C / n_heads; p.gh_k = LQ->g / n_heads; p.gh_v = LV->g / n_heads; p.causal = causal ? 1 : 0;
     p.cl_unit0_k = LQ->d_cl_unit0; p.cl_unit0_v = LV->d_cl_unit0; p.unit_cluster_k = LQ->d_unit_cluster;
     p.unit_sz_q = LQ->d_unit_sz; p.unit_sz_k = LK->d_unit_sz; p.unit_sz_v = LV->d_unit_sz;
     p.src_v = LV->d_src; p.jidx_v = LV->d_jidx;
@@ -352,6 +352,7 @@ extern "C" int rptq_attention(const rptq_layout_t* LQ, const rptq_layout_t* LK, 
     const int n_sm = sm_count(dev);
     if (n_sm == 0) return RPTQ_ERR_CUDA;
     if (attn_decode::fits(p, false)) return attn_decode::launch(p, false, units_k, units_v, n_seq, dev, n_sm, st);
+    return attn_prefill::launch(p, false, units_k, units_v, n_seq, heads_own_their_channels(LV, n_heads), dev, n_sm, st);
 
     const int max_bits = LK->bits > LV->bits ? LK->bits : LV->bits;
     const int raw_pitch = 4 * max_bits * MAX_UNITS + 32;          // a head's packed codes plus the alignment slack, a multiple of 16

@@ -240,17 +240,6 @@ attention_kv_kernel(const AttnParams p)
 }  // namespace attnkv
 }  // namespace rptq
 
-// head h's clusters hold exactly the channels h * hd .. (h + 1) * hd - 1 (the kernel reads a head's query slice by that rule)
-static bool kv_heads_own_their_channels(const rptq_layout_t* L, int H)
-{
-    const int gh = L->g / H, hd = L->C / H;
-    for (int c = 0; c < L->g; ++c) {
-        const size_t i = (size_t)c;
-        if (L->cl_ch_hi[i] >= 0 && (L->cl_ch_lo[i] / hd != c / gh || L->cl_ch_hi[i] / hd != c / gh)) return false;
-    }
-    return true;
-}
-
 extern "C" int rptq_attention_kv(const rptq_layout_t* LK, const rptq_layout_t* LV, int n_heads,
                                  const void* q_f16, int64_t ldq, int Tq, const void* k_codes, const void* v_codes, int Tk, int n_seq,
                                  float qk_scale, int causal, void* out_f16, int64_t ldo, void* stream)
@@ -266,7 +255,7 @@ extern "C" int rptq_attention_kv(const rptq_layout_t* LK, const rptq_layout_t* L
     if (!LK->in_cluster_order || !LV->in_cluster_order) return RPTQ_ERR_UNSUPPORTED;
     const int units_k = max_units_per_head(LK, n_heads), units_v = max_units_per_head(LV, n_heads);
     if (units_k > MAX_UNITS || units_v > MAX_UNITS) return RPTQ_ERR_UNSUPPORTED;
-    if (!kv_heads_own_their_channels(LK, n_heads)) return RPTQ_ERR_INVALID_ARG;
+    if (!heads_own_their_channels(LK, n_heads)) return RPTQ_ERR_INVALID_ARG;
     if (Tq == 0 || n_seq == 0) return RPTQ_OK;
     int dev = -1;
     if (LK->device < 0 || cudaGetDevice(&dev) != cudaSuccess) return RPTQ_ERR_CUDA;
@@ -287,6 +276,7 @@ extern "C" int rptq_attention_kv(const rptq_layout_t* LK, const rptq_layout_t* L
     const int n_sm = sm_count(dev);
     if (n_sm == 0) return RPTQ_ERR_CUDA;
     if (attn_decode::fits(p, true)) return attn_decode::launch(p, true, units_k, units_v, n_seq, dev, n_sm, st);
+    return attn_prefill::launch(p, true, units_k, units_v, n_seq, heads_own_their_channels(LV, n_heads), dev, n_sm, st);
 
     const int smem = (BM + 2 * BN) * PITCH;
     static std::atomic<uint64_t> done{0};

@@ -99,11 +99,27 @@ inline int max_units_per_head(const rptq_layout_t* L, int n_heads)
     return m;
 }
 
+// Head h's clusters hold exactly the channels h * hd .. (h + 1) * hd - 1.
+inline bool heads_own_their_channels(const rptq_layout_t* L, int n_heads)
+{
+    if (L->C % n_heads) return false;
+    const int gh = L->g / n_heads, hd = L->C / n_heads;
+    for (int c = 0; c < L->g; ++c) {
+        const size_t i = (size_t)c;
+        if (L->cl_ch_hi[i] >= 0 && (L->cl_ch_lo[i] / hd != c / gh || L->cl_ch_hi[i] / hd != c / gh)) return false;
+    }
+    return true;
+}
+
 }  // namespace attn
 
 // The decode kernel (attention_decode.cu): few queries per sequence, the keys split over a cluster of blocks.
 namespace attn_decode {
 bool fits(const attn::AttnParams& p, bool kv);     // false: the prefill kernel takes the call
 int launch(const attn::AttnParams& p, bool kv, int units_k, int units_v, int n_seq, int dev, int n_sm, cudaStream_t st);
+}
+// The kernel for more queries (attention_prefill.cu). v_heads_local: head h of V owns the channels h * hd .. (h + 1) * hd - 1.
+namespace attn_prefill {
+int launch(const attn::AttnParams& p, bool kv, int units_k, int units_v, int n_seq, bool v_heads_local, int dev, int n_sm, cudaStream_t st);
 }
 }  // namespace rptq

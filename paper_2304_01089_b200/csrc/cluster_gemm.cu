@@ -41,10 +41,13 @@
 
 #include "pack.cuh"
 #include "rptq_internal.h"
+#include "tc.cuh"
 #include "unpack.cuh"
 
 namespace rptq {
 namespace gemm {
+
+using namespace tc;
 
 constexpr int TILE_M = 128, TILE_N = 256, KBLK = 128;   // TILE_M is per CTA
 constexpr int THREADS = 512;
@@ -57,7 +60,6 @@ constexpr int REGS_WG0 = 40, REGS_UNPACK = 88, REGS_EPI = 192;
 static_assert(128 * (REGS_WG0 + REGS_UNPACK + 2 * REGS_EPI) <= 128 * THREADS, "register pool");
 constexpr int A8_BYTES = TILE_M * KBLK;                  // 16 KiB of 8-bit activation operands per stage
 constexpr int WTILE_BYTES = 8192;                        // one packed weight tile: 128 rows x 64 bytes
-constexpr long long WAIT_BUDGET_CYCLES = 4000000000ll;   // about two seconds at the SM clock
 
 __host__ __device__ constexpr int w_rows(int ncta) { return TILE_N / ncta; }           // weight rows staged per CTA
 // packed weight stages; the single-CTA variant (at most 128 tokens) is a weight stream and takes what shared memory is left
@@ -128,72 +130,6 @@ struct Params {
 };
 
 // ---------------------------------------------------------------- PTX wrappers
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-
-__device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count)
-{
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
-// Arrive on the barrier at the same shared-memory offset in CTA `rank` of the cluster.
-__device__ __forceinline__ void mbar_arrive_remote(uint32_t bar, uint32_t rank)
-{
-    asm volatile(
-        "{\n\t.reg .b32 ra;\n\t"
-        "mapa.shared::cluster.u32 ra, %0, %1;\n\t"
-        "mbarrier.arrive.shared::cluster.b64 _, [ra];\n\t}"
-        ::"r"(bar), "r"(rank) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive_expect_tx(uint32_t bar, uint32_t bytes)
-{
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
-}
-// Bounded wait. Returns false when the budget ran out or another role already gave up. The common
-// case (the phase has already completed, or completes within a few polls) touches no timer; the
-// budget is counted on the SM's cycle counter, read once per batch of polls.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, bool heed_abort = true)
-{
-    auto poll = [&]() { return mbar_try_wait(bar, parity); };
-    if (poll()) return true;
-    if (poll()) return true;
-    const long long t0 = clock64();
-#pragma unroll 1
-    while (true) {
-#pragma unroll 1
-        for (int i = 0; i < 1024; ++i)
-            if (poll()) return true;
-        if (heed_abort && *abort_flag) return false;
-        if (clock64() - t0 > WAIT_BUDGET_CYCLES) { *abort_flag = 1; return false; }
-    }
-}
-// The same wait for a whole warp that must stay converged (the MMA-issuing warp): the lanes vote on
-// every poll, so all of them leave the loop in the same iteration whatever each one saw.
-__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag)
-{
-    if (__any_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-    const long long t0 = clock64();
-#pragma unroll 1
-    while (true) {
-#pragma unroll 1
-        for (int i = 0; i < 1024; ++i)
-            if (__any_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
-        const bool give_up = *abort_flag != 0 || clock64() - t0 > WAIT_BUDGET_CYCLES;
-        if (__any_sync(0xffffffffu, give_up)) { *abort_flag = 1; return false; }
-    }
-}
 __device__ __forceinline__ uint32_t cluster_ctarank()
 {
     uint32_t r;
@@ -222,9 +158,6 @@ __device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool v
 __device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 template <int N>
 __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-__device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 // The two tensor-core instructions below are executed by the WHOLE issuing warp in converged
 // control flow; elect.sync picks the one lane that issues. Measured on an operand-resident loop: a
 // tcgen05.mma issued from a branch that a single lane took costs the issuing thread ~120 clocks,
@@ -286,28 +219,6 @@ __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, ui
             "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
             ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
     }
-}
-__device__ __forceinline__ void tc_ld16(uint32_t taddr, uint32_t (&v)[16])
-{
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-        : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ void tc_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-
-// K-major operand tile with 128-byte rows and the 128-byte swizzle: 8-row groups are 1024 bytes
-// apart (stride byte offset), the leading byte offset is unused for swizzled K-major layouts.
-__device__ __forceinline__ uint64_t smem_desc_sw128(uint32_t addr)
-{
-    uint64_t d = 0;
-    d |= (uint64_t)((addr & 0x3FFFFu) >> 4);        // start address, 16-byte units
-    d |= (uint64_t)1 << 16;                         // leading byte offset (ignored)
-    d |= (uint64_t)(1024 >> 4) << 32;               // stride byte offset
-    d |= (uint64_t)1 << 46;                         // descriptor version of this architecture
-    d |= (uint64_t)2 << 61;                         // 128-byte swizzle
-    return d;
 }
 // kind::i8, D = s32, A = unsigned 8-bit (activation codes), B = signed 8-bit (weights), both
 // K-major, M = 128 per CTA, N = 256.
