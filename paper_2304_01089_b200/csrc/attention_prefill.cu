@@ -8,13 +8,18 @@
 // What bounds it: one exponential per score and pass (the special-function unit gives 16 per clock and SM), then the
 // issue slots of the softmax warps: a score costs one multiply-add per cluster of the head, and five or six
 // instructions more. So everything else is kept off those warps:
-//   warp 0        issues the MMAs: per key tile, one accumulator per CLUSTER of the head (the scales differ), handed over
-//                 slot by slot through a ring in tensor memory; then, in pass 2, P V of the previous tile into the
-//                 head's output accumulator, which stays in tensor memory over the whole pass
+//   warps 0, 1    issue the score MMAs of two STREAMS (integer calls: the halves of a 128-key tile; KV: even and odd tiles
+//                 of 64 keys): one accumulator per CLUSTER of the head (the scales differ), handed over slot by slot
+//                 through the stream's own ring in tensor memory. The streams run on their own, so that one's drains
+//                 fall under the other's exponentials
+//   warp 2        issues P V (pass 2) into the head's output accumulator, which stays in tensor memory
 //   warps 4-7     keys: packed rows arrive by cp.async one tile ahead, are unpacked into the swizzled operand tile; integer
 //                 calls: with the per-key zero-point term -sum_c s^Q s^K z^Q sum_p K_q. They also lay out the queries.
-//   warps 8-11    values: unpacked and transposed into [position][key] (byte permutes on the packed words)
-//   warps 12-19   softmax: thread = (query row, half of the tile's keys); S = sum_c coef_c acc_c in registers
+//   warps 8-11    values: unpacked and transposed into [position][key] (byte permutes on the packed words); and the
+//                 output of an item, while the next item's pass 1 runs (they have nothing else to do there)
+//   warps 12-19   softmax, four per stream: thread = query row, 64 keys; S = sum_c coef_c acc_c in registers. (Sixteen warps
+//                 with 32 keys each were slower, 1418 against 1028 us: the hand-over of a cluster costs as many
+//                 instructions for 32 keys as for 64)
 // Operand types (MODE):
 //   I8   bytes, kind::i8, int32 sums
 //   F8   both codes of at most four bits: a nibble n as an 8-bit E4M3 pattern IS the number n 2^-9, so the same bytes
@@ -23,9 +28,9 @@
 //   KV   fp16 query; codes as fp16 integers n - 8 (n - 128): the centre is a constant per row in the scores and part of the
 //        zero point in the outputs
 // P V is u8 x u8 -> s32 for I8 and F8 (exact), fp16 x fp16 -> fp32 for KV.
-// Key order inside a tile of the second product (both operands are written in it, so the sums do not change):
-// KEYS = 128: byte b of word w is key w + 32 b; KV, 64 keys: see v_tile. It lets the V loader read and
-// write shared memory without bank conflicts.
+// Key order inside a tile of the second product (both operands are written in it, so the sums do not change): within a
+// quarter of 32 keys, byte b of word w is key w + 8 b; KV, quarters of 16 keys: fp16 pair b of chunk y is keys
+// 4 b + 2 y + {0, 1}. It lets the V loader read and write shared memory without bank conflicts.
 //
 // Measured: MEASURED_PREFILL
 #include <type_traits>
@@ -40,12 +45,14 @@ namespace attn_prefill {
 using namespace attn;
 using tc::mbar_arrive;
 using tc::mbar_init;
-using tc::mbar_wait;
-using tc::mbar_wait_warp;
+using tc::mbar_sleep;
+using tc::mbar_sleep_warp;
 
 enum { I8 = 0, F8 = 1, KV = 2 };
 constexpr int BM = 128, THREADS = 640;
 constexpr int K_WARP0 = 4, V_WARP0 = 8, S_WARP0 = 12;
+constexpr int COLS = 64;                                  // keys of a stream's piece of work = columns of a score slot
+constexpr int N_SLOTS = 2;                                // score slots of each stream
 // registers per thread of the five warpgroups (the block is launched with 96 each)
 constexpr int REGS_MMA = 48, REGS_LOAD = 72, REGS_SOFTMAX = 144;
 static_assert(REGS_MMA + 2 * REGS_LOAD + 2 * REGS_SOFTMAX <= 5 * 96, "register pool");
@@ -57,8 +64,8 @@ __host__ __device__ constexpr int keys_of(int mode) { return mode == KV ? 64 : 1
 // Shared memory of a launch (sizes follow the widest head of the layouts).
 struct Plan {
     int n_items, n_qt, n_seq;
-    int off_k, k_stage, off_v, v_stage, v_stages, off_p, off_rawk, pitch_k, off_rawv, pitch_v, off_col, off_x, off_bar, total;
-    int local_v;          // V's heads own their channels and the output tile fits the V region: rows leave through shared memory
+    int off_k, k_stage, off_v, v_stage, v_stages, off_p, p_tiles, off_rawk, rawk_stage, rawk_stages, pitch_k, off_rawv, pitch_v, off_col, off_ml, off_sum, off_bar, total;
+    int local_v;          // V's heads own their channels and the output tile fits the V and P region: rows leave through shared memory
     int out_pitch;
     int* status;
 };
@@ -71,10 +78,16 @@ static int raw_pitch_of(int bits, int units)
     return 16 * (c | 1);
 }
 
-__device__ __forceinline__ void ld8(uint32_t taddr, uint32_t* v)
+__device__ __forceinline__ void ld32(uint32_t taddr, uint32_t (&v)[32])
 {
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(taddr) : "memory");
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
+          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        : "r"(taddr) : "memory");
 }
 __device__ __forceinline__ float2 add2(float2 a, float2 b)
 {
@@ -97,19 +110,21 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
         : "l"(reinterpret_cast<uint64_t&>(a)), "l"(reinterpret_cast<uint64_t&>(b)), "l"(reinterpret_cast<uint64_t&>(c)));
     return d;
 }
-// The whole warp executes these in converged control flow; one elected lane issues.
+// The whole warp executes these in converged control flow; one elected lane issues. a, b: the low words of the operands'
+// descriptors (the high words are the same for every tile).
+constexpr uint32_t DESC_HI = (uint32_t)(1024 >> 4) | (1u << 14) | (2u << 29);       // of smem_desc_sw128
 template <int KIND>       // 0 i8, 1 f8f6f4, 2 f16
-__device__ __forceinline__ void mma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc)
+__device__ __forceinline__ void mma(uint32_t d, uint32_t a, uint32_t b, uint32_t idesc, uint32_t acc)
 {
     if constexpr (KIND == 0)
-        asm volatile("{\n\t.reg .pred p, q;\n\telect.sync _|q, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                     "@q tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n\t}" ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
+        asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\telect.sync _|q, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                     "@q tcgen05.mma.cta_group::1.kind::i8 [%0], da, db, %3, p;\n\t}" ::"r"(d), "r"(a), "r"(b), "r"(idesc), "r"(acc), "r"(DESC_HI) : "memory");
     else if constexpr (KIND == 1)
-        asm volatile("{\n\t.reg .pred p, q;\n\telect.sync _|q, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                     "@q tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], %1, %2, %3, p;\n\t}" ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
+        asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\telect.sync _|q, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                     "@q tcgen05.mma.cta_group::1.kind::f8f6f4 [%0], da, db, %3, p;\n\t}" ::"r"(d), "r"(a), "r"(b), "r"(idesc), "r"(acc), "r"(DESC_HI) : "memory");
     else
-        asm volatile("{\n\t.reg .pred p, q;\n\telect.sync _|q, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-                     "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
+        asm volatile("{\n\t.reg .pred p, q;\n\t.reg .b64 da, db;\n\tmov.b64 da, {%1, %5};\n\tmov.b64 db, {%2, %5};\n\telect.sync _|q, 0xffffffff;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+                     "@q tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n\t}" ::"r"(d), "r"(a), "r"(b), "r"(idesc), "r"(acc), "r"(DESC_HI) : "memory");
 }
 __device__ __forceinline__ void commit(uint32_t bar)
 {
@@ -186,17 +201,19 @@ template <int MODE>
 __global__ void __launch_bounds__(THREADS, 1)
 prefill_kernel(const AttnParams p, const Plan g)
 {
-    constexpr int KEYS = keys_of(MODE), N_SLOTS = (512 - O_COLS) / KEYS;
+    constexpr int KEYS = keys_of(MODE);
+    constexpr bool ALT = MODE == KV;                      // the streams take tiles by turns (otherwise halves of every tile)
+    static_assert(O_COLS + 2 * N_SLOTS * COLS <= 512, "tensor memory");
     constexpr int K_ATOM = KEYS * 128;                    // operand tile of the keys: KEYS rows of 128 bytes per atom
-    constexpr int UNITS_PER_ATOM = MODE == KV ? 2 : 4;    // 64 bytes (fp16) or 32 bytes per unit
+    constexpr int Q_LOADERS = MODE == KV ? 8 : 4;         // warps that lay out the queries
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t* smem = smem_raw + (base - smem_u32(smem_raw));
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + g.off_bar);
-    constexpr int B_QFULL = 0, B_QEMPTY = 1, B_KFULL = 2, B_KEMPTY = 4, B_SFULL = 6, B_SEMPTY = B_SFULL + N_SLOTS, B_PFULL = B_SEMPTY + N_SLOTS,
-                  B_PEMPTY = B_PFULL + 1, B_VFULL = B_PEMPTY + 1, B_VEMPTY = B_VFULL + 2, B_OFULL = B_VEMPTY + 2, B_OEMPTY = B_OFULL + 1,
-                  B_OUT = B_OEMPTY + 1, B_XS = B_OUT + 1, B_XV = B_XS + 1, B_DRAIN = B_XV + 1, N_BARS = B_DRAIN + 1;
-    static_assert(N_BARS * 8 + 16 <= 256, "barrier block");
+    constexpr int B_QFULL = 0, B_QEMPTY = 1, B_KFULL = 2, B_KEMPTY = 4, B_SFULL = 6, B_SEMPTY = B_SFULL + 2 * N_SLOTS, B_PFULL = B_SEMPTY + 2 * N_SLOTS,
+                  B_PEMPTY = B_PFULL + 2, B_VFULL = B_PEMPTY + 2, B_VEMPTY = B_VFULL + 2, B_OFULL = B_VEMPTY + 2, B_OEMPTY = B_OFULL + 1,
+                  B_OUT = B_OEMPTY + 1, B_SUM = B_OUT + 1, B_XS = B_SUM + 1, B_XV = B_XS + 1, B_DRAIN = B_XV + 1, N_BARS = B_DRAIN + 3;
+    static_assert(N_BARS * 8 + 16 <= 512, "barrier block");
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + N_BARS);
     volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
     const uint32_t bar0 = smem_u32(bars);
@@ -204,12 +221,15 @@ prefill_kernel(const AttnParams p, const Plan g)
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
     if (tid == 0) {
-        mbar_init(bar(B_QFULL), 4); mbar_init(bar(B_QEMPTY), 1);
-        for (int i = 0; i < 2; ++i) { mbar_init(bar(B_KFULL + i), 4); mbar_init(bar(B_KEMPTY + i), 1); mbar_init(bar(B_VFULL + i), 4); mbar_init(bar(B_VEMPTY + i), 1); }
-        for (int i = 0; i < N_SLOTS; ++i) { mbar_init(bar(B_SFULL + i), 1); mbar_init(bar(B_SEMPTY + i), 8); }
-        mbar_init(bar(B_PFULL), 8); mbar_init(bar(B_PEMPTY), 1);
-        mbar_init(bar(B_OFULL), 1); mbar_init(bar(B_OEMPTY), 8); mbar_init(bar(B_OUT), 8);
-        mbar_init(bar(B_XS), 8); mbar_init(bar(B_XV), 4); mbar_init(bar(B_DRAIN), 1);
+        mbar_init(bar(B_QFULL), Q_LOADERS); mbar_init(bar(B_QEMPTY), 2);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(bar(B_KFULL + i), 4); mbar_init(bar(B_KEMPTY + i), ALT ? 1 : 2); mbar_init(bar(B_VFULL + i), 4); mbar_init(bar(B_VEMPTY + i), 1);
+            mbar_init(bar(B_PFULL + i), 4); mbar_init(bar(B_PEMPTY + i), 1);
+        }
+        for (int i = 0; i < 2 * N_SLOTS; ++i) { mbar_init(bar(B_SFULL + i), 1); mbar_init(bar(B_SEMPTY + i), 4); }
+        mbar_init(bar(B_OFULL), 1); mbar_init(bar(B_OEMPTY), 4); mbar_init(bar(B_OUT), 4);
+        mbar_init(bar(B_SUM), 8); mbar_init(bar(B_XS), 8); mbar_init(bar(B_XV), 4);
+        for (int i = 0; i < 3; ++i) mbar_init(bar(B_DRAIN + i), 1);
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -223,380 +243,438 @@ prefill_kernel(const AttnParams p, const Plan g)
     __syncthreads();
     tc::tc_fence_after();
     const uint32_t tmem = *s_tmem;
-    const int off = p.Tk - p.Tq;
     float* s_col = reinterpret_cast<float*>(smem + g.off_col);            // [4][KEYS]
-    float2* s_x = reinterpret_cast<float2*>(smem + g.off_x);              // [2][2][BM]: the halves' row statistics
+    float2* s_ml = reinterpret_cast<float2*>(smem + g.off_ml);            // [2][2][BM]: the streams' row maxima and sums
+    uint32_t* s_sum = reinterpret_cast<uint32_t*>(smem + g.off_sum);      // [2][BM]: the streams' sums of probabilities (codes)
 
     if (warp < K_WARP0) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_MMA));
-        if (warp == 0) {
-            // ------------------------------------------------------------ MMA issuer
-            constexpr uint32_t FMT = MODE == I8 ? (2u << 4) : (1u << 4);                          // D: s32 or f32; A, B: u8 / E4M3 / f16
-            constexpr uint32_t ID_QK = FMT | ((uint32_t)(KEYS >> 3) << 17) | (8u << 24);
-            constexpr uint32_t ID_PV = (MODE == KV ? (1u << 4) : (2u << 4)) | (8u << 24);
-            const uint64_t dq = tc::smem_desc_sw128(base), dk = tc::smem_desc_sw128(base + g.off_k), dv = tc::smem_desc_sw128(base + g.off_v),
-                           dp = tc::smem_desc_sw128(base + g.off_p);
-            uint32_t n_k = 0, n_s = 0, n_v = 0, n_item = 0;
-            bool ok = true;
+        auto desc = [&](int off) { return ((base + (uint32_t)off) & 0x3FFFFu) >> 4 | 1u << 16; };
+        bool ok = true;
+        if (warp < 2) {
+            // ------------------------------------------------------------ scores of one stream
+            const int stream = warp;
+            constexpr uint32_t ID = (MODE == I8 ? (2u << 4) : (1u << 4)) | ((uint32_t)(COLS >> 3) << 17) | (8u << 24);   // D: s32 or f32; A, B: u8 / E4M3 / f16
+            constexpr uint32_t LOG_ATOM = ALT ? 1 : 2, STEP = ALT ? 4 : 2;                   // units per atom; a unit's bytes / 16
+            const uint32_t dq = desc(0), dk = desc(g.off_k + (ALT ? 0 : stream * COLS * 128)), k_step = (uint32_t)(g.k_stage >> 4);
+            const uint32_t d0 = tmem + O_COLS + stream * (N_SLOTS * COLS);
+            const uint32_t b_full0 = bar(B_SFULL + stream * N_SLOTS), b_empty0 = bar(B_SEMPTY + stream * N_SLOTS);
+            uint32_t n_k = 0, slot = 0, par = 1, n_item = 0;                    // n_k: my tiles so far
             for (int idx = blockIdx.x; idx < g.n_items && ok; idx += gridDim.x, ++n_item) {
                 const Item it = item_of(p, g, idx, KEYS);
-                const int uk0 = __ldg(p.cl_unit0_k + it.h * p.gh_k), nuk = __ldg(p.cl_unit0_k + (it.h + 1) * p.gh_k) - uk0;
-                const int nuv = __ldg(p.cl_unit0_v + (it.h + 1) * p.gh_v) - __ldg(p.cl_unit0_v + it.h * p.gh_v);
+                const int uk0 = __ldg(p.cl_unit0_k + it.h * p.gh_k), nuk = __ldg(p.cl_unit0_k + (it.h + 1) * p.gh_k) - uk0, nu = units_seen(nuk);
                 // bit u: unit u is the last of its cluster
                 const int cl = lane < nuk ? __ldg(p.unit_cluster_k + uk0 + lane) : -1;
                 const int cl_next = __shfl_down_sync(0xffffffffu, cl, 1);
-                const uint32_t last = __ballot_sync(0xffffffffu, lane < units_seen(nuk) && (lane >= nuk - 1 || cl != cl_next));
-                const uint32_t id_pv = ID_PV | ((uint32_t)(4 * nuv) << 17);
-                if (!mbar_wait_warp(bar(B_QFULL), n_item & 1, s_abort)) { ok = false; break; }
-                auto scores = [&]() {
-                    const uint32_t st = n_k & 1;
-                    if (!mbar_wait_warp(bar(B_KFULL + st), (n_k >> 1) & 1, s_abort)) return false;
-                    tc::tc_fence_after();
-                    const uint64_t kb = dk + (uint64_t)(st * (uint32_t)(g.k_stage >> 4));
-                    bool first = true;
+                const uint32_t last = __ballot_sync(0xffffffffu, lane < nu && (lane >= nuk - 1 || cl != cl_next));
+                if (!mbar_sleep_warp(bar(B_QFULL), n_item & 1, s_abort)) { ok = false; break; }
 #pragma unroll 1
-                    for (int u = 0; u < units_seen(nuk); ++u) {
-                        const uint32_t slot = n_s % N_SLOTS, d = tmem + O_COLS + slot * KEYS;
-                        if (first) {
-                            if (!mbar_wait_warp(bar(B_SEMPTY + slot), ((n_s / N_SLOTS) & 1) ^ 1, s_abort)) return false;
-                            tc::tc_fence_after();
-                        }
-                        const uint32_t atom = (uint32_t)u / UNITS_PER_ATOM, in = (uint32_t)u % UNITS_PER_ATOM;
-                        const uint64_t a = dq + (uint64_t)(atom * (ATOM_Q >> 4)), b = kb + (uint64_t)(atom * (K_ATOM >> 4));
-                        if constexpr (MODE == KV) {
-                            mma<2>(d, a + 4 * in, b + 4 * in, ID_QK, first ? 0u : 1u);
-                            mma<2>(d, a + 4 * in + 2, b + 4 * in + 2, ID_QK, 1u);
-                        } else {
-                            mma<MODE == F8 ? 1 : 0>(d, a + 2 * in, b + 2 * in, ID_QK, first ? 0u : 1u);
-                        }
-                        first = false;
-                        if ((last >> u) & 1u) { commit(bar(B_SFULL + slot)); ++n_s; first = true; }
-                    }
-                    commit(bar(B_KEMPTY + st));
-                    ++n_k;
-                    return true;
-                };
-                auto outputs = [&](bool first) {
-                    const uint32_t st = g.v_stages == 2 ? n_v & 1 : 0u, ph = g.v_stages == 2 ? (n_v >> 1) & 1 : n_v & 1;
-                    if (!mbar_wait_warp(bar(B_VFULL + st), ph, s_abort)) return false;
-                    if (!mbar_wait_warp(bar(B_PFULL), n_v & 1, s_abort)) return false;
-                    tc::tc_fence_after();
-                    const uint64_t b = dv + (uint64_t)(st * (uint32_t)(g.v_stage >> 4));
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        if (nuv > 0) mma<MODE == KV ? 2 : 0>(tmem, dp + 2 * k, b + 2 * k, id_pv, (first && k == 0) ? 0u : 1u);
-                    commit(bar(B_PEMPTY));
-                    commit(bar(B_VEMPTY + st));
-                    ++n_v;
-                    return true;
-                };
-                for (int kt = 0; kt < it.n_kt && ok; ++kt) ok = scores();
-                for (int kt = 0; kt < it.n_kt && ok; ++kt) {
-                    ok = scores();
-                    if (!ok) break;
-                    if (kt == it.n_kt - 1) commit(bar(B_QEMPTY));              // the item's last score product has been issued
-                    if (kt == 1) {                                             // the item's first output product comes next
-                        ok = mbar_wait_warp(bar(B_OEMPTY), (n_item & 1) ^ 1, s_abort);
+                for (int pass = 0; pass < 2 && ok; ++pass) {
+#pragma unroll 1
+                    for (int kt = ALT ? stream : 0; kt < it.n_kt && ok; kt += ALT ? 2 : 1, ++n_k) {
+                        const uint32_t st = ALT ? stream : n_k & 1;            // (KV: a stage belongs to a stream, which so sees all its phases)
+                        if (!mbar_sleep_warp(bar(B_KFULL + st), (ALT ? n_k : n_k >> 1) & 1, s_abort)) { ok = false; break; }
                         tc::tc_fence_after();
+                        const uint32_t kb = dk + st * k_step;
+                        uint32_t acc = 0u;
+#pragma unroll 1
+                        for (uint32_t u = 0; u < (uint32_t)nu; ++u) {
+                            if (acc == 0u) {
+                                if (!mbar_sleep_warp(b_empty0 + 8 * slot, par, s_abort)) { ok = false; break; }
+                                tc::tc_fence_after();
+                            }
+                            const uint32_t d = d0 + slot * COLS, in = (u & ((1u << LOG_ATOM) - 1u)) * STEP;
+                            const uint32_t a = dq + (u >> LOG_ATOM) * (ATOM_Q >> 4) + in, b = kb + (u >> LOG_ATOM) * (K_ATOM >> 4) + in;
+                            if constexpr (MODE == KV) {
+                                mma<2>(d, a, b, ID, acc);
+                                mma<2>(d, a + 2, b + 2, ID, 1u);
+                            } else {
+                                mma<MODE == F8 ? 1 : 0>(d, a, b, ID, acc);
+                            }
+                            acc = 1u;
+                            if ((last >> u) & 1u) {
+                                commit(b_full0 + 8 * slot);
+                                acc = 0u;
+                                slot ^= 1u;
+                                par ^= slot ^ 1u;
+                            }
+                        }
+                        if (ok) commit(bar(B_KEMPTY + st));
                     }
-                    if (kt > 0 && ok) ok = outputs(kt == 1);
                 }
-                if (ok && it.n_kt == 1) { ok = mbar_wait_warp(bar(B_OEMPTY), (n_item & 1) ^ 1, s_abort); tc::tc_fence_after(); }
-                if (ok) ok = outputs(it.n_kt == 1);
+                if (ok) commit(bar(B_QEMPTY));
+            }
+        } else if (warp == 2) {
+            // ------------------------------------------------------------ outputs
+            constexpr uint32_t ID = (MODE == KV ? (1u << 4) : (2u << 4)) | (8u << 24);
+            const uint32_t dv = desc(g.off_v), dp = desc(g.off_p), v_step = (uint32_t)(g.v_stage >> 4);
+            uint32_t n_v = 0, n_item = 0, n_p0 = 0, n_p1 = 0;                  // (KV: tiles of each stream so far)
+            for (int idx = blockIdx.x; idx < g.n_items && ok; idx += gridDim.x, ++n_item) {
+                const Item it = item_of(p, g, idx, KEYS);
+                const int nuv = __ldg(p.cl_unit0_v + (it.h + 1) * p.gh_v) - __ldg(p.cl_unit0_v + it.h * p.gh_v);
+                const uint32_t id = ID | ((uint32_t)(4 * nuv) << 17);
+                if (!mbar_sleep_warp(bar(B_OEMPTY), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
+                uint32_t acc = 0u;
+#pragma unroll 1
+                for (int kt = 0; kt < it.n_kt && ok; ++kt, ++n_v) {
+                    const uint32_t st = g.v_stages == 2 ? n_v & 1 : 0u, ph = g.v_stages == 2 ? (n_v >> 1) & 1 : n_v & 1;
+                    if (!mbar_sleep_warp(bar(B_VFULL + st), ph, s_abort)) { ok = false; break; }
+                    const uint32_t b0 = dv + st * v_step;
+                    if constexpr (ALT) {
+                        const uint32_t stream = kt & 1, n_p = stream ? n_p1 : n_p0;
+                        if (!mbar_sleep_warp(bar(B_PFULL + stream), n_p & 1, s_abort)) { ok = false; break; }
+                        tc::tc_fence_after();
+                        const uint32_t a0 = dp + (g.p_tiles == 2 ? stream * (BM * 128 >> 4) : 0u);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (nuv > 0) mma<2>(tmem, a0 + 2 * k, b0 + 2 * k, id, k == 0 ? acc : 1u);
+                        if (stream) ++n_p1; else ++n_p0;
+                        // one buffer for both streams: it goes to the stream of the tile that follows
+                        commit(bar(B_PEMPTY + (g.p_tiles == 2 ? stream : kt + 1 < it.n_kt ? stream ^ 1u : 0u)));
+                    } else {
+#pragma unroll
+                        for (int half = 0; half < 2; ++half) {
+                            if (!mbar_sleep_warp(bar(B_PFULL + half), n_v & 1, s_abort)) { ok = false; break; }
+                            tc::tc_fence_after();
+                            if (nuv > 0) {
+                                mma<0>(tmem, dp + 4 * half, b0 + 4 * half, id, half == 0 ? acc : 1u);
+                                mma<0>(tmem, dp + 4 * half + 2, b0 + 4 * half + 2, id, 1u);
+                            }
+                            commit(bar(B_PEMPTY + half));
+                        }
+                    }
+                    acc = 1u;
+                    if (ok) commit(bar(B_VEMPTY + st));
+                }
                 if (ok) commit(bar(B_OFULL));
             }
-            if (!ok) {
-                commit(bar(B_DRAIN));
-                mbar_wait(bar(B_DRAIN), 0, s_abort, false);
-            }
         }
-    } else if (warp < V_WARP0) {
-        // ---------------------------------------------------------------- keys (and queries)
+        if (warp < 3 && !ok) {
+            commit(bar(B_DRAIN + warp));
+            tc::mbar_wait(bar(B_DRAIN + warp), 0, s_abort, false);
+        }
+    } else if (warp < S_WARP0) {
+        // ---------------------------------------------------------------- loaders: keys and queries (warps 4-7), values and outputs (8-11)
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_LOAD));
-        const int kw = warp - K_WARP0, kt_id = tid - 32 * K_WARP0;             // 0..3, 0..127
-        constexpr int ROWS_W = KEYS / 4;                                       // key rows that a warp copies and unpacks
-        const bool direct = MODE != KV && p.bits_k == 8;                       // bytes already: copied straight into the operand tile
-        // copies of a tile's packed rows (eight lanes per row), into the raw buffer or, swizzled, into operand stage st
-        auto copy_rows = [&](const Item& it, int kt, uint32_t st) {
-            const int uk0 = __ldg(p.cl_unit0_k + it.h * p.gh_k), nuk = __ldg(p.cl_unit0_k + (it.h + 1) * p.gh_k) - uk0;
-            const int win = (4 * p.bits_k * uk0) & ~15, n16 = ((4 * p.bits_k * uk0 - win) + 4 * p.bits_k * nuk + 15) >> 4;
-            const int r0 = lane >> 3, c0 = lane & 7;
-#pragma unroll 2
-            for (int i = 0; i < ROWS_W / 4; ++i) {
-                const int r = ROWS_W * kw + 4 * i + r0, j = kt * KEYS + r;
-                const bool okr = j < p.Tk;
-                const uint8_t* src = p.k + ((int64_t)it.seq * p.Tk + (okr ? j : 0)) * p.k_row_bytes + win;
-                for (int c = c0; c < n16; c += 8) {
-                    const uint32_t dst = direct ? base + g.off_k + st * g.k_stage + (c >> 3) * K_ATOM + r * 128 + (((c & 7) ^ (r & 7)) << 4)
-                                                : base + g.off_rawk + r * g.pitch_k + 16 * c;
-                    cp_async16(dst, src + 16 * c, okr ? 16 : 0);
+        constexpr int ROWS_W = KEYS / 4;                                       // rows of a tile that a warp copies
+        const int lw = warp & 3, lt = tid & 127;
+        const int r0 = ROWS_W * lw + (lane >> 3), c0 = lane & 7;               // eight lanes per row; my rows are r0 + 4 i
+        bool ok = true;
+        // The tile that is being fetched (`nx`) and the one that is being worked on (`cu`), one tile behind
+        struct Tile { int idx, t, n_t, kt; Item it; int u0, nu; };
+        const bool is_k = warp < V_WARP0;
+        Tile nx, cu;
+        nx.idx = (int)blockIdx.x - (int)gridDim.x; nx.t = 0; nx.n_t = 1; nx.kt = 0;
+        // keys: every item's tiles twice; values: once
+        auto advance = [&]() {
+            ++nx.kt;
+            if (++nx.t == nx.n_t) {
+                nx.idx += gridDim.x;
+                nx.t = 0;
+                if (nx.idx >= g.n_items) return false;
+                nx.it = item_of(p, g, nx.idx, KEYS);
+                nx.n_t = is_k ? 2 * nx.it.n_kt : nx.it.n_kt;
+                const int32_t* u = is_k ? p.cl_unit0_k + nx.it.h * p.gh_k : p.cl_unit0_v + nx.it.h * p.gh_v;
+                nx.u0 = __ldg(u);
+                nx.nu = __ldg(u + (is_k ? p.gh_k : p.gh_v)) - nx.u0;
+            }
+            if (nx.t == 0 || nx.kt == nx.it.n_kt) nx.kt = 0;
+            return true;
+        };
+        const uint8_t* const codes = is_k ? p.k : p.v;
+        const int64_t row_bytes = is_k ? p.k_row_bytes : p.v_row_bytes;
+        const int bits = is_k ? p.bits_k : p.bits_v;
+        // Copies of the packed rows of the tile to fetch: row r goes to dst(r, c), chunk c of 16 bytes. Rows past the last key: zeros.
+        auto copy_rows = [&](auto dst) {
+            const int win = (4 * bits * nx.u0) & ~15, n16 = ((4 * bits * nx.u0 - win) + 4 * bits * nx.nu + 15) >> 4;
+            const int rows = p.Tk - nx.kt * KEYS;
+            const uint8_t* from = codes + ((int64_t)nx.it.seq * p.Tk + nx.kt * KEYS + r0) * row_bytes + win + 16 * c0;
+#pragma unroll 1
+            for (int c = c0; c < n16; c += 8, from += 128) {
+                const uint8_t* f = from;
+#pragma unroll
+                for (int i = 0; i < ROWS_W / 4; ++i, f += 4 * row_bytes) {
+                    const bool in = r0 + 4 * i < rows;
+                    cp_async16(dst(r0 + 4 * i, c), in ? f : codes, in ? 16 : 0);       // (size 0 reads nothing)
                 }
             }
         };
-        uint32_t n_k = 0, n_item = 0;
-        bool ok = true;
-        int idx = blockIdx.x;
-        if (idx < g.n_items) copy_rows(item_of(p, g, idx, KEYS), 0, 0u);       // (stage 0 is free at the start)
-        cp_async_commit();
-        for (; idx < g.n_items && ok; idx += gridDim.x, ++n_item) {
-            const Item it = item_of(p, g, idx, KEYS);
-            const int uk0 = __ldg(p.cl_unit0_k + it.h * p.gh_k), nuk = __ldg(p.cl_unit0_k + (it.h + 1) * p.gh_k) - uk0;
-            const int off_b = (4 * p.bits_k * uk0) & 15;
-            // ---- the item's queries
-            if (!mbar_wait(bar(B_QEMPTY), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
-            const int i0 = it.qt * BM;
-            if constexpr (MODE == KV) {
-                // a lane takes up to four pairs of positions (operand order: codes 0, 2, 1, 3, 4, 6, 5, 7 of every eight, the order
-                // in which the key codes come out of their words) and gathers their channels row by row
-                int ca[4], cb[4];
+        // KV: the queries as fp16 in operand order (codes 0, 2, 1, 3, 4, 6, 5, 7 of every eight positions, the order in which
+        // the key codes come out of their words). Eight warps; a lane takes up to four pairs of positions and gathers their
+        // channels row by row.
+        auto gather_queries = [&](const Item& it, uint32_t n_item) {
+            const int uk0 = __ldg(p.cl_unit0_k + it.h * p.gh_k), nuk = __ldg(p.cl_unit0_k + (it.h + 1) * p.gh_k) - uk0, nu = units_seen(nuk);
+            int ca[4], cb[4];
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int p2 = lane + 32 * k, code = (p2 >> 2) * 8 + (p2 & 1) + 4 * ((p2 >> 1) & 1), pos = 32 * uk0 + code;
-                    const bool in = p2 < 16 * nuk;            // (a head without channels: no pair is, zeros are written)
-                    ca[k] = in && __ldg(p.jidx_k + pos) >= 0 ? (int)__ldg(p.src_k + pos) : -1;
-                    cb[k] = in && __ldg(p.jidx_k + pos + 2) >= 0 ? (int)__ldg(p.src_k + pos + 2) : -1;
-                }
-#pragma unroll 2
-                for (int r = kw; r < BM; r += 4) {
-                    const bool okr = i0 + r < p.Tq;
-                    const __half* row = p.q_f16 + ((int64_t)it.seq * p.Tq + (okr ? i0 + r : 0)) * p.ldq;
+            for (int k = 0; k < 4; ++k) {
+                const int p2 = lane + 32 * k, code = (p2 >> 2) * 8 + (p2 & 1) + 4 * ((p2 >> 1) & 1), pos = 32 * uk0 + code;
+                const bool in = p2 < 16 * nuk;                // (a head without channels: no pair is, zeros are written)
+                ca[k] = in && __ldg(p.jidx_k + pos) >= 0 ? (int)__ldg(p.src_k + pos) : -1;
+                cb[k] = in && __ldg(p.jidx_k + pos + 2) >= 0 ? (int)__ldg(p.src_k + pos + 2) : -1;
+            }
+            if (!mbar_sleep(bar(B_QEMPTY), (n_item & 1) ^ 1, s_abort)) return false;
+            const int i0 = it.qt * BM;
+#pragma unroll 1
+            for (int r4 = (warp - K_WARP0) * 16; r4 < (warp - K_WARP0) * 16 + 16; r4 += 2) {
+                uint32_t v[2][4];
+#pragma unroll
+                for (int rr = 0; rr < 2; ++rr) {
+                    const bool okr = i0 + r4 + rr < p.Tq;
+                    const __half* row = p.q_f16 + ((int64_t)it.seq * p.Tq + (okr ? i0 + r4 + rr : 0)) * p.ldq;
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        const int p2 = lane + 32 * k;
-                        if (p2 < 16 * units_seen(nuk)) {
-                            const uint32_t lo = okr && ca[k] >= 0 ? (uint32_t)__half_as_ushort(row[ca[k]]) : 0u;
-                            const uint32_t hi = okr && cb[k] >= 0 ? (uint32_t)__half_as_ushort(row[cb[k]]) : 0u;
-                            sts32(base + k * ATOM_Q + r * 128 + (((lane >> 2) ^ (r & 7)) << 4) + 4 * (lane & 3), lo | (hi << 16));
-                        }
+                        const uint32_t lo = okr && ca[k] >= 0 ? (uint32_t)__half_as_ushort(row[ca[k]]) : 0u;
+                        const uint32_t hi = okr && cb[k] >= 0 ? (uint32_t)__half_as_ushort(row[cb[k]]) : 0u;
+                        v[rr][k] = lo | (hi << 16);
                     }
                 }
-            } else {
-#pragma unroll 2
-                for (int i = kt_id; i < BM * units_seen(nuk); i += 128) {
-                    const int r = i / units_seen(nuk), u = i - r * units_seen(nuk);
-                    uint32_t o[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-                    if (u < nuk && i0 + r < p.Tq) load_unit(p.q + ((int64_t)it.seq * p.Tq + i0 + r) * p.q_row_bytes, uk0 + u, p.bits_q, o);
-                    const uint32_t d = base + (u >> 2) * ATOM_Q + r * 128, c = 2 * (u & 3), sw = r & 7;
-                    sts128(d + ((c ^ sw) << 4), o[0], o[1], o[2], o[3]);
-                    sts128(d + (((c + 1) ^ sw) << 4), o[4], o[5], o[6], o[7]);
-                }
+#pragma unroll
+                for (int rr = 0; rr < 2; ++rr)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        if (lane + 32 * k < 16 * nu) sts32(base + k * ATOM_Q + (r4 + rr) * 128 + (((lane >> 2) ^ ((r4 + rr) & 7)) << 4) + 4 * (lane & 3), v[rr][k]);
             }
             tc::fence_proxy_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(B_QFULL));
-            // integer calls: -s^Q s^K z^Q qk_scale log2(e) of unit `lane`
-            float czq = 0.f;
-            if constexpr (MODE != KV) {
-                if (lane < nuk) {
-                    const float2 q = __ldg(p.unit_sz_q + uk0 + lane), k = __ldg(p.unit_sz_k + uk0 + lane);
-                    czq = -(q.x * k.x * p.qk_scale_log2e) * q.y;
-                }
-            }
-            // ---- the key tiles, twice
-            const int n_tiles = 2 * it.n_kt;
+            return true;
+        };
+        bool have = advance();
+        uint32_t n_item = 0;
+        if (is_k) {
+            // ------------------------------------------------------------ keys
+            const bool direct = MODE != KV && p.bits_k == 8;                   // bytes already: copied straight into the operand tile
+            float czq = 0.f;                      // integer calls: -s^Q s^K z^Q qk_scale log2(e) of unit `lane`
+            uint32_t seq[2] = {0, 0};             // KV: tiles of each stage (stream) so far
+            // iteration n fetches tile n and works on tile n - 1
 #pragma unroll 1
-            for (int t = 0; t < n_tiles; ++t, ++n_k) {
-                const uint32_t st = n_k & 1;
-                const uint32_t tile = base + g.off_k + st * g.k_stage;
-                // the copies of the tile after this one (of the next item after the last)
-                auto copy_next = [&]() {
-                    if (t + 1 < n_tiles) copy_rows(it, t + 1 < it.n_kt ? t + 1 : t + 1 - it.n_kt, st ^ 1u);
-                    else if (idx + (int)gridDim.x < g.n_items) copy_rows(item_of(p, g, idx + gridDim.x, KEYS), 0, st ^ 1u);
-                    cp_async_commit();
-                };
-                if constexpr (MODE == KV) {
-                    // thread = (row, parity of the unit): up to four units, as nibble words or bytes
-                    const int r = kt_id >> 1, odd = kt_id & 1;
-                    const uint32_t raw = base + g.off_rawk + r * g.pitch_k + off_b;
-                    uint4 w[4][2];
-                    cp_async_wait<0>();
-                    __syncwarp();
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const int u = 2 * i + odd;
-                        w[i][0] = w[i][1] = make_uint4(0u, 0u, 0u, 0u);
-                        if (u < nuk) {
-                            if (p.bits_k == 8) { w[i][0] = lds128(raw + 32 * u); w[i][1] = lds128(raw + 32 * u + 16); }
-                            else w[i][0] = nibbles(raw, u, p.bits_k);
-                        }
-                    }
-                    __syncwarp();
-                    copy_next();
-                    if (!mbar_wait(bar(B_KEMPTY + st), ((n_k >> 1) & 1) ^ 1, s_abort)) { ok = false; break; }
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        if (2 * i + odd < units_seen(nuk)) {
-                            const uint32_t d = tile + i * K_ATOM + r * 128, sw = r & 7;
-                            const uint32_t a[8] = {w[i][0].x, w[i][0].y, w[i][0].z, w[i][0].w, w[i][1].x, w[i][1].y, w[i][1].z, w[i][1].w};
-#pragma unroll
-                            for (int c = 0; c < 4; ++c) {                          // eight codes = one chunk
-                                const uint32_t at = d + (((4 * odd + c) ^ sw) << 4);
-                                if (p.bits_k == 8) sts128(at, byte_half<0>(a[2 * c]), byte_half<8>(a[2 * c]), byte_half<0>(a[2 * c + 1]), byte_half<8>(a[2 * c + 1]));
-                                else sts128(at, nib_half<0>(a[c]), nib_half<8>(a[c]), nib_half<4>(a[c]), nib_half<12>(a[c]));
-                            }
-                        }
-                    }
-                } else {
-                    const int r = kt_id, sw = r & 7;
-                    float col = 0.f;
+            for (uint32_t n = 0; ok; ++n) {
+                auto fetch = [&]() {
                     if (direct) {
-                        // the next tile's copies go into the other stage: its products must have read it
-                        const bool more = t + 1 < n_tiles || idx + (int)gridDim.x < g.n_items;
-                        if (more && !mbar_wait(bar(B_KEMPTY + (st ^ 1u)), (((n_k + 1) >> 1) & 1) ^ 1, s_abort)) { ok = false; break; }
-                        copy_next();
-                        cp_async_wait<1>();
-                        __syncwarp();
-#pragma unroll 1
-                        for (int u = 0; u < nuk; ++u) {
-                            const uint32_t d = tile + (u >> 2) * K_ATOM + r * 128, c = 2 * (u & 3);
-                            const uint4 a = lds128(d + ((c ^ sw) << 4)), b = lds128(d + (((c + 1) ^ sw) << 4));
-                            unsigned s = __dp4a(a.x, 0x01010101u, 0u);
-                            s = __dp4a(a.y, 0x01010101u, s); s = __dp4a(a.z, 0x01010101u, s); s = __dp4a(a.w, 0x01010101u, s);
-                            s = __dp4a(b.x, 0x01010101u, s); s = __dp4a(b.y, 0x01010101u, s); s = __dp4a(b.z, 0x01010101u, s); s = __dp4a(b.w, 0x01010101u, s);
-                            col = __fmaf_rn(__shfl_sync(0xffffffffu, czq, u), (float)s, col);
-                        }
+                        const uint32_t to = base + g.off_k + (n & 1) * g.k_stage;
+                        copy_rows([&](int r, int c) { return to + (c >> 3) * K_ATOM + r * 128 + (((c & 7) ^ (r & 7)) << 4); });
                     } else {
-                        const uint32_t raw = base + g.off_rawk + r * g.pitch_k + off_b;
-                        uint4 w[MAX_UNITS];
-                        cp_async_wait<0>();
-                        __syncwarp();
-#pragma unroll
-                        for (int u = 0; u < MAX_UNITS; ++u) w[u] = u < nuk ? nibbles(raw, u, p.bits_k) : make_uint4(0u, 0u, 0u, 0u);
-                        __syncwarp();
-                        copy_next();
-                        if (!mbar_wait(bar(B_KEMPTY + st), ((n_k >> 1) & 1) ^ 1, s_abort)) { ok = false; break; }
-#pragma unroll
-                        for (int u = 0; u < MAX_UNITS; ++u) {
-                            if (u < units_seen(nuk)) {
-                                const uint32_t d = tile + (u >> 2) * K_ATOM + r * 128, c = 2 * (u & 3);
-                                const uint32_t o[8] = {w[u].x & 0x0F0F0F0Fu, (w[u].x >> 4) & 0x0F0F0F0Fu, w[u].y & 0x0F0F0F0Fu, (w[u].y >> 4) & 0x0F0F0F0Fu,
-                                                       w[u].z & 0x0F0F0F0Fu, (w[u].z >> 4) & 0x0F0F0F0Fu, w[u].w & 0x0F0F0F0Fu, (w[u].w >> 4) & 0x0F0F0F0Fu};
+                        const uint32_t to = base + g.off_rawk + (g.rawk_stages == 2 ? (n & 1) * g.rawk_stage : 0);
+                        copy_rows([&](int r, int c) { return to + r * g.pitch_k + 16 * c; });
+                    }
+                };
+                const bool ahead = direct || g.rawk_stages == 2 || n == 0;     // (one raw buffer: it is refilled after it was read)
+                if (have && ahead) {
+                    // (copied into the operand tile itself: its products must have read it)
+                    if (direct && !mbar_sleep(bar(B_KEMPTY + (n & 1)), ((n >> 1) & 1) ^ 1, s_abort)) { ok = false; break; }
+                    fetch();
+                }
+                cp_async_commit();
+                if (n > 0) {
+                    const uint32_t m = n - 1, st = ALT ? cu.kt & 1 : m & 1, ph = ALT ? (st ? seq[1]++ : seq[0]++) : m >> 1;
+                    const uint32_t tile = base + g.off_k + st * g.k_stage;
+                    const int nuk = cu.nu, nu = units_seen(nuk);
+                    if (cu.t == 0) {
+                        // ---- a new item's queries
+                        if constexpr (MODE == KV) {
+                            if (!gather_queries(cu.it, n_item)) { ok = false; break; }
+                        } else {
+                            const int i = cu.it.qt * BM + lt;
+                            const uint8_t* q_row = p.q + ((int64_t)cu.it.seq * p.Tq + (i < p.Tq ? i : 0)) * p.q_row_bytes;
+                            czq = 0.f;
+                            if (lane < nuk) {
+                                const float2 q = __ldg(p.unit_sz_q + cu.u0 + lane), k = __ldg(p.unit_sz_k + cu.u0 + lane);
+                                czq = -(q.x * k.x * p.qk_scale_log2e) * q.y;
+                            }
+                            if (!mbar_sleep(bar(B_QEMPTY), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
+#pragma unroll 2
+                            for (int u = 0; u < nu; ++u) {
+                                uint32_t o[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+                                if (u < nuk && i < p.Tq) load_unit(q_row, cu.u0 + u, p.bits_q, o);
+                                const uint32_t d = base + (u >> 2) * ATOM_Q + lt * 128, c = 2 * (u & 3), sw = lt & 7;
                                 sts128(d + ((c ^ sw) << 4), o[0], o[1], o[2], o[3]);
                                 sts128(d + (((c + 1) ^ sw) << 4), o[4], o[5], o[6], o[7]);
-                                unsigned s = 0u;
-#pragma unroll
-                                for (int e = 0; e < 8; ++e) s = __dp4a(o[e], 0x01010101u, s);
-                                col = __fmaf_rn(__shfl_sync(0xffffffffu, czq, u), (float)s, col);
                             }
+                            tc::fence_proxy_async();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive(bar(B_QFULL));
                         }
+                        ++n_item;
                     }
-                    s_col[(n_k & 3) * KEYS + r] = col;
-                }
-                tc::fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar(B_KFULL + st));
-            }
-        }
-        cp_async_wait<0>();
-    } else if (warp < S_WARP0) {
-        // ---------------------------------------------------------------- values
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_LOAD));
-        const int vw = warp - V_WARP0;
-        constexpr int ROWS_W = KEYS / 4;
-        auto copy_rows = [&](const Item& it, int kt) {
-            const int uv0 = __ldg(p.cl_unit0_v + it.h * p.gh_v), nuv = __ldg(p.cl_unit0_v + (it.h + 1) * p.gh_v) - uv0;
-            const int win = (4 * p.bits_v * uv0) & ~15, n16 = ((4 * p.bits_v * uv0 - win) + 4 * p.bits_v * nuv + 15) >> 4;
-            const int r0 = lane >> 3, c0 = lane & 7;
+                    if (ahead && have) cp_async_wait<1>(); else cp_async_wait<0>();
+                    __syncwarp();                                              // (a warp unpacks the rows that it copied)
+                    if (!direct && !mbar_sleep(bar(B_KEMPTY + st), (ph & 1) ^ 1, s_abort)) { ok = false; break; }
+                    const uint32_t raw0 = base + g.off_rawk + (g.rawk_stages == 2 ? (m & 1) * g.rawk_stage : 0) + ((4 * p.bits_k * cu.u0) & 15);
+                    if constexpr (MODE == KV) {
+                        // thread = (row, parity of the unit)
+                        const int r = lt >> 1, odd = lt & 1, sw = r & 7;
+                        const uint32_t raw = raw0 + r * g.pitch_k;
 #pragma unroll 2
-            for (int i = 0; i < ROWS_W / 4; ++i) {
-                const int r = ROWS_W * vw + 4 * i + r0, j = kt * KEYS + r;
-                const bool okr = j < p.Tk;
-                const uint8_t* src = p.v + ((int64_t)it.seq * p.Tk + (okr ? j : 0)) * p.v_row_bytes + win;
-                for (int c = c0; c < n16; c += 8) cp_async16(base + g.off_rawv + r * g.pitch_v + 16 * c, src + 16 * c, okr ? 16 : 0);
-            }
-        };
-        uint32_t n_v = 0, n_x = 0, n_item = 0;
-        bool ok = true;
-        // all four warps have passed this point (bounded, unlike a named barrier)
-        auto group_sync = [&]() {
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(B_XV));
-            const bool done = mbar_wait(bar(B_XV), n_x & 1, s_abort);
-            ++n_x;
-            return done;
-        };
-        int idx = blockIdx.x;
-        if (idx < g.n_items) copy_rows(item_of(p, g, idx, KEYS), 0);
-        cp_async_commit();
-        for (; idx < g.n_items && ok; idx += gridDim.x, ++n_item) {
-            const Item it = item_of(p, g, idx, KEYS);
-            const int uv0 = __ldg(p.cl_unit0_v + it.h * p.gh_v), nuv = __ldg(p.cl_unit0_v + (it.h + 1) * p.gh_v) - uv0;
-            const int off_b = (4 * p.bits_v * uv0) & 15;
-            // the previous item's output rows have left the region
-            if (!mbar_wait(bar(B_OUT), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
-#pragma unroll 1
-            for (int kt = 0; kt < it.n_kt; ++kt, ++n_v) {
-                const uint32_t st = g.v_stages == 2 ? n_v & 1 : 0u, ph = g.v_stages == 2 ? (n_v >> 1) & 1 : n_v & 1;
-                cp_async_wait<0>();
-                if (!group_sync()) { ok = false; break; }                      // everyone's copies of the tile have landed
-                if (!mbar_wait(bar(B_VEMPTY + st), ph ^ 1, s_abort)) { ok = false; break; }
-                const uint32_t tile = base + g.off_v + st * g.v_stage, raw = base + g.off_rawv + off_b;
-                if constexpr (MODE == KV) {
-                    // lane = (chunk c8 = 4 hf + v of the 64 slots, word j of the unit): keys 16 a + 8 hf + 2 v + {0, 1}, a = 0..3
-                    const int c8 = lane & 7, j = lane >> 3, key0 = 8 * (c8 >> 2) + 2 * (c8 & 3);
-#pragma unroll 1
-                    for (int u = vw; u < nuv; u += 4) {
-                        uint32_t lo[8], hi[8];                                 // my eight codes of the eight keys (hi: bytes 4..7 of 8-bit codes)
+                        for (int u = odd; u < nu; u += 2) {
+                            const uint32_t d = tile + (u >> 1) * K_ATOM + r * 128;
+                            if (p.bits_k == 8) {
+                                uint4 w[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
+                                if (u < nuk) { w[0] = lds128(raw + 32 * u); w[1] = lds128(raw + 32 * u + 16); }
+                                const uint32_t a[8] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w};
 #pragma unroll
-                        for (int a = 0; a < 8; ++a) {
-                            const uint32_t row = raw + (16 * (a >> 1) + key0 + (a & 1)) * g.pitch_v;
-                            hi[a] = 0u;
-                            if (p.bits_v == 8) { lo[a] = lds32(row + 32 * u + 8 * j); hi[a] = lds32(row + 32 * u + 8 * j + 4); }
-                            else if (p.bits_v == 4) lo[a] = lds32(row + 16 * u + 4 * j);
-                            else {
-                                const uint32_t x = lds32(row + 12 * u), y = lds32(row + 12 * u + 4), z = lds32(row + 12 * u + 8);
-                                const uint32_t tail = ((x >> 3) & 0x11111111u) | ((y >> 2) & 0x22222222u) | ((z >> 1) & 0x44444444u);
-                                lo[a] = j == 3 ? tail : (j == 0 ? x : j == 1 ? y : z) & 0x77777777u;
+                                for (int c = 0; c < 4; ++c)                        // eight codes = one chunk
+                                    sts128(d + (((4 * odd + c) ^ sw) << 4), byte_half<0>(a[2 * c]), byte_half<8>(a[2 * c]), byte_half<0>(a[2 * c + 1]), byte_half<8>(a[2 * c + 1]));
+                            } else {
+                                const uint4 w = u < nuk ? nibbles(raw, u, p.bits_k) : make_uint4(0u, 0u, 0u, 0u);
+                                const uint32_t a[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+                                for (int c = 0; c < 4; ++c)
+                                    sts128(d + (((4 * odd + c) ^ sw) << 4), nib_half<0>(a[c]), nib_half<8>(a[c]), nib_half<4>(a[c]), nib_half<12>(a[c]));
                             }
                         }
-                        const uint32_t d = tile + (32 * u + 8 * j) * 128;
-                        // codes e and e + 4 (nibbles) or e (bytes) of the four key pairs = one chunk of position row 8 j + e; row & 7 = e
-                        auto put = [&](int e, const uint32_t (&h4)[4]) { sts128(d + e * 128 + ((c8 ^ e) << 4), h4[0], h4[1], h4[2], h4[3]); };
-                        if (p.bits_v == 8) {
-#pragma unroll
-                            for (int half = 0; half < 4; ++half) {             // codes 2 half, 2 half + 1
-                                uint32_t x[4], h0[4], h1[4];
-#pragma unroll
-                                for (int a = 0; a < 4; ++a) {
-                                    const uint32_t p0 = half < 2 ? lo[2 * a] : hi[2 * a], p1 = half < 2 ? lo[2 * a + 1] : hi[2 * a + 1];
-                                    x[a] = __byte_perm(p0, p1, (half & 1) ? 0x7632 : 0x5410);
-                                    h0[a] = byte_half<0>(x[a]); h1[a] = byte_half<8>(x[a]);
-                                }
-                                put(2 * half, h0); put(2 * half + 1, h1);
+                    } else {
+                        const int r = lt, sw = r & 7;
+                        const uint32_t raw = raw0 + r * g.pitch_k;
+                        float col = 0.f;
+#pragma unroll 2
+                        for (int u = 0; u < nu; ++u) {
+                            const uint32_t d = tile + (u >> 2) * K_ATOM + r * 128, c = 2 * (u & 3);
+                            uint32_t o[8];
+                            if (direct) {
+                                const uint4 a = lds128(d + ((c ^ sw) << 4)), b = lds128(d + (((c + 1) ^ sw) << 4));
+                                o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
+                            } else {
+                                const uint4 w = u < nuk ? nibbles(raw, u, p.bits_k) : make_uint4(0u, 0u, 0u, 0u);
+                                o[0] = w.x & 0x0F0F0F0Fu; o[1] = (w.x >> 4) & 0x0F0F0F0Fu; o[2] = w.y & 0x0F0F0F0Fu; o[3] = (w.y >> 4) & 0x0F0F0F0Fu;
+                                o[4] = w.z & 0x0F0F0F0Fu; o[5] = (w.z >> 4) & 0x0F0F0F0Fu; o[6] = w.w & 0x0F0F0F0Fu; o[7] = (w.w >> 4) & 0x0F0F0F0Fu;
+                                sts128(d + ((c ^ sw) << 4), o[0], o[1], o[2], o[3]);
+                                sts128(d + (((c + 1) ^ sw) << 4), o[4], o[5], o[6], o[7]);
                             }
-                        } else {
+                            unsigned s = 0u;
 #pragma unroll
-                            for (int half = 0; half < 2; ++half) {             // codes 2 half, 2 half + 1 and those + 4
-                                uint32_t x[4], h0[4], h1[4], h4[4], h5[4];
-#pragma unroll
-                                for (int a = 0; a < 4; ++a) {
-                                    x[a] = __byte_perm(lo[2 * a], lo[2 * a + 1], half ? 0x7632 : 0x5410);
-                                    h0[a] = nib_half<0>(x[a]); h4[a] = nib_half<4>(x[a]); h1[a] = nib_half<8>(x[a]); h5[a] = nib_half<12>(x[a]);
-                                }
-                                put(2 * half, h0); put(2 * half + 1, h1); put(2 * half + 4, h4); put(2 * half + 5, h5);
-                            }
+                            for (int e = 0; e < 8; ++e) s = __dp4a(o[e], 0x01010101u, s);
+                            col = __fmaf_rn(__shfl_sync(0xffffffffu, czq, u), (float)s, col);
                         }
+                        s_col[(m & 3) * KEYS + r] = col;
                     }
-                } else {
-                    // lane w: keys w, w + 32, w + 64, w + 96 of unit u; word w of the 32 positions' rows
-                    const uint32_t wc = (uint32_t)lane >> 2, wo = 4 * ((uint32_t)lane & 3);
+                    tc::fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(B_KFULL + st));
+                    if (have && !ahead) { fetch(); cp_async_commit(); }
+                }
+                if (!have) break;
+                cu = nx;
+                have = advance();
+            }
+        } else {
+            // ------------------------------------------------------------ values and outputs
+            // KV: row r of the tile is staged at row blk + 4 y + 8 (2 b + s), r = 16 blk + 4 b + 2 y + s (see v_tile below)
+            auto staged_row = [](int r) { return MODE == KV ? (r >> 4) + 4 * ((r >> 1) & 1) + 8 * (2 * ((r >> 2) & 3) + (r & 1)) : r; };
+            uint32_t n_x = 0;
+            // all four warps have passed this point (bounded, unlike a named barrier)
+            auto group_sync = [&]() {
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(B_XV));
+                const bool done = mbar_sleep(bar(B_XV), n_x & 1, s_abort);
+                ++n_x;
+                return done;
+            };
+            // iteration n works on tile n - 1, then fetches tile n
 #pragma unroll 1
-                    for (int u = vw; u < nuv; u += 4) {
-                        const uint32_t d = tile + 32 * u * 128 + wo;
-                        auto put = [&](int pos, uint32_t x) { sts32(d + pos * 128 + ((wc ^ (pos & 7)) << 4), x); };
-                        // 4 x 4 byte transpose: out[i] = byte i of the four rows
-                        auto transpose = [](uint32_t a, uint32_t b, uint32_t c, uint32_t e, uint32_t (&out)[4]) {
-                            const uint32_t x01l = __byte_perm(a, b, 0x5140), x01h = __byte_perm(a, b, 0x7362);
-                            const uint32_t x23l = __byte_perm(c, e, 0x5140), x23h = __byte_perm(c, e, 0x7362);
-                            out[0] = __byte_perm(x01l, x23l, 0x5410); out[1] = __byte_perm(x01l, x23l, 0x7632);
-                            out[2] = __byte_perm(x01h, x23h, 0x5410); out[3] = __byte_perm(x01h, x23h, 0x7632);
-                        };
-                        if (p.bits_v == 8) {
+            for (uint32_t n = 0; ok; ++n) {
+                const int uv0 = cu.u0, nuv = cu.nu;
+                const Item& it = cu.it;
+                if (n > 0) {
+                    const uint32_t raw = base + g.off_rawv + ((4 * p.bits_v * uv0) & 15), n_v = n - 1;
+                    const uint32_t st = g.v_stages == 2 ? n_v & 1 : 0u, ph = g.v_stages == 2 ? (n_v >> 1) & 1 : n_v & 1;
+                    cp_async_wait<0>();
+                    if (!group_sync()) { ok = false; break; }                  // everyone's copies of the tile have landed
+                    if (!mbar_sleep(bar(B_VEMPTY + st), ph ^ 1, s_abort)) { ok = false; break; }
+                    const uint32_t tile = base + g.off_v + st * g.v_stage;
+                    if constexpr (MODE == KV) {
+                        // lane = (chunk c8 of the 64 slots, word j of the unit). Chunk c8 = 2 blk + y holds the pairs b = 0..3 of keys
+                        // 16 blk + 4 b + 2 y + {0, 1}: staged rows blk + 4 y + 8 (2 b + s), so the eight chunks' rows are in different banks
+                        const int c8 = lane & 7, j = lane >> 3;
+                        const uint32_t rows = raw + ((c8 >> 1) + 4 * (c8 & 1)) * g.pitch_v;
+#pragma unroll 1
+                        for (int u = lw; u < nuv; u += 4) {
+                            const uint32_t d = tile + (32 * u + 8 * j) * 128;
+                            // one chunk of position row 8 j + e; row & 7 = e
+                            auto put = [&](int e, const uint32_t (&h4)[4]) { sts128(d + e * 128 + ((c8 ^ e) << 4), h4[0], h4[1], h4[2], h4[3]); };
+                            if (p.bits_v == 8) {
 #pragma unroll
-                            for (int half = 0; half < 2; ++half) {
+                                for (int half = 0; half < 2; ++half) {             // codes 4 half .. 4 half + 3
+                                    uint32_t x[8];
+#pragma unroll
+                                    for (int a = 0; a < 8; ++a) x[a] = lds32(rows + 8 * a * g.pitch_v + 32 * u + 8 * j + 4 * half);
+#pragma unroll
+                                    for (int q = 0; q < 2; ++q) {
+                                        uint32_t h0[4], h1[4];
+#pragma unroll
+                                        for (int b = 0; b < 4; ++b) {
+                                            const uint32_t y = __byte_perm(x[2 * b], x[2 * b + 1], q ? 0x7632 : 0x5410);
+                                            h0[b] = byte_half<0>(y); h1[b] = byte_half<8>(y);
+                                        }
+                                        put(4 * half + 2 * q, h0); put(4 * half + 2 * q + 1, h1);
+                                    }
+                                }
+                            } else {
+                                uint32_t x[8];
+#pragma unroll
+                                for (int a = 0; a < 8; ++a) {
+                                    const uint32_t row = rows + 8 * a * g.pitch_v;
+                                    if (p.bits_v == 4) x[a] = lds32(row + 16 * u + 4 * j);
+                                    else {
+                                        const uint32_t w0 = lds32(row + 12 * u), w1 = lds32(row + 12 * u + 4), w2 = lds32(row + 12 * u + 8);
+                                        const uint32_t tail = ((w0 >> 3) & 0x11111111u) | ((w1 >> 2) & 0x22222222u) | ((w2 >> 1) & 0x44444444u);
+                                        x[a] = j == 3 ? tail : (j == 0 ? w0 : j == 1 ? w1 : w2) & 0x77777777u;
+                                    }
+                                }
+#pragma unroll
+                                for (int q = 0; q < 2; ++q) {                      // codes 2 q, 2 q + 1 and those + 4
+                                    uint32_t y[4], h[4];
+#pragma unroll
+                                    for (int b = 0; b < 4; ++b) y[b] = __byte_perm(x[2 * b], x[2 * b + 1], q ? 0x7632 : 0x5410);
+#pragma unroll
+                                    for (int b = 0; b < 4; ++b) h[b] = nib_half<0>(y[b]);
+                                    put(2 * q, h);
+#pragma unroll
+                                    for (int b = 0; b < 4; ++b) h[b] = nib_half<8>(y[b]);
+                                    put(2 * q + 1, h);
+#pragma unroll
+                                    for (int b = 0; b < 4; ++b) h[b] = nib_half<4>(y[b]);
+                                    put(2 * q + 4, h);
+#pragma unroll
+                                    for (int b = 0; b < 4; ++b) h[b] = nib_half<12>(y[b]);
+                                    put(2 * q + 5, h);
+                                }
+                            }
+                        }
+                    } else {
+                        // lane = word w of the positions' rows: keys 32 (w / 8) + w % 8 + 8 b
+                        const uint32_t wc = (uint32_t)lane >> 2, wo = 4 * ((uint32_t)lane & 3);
+                        const uint32_t rows = raw + (32 * (lane >> 3) + (lane & 7)) * g.pitch_v;
+#pragma unroll 1
+                        for (int u = lw; u < nuv; u += 4) {
+                            const uint32_t d = tile + 32 * u * 128 + wo;
+                            auto put = [&](int pos, uint32_t x) { sts32(d + pos * 128 + ((wc ^ (pos & 7)) << 4), x); };
+                            // 4 x 4 byte transpose: out[i] = byte i of the four rows
+                            auto transpose = [](uint32_t a, uint32_t b, uint32_t c, uint32_t e, uint32_t (&out)[4]) {
+                                const uint32_t x01l = __byte_perm(a, b, 0x5140), x01h = __byte_perm(a, b, 0x7362);
+                                const uint32_t x23l = __byte_perm(c, e, 0x5140), x23h = __byte_perm(c, e, 0x7362);
+                                out[0] = __byte_perm(x01l, x23l, 0x5410); out[1] = __byte_perm(x01l, x23l, 0x7632);
+                                out[2] = __byte_perm(x01h, x23h, 0x5410); out[3] = __byte_perm(x01h, x23h, 0x7632);
+                            };
+                            if (p.bits_v == 8) {
+#pragma unroll
+                                for (int half = 0; half < 2; ++half) {
+                                    uint4 rw[4];
+#pragma unroll
+                                    for (int b = 0; b < 4; ++b) rw[b] = lds128(rows + 8 * b * g.pitch_v + 32 * u + 16 * half);
+                                    const uint32_t a[4][4] = {{rw[0].x, rw[0].y, rw[0].z, rw[0].w}, {rw[1].x, rw[1].y, rw[1].z, rw[1].w},
+                                                              {rw[2].x, rw[2].y, rw[2].z, rw[2].w}, {rw[3].x, rw[3].y, rw[3].z, rw[3].w}};
+#pragma unroll
+                                    for (int k = 0; k < 4; ++k) {
+                                        uint32_t o[4];
+                                        transpose(a[0][k], a[1][k], a[2][k], a[3][k], o);
+#pragma unroll
+                                        for (int i = 0; i < 4; ++i) put(16 * half + 4 * k + i, o[i]);
+                                    }
+                                }
+                            } else {
                                 uint4 rw[4];
 #pragma unroll
-                                for (int b = 0; b < 4; ++b) rw[b] = lds128(raw + (lane + 32 * b) * g.pitch_v + 32 * u + 16 * half);
+                                for (int b = 0; b < 4; ++b) rw[b] = nibbles(rows + 8 * b * g.pitch_v, u, p.bits_v);
                                 const uint32_t a[4][4] = {{rw[0].x, rw[0].y, rw[0].z, rw[0].w}, {rw[1].x, rw[1].y, rw[1].z, rw[1].w},
                                                           {rw[2].x, rw[2].y, rw[2].z, rw[2].w}, {rw[3].x, rw[3].y, rw[3].z, rw[3].w}};
 #pragma unroll
@@ -604,296 +682,306 @@ prefill_kernel(const AttnParams p, const Plan g)
                                     uint32_t o[4];
                                     transpose(a[0][k], a[1][k], a[2][k], a[3][k], o);
 #pragma unroll
-                                    for (int i = 0; i < 4; ++i) put(16 * half + 4 * k + i, o[i]);
+                                    for (int i = 0; i < 4; ++i) { put(8 * k + i, o[i] & 0x0F0F0F0Fu); put(8 * k + 4 + i, (o[i] >> 4) & 0x0F0F0F0Fu); }
                                 }
-                            }
-                        } else {
-                            uint4 rw[4];
-#pragma unroll
-                            for (int b = 0; b < 4; ++b) rw[b] = nibbles(raw + (lane + 32 * b) * g.pitch_v, u, p.bits_v);
-                            const uint32_t a[4][4] = {{rw[0].x, rw[0].y, rw[0].z, rw[0].w}, {rw[1].x, rw[1].y, rw[1].z, rw[1].w},
-                                                      {rw[2].x, rw[2].y, rw[2].z, rw[2].w}, {rw[3].x, rw[3].y, rw[3].z, rw[3].w}};
-#pragma unroll
-                            for (int k = 0; k < 4; ++k) {
-                                uint32_t o[4];
-                                transpose(a[0][k], a[1][k], a[2][k], a[3][k], o);
-#pragma unroll
-                                for (int i = 0; i < 4; ++i) { put(8 * k + i, o[i] & 0x0F0F0F0Fu); put(8 * k + 4 + i, (o[i] >> 4) & 0x0F0F0F0Fu); }
                             }
                         }
                     }
+                    tc::fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(B_VFULL + st));
+                    if (!group_sync()) { ok = false; break; }                  // the raw rows have been read
                 }
-                tc::fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar(B_VFULL + st));
-                if (!group_sync()) { ok = false; break; }                      // the raw rows have been read
-                if (kt + 1 < it.n_kt) copy_rows(it, kt + 1);
-                else if (idx + (int)gridDim.x < g.n_items) copy_rows(item_of(p, g, idx + gridDim.x, KEYS), 0);
+                if (have) copy_rows([&](int r, int c) { return base + g.off_rawv + staged_row(r) * g.pitch_v + 16 * c; });
                 cp_async_commit();
+                if constexpr (MODE == KV) {
+                    if (have && nx.t == 0 && !gather_queries(nx.it, n == 0 ? 0u : n_item + 1)) { ok = false; break; }
+                }
+                if (n > 0 && cu.t == cu.n_t - 1) {
+                // ---- the item's output rows: warp = lane quarter of the accumulator, thread = row
+                if (!mbar_sleep(bar(B_SUM), n_item & 1, s_abort) || !mbar_sleep(bar(B_OFULL), n_item & 1, s_abort)) { ok = false; break; }
+                __syncwarp();
+                tc::tc_fence_after();
+                const int row = 32 * lw + lane, i0 = it.qt * BM, i = i0 + row;
+                const bool live = i0 + 32 * lw < p.Tq;                         // some row of my warp exists
+                if (live) {
+                    float inv_l = 0.f;
+                    int rs = 0;
+                    if constexpr (MODE == KV) {
+                        float l = 0.f;
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) l += __uint_as_float(s_sum[q * BM + row]);
+                        inv_l = 1.0f / l;
+                    } else {
+#pragma unroll
+                        for (int q = 0; q < 2; ++q) rs += (int)s_sum[q * BM + row];
+                    }
+                    const uint32_t stage = base + g.off_v, o_row = stage + row * g.out_pitch;
+                    __half* out_row = p.out + ((int64_t)it.seq * p.Tq + i) * p.ldo;
+#pragma unroll 1
+                    for (int u = 0; u < nuv; ++u) {
+                        // channel of position `lane` of the unit
+                        const int pos = 32 * (uv0 + u) + lane;
+                        int ch = __ldg(p.jidx_v + pos) >= 0 ? (int)__ldg(p.src_v + pos) : -1;
+                        const float2 sz = __ldg(p.unit_sz_v + uv0 + u);
+                        const float sc = MODE == KV ? sz.x * inv_l : p.s_P * sz.x, zf = sz.x * (sz.y - (p.bits_v == 8 ? 128.0f : 8.0f));
+                        const int zi = (int)sz.y * rs;
+                        if (g.local_v && ch >= 0) ch = 2 * (ch - it.h * p.hd);         // its byte within a staged row
+#pragma unroll 1
+                        for (int part = 0; part < 2; ++part) {
+                            uint32_t v[16];
+                            tc::tc_ld16(tmem + ((uint32_t)(32 * lw) << 16) + 32 * u + 16 * part, v);
+                            tc::tc_wait_ld();
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) {
+                                const int c = __shfl_sync(0xffffffffu, ch, 16 * part + e);
+                                if (c < 0) continue;
+                                float o;
+                                if constexpr (MODE == KV) o = __fmaf_rn(__uint_as_float(v[e]), sc, -zf);
+                                else o = sc * (float)((int)v[e] - zi);
+                                const uint16_t oh = __half_as_ushort(__float2half_rn(o));
+                                // (the staged words of row r are exchanged by r & 31: no bank conflicts)
+                                if (g.local_v) sts16(o_row + ((uint32_t)c ^ ((uint32_t)lane << 2)), oh);
+                                else if (i < p.Tq) out_row[c] = __ushort_as_half(oh);
+                            }
+                        }
+                    }
+                    tc::tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(B_OEMPTY));
+                    if (g.local_v) {
+                        const int n_rows = min(32, p.Tq - i0 - 32 * lw);
+                        const uint32_t src = stage + 32 * lw * g.out_pitch;
+                        __half* dst = p.out + ((int64_t)it.seq * p.Tq + i0 + 32 * lw) * p.ldo + it.h * p.hd;
+                        const bool pairs = (((uintptr_t)p.out & 3u) == 0) && (p.ldo & 1) == 0 && (p.hd & 1) == 0;
+                        if (pairs) {
+#pragma unroll 4
+                            for (int r = 0; r < n_rows; ++r, dst += p.ldo)
+                                for (int c = lane; c < p.hd / 2; c += 32) reinterpret_cast<uint32_t*>(dst)[c] = lds32(src + r * g.out_pitch + ((c ^ r) << 2));
+                        } else {
+                            for (int r = 0; r < n_rows; ++r, dst += p.ldo)
+                                for (int c = lane; c < p.hd; c += 32) dst[c] = __ushort_as_half(lds16(src + r * g.out_pitch + (((c >> 1) ^ r) << 2) + 2 * (c & 1)));
+                        }
+                    }
+                } else if (lane == 0) {
+                    mbar_arrive(bar(B_OEMPTY));
+                }
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(B_OUT));
+                ++n_item;
+                }
+                if (!have) break;
+                cu = nx;
+                have = advance();
             }
         }
         cp_async_wait<0>();
     } else {
         // ---------------------------------------------------------------- softmax
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX));
-        const int sw_ = warp - S_WARP0, q4 = sw_ & 3, hf = sw_ >> 2;           // lane quarter of the accumulators, half of the keys
+        const int q4 = warp & 3, stream = (warp - S_WARP0) >> 2;               // lane quarter of the accumulators
         const int row = 32 * q4 + lane;                                        // query row within the tile
-        constexpr int RUN = KEYS / 8;                                          // my keys: KEYS / 4 * b + RUN * hf + 0 .. RUN - 1, b = 0..3
-        const uint32_t t_lane = tmem + ((uint32_t)(32 * q4) << 16);
-        uint32_t n_k = 0, n_s = 0, n_p = 0, n_x = 0, n_item = 0;
+        const uint32_t t_col = tmem + ((uint32_t)(32 * q4) << 16) + O_COLS + stream * (N_SLOTS * COLS);
+        const uint32_t b_full0 = bar(B_SFULL + stream * N_SLOTS), b_empty0 = bar(B_SEMPTY + stream * N_SLOTS);
+        uint32_t n_k0 = 0, slot = 0, par = 0, n_s = 0, n_item = 0;   // n_s: my stream's tiles of pass 2 so far
         bool ok = true;
-        auto group_sync = [&]() {
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(B_XS));
-            const bool done = mbar_wait(bar(B_XS), n_x & 1, s_abort);
-            ++n_x;
-            return done;
-        };
         for (int idx = blockIdx.x; idx < g.n_items && ok; idx += gridDim.x, ++n_item) {
             const Item it = item_of(p, g, idx, KEYS);
-            const int uk0 = __ldg(p.cl_unit0_k + it.h * p.gh_k), nuk = __ldg(p.cl_unit0_k + (it.h + 1) * p.gh_k) - uk0;
-            const int uv0 = __ldg(p.cl_unit0_v + it.h * p.gh_v), nuv = __ldg(p.cl_unit0_v + (it.h + 1) * p.gh_v) - uv0;
-            const int i0 = it.qt * BM, i = i0 + row;
+            const int i0 = it.qt * BM, i = i0 + row, off = p.Tk - p.Tq;
             const bool live = i0 + 32 * q4 < p.Tq;                             // some row of my warp exists
             const int vis = p.causal ? min(p.Tk - 1, i + off) : p.Tk - 1;      // my last visible key
             const int vis_all = p.causal ? min(p.Tk - 1, i0 + 32 * q4 + off) : p.Tk - 1;    // of the warp's first row
             // coefficient of unit `lane`'s cluster; bit u of last: unit u is the last of its cluster
             float coef = 0.f;
-            int cl = -1;
-            if (lane < nuk) {
-                cl = __ldg(p.unit_cluster_k + uk0 + lane);
-                coef = __ldg(&p.unit_sz_k[uk0 + lane].x) * p.qk_scale_log2e;
-                if constexpr (MODE != KV) coef = __ldg(&p.unit_sz_q[uk0 + lane].x) * __ldg(&p.unit_sz_k[uk0 + lane].x) * p.qk_scale_log2e;
-                if constexpr (MODE == F8) coef *= 262144.0f;                   // both operands are n 2^-9
-            }
-            const int cl_next = __shfl_down_sync(0xffffffffu, cl, 1);
-            const uint32_t last = __ballot_sync(0xffffffffu, lane < units_seen(nuk) && (lane >= nuk - 1 || cl != cl_next));
-
-            float2 S[4][RUN / 2];
-            // scores of my row against my keys of tile kt, times log2(e); hidden keys at NEG_BIG
-            auto scores = [&](int kt) {
-                const float* col = s_col + (n_k & 3) * KEYS;
-                bool first = true;
-                uint32_t m = last;                                             // (at least one bit)
-                do {
-                    const uint32_t slot = n_s % N_SLOTS;
-                    const float c = __shfl_sync(0xffffffffu, coef, __ffs(m) - 1);
-                    if (!mbar_wait(bar(B_SFULL + slot), (n_s / N_SLOTS) & 1, s_abort)) return false;
-                    ++n_s;
-                    __syncwarp();
-                    tc::tc_fence_after();
-                    if (live) {
-                        if (first) {
-                            if constexpr (MODE == KV) {
-#pragma unroll
-                                for (int b = 0; b < 4; ++b)
-#pragma unroll
-                                    for (int e = 0; e < RUN / 2; ++e) S[b][e] = make_float2(0.f, 0.f);
-                            } else {
-#pragma unroll
-                                for (int b = 0; b < 4; ++b)
-#pragma unroll
-                                    for (int e = 0; e < RUN / 2; e += 2) {
-                                        const float4 v = *reinterpret_cast<const float4*>(col + KEYS / 4 * b + RUN * hf + 2 * e);
-                                        S[b][e] = make_float2(v.x, v.y); S[b][e + 1] = make_float2(v.z, v.w);
-                                    }
-                            }
-                        }
-                        const float2 c2 = make_float2(c, c);
-                        const uint32_t ta = t_lane + O_COLS + slot * KEYS + RUN * hf;
-                        uint32_t v[2][RUN];
-                        auto load = [&](int b) {
-                            if constexpr (RUN == 16) tc::tc_ld16(ta + KEYS / 4 * b, reinterpret_cast<uint32_t(&)[16]>(v[b & 1]));
-                            else ld8(ta + KEYS / 4 * b, v[b & 1]);
-                        };
-                        load(0);
-#pragma unroll
-                        for (int b = 0; b < 4; ++b) {
-                            tc::tc_wait_ld();
-                            if (b < 3) load(b + 1);
-#pragma unroll
-                            for (int e = 0; e < RUN / 2; ++e) {
-                                float2 x;
-                                if constexpr (MODE == I8) x = make_float2((float)(int)v[b & 1][2 * e], (float)(int)v[b & 1][2 * e + 1]);
-                                else x = make_float2(__uint_as_float(v[b & 1][2 * e]), __uint_as_float(v[b & 1][2 * e + 1]));
-                                S[b][e] = fma2(c2, x, S[b][e]);
-                            }
-                        }
-                    }
-                    first = false;
-                    tc::tc_fence_before();
-                    __syncwarp();
-                    if (lane == 0) mbar_arrive(bar(B_SEMPTY + slot));
-                    m &= m - 1;
-                } while (m);
-                ++n_k;
-                const int j0 = kt * KEYS;
-                if (live && j0 + KEYS - 1 > vis_all) {
-#pragma unroll
-                    for (int b = 0; b < 4; ++b)
-#pragma unroll
-                        for (int e = 0; e < RUN / 2; ++e) {
-                            const int j = j0 + KEYS / 4 * b + RUN * hf + 2 * e;
-                            if (j > vis) S[b][e].x = NEG_BIG;
-                            if (j + 1 > vis) S[b][e].y = NEG_BIG;
-                        }
+            uint32_t last;
+            {
+                const int uk0 = __ldg(p.cl_unit0_k + it.h * p.gh_k), nuk = __ldg(p.cl_unit0_k + (it.h + 1) * p.gh_k) - uk0;
+                int cl = -1;
+                if (lane < nuk) {
+                    cl = __ldg(p.unit_cluster_k + uk0 + lane);
+                    if constexpr (MODE == KV) coef = __ldg(&p.unit_sz_k[uk0 + lane].x) * p.qk_scale_log2e;
+                    else coef = __ldg(&p.unit_sz_q[uk0 + lane].x) * __ldg(&p.unit_sz_k[uk0 + lane].x) * p.qk_scale_log2e;
+                    if constexpr (MODE == F8) coef *= 262144.0f;               // both operands are n 2^-9
                 }
-                return true;
-            };
-
-            // ---- pass 1: row maximum (integer calls: and row sum) over my keys
-            float m = NEG_BIG, l = 0.f;
-            for (int kt = 0; kt < it.n_kt; ++kt) {
-                if (!scores(kt)) { ok = false; break; }
-                if (live) {
-                    float x0 = NEG_BIG, x1 = NEG_BIG;
-#pragma unroll
-                    for (int b = 0; b < 4; ++b)
-#pragma unroll
-                        for (int e = 0; e < RUN / 2; e += 2) {
-                            x0 = fmaxf(x0, fmaxf(S[b][e].x, S[b][e].y));
-                            x1 = fmaxf(x1, fmaxf(S[b][e + 1].x, S[b][e + 1].y));
-                        }
-                    const float n = fmaxf(m, fmaxf(x0, x1));
+                const int cl_next = __shfl_down_sync(0xffffffffu, cl, 1);
+                last = __ballot_sync(0xffffffffu, lane < units_seen(nuk) && (lane >= nuk - 1 || cl != cl_next));
+            }
+            float m = NEG_BIG, l = 0.f, f = 0.f, lsum = 0.f;
+            uint32_t rsum = 0u;
+#pragma unroll 1
+            for (int pass = 0; pass < 2 && ok; ++pass, n_k0 += it.n_kt) {
+                if (pass == 1) {
+                    // the streams' statistics meet (two sets by turns: a warp may be an item ahead of another)
+                    float2* ml = s_ml + (n_item & 1) * 2 * BM;
+                    ml[stream * BM + row] = make_float2(m, l);
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(B_XS));
+                    if (!mbar_sleep(bar(B_XS), n_item & 1, s_abort)) { ok = false; break; }
+                    const float2 o = ml[(stream ^ 1) * BM + row];
+                    const float n = fmaxf(m, o.x);
                     if constexpr (MODE != KV) {
-                        const float2 nn = make_float2(-n, -n);
-                        float2 a0 = make_float2(0.f, 0.f), a1 = a0;
-#pragma unroll
-                        for (int b = 0; b < 4; ++b)
-#pragma unroll
-                            for (int e = 0; e < RUN / 2; e += 2) {
-                                const float2 y = add2(S[b][e], nn), z = add2(S[b][e + 1], nn);
-                                a0 = add2(a0, make_float2(ex2(y.x), ex2(y.y)));
-                                a1 = add2(a1, make_float2(ex2(z.x), ex2(z.y)));
-                            }
-                        l = l * ex2(m - n) + ((a0.x + a0.y) + (a1.x + a1.y));
+                        l = l * ex2(m - n) + o.y * ex2(o.x - n);               // (a stream without a visible key weighs 0)
+                        f = p.inv_sP / l * 1.7763568394002505e-15f;            // times 2^-49: see below
                     }
                     m = n;
                 }
-            }
-            if (!ok) break;
-            s_x[hf * BM + row] = make_float2(m, l);
-            if (!group_sync()) { ok = false; break; }
-            {
-                const float2 o = s_x[(hf ^ 1) * BM + row];
-                const float n = fmaxf(m, o.x);
-                if constexpr (MODE != KV) l = l * ex2(m - n) + o.y * ex2(o.x - n);     // (a half without a visible key weighs 0)
-                m = n;
-            }
-            // ---- pass 2: probabilities
-            const float2 nm = make_float2(-m, -m);
-            const float f = MODE == KV ? 0.f : p.inv_sP / l * 1.7763568394002505e-15f;   // times 2^-49: see below
-            const float2 f2 = make_float2(f, f), k100 = make_float2(7.888609052210118e-31f, 7.888609052210118e-31f);   // 2^-100
-            float lsum = 0.f;
-            uint32_t rsum = 0u;
-            const uint32_t p_row = base + g.off_p + row * 128, p_sw = row & 7;
-            for (int kt = 0; kt < it.n_kt; ++kt, ++n_p) {
-                if (!scores(kt)) { ok = false; break; }
-                uint32_t w[16];
-                if (live) {
-                    if constexpr (MODE == KV) {
+#pragma unroll 1
+                for (int kt = ALT ? stream : 0; kt < it.n_kt; kt += ALT ? 2 : 1) {
+                    // ---- scores of my row against my keys of the tile, times log2(e); hidden keys at NEG_BIG
+                    float2 S[COLS / 2];
+                    const float* col = s_col + ((n_k0 + kt) & 3) * KEYS + stream * COLS;
+                    bool first = true;
+                    uint32_t left = last;                                      // (at least one bit)
+                    do {
+                        const float c = __shfl_sync(0xffffffffu, coef, __ffs(left) - 1);
+                        if (!mbar_sleep(b_full0 + 8 * slot, par, s_abort)) { ok = false; break; }
+                        __syncwarp();
+                        tc::tc_fence_after();
+                        if (live) {
+                            uint32_t v[32];
+                            ld32(t_col + slot * COLS, v);
+                            if (first) {
+                                if constexpr (MODE == KV) {
 #pragma unroll
-                        for (int b = 0; b < 4; ++b)
+                                    for (int e = 0; e < COLS / 2; ++e) S[e] = make_float2(0.f, 0.f);
+                                } else {
 #pragma unroll
-                            for (int e = 0; e < RUN / 2; ++e) {
-                                const float2 y = add2(S[b][e], nm);
-                                w[4 * e + b] = pack_half2(ex2(y.x), ex2(y.y));         // chunk e: the four pairs b
-                                const float2 r = __half22float2(*reinterpret_cast<const __half2*>(&w[4 * e + b]));
-                                lsum += r.x + r.y;           // the rounded values: the division normalises what was multiplied
-                            }
-                    } else {
-                        // code = min(rne(2^(S - m) / (s_P l)), 255): the product scaled by 2^-149 is rounded once, half to even, to the
-                        // grid of the subnormals, whose bit pattern is the integer itself; the saturating pack clamps it
-#pragma unroll
-                        for (int e = 0; e < RUN / 2; ++e) {
-                            int q[4][2];
-#pragma unroll
-                            for (int b = 0; b < 4; ++b) {
-                                const float2 y = add2(S[b][e], nm);
-                                const float2 t = mul2(mul2(make_float2(ex2(y.x), ex2(y.y)), f2), k100);
-                                q[b][0] = __float_as_int(t.x); q[b][1] = __float_as_int(t.y);
-                            }
-#pragma unroll
-                            for (int k = 0; k < 2; ++k) {
-                                w[2 * e + k] = sat_pack_u8(q[1][k], q[0][k], sat_pack_u8(q[3][k], q[2][k], 0u));
-                                rsum = __dp4a(w[2 * e + k], 0x01010101u, rsum);
-                            }
-                        }
-                        if (p.p_dbg && i < p.Tq) {
-                            uint8_t* dst = p.p_dbg + (((int64_t)it.seq * p.H + it.h) * p.Tq + i) * p.Tk;
-#pragma unroll
-                            for (int e = 0; e < 16; ++e)
-#pragma unroll
-                                for (int b = 0; b < 4; ++b) {
-                                    const int j = kt * KEYS + KEYS / 4 * b + RUN * hf + e;
-                                    if (j < p.Tk) dst[j] = (uint8_t)(w[e] >> (8 * b));
+                                    for (int e = 0; e < COLS / 2; e += 2) {
+                                        const float4 x = *reinterpret_cast<const float4*>(col + 2 * e);
+                                        S[e] = make_float2(x.x, x.y); S[e + 1] = make_float2(x.z, x.w);
+                                    }
                                 }
+                            }
+                            const float2 c2 = make_float2(c, c);
+#pragma unroll
+                            for (int part = 0; part < 2; ++part) {
+                                tc::tc_wait_ld();
+#pragma unroll
+                                for (int e = 0; e < 16; ++e) {
+                                    float2 x;
+                                    if constexpr (MODE == I8) x = make_float2((float)(int)v[2 * e], (float)(int)v[2 * e + 1]);
+                                    else x = make_float2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
+                                    S[16 * part + e] = fma2(c2, x, S[16 * part + e]);
+                                }
+                                if (part == 0) ld32(t_col + slot * COLS + 32, v);
+                            }
+                        }
+                        first = false;
+                        tc::tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) mbar_arrive(b_empty0 + 8 * slot);
+                        slot ^= 1u;
+                        par ^= slot ^ 1u;
+                        left &= left - 1;
+                    } while (left);
+                    if (!ok) break;
+                    const int j0 = kt * KEYS + (ALT ? 0 : stream * COLS);
+                    if (live && j0 + COLS - 1 > vis_all) {
+                        const int n_vis = vis - j0;                            // my last visible column
+#pragma unroll
+                        for (int e = 0; e < COLS / 2; ++e) {
+                            if (2 * e > n_vis) S[e].x = NEG_BIG;
+                            if (2 * e + 1 > n_vis) S[e].y = NEG_BIG;
                         }
                     }
-                }
-                if (!mbar_wait(bar(B_PEMPTY), (n_p & 1) ^ 1, s_abort)) { ok = false; break; }
-                if (live) {
+                    if (pass == 0) {
+                        // ---- pass 1: row maximum (integer calls: and row sum) over my keys
+                        if (live) {
+                            float x0 = NEG_BIG, x1 = NEG_BIG;
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) sts128(p_row + (((4 * hf + c) ^ p_sw) << 4), w[4 * c], w[4 * c + 1], w[4 * c + 2], w[4 * c + 3]);
+                            for (int e = 0; e < COLS / 2; e += 2) {
+                                x0 = fmaxf(x0, fmaxf(S[e].x, S[e].y));
+                                x1 = fmaxf(x1, fmaxf(S[e + 1].x, S[e + 1].y));
+                            }
+                            const float n = fmaxf(m, fmaxf(x0, x1));
+                            if constexpr (MODE != KV) {
+                                const float2 nn = make_float2(-n, -n);
+                                float2 a0 = make_float2(0.f, 0.f), a1 = a0;
+#pragma unroll
+                                for (int e = 0; e < COLS / 2; e += 2) {
+                                    const float2 y = add2(S[e], nn), z = add2(S[e + 1], nn);
+                                    a0 = add2(a0, make_float2(ex2(y.x), ex2(y.y)));
+                                    a1 = add2(a1, make_float2(ex2(z.x), ex2(z.y)));
+                                }
+                                l = l * ex2(m - n) + ((a0.x + a0.y) + (a1.x + a1.y));
+                            }
+                            m = n;
+                        }
+                        continue;
+                    }
+                    // ---- pass 2: probabilities. P's region also stages the previous item's output
+                    if (kt < 2 && !mbar_sleep(bar(B_OUT), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
+                    // the buffer's previous tile has been multiplied
+                    // (one buffer for both streams: stream 1's first tile waits for stream 0's)
+                    const uint32_t behind = ALT && g.p_tiles == 1 && stream == 1 ? 0u : 1u;
+                    if (!mbar_sleep(bar(B_PEMPTY + stream), (n_s & 1) ^ behind, s_abort)) { ok = false; break; }
+                    ++n_s;
+                    if (live) {
+                        const float2 nm = make_float2(-m, -m);
+                        if constexpr (MODE == KV) {
+                            const uint32_t p_row = base + g.off_p + (g.p_tiles == 2 ? stream * (BM * 128) : 0) + row * 128;
+#pragma unroll
+                            for (int blk = 0; blk < 4; ++blk)
+#pragma unroll
+                                for (int y = 0; y < 2; ++y) {                  // chunk 2 blk + y: keys 16 blk + 4 b + 2 y + {0, 1}
+                                    uint32_t w[4];
+#pragma unroll
+                                    for (int b = 0; b < 4; ++b) {
+                                        const float2 x = add2(S[8 * blk + 2 * b + y], nm);
+                                        w[b] = pack_half2(ex2(x.x), ex2(x.y));
+                                        const float2 r = __half22float2(*reinterpret_cast<const __half2*>(&w[b]));
+                                        lsum += r.x + r.y;   // the rounded values: the division normalises what was multiplied
+                                    }
+                                    sts128(p_row + (((2 * blk + y) ^ (row & 7)) << 4), w[0], w[1], w[2], w[3]);
+                                }
+                        } else {
+                            // code = min(rne(2^(S - m) / (s_P l)), 255): the product scaled by 2^-149 is rounded once, half to even, to the
+                            // grid of the subnormals, whose bit pattern is the integer itself; the saturating pack clamps it
+                            const float2 f2 = make_float2(f, f), k100 = make_float2(7.888609052210118e-31f, 7.888609052210118e-31f);   // 2^-100
+                            const uint32_t p_row = base + g.off_p + row * 128;
+#pragma unroll
+                            for (int blk = 0; blk < 2; ++blk) {                // 32 keys: word x has keys x + 8 b
+                                uint32_t w[8];
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) {
+                                    int q[4][2];
+#pragma unroll
+                                    for (int b = 0; b < 4; ++b) {
+                                        const float2 y = add2(S[16 * blk + 4 * b + e], nm);
+                                        const float2 t = mul2(mul2(make_float2(ex2(y.x), ex2(y.y)), f2), k100);
+                                        q[b][0] = __float_as_int(t.x); q[b][1] = __float_as_int(t.y);
+                                    }
+#pragma unroll
+                                    for (int k = 0; k < 2; ++k) {
+                                        w[2 * e + k] = sat_pack_u8(q[1][k], q[0][k], sat_pack_u8(q[3][k], q[2][k], 0u));
+                                        rsum = __dp4a(w[2 * e + k], 0x01010101u, rsum);
+                                    }
+                                }
+                                const int c = 4 * stream + 2 * blk;
+                                sts128(p_row + ((c ^ (row & 7)) << 4), w[0], w[1], w[2], w[3]);
+                                sts128(p_row + (((c + 1) ^ (row & 7)) << 4), w[4], w[5], w[6], w[7]);
+                            }
+                            if (p.p_dbg && i < p.Tq) {                         // key k of the stream: byte (k & 31) / 8 of word k & 7 of block k / 32
+                                uint8_t* dst = p.p_dbg + (((int64_t)it.seq * p.H + it.h) * p.Tq + i) * p.Tk;
+#pragma unroll 1
+                                for (int k = 0; k < COLS && j0 + k < p.Tk; ++k) {
+                                    const int c = 4 * stream + 2 * (k >> 5) + ((k & 7) >> 2);
+                                    dst[j0 + k] = (uint8_t)(lds32(p_row + ((c ^ (row & 7)) << 4) + 4 * (k & 3)) >> (8 * ((k & 31) >> 3)));
+                                }
+                            }
+                        }
+                    }
+                    tc::fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(B_PFULL + stream));
                 }
-                tc::fence_proxy_async();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar(B_PFULL));
             }
             if (!ok) break;
-            // ---- outputs
-            s_x[2 * BM + hf * BM + row] = make_float2(lsum, __uint_as_float(rsum));
-            if (!group_sync()) { ok = false; break; }
-            const float2 part = s_x[2 * BM + (hf ^ 1) * BM + row];
-            const float inv_l = MODE == KV ? 1.0f / (lsum + part.x) : 0.f;
-            const int rs = (int)(rsum + __float_as_uint(part.y));
-            if (!mbar_wait(bar(B_OFULL), n_item & 1, s_abort)) { ok = false; break; }
+            // (a stream without a tile of its own has not waited for the previous item's sums to be read)
+            if (ALT && it.n_kt == 1 && !mbar_sleep(bar(B_OUT), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
+            s_sum[stream * BM + row] = MODE == KV ? __float_as_uint(lsum) : rsum;
             __syncwarp();
-            tc::tc_fence_after();
-            const uint32_t stage = base + g.off_v, o_row = stage + row * g.out_pitch;
-            __half* out_row = p.out + ((int64_t)it.seq * p.Tq + i) * p.ldo;
-            for (int u = hf; u < nuv; u += 2) {
-                // channel of position `lane` of the unit
-                const int pos = 32 * (uv0 + u) + lane;
-                const int ch = __ldg(p.jidx_v + pos) >= 0 ? (int)__ldg(p.src_v + pos) : -1;
-                const float2 sz = __ldg(p.unit_sz_v + uv0 + u);
-#pragma unroll
-                for (int half = 0; half < 2; ++half) {
-                    uint32_t v[16];
-                    if (live) { tc::tc_ld16(t_lane + 32 * u + 16 * half, v); tc::tc_wait_ld(); }
-#pragma unroll
-                    for (int e = 0; e < 16; ++e) {
-                        const int c = __shfl_sync(0xffffffffu, ch, 16 * half + e);
-                        if (!live || c < 0) continue;
-                        float o;
-                        if constexpr (MODE == KV) o = sz.x * (__uint_as_float(v[e]) * inv_l - (sz.y - (p.bits_v == 8 ? 128.0f : 8.0f)));
-                        else o = p.s_P * sz.x * (float)((int)v[e] - (int)sz.y * rs);
-                        const __half oh = __float2half_rn(o);
-                        if (g.local_v) sts16(o_row + 2 * (c - it.h * p.hd), __half_as_ushort(oh));
-                        else if (i < p.Tq) out_row[c] = oh;
-                    }
-                }
-            }
-            tc::tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive(bar(B_OEMPTY));
-            if (g.local_v) {
-                if (!group_sync()) { ok = false; break; }                      // (a row's units are spread over both halves)
-                __half* out0 = p.out + ((int64_t)it.seq * p.Tq + i0) * p.ldo + it.h * p.hd;
-                const int n_rows = min(BM, p.Tq - i0);
-                const bool pairs = (((uintptr_t)p.out & 3u) == 0) && (p.ldo & 1) == 0 && (p.hd & 1) == 0;
-                for (int r = sw_; r < n_rows; r += 8) {
-                    const uint32_t src = stage + r * g.out_pitch;
-                    if (pairs) {
-                        uint32_t* dst = reinterpret_cast<uint32_t*>(out0 + (int64_t)r * p.ldo);
-                        for (int c = lane; c < p.hd / 2; c += 32) dst[c] = lds32(src + 4 * c);
-                    } else {
-                        for (int c = lane; c < p.hd; c += 32) out0[(int64_t)r * p.ldo + c] = __ushort_as_half(lds16(src + 2 * c));
-                    }
-                }
-                __syncwarp();
-            }
-            if (lane == 0) mbar_arrive(bar(B_OUT));
+            if (lane == 0) mbar_arrive(bar(B_SUM));
         }
     }
 
@@ -920,24 +1008,31 @@ static int launch_one(const AttnParams& p, int units_k, int units_v, int n_seq, 
     g.k_stage = atoms * KEYS * 128;
     g.off_v = g.off_k + 2 * g.k_stage;
     g.v_stage = units_v * 32 * 128;
-    const int raw_k = MODE != KV && p.bits_k == 8 ? 0 : KEYS * raw_pitch_of(p.bits_k, units_k);
     g.pitch_k = raw_pitch_of(p.bits_k, units_k);
     g.pitch_v = raw_pitch_of(p.bits_v, units_v);
-    const int rest = BM * 128 + raw_k + KEYS * g.pitch_v + 4 * KEYS * 4 + 4 * BM * 8 + 256;
+    g.rawk_stage = MODE != KV && p.bits_k == 8 ? 0 : KEYS * g.pitch_k;
+    const int rest = BM * 128 + KEYS * g.pitch_v + 4 * KEYS * 4 + 4 * BM * 8 + 2 * BM * 4 + 512;
     constexpr int LIMIT = 226 * 1024;                     // (with 1 KiB for the alignment: the most a block may have)
-    g.v_stages = g.off_v + 2 * g.v_stage + rest <= LIMIT ? 2 : 1;
+    // a second packed key tile first (the copies of a tile then have a whole tile's time), then (KV) a probability tile for each
+    // stream, then a second value tile
+    int used = g.off_v + g.v_stage + g.rawk_stage + rest;
+    g.rawk_stages = used + g.rawk_stage <= LIMIT ? 2 : 1;
+    used += (g.rawk_stages - 1) * g.rawk_stage;
+    g.p_tiles = MODE == KV && used + BM * 128 <= LIMIT ? 2 : 1;
+    used += (g.p_tiles - 1) * BM * 128;
+    g.v_stages = used + g.v_stage <= LIMIT ? 2 : 1;
     g.off_p = g.off_v + g.v_stages * g.v_stage;
-    g.off_rawk = g.off_p + BM * 128;
-    g.off_rawv = g.off_rawk + raw_k;
+    g.off_rawk = g.off_p + g.p_tiles * BM * 128;
+    g.off_rawv = g.off_rawk + g.rawk_stages * g.rawk_stage;
     g.off_col = g.off_rawv + KEYS * g.pitch_v;
-    g.off_x = g.off_col + 4 * KEYS * 4;
-    g.off_bar = g.off_x + 4 * BM * 8;
-    g.total = g.off_bar + 256;
+    g.off_ml = g.off_col + 4 * KEYS * 4;
+    g.off_sum = g.off_ml + 4 * BM * 8;
+    g.off_bar = g.off_sum + 2 * BM * 4;
+    g.total = g.off_bar + 512;
     if (g.total > LIMIT) return RPTQ_ERR_UNSUPPORTED;
-    // an output tile in the V and P region: an odd number of words per row keeps a warp's rows in different banks
-    const int words = (p.hd + 1) / 2;
-    g.out_pitch = 4 * (words | 1);
-    g.local_v = v_heads_local && BM * g.out_pitch <= g.v_stages * g.v_stage + BM * 128;
+    // the output tile is staged in the V and P region (rows of a multiple of 128 bytes: see the staging stores)
+    g.out_pitch = (2 * p.hd + 127) / 128 * 128;
+    g.local_v = v_heads_local && BM * g.out_pitch <= g.v_stages * g.v_stage + g.p_tiles * BM * 128;
     g.status = device_status_word();
     const void* fn = reinterpret_cast<const void*>(prefill_kernel<MODE>);
     static std::atomic<uint64_t> done{0}, pool_ok{0};

@@ -41,6 +41,43 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
+// The same test, but the thread may stay suspended in it for up to `ns` nanoseconds while the phase has not completed.
+__device__ __forceinline__ bool mbar_try_wait_for(uint32_t bar, uint32_t parity, uint32_t ns)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity), "r"(ns) : "memory");
+    return ok != 0;
+}
+// Bounded wait for kernels with many waiting warps: sleeps in the barrier instruction instead of polling it, and takes few
+// instructions at each of its many call sites. The limit is a number of wake-ups (each at most about a microsecond: two
+// seconds in all).
+__device__ __forceinline__ bool mbar_sleep(uint32_t bar, uint32_t parity, volatile int* abort_flag)
+{
+    if (mbar_try_wait(bar, parity)) return true;
+#pragma unroll 1
+    for (int i = 0; i < (1 << 21); ++i) {
+        if (mbar_try_wait_for(bar, parity, 1000u)) return true;
+        if (*abort_flag) return false;
+    }
+    *abort_flag = 1;
+    return false;
+}
+// For a whole warp that must stay converged: every lane leaves in the same iteration.
+__device__ __forceinline__ bool mbar_sleep_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag)
+{
+    if (__any_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+#pragma unroll 1
+    for (int i = 0; i < (1 << 21); ++i) {
+        if (__any_sync(0xffffffffu, mbar_try_wait_for(bar, parity, 1000u))) return true;
+        if (__any_sync(0xffffffffu, *abort_flag != 0)) return false;
+    }
+    *abort_flag = 1;
+    return false;
+}
 // Bounded wait. Returns false when the budget ran out or another role already gave up. The common
 // case (the phase has already completed, or completes within a few polls) touches no timer; the
 // budget is counted on the SM's cycle counter, read once per batch of polls.
