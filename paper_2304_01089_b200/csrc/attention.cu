@@ -352,7 +352,7 @@ extern "C" int rptq_attention(const rptq_layout_t* LQ, const rptq_layout_t* LK, 
     const int n_sm = sm_count(dev);
     if (n_sm == 0) return RPTQ_ERR_CUDA;
     if (attn_decode::fits(p, false)) return attn_decode::launch(p, false, units_k, units_v, n_seq, dev, n_sm, st);
-    return attn_prefill::launch(p, false, units_k, units_v, n_seq, heads_own_their_channels(LV, n_heads), dev, n_sm, st);
+    return attn_prefill::launch(p, false, LQ->z_min, LQ->z_max, units_k, units_v, n_seq, heads_own_their_channels(LV, n_heads), dev, n_sm, st);
 
     const int max_bits = LK->bits > LV->bits ? LK->bits : LV->bits;
     const int raw_pitch = 4 * max_bits * MAX_UNITS + 32;          // a head's packed codes plus the alignment slack, a multiple of 16

@@ -276,7 +276,7 @@ extern "C" int rptq_attention_kv(const rptq_layout_t* LK, const rptq_layout_t* L
     const int n_sm = sm_count(dev);
     if (n_sm == 0) return RPTQ_ERR_CUDA;
     if (attn_decode::fits(p, true)) return attn_decode::launch(p, true, units_k, units_v, n_seq, dev, n_sm, st);
-    return attn_prefill::launch(p, true, units_k, units_v, n_seq, heads_own_their_channels(LV, n_heads), dev, n_sm, st);
+    return attn_prefill::launch(p, true, 0, 0, units_k, units_v, n_seq, heads_own_their_channels(LV, n_heads), dev, n_sm, st);
 
     const int smem = (BM + 2 * BN) * PITCH;
     static std::atomic<uint64_t> done{0};

@@ -13,8 +13,9 @@
 //                 through the stream's own ring in tensor memory. The streams run on their own, so that one's drains
 //                 fall under the other's exponentials
 //   warp 2        issues P V (pass 2) into the head's output accumulator, which stays in tensor memory
-//   warps 4-7     keys: packed rows arrive by cp.async one tile ahead, are unpacked into the swizzled operand tile; integer
-//                 calls: with the per-key zero-point term -sum_c s^Q s^K z^Q sum_p K_q. They also lay out the queries.
+//   warps 4-7     keys: packed rows arrive by cp.async one tile ahead, are unpacked into the swizzled operand tile; they
+//                 also lay out the queries: integer calls store q - z^Q where that fits the operand type (a byte; 16 in
+//                 magnitude for E4M3), otherwise q, and form the per-key term -sum_c s^Q s^K z^Q sum_p K_q
 //   warps 8-11    values: unpacked and transposed into [position][key] (byte permutes on the packed words); and the
 //                 output of an item, while the next item's pass 1 runs (they have nothing else to do there)
 //   warps 12-19   softmax, four per stream: thread = query row, 64 keys; S = sum_c coef_c acc_c in registers. (Sixteen warps
@@ -49,13 +50,17 @@ using tc::mbar_sleep;
 using tc::mbar_sleep_warp;
 
 enum { I8 = 0, F8 = 1, KV = 2 };
-constexpr int BM = 128, THREADS = 640;
+constexpr int SUB = 1;                                    // softmax warps that share a stream's piece of work (and a lane quarter)
+constexpr int BM = 128, THREADS = 384 + 256 * SUB;
 constexpr int K_WARP0 = 4, V_WARP0 = 8, S_WARP0 = 12;
 constexpr int COLS = 64;                                  // keys of a stream's piece of work = columns of a score slot
+constexpr int CT = COLS / SUB;                            // keys of a thread
 constexpr int N_SLOTS = 2;                                // score slots of each stream
-// registers per thread of the five warpgroups (the block is launched with 96 each)
-constexpr int REGS_MMA = 48, REGS_LOAD = 72, REGS_SOFTMAX = 144;
-static_assert(REGS_MMA + 2 * REGS_LOAD + 2 * REGS_SOFTMAX <= 5 * 96, "register pool");
+constexpr int S_WARPS = 8 * SUB, PARTS = 2 * SUB;         // softmax warps; threads that share a row
+// registers per thread of the warpgroups: MMA issuers, two of loaders, 2 SUB of softmax (the block is launched with 72 or 96 each)
+constexpr int REGS_MMA = SUB == 2 ? 40 : 48, REGS_LOAD = SUB == 2 ? 56 : 72, REGS_SOFTMAX = SUB == 2 ? 88 : 144;
+constexpr int REGS_ALL = REGS_MMA + 2 * REGS_LOAD + 2 * SUB * REGS_SOFTMAX;
+static_assert(REGS_ALL <= (SUB == 2 ? 7 * 72 : 5 * 96), "register pool");
 constexpr int O_COLS = 32 * MAX_UNITS;                    // tensor memory: the output accumulator, then the score slots
 constexpr int ATOM_Q = BM * 128;                          // 128 rows of 128 bytes
 
@@ -63,10 +68,12 @@ __host__ __device__ constexpr int keys_of(int mode) { return mode == KV ? 64 : 1
 
 // Shared memory of a launch (sizes follow the widest head of the layouts).
 struct Plan {
-    int n_items, n_qt, n_seq;
+    int n_items, n_qt, per_qt;        // per_qt: items of a query tile (heads x sequences)
+    uint32_t inv_per_qt, inv_h;       // ceil(2^32 / per_qt), ceil(2^32 / H)
     int off_k, k_stage, off_v, v_stage, v_stages, off_p, p_tiles, off_rawk, rawk_stage, rawk_stages, pitch_k, off_rawv, pitch_v, off_col, off_ml, off_sum, off_bar, total;
     int local_v;          // V's heads own their channels and the output tile fits the V and P region: rows leave through shared memory
     int out_pitch;
+    int folded;           // integer calls: the queries are stored as q - z^Q (it fits the operand type): no per-key term
     int* status;
 };
 
@@ -151,7 +158,10 @@ __device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, ui
     asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
 }
 __device__ __forceinline__ void sts32(uint32_t addr, uint32_t a) { asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(a) : "memory"); }
-__device__ __forceinline__ void sts16(uint32_t addr, uint16_t a) { asm volatile("st.shared.b16 [%0], %1;" ::"r"(addr), "h"(a) : "memory"); }
+__device__ __forceinline__ void sts16_if(bool p, uint32_t addr, uint16_t a)
+{
+    asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q st.shared.b16 [%0], %1;\n\t}" ::"r"(addr), "h"(a), "r"((int)p) : "memory");
+}
 __device__ __forceinline__ uint4 lds128(uint32_t addr)
 {
     uint4 v;
@@ -188,16 +198,25 @@ struct Item { int qt, h, seq, n_kt; };
 __device__ __forceinline__ Item item_of(const AttnParams& p, const Plan& g, int idx, int keys)
 {
     Item it;
-    const int per = p.H * g.n_seq, q = idx / per, r = idx - q * per;
-    it.qt = g.n_qt - 1 - q;
-    it.seq = r / p.H;
-    it.h = r - it.seq * p.H;
+    // quotients by multiplication with ceil(2^32 / divisor): at most one too large
+    auto divide = [](int n, int d, uint32_t inv, int& rest) {
+        int q = d == 1 ? n : (int)__umulhi((uint32_t)n, inv);
+        rest = n - q * d;
+        if (rest < 0) { --q; rest += d; }
+        return q;
+    };
+    int r;
+    it.qt = g.n_qt - 1 - divide(idx, g.per_qt, g.inv_per_qt, r);
+    it.seq = divide(r, p.H, g.inv_h, it.h);
     const int last = p.causal ? min(p.Tk - 1, it.qt * BM + BM - 1 + p.Tk - p.Tq) : p.Tk - 1;
     it.n_kt = last / keys + 1;
     return it;
 }
 
-template <int MODE>
+// K8, V8: 8-bit key / value codes (otherwise 3 or 4 bits). Separate instances keep each one's code well inside the instruction
+// cache, which this kernel's five roles share (at 188 KB of code every warp issued one instruction per 10 to 15 clocks:
+// 1285 us against 886).
+template <int MODE, bool K8, bool V8>
 __global__ void __launch_bounds__(THREADS, 1)
 prefill_kernel(const AttnParams p, const Plan g)
 {
@@ -224,11 +243,11 @@ prefill_kernel(const AttnParams p, const Plan g)
         mbar_init(bar(B_QFULL), Q_LOADERS); mbar_init(bar(B_QEMPTY), 2);
         for (int i = 0; i < 2; ++i) {
             mbar_init(bar(B_KFULL + i), 4); mbar_init(bar(B_KEMPTY + i), ALT ? 1 : 2); mbar_init(bar(B_VFULL + i), 4); mbar_init(bar(B_VEMPTY + i), 1);
-            mbar_init(bar(B_PFULL + i), 4); mbar_init(bar(B_PEMPTY + i), 1);
+            mbar_init(bar(B_PFULL + i), 4 * SUB); mbar_init(bar(B_PEMPTY + i), 1);
         }
-        for (int i = 0; i < 2 * N_SLOTS; ++i) { mbar_init(bar(B_SFULL + i), 1); mbar_init(bar(B_SEMPTY + i), 4); }
+        for (int i = 0; i < 2 * N_SLOTS; ++i) { mbar_init(bar(B_SFULL + i), 1); mbar_init(bar(B_SEMPTY + i), 4 * SUB); }
         mbar_init(bar(B_OFULL), 1); mbar_init(bar(B_OEMPTY), 4); mbar_init(bar(B_OUT), 4);
-        mbar_init(bar(B_SUM), 8); mbar_init(bar(B_XS), 8); mbar_init(bar(B_XV), 4);
+        mbar_init(bar(B_SUM), S_WARPS); mbar_init(bar(B_XS), S_WARPS); mbar_init(bar(B_XV), 4);
         for (int i = 0; i < 3; ++i) mbar_init(bar(B_DRAIN + i), 1);
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -244,8 +263,8 @@ prefill_kernel(const AttnParams p, const Plan g)
     tc::tc_fence_after();
     const uint32_t tmem = *s_tmem;
     float* s_col = reinterpret_cast<float*>(smem + g.off_col);            // [4][KEYS]
-    float2* s_ml = reinterpret_cast<float2*>(smem + g.off_ml);            // [2][2][BM]: the streams' row maxima and sums
-    uint32_t* s_sum = reinterpret_cast<uint32_t*>(smem + g.off_sum);      // [2][BM]: the streams' sums of probabilities (codes)
+    float2* s_ml = reinterpret_cast<float2*>(smem + g.off_ml);            // [2][PARTS][BM]: row maxima and sums of the parts
+    uint32_t* s_sum = reinterpret_cast<uint32_t*>(smem + g.off_sum);      // [PARTS][BM]: sums of probabilities (codes)
 
     if (warp < K_WARP0) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_MMA));
@@ -258,6 +277,7 @@ prefill_kernel(const AttnParams p, const Plan g)
             constexpr uint32_t LOG_ATOM = ALT ? 1 : 2, STEP = ALT ? 4 : 2;                   // units per atom; a unit's bytes / 16
             const uint32_t dq = desc(0), dk = desc(g.off_k + (ALT ? 0 : stream * COLS * 128)), k_step = (uint32_t)(g.k_stage >> 4);
             const uint32_t d0 = tmem + O_COLS + stream * (N_SLOTS * COLS);
+            const uint32_t id = MODE == I8 && g.folded ? ID | (1u << 7) : ID;                // (signed bytes)
             const uint32_t b_full0 = bar(B_SFULL + stream * N_SLOTS), b_empty0 = bar(B_SEMPTY + stream * N_SLOTS);
             uint32_t n_k = 0, slot = 0, par = 1, n_item = 0;                    // n_k: my tiles so far
             for (int idx = blockIdx.x; idx < g.n_items && ok; idx += gridDim.x, ++n_item) {
@@ -286,10 +306,10 @@ prefill_kernel(const AttnParams p, const Plan g)
                             const uint32_t d = d0 + slot * COLS, in = (u & ((1u << LOG_ATOM) - 1u)) * STEP;
                             const uint32_t a = dq + (u >> LOG_ATOM) * (ATOM_Q >> 4) + in, b = kb + (u >> LOG_ATOM) * (K_ATOM >> 4) + in;
                             if constexpr (MODE == KV) {
-                                mma<2>(d, a, b, ID, acc);
-                                mma<2>(d, a + 2, b + 2, ID, 1u);
+                                mma<2>(d, a, b, id, acc);
+                                mma<2>(d, a + 2, b + 2, id, 1u);
                             } else {
-                                mma<MODE == F8 ? 1 : 0>(d, a, b, ID, acc);
+                                mma<MODE == F8 ? 1 : 0>(d, a, b, id, acc);
                             }
                             acc = 1u;
                             if ((last >> u) & 1u) {
@@ -385,17 +405,17 @@ prefill_kernel(const AttnParams p, const Plan g)
         const int64_t row_bytes = is_k ? p.k_row_bytes : p.v_row_bytes;
         const int bits = is_k ? p.bits_k : p.bits_v;
         // Copies of the packed rows of the tile to fetch: row r goes to dst(r, c), chunk c of 16 bytes. Rows past the last key: zeros.
-        auto copy_rows = [&](auto dst) {
+        auto copy_rows = [&](const Tile& nx, auto dst) {
             const int win = (4 * bits * nx.u0) & ~15, n16 = ((4 * bits * nx.u0 - win) + 4 * bits * nx.nu + 15) >> 4;
             const int rows = p.Tk - nx.kt * KEYS;
             const uint8_t* from = codes + ((int64_t)nx.it.seq * p.Tk + nx.kt * KEYS + r0) * row_bytes + win + 16 * c0;
+            const uint32_t rb = (uint32_t)row_bytes;
 #pragma unroll 1
             for (int c = c0; c < n16; c += 8, from += 128) {
-                const uint8_t* f = from;
 #pragma unroll
-                for (int i = 0; i < ROWS_W / 4; ++i, f += 4 * row_bytes) {
+                for (int i = 0; i < ROWS_W / 4; ++i) {
                     const bool in = r0 + 4 * i < rows;
-                    cp_async16(dst(r0 + 4 * i, c), in ? f : codes, in ? 16 : 0);       // (size 0 reads nothing)
+                    cp_async16(dst(r0 + 4 * i, c), in ? from + (uint64_t)(4 * i) * rb : codes, in ? 16 : 0);       // (size 0 reads nothing)
                 }
             }
         };
@@ -415,24 +435,25 @@ prefill_kernel(const AttnParams p, const Plan g)
             if (!mbar_sleep(bar(B_QEMPTY), (n_item & 1) ^ 1, s_abort)) return false;
             const int i0 = it.qt * BM;
 #pragma unroll 1
-            for (int r4 = (warp - K_WARP0) * 16; r4 < (warp - K_WARP0) * 16 + 16; r4 += 2) {
-                uint32_t v[2][4];
+            for (int r4 = (warp - K_WARP0) * 16; r4 < (warp - K_WARP0) * 16 + 16; r4 += 4) {
+                uint16_t v[4][4][2];                          // (all loads first: they are bound by latency)
 #pragma unroll
-                for (int rr = 0; rr < 2; ++rr) {
+                for (int rr = 0; rr < 4; ++rr) {
                     const bool okr = i0 + r4 + rr < p.Tq;
-                    const __half* row = p.q_f16 + ((int64_t)it.seq * p.Tq + (okr ? i0 + r4 + rr : 0)) * p.ldq;
+                    const uint16_t* row = reinterpret_cast<const uint16_t*>(p.q_f16) + ((int64_t)it.seq * p.Tq + (okr ? i0 + r4 + rr : 0)) * p.ldq;
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        const uint32_t lo = okr && ca[k] >= 0 ? (uint32_t)__half_as_ushort(row[ca[k]]) : 0u;
-                        const uint32_t hi = okr && cb[k] >= 0 ? (uint32_t)__half_as_ushort(row[cb[k]]) : 0u;
-                        v[rr][k] = lo | (hi << 16);
+                        v[rr][k][0] = v[rr][k][1] = 0;
+                        if (okr && ca[k] >= 0) v[rr][k][0] = __ldg(row + ca[k]);
+                        if (okr && cb[k] >= 0) v[rr][k][1] = __ldg(row + cb[k]);
                     }
                 }
 #pragma unroll
-                for (int rr = 0; rr < 2; ++rr)
+                for (int rr = 0; rr < 4; ++rr)
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
-                        if (lane + 32 * k < 16 * nu) sts32(base + k * ATOM_Q + (r4 + rr) * 128 + (((lane >> 2) ^ ((r4 + rr) & 7)) << 4) + 4 * (lane & 3), v[rr][k]);
+                        if (lane + 32 * k < 16 * nu)
+                            sts32(base + k * ATOM_Q + (r4 + rr) * 128 + (((lane >> 2) ^ ((r4 + rr) & 7)) << 4) + 4 * (lane & 3), v[rr][k][0] | ((uint32_t)v[rr][k][1] << 16));
             }
             tc::fence_proxy_async();
             __syncwarp();
@@ -443,26 +464,24 @@ prefill_kernel(const AttnParams p, const Plan g)
         uint32_t n_item = 0;
         if (is_k) {
             // ------------------------------------------------------------ keys
-            const bool direct = MODE != KV && p.bits_k == 8;                   // bytes already: copied straight into the operand tile
+            constexpr bool direct = MODE != KV && K8;                   // bytes already: copied straight into the operand tile
             float czq = 0.f;                      // integer calls: -s^Q s^K z^Q qk_scale log2(e) of unit `lane`
             uint32_t seq[2] = {0, 0};             // KV: tiles of each stage (stream) so far
             // iteration n fetches tile n and works on tile n - 1
 #pragma unroll 1
             for (uint32_t n = 0; ok; ++n) {
-                auto fetch = [&]() {
-                    if (direct) {
+                // (with one raw buffer a tile is fetched just before it is worked on)
+                const bool ahead = direct || g.rawk_stages == 2;
+                if (ahead ? have : n > 0) {
+                    if constexpr (direct) {
+                        // (copied into the operand tile itself: its products must have read it)
+                        if (!mbar_sleep(bar(B_KEMPTY + (n & 1)), ((n >> 1) & 1) ^ 1, s_abort)) { ok = false; break; }
                         const uint32_t to = base + g.off_k + (n & 1) * g.k_stage;
-                        copy_rows([&](int r, int c) { return to + (c >> 3) * K_ATOM + r * 128 + (((c & 7) ^ (r & 7)) << 4); });
+                        copy_rows(nx, [&](int r, int c) { return to + (c >> 3) * K_ATOM + r * 128 + (((c & 7) ^ (r & 7)) << 4); });
                     } else {
-                        const uint32_t to = base + g.off_rawk + (g.rawk_stages == 2 ? (n & 1) * g.rawk_stage : 0);
-                        copy_rows([&](int r, int c) { return to + r * g.pitch_k + 16 * c; });
+                        const uint32_t to = base + g.off_rawk + (ahead ? (n & 1) * g.rawk_stage : 0);
+                        copy_rows(ahead ? nx : cu, [&](int r, int c) { return to + r * g.pitch_k + 16 * c; });
                     }
-                };
-                const bool ahead = direct || g.rawk_stages == 2 || n == 0;     // (one raw buffer: it is refilled after it was read)
-                if (have && ahead) {
-                    // (copied into the operand tile itself: its products must have read it)
-                    if (direct && !mbar_sleep(bar(B_KEMPTY + (n & 1)), ((n >> 1) & 1) ^ 1, s_abort)) { ok = false; break; }
-                    fetch();
                 }
                 cp_async_commit();
                 if (n > 0) {
@@ -485,7 +504,24 @@ prefill_kernel(const AttnParams p, const Plan g)
 #pragma unroll 2
                             for (int u = 0; u < nu; ++u) {
                                 uint32_t o[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-                                if (u < nuk && i < p.Tq) load_unit(q_row, cu.u0 + u, p.bits_q, o);
+                                if (u < nuk && i < p.Tq) {
+                                    load_unit(q_row, cu.u0 + u, p.bits_q, o);
+                                    if (g.folded) {
+                                        // 128 + q - z of every byte, then two's complement (I8), or sign and magnitude: the E4M3 pattern of
+                                        // (q - z) 2^-9. Pads hold some constant; the keys' pads are 0
+                                        const uint32_t z4 = (uint32_t)(int)__ldg(&p.unit_sz_q[cu.u0 + u].y) * 0x01010101u;
+#pragma unroll
+                                        for (int e = 0; e < 8; ++e) {
+                                            if (MODE == I8 && p.bits_q == 8) { o[e] ^= 0x80808080u; continue; }          // (z = 128)
+                                            const uint32_t t = (o[e] | 0x80808080u) - z4;
+                                            if constexpr (MODE == I8) o[e] = t ^ 0x80808080u;
+                                            else {
+                                                const uint32_t neg = ~t & 0x80808080u, one = neg >> 7;
+                                                o[e] = ((t ^ 0x80808080u ^ (one * 255u)) + one) | neg;
+                                            }
+                                        }
+                                    }
+                                }
                                 const uint32_t d = base + (u >> 2) * ATOM_Q + lt * 128, c = 2 * (u & 3), sw = lt & 7;
                                 sts128(d + ((c ^ sw) << 4), o[0], o[1], o[2], o[3]);
                                 sts128(d + (((c + 1) ^ sw) << 4), o[4], o[5], o[6], o[7]);
@@ -499,58 +535,73 @@ prefill_kernel(const AttnParams p, const Plan g)
                     if (ahead && have) cp_async_wait<1>(); else cp_async_wait<0>();
                     __syncwarp();                                              // (a warp unpacks the rows that it copied)
                     if (!direct && !mbar_sleep(bar(B_KEMPTY + st), (ph & 1) ^ 1, s_abort)) { ok = false; break; }
-                    const uint32_t raw0 = base + g.off_rawk + (g.rawk_stages == 2 ? (m & 1) * g.rawk_stage : 0) + ((4 * p.bits_k * cu.u0) & 15);
+                    const uint32_t raw0 = base + g.off_rawk + (ahead ? (m & 1) * g.rawk_stage : 0) + ((4 * p.bits_k * cu.u0) & 15);
                     if constexpr (MODE == KV) {
                         // thread = (row, parity of the unit)
                         const int r = lt >> 1, odd = lt & 1, sw = r & 7;
-                        const uint32_t raw = raw0 + r * g.pitch_k;
+                        const uint32_t raw = raw0 + r * g.pitch_k, d = tile + r * 128;
+                        if constexpr (K8) {
 #pragma unroll 2
-                        for (int u = odd; u < nu; u += 2) {
-                            const uint32_t d = tile + (u >> 1) * K_ATOM + r * 128;
-                            if (p.bits_k == 8) {
+                            for (int u = odd; u < nu; u += 2) {
                                 uint4 w[2] = {make_uint4(0u, 0u, 0u, 0u), make_uint4(0u, 0u, 0u, 0u)};
                                 if (u < nuk) { w[0] = lds128(raw + 32 * u); w[1] = lds128(raw + 32 * u + 16); }
                                 const uint32_t a[8] = {w[0].x, w[0].y, w[0].z, w[0].w, w[1].x, w[1].y, w[1].z, w[1].w};
 #pragma unroll
                                 for (int c = 0; c < 4; ++c)                        // eight codes = one chunk
-                                    sts128(d + (((4 * odd + c) ^ sw) << 4), byte_half<0>(a[2 * c]), byte_half<8>(a[2 * c]), byte_half<0>(a[2 * c + 1]), byte_half<8>(a[2 * c + 1]));
-                            } else {
-                                const uint4 w = u < nuk ? nibbles(raw, u, p.bits_k) : make_uint4(0u, 0u, 0u, 0u);
-                                const uint32_t a[4] = {w.x, w.y, w.z, w.w};
+                                    sts128(d + (u >> 1) * K_ATOM + (((4 * odd + c) ^ sw) << 4),
+                                           byte_half<0>(a[2 * c]), byte_half<8>(a[2 * c]), byte_half<0>(a[2 * c + 1]), byte_half<8>(a[2 * c + 1]));
+                            }
+                        } else {
+                            uint4 w[4];                                        // (all loads first: a warp on its own is bound by latency)
 #pragma unroll
-                                for (int c = 0; c < 4; ++c)
-                                    sts128(d + (((4 * odd + c) ^ sw) << 4), nib_half<0>(a[c]), nib_half<8>(a[c]), nib_half<4>(a[c]), nib_half<12>(a[c]));
+                            for (int i = 0; i < 4; ++i) w[i] = 2 * i + odd < nuk ? nibbles(raw, 2 * i + odd, p.bits_k) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                            for (int i = 0; i < 4; ++i) {
+                                if (2 * i + odd < nu) {
+                                    const uint32_t a[4] = {w[i].x, w[i].y, w[i].z, w[i].w};
+#pragma unroll
+                                    for (int c = 0; c < 4; ++c)
+                                        sts128(d + i * K_ATOM + (((4 * odd + c) ^ sw) << 4), nib_half<0>(a[c]), nib_half<8>(a[c]), nib_half<4>(a[c]), nib_half<12>(a[c]));
+                                }
                             }
                         }
                     } else {
                         const int r = lt, sw = r & 7;
-                        const uint32_t raw = raw0 + r * g.pitch_k;
-                        float col = 0.f;
-#pragma unroll 2
-                        for (int u = 0; u < nu; ++u) {
-                            const uint32_t d = tile + (u >> 2) * K_ATOM + r * 128, c = 2 * (u & 3);
-                            uint32_t o[8];
-                            if (direct) {
-                                const uint4 a = lds128(d + ((c ^ sw) << 4)), b = lds128(d + (((c + 1) ^ sw) << 4));
-                                o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
-                            } else {
-                                const uint4 w = u < nuk ? nibbles(raw, u, p.bits_k) : make_uint4(0u, 0u, 0u, 0u);
-                                o[0] = w.x & 0x0F0F0F0Fu; o[1] = (w.x >> 4) & 0x0F0F0F0Fu; o[2] = w.y & 0x0F0F0F0Fu; o[3] = (w.y >> 4) & 0x0F0F0F0Fu;
-                                o[4] = w.z & 0x0F0F0F0Fu; o[5] = (w.z >> 4) & 0x0F0F0F0Fu; o[6] = w.w & 0x0F0F0F0Fu; o[7] = (w.w >> 4) & 0x0F0F0F0Fu;
-                                sts128(d + ((c ^ sw) << 4), o[0], o[1], o[2], o[3]);
-                                sts128(d + (((c + 1) ^ sw) << 4), o[4], o[5], o[6], o[7]);
-                            }
-                            unsigned s = 0u;
+                        const uint32_t raw = raw0 + r * g.pitch_k, d = tile + r * 128;
+                        if constexpr (!direct) {
 #pragma unroll
-                            for (int e = 0; e < 8; ++e) s = __dp4a(o[e], 0x01010101u, s);
-                            col = __fmaf_rn(__shfl_sync(0xffffffffu, czq, u), (float)s, col);
+                            for (int h = 0; h < 2; ++h) {                      // one atom: four units, all loads first
+                                uint4 w[4];
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) w[i] = 4 * h + i < nuk ? nibbles(raw, 4 * h + i, p.bits_k) : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+                                for (int i = 0; i < 4; ++i) {
+                                    if (4 * h + i < nu) {
+                                        const uint32_t at = d + h * K_ATOM;
+                                        sts128(at + (((2 * i) ^ sw) << 4), w[i].x & 0x0F0F0F0Fu, (w[i].x >> 4) & 0x0F0F0F0Fu, w[i].y & 0x0F0F0F0Fu, (w[i].y >> 4) & 0x0F0F0F0Fu);
+                                        sts128(at + (((2 * i + 1) ^ sw) << 4), w[i].z & 0x0F0F0F0Fu, (w[i].z >> 4) & 0x0F0F0F0Fu, w[i].w & 0x0F0F0F0Fu, (w[i].w >> 4) & 0x0F0F0F0Fu);
+                                    }
+                                }
+                            }
                         }
-                        s_col[(m & 3) * KEYS + r] = col;
+                        if (!g.folded) {
+                            float col = 0.f;
+#pragma unroll 1
+                            for (int u = 0; u < nu; ++u) {
+                                const uint32_t at = d + (u >> 2) * K_ATOM, c = 2 * (u & 3);
+                                const uint4 a = lds128(at + ((c ^ sw) << 4)), b = lds128(at + (((c + 1) ^ sw) << 4));
+                                unsigned s0 = __dp4a(a.x, 0x01010101u, 0u), s1 = __dp4a(b.x, 0x01010101u, 0u);
+                                s0 = __dp4a(a.y, 0x01010101u, s0); s1 = __dp4a(b.y, 0x01010101u, s1);
+                                s0 = __dp4a(a.z, 0x01010101u, s0); s1 = __dp4a(b.z, 0x01010101u, s1);
+                                s0 = __dp4a(a.w, 0x01010101u, s0); s1 = __dp4a(b.w, 0x01010101u, s1);
+                                col = __fmaf_rn(__shfl_sync(0xffffffffu, czq, u), (float)(s0 + s1), col);
+                            }
+                            s_col[(m & 3) * KEYS + r] = col;
+                        }
                     }
                     tc::fence_proxy_async();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(B_KFULL + st));
-                    if (have && !ahead) { fetch(); cp_async_commit(); }
                 }
                 if (!have) break;
                 cu = nx;
@@ -591,7 +642,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                             const uint32_t d = tile + (32 * u + 8 * j) * 128;
                             // one chunk of position row 8 j + e; row & 7 = e
                             auto put = [&](int e, const uint32_t (&h4)[4]) { sts128(d + e * 128 + ((c8 ^ e) << 4), h4[0], h4[1], h4[2], h4[3]); };
-                            if (p.bits_v == 8) {
+                            if constexpr (V8) {
 #pragma unroll
                                 for (int half = 0; half < 2; ++half) {             // codes 4 half .. 4 half + 3
                                     uint32_t x[8];
@@ -646,8 +697,11 @@ prefill_kernel(const AttnParams p, const Plan g)
                         const uint32_t rows = raw + (32 * (lane >> 3) + (lane & 7)) * g.pitch_v;
 #pragma unroll 1
                         for (int u = lw; u < nuv; u += 4) {
-                            const uint32_t d = tile + 32 * u * 128 + wo;
-                            auto put = [&](int pos, uint32_t x) { sts32(d + pos * 128 + ((wc ^ (pos & 7)) << 4), x); };
+                            // position 8 k + i of the unit: row base at[i] + 1024 k (the swizzle depends on i alone)
+                            uint32_t at[8];
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) at[i] = tile + 32 * u * 128 + wo + i * 128 + ((wc ^ i) << 4);
+                            auto put = [&](int pos, uint32_t x) { sts32(at[pos & 7] + (pos >> 3) * 1024, x); };
                             // 4 x 4 byte transpose: out[i] = byte i of the four rows
                             auto transpose = [](uint32_t a, uint32_t b, uint32_t c, uint32_t e, uint32_t (&out)[4]) {
                                 const uint32_t x01l = __byte_perm(a, b, 0x5140), x01h = __byte_perm(a, b, 0x7362);
@@ -655,7 +709,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                                 out[0] = __byte_perm(x01l, x23l, 0x5410); out[1] = __byte_perm(x01l, x23l, 0x7632);
                                 out[2] = __byte_perm(x01h, x23h, 0x5410); out[3] = __byte_perm(x01h, x23h, 0x7632);
                             };
-                            if (p.bits_v == 8) {
+                            if constexpr (V8) {
 #pragma unroll
                                 for (int half = 0; half < 2; ++half) {
                                     uint4 rw[4];
@@ -692,7 +746,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                     if (lane == 0) mbar_arrive(bar(B_VFULL + st));
                     if (!group_sync()) { ok = false; break; }                  // the raw rows have been read
                 }
-                if (have) copy_rows([&](int r, int c) { return base + g.off_rawv + staged_row(r) * g.pitch_v + 16 * c; });
+                if (have) copy_rows(nx, [&](int r, int c) { return base + g.off_rawv + staged_row(r) * g.pitch_v + 16 * c; });
                 cp_async_commit();
                 if constexpr (MODE == KV) {
                     if (have && nx.t == 0 && !gather_queries(nx.it, n == 0 ? 0u : n_item + 1)) { ok = false; break; }
@@ -710,11 +764,11 @@ prefill_kernel(const AttnParams p, const Plan g)
                     if constexpr (MODE == KV) {
                         float l = 0.f;
 #pragma unroll
-                        for (int q = 0; q < 2; ++q) l += __uint_as_float(s_sum[q * BM + row]);
+                        for (int q = 0; q < PARTS; ++q) l += __uint_as_float(s_sum[q * BM + row]);
                         inv_l = 1.0f / l;
                     } else {
 #pragma unroll
-                        for (int q = 0; q < 2; ++q) rs += (int)s_sum[q * BM + row];
+                        for (int q = 0; q < PARTS; ++q) rs += (int)s_sum[q * BM + row];
                     }
                     const uint32_t stage = base + g.off_v, o_row = stage + row * g.out_pitch;
                     __half* out_row = p.out + ((int64_t)it.seq * p.Tq + i) * p.ldo;
@@ -724,25 +778,35 @@ prefill_kernel(const AttnParams p, const Plan g)
                         const int pos = 32 * (uv0 + u) + lane;
                         int ch = __ldg(p.jidx_v + pos) >= 0 ? (int)__ldg(p.src_v + pos) : -1;
                         const float2 sz = __ldg(p.unit_sz_v + uv0 + u);
-                        const float sc = MODE == KV ? sz.x * inv_l : p.s_P * sz.x, zf = sz.x * (sz.y - (p.bits_v == 8 ? 128.0f : 8.0f));
+                        const float sc = MODE == KV ? sz.x * inv_l : p.s_P * sz.x, zf = sz.x * (sz.y - (V8 ? 128.0f : 8.0f));
                         const int zi = (int)sz.y * rs;
                         if (g.local_v && ch >= 0) ch = 2 * (ch - it.h * p.hd);         // its byte within a staged row
+                        auto value = [&](uint32_t v) {
+                            if constexpr (MODE == KV) return __half_as_ushort(__float2half_rn(__fmaf_rn(__uint_as_float(v), sc, -zf)));
+                            else return __half_as_ushort(__float2half_rn(sc * (float)((int)v - zi)));
+                        };
+                        const uint32_t t_unit = tmem + ((uint32_t)(32 * lw) << 16) + 32 * u;
+                        if (!g.local_v) {                                      // straight to the channel, column by column (rare layouts)
 #pragma unroll 1
-                        for (int part = 0; part < 2; ++part) {
+                            for (int e = 0; e < 32; ++e) {
+                                const int c = __shfl_sync(0xffffffffu, ch, e);
+                                uint32_t v;
+                                asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(v) : "r"(t_unit + e) : "memory");
+                                tc::tc_wait_ld();
+                                if (c >= 0 && i < p.Tq) out_row[c] = __ushort_as_half(value(v));
+                            }
+                            continue;
+                        }
+#pragma unroll 1
+                        for (int h = 0; h < 2; ++h) {
                             uint32_t v[16];
-                            tc::tc_ld16(tmem + ((uint32_t)(32 * lw) << 16) + 32 * u + 16 * part, v);
+                            tc::tc_ld16(t_unit + 16 * h, v);
                             tc::tc_wait_ld();
+                            // (the staged words of row r are exchanged by r & 31: no bank conflicts)
 #pragma unroll
                             for (int e = 0; e < 16; ++e) {
-                                const int c = __shfl_sync(0xffffffffu, ch, 16 * part + e);
-                                if (c < 0) continue;
-                                float o;
-                                if constexpr (MODE == KV) o = __fmaf_rn(__uint_as_float(v[e]), sc, -zf);
-                                else o = sc * (float)((int)v[e] - zi);
-                                const uint16_t oh = __half_as_ushort(__float2half_rn(o));
-                                // (the staged words of row r are exchanged by r & 31: no bank conflicts)
-                                if (g.local_v) sts16(o_row + ((uint32_t)c ^ ((uint32_t)lane << 2)), oh);
-                                else if (i < p.Tq) out_row[c] = __ushort_as_half(oh);
+                                const int c = __shfl_sync(0xffffffffu, ch, 16 * h + e);
+                                sts16_if(c >= 0, o_row + ((uint32_t)c ^ ((uint32_t)lane << 2)), value(v[e]));
                             }
                         }
                     }
@@ -779,9 +843,9 @@ prefill_kernel(const AttnParams p, const Plan g)
     } else {
         // ---------------------------------------------------------------- softmax
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX));
-        const int q4 = warp & 3, stream = (warp - S_WARP0) >> 2;               // lane quarter of the accumulators
+        const int q4 = warp & 3, part = (warp - S_WARP0) >> 2, stream = part / SUB, sub = part % SUB;      // q4: lane quarter of the accumulators
         const int row = 32 * q4 + lane;                                        // query row within the tile
-        const uint32_t t_col = tmem + ((uint32_t)(32 * q4) << 16) + O_COLS + stream * (N_SLOTS * COLS);
+        const uint32_t t_col = tmem + ((uint32_t)(32 * q4) << 16) + O_COLS + stream * (N_SLOTS * COLS) + sub * CT;
         const uint32_t b_full0 = bar(B_SFULL + stream * N_SLOTS), b_empty0 = bar(B_SEMPTY + stream * N_SLOTS);
         uint32_t n_k0 = 0, slot = 0, par = 0, n_s = 0, n_item = 0;   // n_s: my stream's tiles of pass 2 so far
         bool ok = true;
@@ -811,25 +875,26 @@ prefill_kernel(const AttnParams p, const Plan g)
 #pragma unroll 1
             for (int pass = 0; pass < 2 && ok; ++pass, n_k0 += it.n_kt) {
                 if (pass == 1) {
-                    // the streams' statistics meet (two sets by turns: a warp may be an item ahead of another)
-                    float2* ml = s_ml + (n_item & 1) * 2 * BM;
-                    ml[stream * BM + row] = make_float2(m, l);
+                    // the parts' statistics meet (two sets by turns: a warp may be an item ahead of another)
+                    float2* ml = s_ml + (n_item & 1) * PARTS * BM + row;
+                    ml[part * BM] = make_float2(m, l);
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(B_XS));
                     if (!mbar_sleep(bar(B_XS), n_item & 1, s_abort)) { ok = false; break; }
-                    const float2 o = ml[(stream ^ 1) * BM + row];
-                    const float n = fmaxf(m, o.x);
+#pragma unroll
+                    for (int q = 0; q < PARTS; ++q) m = fmaxf(m, ml[q * BM].x);
                     if constexpr (MODE != KV) {
-                        l = l * ex2(m - n) + o.y * ex2(o.x - n);               // (a stream without a visible key weighs 0)
+                        l = 0.f;
+#pragma unroll
+                        for (int q = 0; q < PARTS; ++q) l = __fmaf_rn(ml[q * BM].y, ex2(ml[q * BM].x - m), l);     // (a part without a visible key weighs 0)
                         f = p.inv_sP / l * 1.7763568394002505e-15f;            // times 2^-49: see below
                     }
-                    m = n;
                 }
 #pragma unroll 1
                 for (int kt = ALT ? stream : 0; kt < it.n_kt; kt += ALT ? 2 : 1) {
                     // ---- scores of my row against my keys of the tile, times log2(e); hidden keys at NEG_BIG
-                    float2 S[COLS / 2];
-                    const float* col = s_col + ((n_k0 + kt) & 3) * KEYS + stream * COLS;
+                    float2 S[CT / 2];
+                    const float* col = s_col + ((n_k0 + kt) & 3) * KEYS + stream * COLS + sub * CT;
                     bool first = true;
                     uint32_t left = last;                                      // (at least one bit)
                     do {
@@ -841,12 +906,11 @@ prefill_kernel(const AttnParams p, const Plan g)
                             uint32_t v[32];
                             ld32(t_col + slot * COLS, v);
                             if (first) {
-                                if constexpr (MODE == KV) {
 #pragma unroll
-                                    for (int e = 0; e < COLS / 2; ++e) S[e] = make_float2(0.f, 0.f);
-                                } else {
+                                for (int e = 0; e < CT / 2; ++e) S[e] = make_float2(0.f, 0.f);
+                                if (MODE != KV && !g.folded) {
 #pragma unroll
-                                    for (int e = 0; e < COLS / 2; e += 2) {
+                                    for (int e = 0; e < CT / 2; e += 2) {
                                         const float4 x = *reinterpret_cast<const float4*>(col + 2 * e);
                                         S[e] = make_float2(x.x, x.y); S[e + 1] = make_float2(x.z, x.w);
                                     }
@@ -854,16 +918,16 @@ prefill_kernel(const AttnParams p, const Plan g)
                             }
                             const float2 c2 = make_float2(c, c);
 #pragma unroll
-                            for (int part = 0; part < 2; ++part) {
+                            for (int h = 0; h < CT / 32; ++h) {
                                 tc::tc_wait_ld();
 #pragma unroll
                                 for (int e = 0; e < 16; ++e) {
                                     float2 x;
                                     if constexpr (MODE == I8) x = make_float2((float)(int)v[2 * e], (float)(int)v[2 * e + 1]);
                                     else x = make_float2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
-                                    S[16 * part + e] = fma2(c2, x, S[16 * part + e]);
+                                    S[16 * h + e] = fma2(c2, x, S[16 * h + e]);
                                 }
-                                if (part == 0) ld32(t_col + slot * COLS + 32, v);
+                                if (h + 1 < CT / 32) ld32(t_col + slot * COLS + 32, v);
                             }
                         }
                         first = false;
@@ -875,11 +939,11 @@ prefill_kernel(const AttnParams p, const Plan g)
                         left &= left - 1;
                     } while (left);
                     if (!ok) break;
-                    const int j0 = kt * KEYS + (ALT ? 0 : stream * COLS);
-                    if (live && j0 + COLS - 1 > vis_all) {
+                    const int j0 = kt * KEYS + (ALT ? 0 : stream * COLS) + sub * CT;
+                    if (live && j0 + CT - 1 > vis_all) {
                         const int n_vis = vis - j0;                            // my last visible column
 #pragma unroll
-                        for (int e = 0; e < COLS / 2; ++e) {
+                        for (int e = 0; e < CT / 2; ++e) {
                             if (2 * e > n_vis) S[e].x = NEG_BIG;
                             if (2 * e + 1 > n_vis) S[e].y = NEG_BIG;
                         }
@@ -889,7 +953,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                         if (live) {
                             float x0 = NEG_BIG, x1 = NEG_BIG;
 #pragma unroll
-                            for (int e = 0; e < COLS / 2; e += 2) {
+                            for (int e = 0; e < CT / 2; e += 2) {
                                 x0 = fmaxf(x0, fmaxf(S[e].x, S[e].y));
                                 x1 = fmaxf(x1, fmaxf(S[e + 1].x, S[e + 1].y));
                             }
@@ -898,7 +962,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                                 const float2 nn = make_float2(-n, -n);
                                 float2 a0 = make_float2(0.f, 0.f), a1 = a0;
 #pragma unroll
-                                for (int e = 0; e < COLS / 2; e += 2) {
+                                for (int e = 0; e < CT / 2; e += 2) {
                                     const float2 y = add2(S[e], nn), z = add2(S[e + 1], nn);
                                     a0 = add2(a0, make_float2(ex2(y.x), ex2(y.y)));
                                     a1 = add2(a1, make_float2(ex2(z.x), ex2(z.y)));
@@ -921,7 +985,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                         if constexpr (MODE == KV) {
                             const uint32_t p_row = base + g.off_p + (g.p_tiles == 2 ? stream * (BM * 128) : 0) + row * 128;
 #pragma unroll
-                            for (int blk = 0; blk < 4; ++blk)
+                            for (int blk = 0; blk < CT / 16; ++blk)
 #pragma unroll
                                 for (int y = 0; y < 2; ++y) {                  // chunk 2 blk + y: keys 16 blk + 4 b + 2 y + {0, 1}
                                     uint32_t w[4];
@@ -932,7 +996,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                                         const float2 r = __half22float2(*reinterpret_cast<const __half2*>(&w[b]));
                                         lsum += r.x + r.y;   // the rounded values: the division normalises what was multiplied
                                     }
-                                    sts128(p_row + (((2 * blk + y) ^ (row & 7)) << 4), w[0], w[1], w[2], w[3]);
+                                    sts128(p_row + (((CT / 8 * sub + 2 * blk + y) ^ (row & 7)) << 4), w[0], w[1], w[2], w[3]);
                                 }
                         } else {
                             // code = min(rne(2^(S - m) / (s_P l)), 255): the product scaled by 2^-149 is rounded once, half to even, to the
@@ -940,7 +1004,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                             const float2 f2 = make_float2(f, f), k100 = make_float2(7.888609052210118e-31f, 7.888609052210118e-31f);   // 2^-100
                             const uint32_t p_row = base + g.off_p + row * 128;
 #pragma unroll
-                            for (int blk = 0; blk < 2; ++blk) {                // 32 keys: word x has keys x + 8 b
+                            for (int blk = 0; blk < CT / 32; ++blk) {          // 32 keys: word x has keys x + 8 b
                                 uint32_t w[8];
 #pragma unroll
                                 for (int e = 0; e < 4; ++e) {
@@ -957,15 +1021,15 @@ prefill_kernel(const AttnParams p, const Plan g)
                                         rsum = __dp4a(w[2 * e + k], 0x01010101u, rsum);
                                     }
                                 }
-                                const int c = 4 * stream + 2 * blk;
+                                const int c = 4 * stream + CT / 16 * sub + 2 * blk;
                                 sts128(p_row + ((c ^ (row & 7)) << 4), w[0], w[1], w[2], w[3]);
                                 sts128(p_row + (((c + 1) ^ (row & 7)) << 4), w[4], w[5], w[6], w[7]);
                             }
                             if (p.p_dbg && i < p.Tq) {                         // key k of the stream: byte (k & 31) / 8 of word k & 7 of block k / 32
                                 uint8_t* dst = p.p_dbg + (((int64_t)it.seq * p.H + it.h) * p.Tq + i) * p.Tk;
 #pragma unroll 1
-                                for (int k = 0; k < COLS && j0 + k < p.Tk; ++k) {
-                                    const int c = 4 * stream + 2 * (k >> 5) + ((k & 7) >> 2);
+                                for (int k = 0; k < CT && j0 + k < p.Tk; ++k) {
+                                    const int c = 4 * stream + CT / 16 * sub + 2 * (k >> 5) + ((k & 7) >> 2);
                                     dst[j0 + k] = (uint8_t)(lds32(p_row + ((c ^ (row & 7)) << 4) + 4 * (k & 3)) >> (8 * ((k & 31) >> 3)));
                                 }
                             }
@@ -979,7 +1043,7 @@ prefill_kernel(const AttnParams p, const Plan g)
             if (!ok) break;
             // (a stream without a tile of its own has not waited for the previous item's sums to be read)
             if (ALT && it.n_kt == 1 && !mbar_sleep(bar(B_OUT), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
-            s_sum[stream * BM + row] = MODE == KV ? __float_as_uint(lsum) : rsum;
+            s_sum[part * BM + row] = MODE == KV ? __float_as_uint(lsum) : rsum;
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(B_SUM));
         }
@@ -993,16 +1057,20 @@ prefill_kernel(const AttnParams p, const Plan g)
     if (tid == 0 && *s_abort && g.status) atomicExch(g.status, RPTQ_ERR_DEVICE_TIMEOUT);
 }
 
-template <int MODE>
-static int launch_one(const AttnParams& p, int units_k, int units_v, int n_seq, bool v_heads_local, int dev, int n_sm, cudaStream_t st)
+template <int MODE, bool K8, bool V8>
+static int launch_one(const AttnParams& p, int zq_min, int zq_max, int units_k, int units_v, int n_seq, bool v_heads_local, int dev, int n_sm, cudaStream_t st)
 {
     constexpr int KEYS = keys_of(MODE);
+    const int qmax_q = (1 << p.bits_q) - 1;
     Plan g{};
     g.n_qt = (p.Tq + BM - 1) / BM;
-    g.n_seq = n_seq;
     const int64_t items = (int64_t)g.n_qt * p.H * n_seq;
     if (items > 2147483647ll) return RPTQ_ERR_UNSUPPORTED;
     g.n_items = (int)items;
+    g.per_qt = p.H * n_seq;
+    auto inverse = [](uint32_t d) { return (uint32_t)(((uint64_t(1) << 32) + d - 1) / d); };       // (d = 1 is not divided by)
+    g.inv_per_qt = inverse((uint32_t)g.per_qt);
+    g.inv_h = inverse((uint32_t)p.H);
     const int atoms = MODE == KV ? (units_k + 1) / 2 : (units_k + 3) / 4;
     g.off_k = atoms * ATOM_Q;
     g.k_stage = atoms * KEYS * 128;
@@ -1011,7 +1079,7 @@ static int launch_one(const AttnParams& p, int units_k, int units_v, int n_seq, 
     g.pitch_k = raw_pitch_of(p.bits_k, units_k);
     g.pitch_v = raw_pitch_of(p.bits_v, units_v);
     g.rawk_stage = MODE != KV && p.bits_k == 8 ? 0 : KEYS * g.pitch_k;
-    const int rest = BM * 128 + KEYS * g.pitch_v + 4 * KEYS * 4 + 4 * BM * 8 + 2 * BM * 4 + 512;
+    const int rest = BM * 128 + KEYS * g.pitch_v + 4 * KEYS * 4 + 2 * PARTS * BM * 8 + PARTS * BM * 4 + 512;
     constexpr int LIMIT = 226 * 1024;                     // (with 1 KiB for the alignment: the most a block may have)
     // a second packed key tile first (the copies of a tile then have a whole tile's time), then (KV) a probability tile for each
     // stream, then a second value tile
@@ -1026,33 +1094,49 @@ static int launch_one(const AttnParams& p, int units_k, int units_v, int n_seq, 
     g.off_rawv = g.off_rawk + g.rawk_stages * g.rawk_stage;
     g.off_col = g.off_rawv + KEYS * g.pitch_v;
     g.off_ml = g.off_col + 4 * KEYS * 4;
-    g.off_sum = g.off_ml + 4 * BM * 8;
-    g.off_bar = g.off_sum + 2 * BM * 4;
+    g.off_sum = g.off_ml + 2 * PARTS * BM * 8;
+    g.off_bar = g.off_sum + PARTS * BM * 4;
     g.total = g.off_bar + 512;
     if (g.total > LIMIT) return RPTQ_ERR_UNSUPPORTED;
     // the output tile is staged in the V and P region (rows of a multiple of 128 bytes: see the staging stores)
     g.out_pitch = (2 * p.hd + 127) / 128 * 128;
     g.local_v = v_heads_local && BM * g.out_pitch <= g.v_stages * g.v_stage + g.p_tiles * BM * 128;
+    g.folded = MODE == F8 ? zq_min >= qmax_q - 16 && zq_max <= 16 : MODE == I8 ? zq_min >= qmax_q - 127 && zq_max <= 128 : 0;
     g.status = device_status_word();
-    const void* fn = reinterpret_cast<const void*>(prefill_kernel<MODE>);
+    const void* fn = reinterpret_cast<const void*>(prefill_kernel<MODE, K8, V8>);
     static std::atomic<uint64_t> done{0}, pool_ok{0};
     if (!(pool_ok.load(std::memory_order_acquire) >> (dev & 63) & 1u)) {
         cudaFuncAttributes attr;
         if (cudaFuncGetAttributes(&attr, fn) != cudaSuccess) return RPTQ_ERR_CUDA;
         // the register re-partition (setmaxnreg) draws on what the block is launched with
-        if (attr.numRegs * THREADS < 128 * (REGS_MMA + 2 * REGS_LOAD + 2 * REGS_SOFTMAX)) return RPTQ_ERR_UNSUPPORTED;
+        if (attr.numRegs * THREADS < 128 * REGS_ALL) return RPTQ_ERR_UNSUPPORTED;
         if (dev >= 0 && dev < 64) pool_ok.fetch_or(uint64_t(1) << dev, std::memory_order_release);
     }
     if (allow_smem(fn, dev, 227 * 1024, done) != RPTQ_OK) return RPTQ_ERR_CUDA;
     const int grid = g.n_items < n_sm ? g.n_items : n_sm;
-    return launch_kernel(prefill_kernel<MODE>, dim3((unsigned)grid), THREADS, (size_t)g.total + 1024, 0, st, p, g);
+    return launch_kernel(prefill_kernel<MODE, K8, V8>, dim3((unsigned)grid), THREADS, (size_t)g.total + 1024, 0, st, p, g);
 }
 
-int launch(const AttnParams& p, bool kv, int units_k, int units_v, int n_seq, bool v_heads_local, int dev, int n_sm, cudaStream_t st)
+int launch(const AttnParams& p, bool kv, int zq_min, int zq_max, int units_k, int units_v, int n_seq, bool v_heads_local, int dev, int n_sm, cudaStream_t st)
 {
-    if (kv) return launch_one<KV>(p, units_k, units_v, n_seq, v_heads_local, dev, n_sm, st);
-    if (p.bits_q <= 4 && p.bits_k <= 4) return launch_one<F8>(p, units_k, units_v, n_seq, v_heads_local, dev, n_sm, st);
-    return launch_one<I8>(p, units_k, units_v, n_seq, v_heads_local, dev, n_sm, st);
+    const bool k8 = p.bits_k == 8, v8 = p.bits_v == 8;
+    auto go = [&](auto mode, auto ek, auto ev) {
+        return launch_one<decltype(mode)::value, decltype(ek)::value, decltype(ev)::value>(p, zq_min, zq_max, units_k, units_v, n_seq, v_heads_local, dev, n_sm, st);
+    };
+    using std::false_type;
+    using std::true_type;
+    if (kv) {
+        const std::integral_constant<int, KV> mode;
+        if (k8) return v8 ? go(mode, true_type(), true_type()) : go(mode, true_type(), false_type());
+        return v8 ? go(mode, false_type(), true_type()) : go(mode, false_type(), false_type());
+    }
+    if (p.bits_q <= 4 && !k8) {
+        const std::integral_constant<int, F8> mode;
+        return v8 ? go(mode, false_type(), true_type()) : go(mode, false_type(), false_type());
+    }
+    const std::integral_constant<int, I8> mode;
+    if (k8) return v8 ? go(mode, true_type(), true_type()) : go(mode, true_type(), false_type());
+    return v8 ? go(mode, false_type(), true_type()) : go(mode, false_type(), false_type());
 }
 
 }  // namespace attn_prefill

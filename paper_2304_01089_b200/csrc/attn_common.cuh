@@ -118,8 +118,9 @@ namespace attn_decode {
 bool fits(const attn::AttnParams& p, bool kv);     // false: the prefill kernel takes the call
 int launch(const attn::AttnParams& p, bool kv, int units_k, int units_v, int n_seq, int dev, int n_sm, cudaStream_t st);
 }
-// The kernel for more queries (attention_prefill.cu). v_heads_local: head h of V owns the channels h * hd .. (h + 1) * hd - 1.
+// The kernel for more queries (attention_prefill.cu). zq_min, zq_max: the range of the query's zero points (integer calls);
+// v_heads_local: head h of V owns the channels h * hd .. (h + 1) * hd - 1.
 namespace attn_prefill {
-int launch(const attn::AttnParams& p, bool kv, int units_k, int units_v, int n_seq, bool v_heads_local, int dev, int n_sm, cudaStream_t st);
+int launch(const attn::AttnParams& p, bool kv, int zq_min, int zq_max, int units_k, int units_v, int n_seq, bool v_heads_local, int dev, int n_sm, cudaStream_t st);
 }
 }  // namespace rptq

@@ -266,6 +266,13 @@ int rptq_layout_create(rptq_layout_t** out, int C, int g, int bits, const int32_
             ui.nvalid = (n - 32 * uc) < 32 ? (n - 32 * uc) : 32;
         }
     }
+    bool first_z = true;
+    for (int c = 0; c < g; ++c) {
+        if (cluster_size[c] == 0) continue;
+        L->z_min = first_z ? zero_host[c] : std::min(L->z_min, zero_host[c]);
+        L->z_max = first_z ? zero_host[c] : std::max(L->z_max, zero_host[c]);
+        first_z = false;
+    }
     // ---- what the attention entry points ask about per-head layouts on every call
     L->in_cluster_order = true;
     for (int u = 1; u < cur; ++u)

@@ -38,6 +38,7 @@ struct rptq_layout {
     int n_units = 0;   // K_pad / 32
     int n_seg = 0;     // clusters with n_c > 0
     std::vector<int32_t> perm, size, zero;
+    int z_min = 0, z_max = 0;            // over the non-empty clusters
     std::vector<int32_t> pos;            // [C]       padded position of reordered channel j
     std::vector<int32_t> unit_cluster;   // [n_units] owning cluster, -1 past the last cluster
     std::vector<float> scale;
