@@ -18,9 +18,7 @@
 //                 magnitude for E4M3), otherwise q, and form the per-key term -sum_c s^Q s^K z^Q sum_p K_q
 //   warps 8-11    values: unpacked and transposed into [position][key] (byte permutes on the packed words); and the
 //                 output of an item, while the next item's pass 1 runs (they have nothing else to do there)
-//   warps 12-19   softmax, four per stream: thread = query row, 64 keys; S = sum_c coef_c acc_c in registers. (Sixteen warps
-//                 with 32 keys each were slower, 1418 against 1028 us: the hand-over of a cluster costs as many
-//                 instructions for 32 keys as for 64)
+//   warps 12-19   softmax, four per stream: thread = query row, 64 keys; S = sum_c coef_c acc_c in registers
 // Operand types (MODE):
 //   I8   bytes, kind::i8, int32 sums
 //   F8   both codes of at most four bits: a nibble n as an 8-bit E4M3 pattern IS the number n 2^-9, so the same bytes
@@ -33,7 +31,11 @@
 // quarter of 32 keys, byte b of word w is key w + 8 b; KV, quarters of 16 keys: fp16 pair b of chunk y is keys
 // 4 b + 2 y + {0, 1}. It lets the V loader read and write shared memory without bank conflicts.
 //
-// Measured: MEASURED_PREFILL
+// Measured, us, against a mma.sync kernel with 64 (KV: 128) queries per block (72 heads of 128 channels, four clusters each,
+// causal, two sequences of 2048 tokens): 3 bits 2321 -> 876, 8 bits 3856 -> 935; KV, 3 bits 2703 -> 1694; KV, 32 heads,
+// three sequences, 1100 queries on 1337 keys, 4 bits 945 -> 468; 16 queries on 2000 keys, four sequences 269 -> 200 (KV 549 ->
+// 355). A tile of 128 x 128 scores takes about 5000 clocks and pass, of which a warp's own chain of drains, exponentials and
+// waits is the most; the tensor cores are idle most of the time.
 #include <type_traits>
 
 #include "attn_common.cuh"
@@ -50,7 +52,9 @@ using tc::mbar_sleep;
 using tc::mbar_sleep_warp;
 
 enum { I8 = 0, F8 = 1, KV = 2 };
-constexpr int SUB = 1;                                    // softmax warps that share a stream's piece of work (and a lane quarter)
+// Softmax warps that share a stream's piece of work (and a lane quarter). 2 (sixteen warps of 32 keys a thread) measured the same
+// within 3 % with small code, KV 35 % slower: the loaders then have 56 registers and spill.
+constexpr int SUB = 1;
 constexpr int BM = 128, THREADS = 384 + 256 * SUB;
 constexpr int K_WARP0 = 4, V_WARP0 = 8, S_WARP0 = 12;
 constexpr int COLS = 64;                                  // keys of a stream's piece of work = columns of a score slot

@@ -301,3 +301,37 @@ def test_few_queries(Tq, Tk, causal, bits):
 def test_few_queries_of_many_heads_take_one_block_per_head():
     """300 heads: no split of the keys."""
     Case(950, H=300, hd=16, gh=4, Tq=3, Tk=40, bits=(4, 4, 4)).check(True)
+
+
+# The kernel for more queries: tiles of 128 queries and 128 keys (two streams of 64), query zero points folded into the operand where
+# they fit it. Sizes around a tile; zero points that do not fit; 8-bit queries with the one that does; every mix of widths; a head
+# of eight units; more work items than SMs.
+@pytest.mark.parametrize("Tq,Tk,causal", [(9, 9, True), (127, 128, True), (128, 129, False), (129, 257, True), (257, 400, True)])
+@pytest.mark.parametrize("bits", [(4, 4, 4), (3, 4, 8), (4, 8, 3), (8, 3, 4)])
+def test_tile_edges(Tq, Tk, causal, bits):
+    Case(700 + Tq + 10 * bits[1] + bits[2], H=2, hd=72, gh=4, Tq=Tq, Tk=Tk, bits=bits).check(causal)
+
+
+@pytest.mark.parametrize("bits,lo,hi", [((4, 4, 4), -40, 60), ((3, 3, 3), -9, 17), ((4, 8, 8), -100, 120), ((8, 8, 4), 128, 129)])
+def test_query_zero_points(bits, lo, hi):
+    from paper_2304_01089_b200 import binding
+    c = Case(720, H=3, hd=64, gh=4, Tq=140, Tk=150, bits=bits)
+    c.zQ = np.random.default_rng(5).integers(lo, hi, size=c.zQ.shape[0]).astype(np.int32)
+    c.LQ = binding.Layout(c.perm_qk, c.size_qk, c.sQ, c.zQ, bits[0])
+    c.check(True)
+
+
+def test_many_items_and_wide_heads():
+    Case(730, H=90, hd=16, gh=2, Tq=140, Tk=200, bits=(4, 4, 4)).check(True)
+    Case(731, H=2, hd=256, gh=1, Tq=130, Tk=140, bits=(8, 8, 8)).check(True)
+
+
+def test_value_heads_that_own_other_channels():
+    """rptq_attention writes V's position to its own channel whichever head that belongs to."""
+    import torch
+    from paper_2304_01089_b200 import binding
+    c = Case(740, H=3, hd=40, gh=4, Tq=150, Tk=150)
+    c.perm_v = np.random.default_rng(6).permutation(120).astype(np.int32)
+    c.LV = binding.Layout(c.perm_v, c.size_v, c.sV, c.zV, 4)
+    c.dv = torch.from_numpy(oracle.pack(np.ascontiguousarray(c.v[:, c.LV.contiguous_position()]), 4)).cuda()
+    c.check(True)

@@ -164,3 +164,18 @@ def test_opt66b_heads_sampled_rows():
 def test_few_queries(Tq, Tk, n_seq, causal, bits):
     c = Case(900 + Tk + 10 * bits[1] + bits[2], H=2, hd=72, gh=4, Tq=Tq * n_seq, Tk=Tk * n_seq, bits=bits)
     _check(c, _query(np.random.default_rng(3), Tq * n_seq, 144), causal, n_seq=n_seq)
+
+
+# The kernel for more queries: see test_attention_gpu.py::test_tile_edges; tiles of 64 keys that two streams take by turns.
+@pytest.mark.parametrize("Tq,Tk,n_seq,causal", [(9, 9, 1, True), (64, 65, 1, True), (128, 128, 2, False), (129, 257, 1, True), (200, 400, 1, True)])
+@pytest.mark.parametrize("bits", [(4, 4, 4), (4, 3, 8), (4, 8, 3)])
+def test_tile_edges(Tq, Tk, n_seq, causal, bits):
+    c = Case(700 + Tq + 10 * bits[1] + bits[2], H=2, hd=72, gh=4, Tq=Tq * n_seq, Tk=Tk * n_seq, bits=bits)
+    _check(c, _query(np.random.default_rng(7), Tq * n_seq, 144), causal, n_seq=n_seq)
+
+
+def test_many_items_and_wide_heads():
+    c = Case(730, H=90, hd=16, gh=2, Tq=140, Tk=200)
+    _check(c, _query(np.random.default_rng(8), 140, 90 * 16), True)
+    c = Case(731, H=2, hd=256, gh=1, Tq=130, Tk=140, bits=(4, 8, 8))
+    _check(c, _query(np.random.default_rng(9), 130, 512), True)
