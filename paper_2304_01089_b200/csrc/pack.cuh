@@ -7,16 +7,11 @@ namespace rptq {
 
 // The quantiser decision of the GEMM's re-quantising epilogue (Eq. 1 with codes re-based to
 // [0, 2^bits - 1]): t = y * inv_s rounded ONCE to an integer, half to even (the fused multiply-add
-// forms the product exactly; adding 1.5 * 2^23 leaves the rounded integer in the low mantissa bits
-// for |t| < 2^22; larger t keep their order, and everything below -2^22, the negative sums whose bit
+// v = y * inv_s + 1.5 * 2^23 forms the product exactly and leaves the rounded integer in the low mantissa
+// bits for |t| < 2^22; larger t keep their order, and everything below -2^22, the negative sums whose bit
 // patterns would wrap included, is raised to 2^23, i.e. to an integer far below any zero point),
-// then + z_c and clamp. zc = z_c - 0x4B400000 (the bit pattern of 1.5 * 2^23); |z_c| < 2^21.
-__device__ __forceinline__ uint32_t quant_code(float y, float inv_s, int zc, int qmax)
-{
-    const float v = fmaxf(__fmaf_rn(y, inv_s, 12582912.0f), 8388608.0f);
-    const int q = __float_as_int(v) + zc;
-    return (uint32_t)min(max(q, 0), qmax);
-}
+// then + z_c; the saturating pack clamps. zc = z_c - 0x4B400000 (the bit pattern of 1.5 * 2^23); |z_c| < 2^21.
+__device__ __forceinline__ int quant_int(float v, int zc) { return __float_as_int(fmaxf(v, 8388608.0f)) + zc; }
 
 __device__ __forceinline__ uint32_t nibble_word(const uint32_t* q)   // 8 codes -> one 4-bit-layout word
 {
