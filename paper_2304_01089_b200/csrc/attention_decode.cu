@@ -157,7 +157,7 @@ decode_kernel(const AttnParams p, int keys_block, int units_k_max, int units_v_m
     __shared__ __align__(16) uint32_t s_q[MODE == HALF ? MAX_Q * 16 * MAX_UNITS : MODE == LIMB ? LIMB_Q * 32 * MAX_UNITS : 4];
     __shared__ __align__(16) uint32_t s_qb[32 * MAX_UNITS][MODE == HALF ? 4 : 2];
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g8 = lane >> 2, t4 = lane & 3;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, g8 = lane >> 2, t4 = lane & 3;
     const int h = blockIdx.y;
     const uint32_t rank = cluster_rank(), n_ranks = cluster_size();
     const int64_t q_row0 = (int64_t)blockIdx.z * p.Tq, k_row0 = (int64_t)blockIdx.z * p.Tk;

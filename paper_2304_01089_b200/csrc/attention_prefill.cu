@@ -241,7 +241,7 @@ prefill_kernel(const AttnParams p, const Plan g)
     volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
     const uint32_t bar0 = smem_u32(bars);
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
 
     if (tid == 0) {
         mbar_init(bar(B_QFULL), Q_LOADERS); mbar_init(bar(B_QEMPTY), 2);

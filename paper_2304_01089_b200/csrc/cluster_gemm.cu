@@ -342,7 +342,7 @@ cluster_gemm_kernel(const Params p)
     const uint32_t bar0 = smem_u32(bars);
     auto bar = [&](int i) { return bar0 + 8u * (uint32_t)i; };
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int n_steps = p.n_kb * 4;
     const uint32_t cta_rank = NCTA == 2 ? cluster_ctarank() : 0u;       // rank 0 issues the MMAs
     const int pair_id = (int)blockIdx.x / NCTA, n_pairs = (int)gridDim.x / NCTA;

@@ -144,7 +144,7 @@ ln_reorder_quant_kernel(const LnParams p)
     const uint32_t tx_extra = SELFTEST ? c_selftest_tx_extra : 0u;
     extern __shared__ __align__(128) uint8_t smem_raw[];
     const int T = blockDim.x, C = p.C, D = p.depth, S = p.n_stats_warps;
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const uint32_t row_bytes_in = 2u * (uint32_t)C;
     const uint32_t pitch = row_bytes_in + 16u;            // 16 spare bytes keep successive slots 4 banks apart
     uint8_t* ring = smem_raw;

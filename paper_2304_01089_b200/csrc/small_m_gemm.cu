@@ -92,7 +92,7 @@ small_m_kernel(const SmallMParams p)
     __shared__ int s_abort_flag;
     volatile int* s_abort = &s_abort_flag;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g8 = lane >> 2, t4 = lane & 3;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, g8 = lane >> 2, t4 = lane & 3;
     const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES);
 
     if (tid == 0) {
