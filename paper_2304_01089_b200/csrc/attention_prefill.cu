@@ -32,10 +32,11 @@
 // 4 b + 2 y + {0, 1}. It lets the V loader read and write shared memory without bank conflicts.
 //
 // Measured, us, against a mma.sync kernel with 64 (KV: 128) queries per block (72 heads of 128 channels, four clusters each,
-// causal, two sequences of 2048 tokens): 3 bits 2321 -> 876, 8 bits 3856 -> 935; KV, 3 bits 2703 -> 1694; KV, 32 heads,
-// three sequences, 1100 queries on 1337 keys, 4 bits 945 -> 468; 16 queries on 2000 keys, four sequences 269 -> 200 (KV 549 ->
-// 355). A tile of 128 x 128 scores takes about 5000 clocks and pass, of which a warp's own chain of drains, exponentials and
-// waits is the most; the tensor cores are idle most of the time.
+// causal, two sequences of 2048 tokens): 3 bits 2321 -> 772; KV, 32 heads, three sequences, 1100 queries on 1337 keys, 4 bits
+// 945 -> 369. What bounds it is the instruction cache before any pipe: five roles run side by side, and a warp on its own executes
+// one instruction per 6 to 10 clocks (scheduler slots 48 % busy). Whatever shortens the code that runs at the same time helps
+// more than shortening a chain: the compiler told that the warp index is uniform 916 -> 790 (93 -> 83 KB of code), the output
+// rows' store loops not unrolled 790 -> 772; a first cluster's drain of its own (two copies of the loop) 790 -> 830.
 #include <type_traits>
 
 #include "attn_common.cuh"
@@ -77,6 +78,7 @@ struct Plan {
     int off_k, k_stage, off_v, v_stage, v_stages, off_p, p_tiles, off_rawk, rawk_stage, rawk_stages, pitch_k, off_rawv, pitch_v, off_col, off_ml, off_sum, off_bar, total;
     int local_v;          // V's heads own their channels and the output tile fits the V and P region: rows leave through shared memory
     int out_pitch;
+    int q_staged;         // KV (whose heads own their channels): a head's queries are copied in rows of its own channels, in pieces of 16 bytes
     int folded;           // integer calls: the queries are stored as q - z^Q (it fits the operand type): no per-key term
     int* status;
 };
@@ -424,40 +426,64 @@ prefill_kernel(const AttnParams p, const Plan g)
             }
         };
         // KV: the queries as fp16 in operand order (codes 0, 2, 1, 3, 4, 6, 5, 7 of every eight positions, the order in which
-        // the key codes come out of their words). Eight warps; a lane takes up to four pairs of positions and gathers their
-        // channels row by row.
+        // the key codes come out of their words). Eight warps of 16 rows; a lane takes up to four pairs of positions. The head's
+        // channels of a row are copied as they are into the row's own place in the operand tile and permuted there, four rows at
+        // a time (read, then written): gathered from global memory they took 22700 clocks an item, every load's latency in turn.
         auto gather_queries = [&](const Item& it, uint32_t n_item) {
             const int uk0 = __ldg(p.cl_unit0_k + it.h * p.gh_k), nuk = __ldg(p.cl_unit0_k + (it.h + 1) * p.gh_k) - uk0, nu = units_seen(nuk);
-            int ca[4], cb[4];
+            const int r0 = (warp - K_WARP0) * 16, rows = p.Tq - it.qt * BM - r0;               // rows: how many of my rows exist
+            const __half* q_rows = p.q_f16 + ((int64_t)it.seq * p.Tq + it.qt * BM + r0) * p.ldq;
+            int ca[4], cb[4];                                 // channels of my pairs (staged: their place in the row), -1: none
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int p2 = lane + 32 * k, code = (p2 >> 2) * 8 + (p2 & 1) + 4 * ((p2 >> 1) & 1), pos = 32 * uk0 + code;
                 const bool in = p2 < 16 * nuk;                // (a head without channels: no pair is, zeros are written)
-                ca[k] = in && __ldg(p.jidx_k + pos) >= 0 ? (int)__ldg(p.src_k + pos) : -1;
-                cb[k] = in && __ldg(p.jidx_k + pos + 2) >= 0 ? (int)__ldg(p.src_k + pos + 2) : -1;
+                auto place = [&](int at) {
+                    if (!in || __ldg(p.jidx_k + at) < 0) return -1;
+                    const int c = (int)__ldg(p.src_k + at);
+                    return g.q_staged ? ((c - it.h * p.hd) >> 6) * ATOM_Q + 2 * ((c - it.h * p.hd) & 63) : c;
+                };
+                ca[k] = place(pos);
+                cb[k] = place(pos + 2);
             }
             if (!mbar_sleep(bar(B_QEMPTY), (n_item & 1) ^ 1, s_abort)) return false;
-            const int i0 = it.qt * BM;
+            if (g.q_staged) {
+                const int per_row = p.hd / 8;                 // 16-byte chunks
 #pragma unroll 1
-            for (int r4 = (warp - K_WARP0) * 16; r4 < (warp - K_WARP0) * 16 + 16; r4 += 4) {
-                uint16_t v[4][4][2];                          // (all loads first: they are bound by latency)
+                for (int i = lane; i < 16 * per_row; i += 32) {
+                    const int r = i / per_row, c = i - r * per_row;
+                    cp_async16(base + (c >> 3) * ATOM_Q + (r0 + r) * 128 + 16 * (c & 7), r < rows ? q_rows + r * p.ldq + it.h * p.hd + 8 * c : p.q_f16, r < rows ? 16 : 0);
+                }
+                cp_async_commit();
+                cp_async_wait<0>();
+                __syncwarp();
+            }
+#pragma unroll 1
+            for (int r4 = 0; r4 < 16; r4 += 4) {
+                uint32_t v[4][4];
 #pragma unroll
-                for (int rr = 0; rr < 4; ++rr) {
-                    const bool okr = i0 + r4 + rr < p.Tq;
-                    const uint16_t* row = reinterpret_cast<const uint16_t*>(p.q_f16) + ((int64_t)it.seq * p.Tq + (okr ? i0 + r4 + rr : 0)) * p.ldq;
+                for (int rr = 0; rr < 4; ++rr)
 #pragma unroll
                     for (int k = 0; k < 4; ++k) {
-                        v[rr][k][0] = v[rr][k][1] = 0;
-                        if (okr && ca[k] >= 0) v[rr][k][0] = __ldg(row + ca[k]);
-                        if (okr && cb[k] >= 0) v[rr][k][1] = __ldg(row + cb[k]);
+                        uint16_t x = 0, y = 0;
+                        if (g.q_staged) {
+                            const uint32_t row = base + (r0 + r4 + rr) * 128;
+                            if (ca[k] >= 0) x = lds16(row + ca[k]);
+                            if (cb[k] >= 0) y = lds16(row + cb[k]);
+                        } else if (r4 + rr < rows) {          // (layouts whose heads share channels, rows without alignment)
+                            const uint16_t* row = reinterpret_cast<const uint16_t*>(q_rows) + (r4 + rr) * p.ldq;
+                            if (ca[k] >= 0) x = __ldg(row + ca[k]);
+                            if (cb[k] >= 0) y = __ldg(row + cb[k]);
+                        }
+                        v[rr][k] = x | ((uint32_t)y << 16);
                     }
-                }
+                __syncwarp();
 #pragma unroll
                 for (int rr = 0; rr < 4; ++rr)
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
                         if (lane + 32 * k < 16 * nu)
-                            sts32(base + k * ATOM_Q + (r4 + rr) * 128 + (((lane >> 2) ^ ((r4 + rr) & 7)) << 4) + 4 * (lane & 3), v[rr][k][0] | ((uint32_t)v[rr][k][1] << 16));
+                            sts32(base + k * ATOM_Q + (r0 + r4 + rr) * 128 + (((lane >> 2) ^ ((r4 + rr) & 7)) << 4) + 4 * (lane & 3), v[rr][k]);
             }
             tc::fence_proxy_async();
             __syncwarp();
@@ -823,11 +849,14 @@ prefill_kernel(const AttnParams p, const Plan g)
                         __half* dst = p.out + ((int64_t)it.seq * p.Tq + i0 + 32 * lw) * p.ldo + it.h * p.hd;
                         const bool pairs = (((uintptr_t)p.out & 3u) == 0) && (p.ldo & 1) == 0 && (p.hd & 1) == 0;
                         if (pairs) {
-#pragma unroll 4
+#pragma unroll 1
                             for (int r = 0; r < n_rows; ++r, dst += p.ldo)
+#pragma unroll 1
                                 for (int c = lane; c < p.hd / 2; c += 32) reinterpret_cast<uint32_t*>(dst)[c] = lds32(src + r * g.out_pitch + ((c ^ r) << 2));
                         } else {
+                            #pragma unroll 1
                             for (int r = 0; r < n_rows; ++r, dst += p.ldo)
+#pragma unroll 1
                                 for (int c = lane; c < p.hd; c += 32) dst[c] = __ushort_as_half(lds16(src + r * g.out_pitch + (((c >> 1) ^ r) << 2) + 2 * (c & 1)));
                         }
                     }
@@ -1105,6 +1134,7 @@ static int launch_one(const AttnParams& p, int zq_min, int zq_max, int units_k, 
     // the output tile is staged in the V and P region (rows of a multiple of 128 bytes: see the staging stores)
     g.out_pitch = (2 * p.hd + 127) / 128 * 128;
     g.local_v = v_heads_local && BM * g.out_pitch <= g.v_stages * g.v_stage + g.p_tiles * BM * 128;
+    g.q_staged = MODE == KV && p.hd % 8 == 0 && p.ldq % 8 == 0 && aligned16(p.q_f16);
     g.folded = MODE == F8 ? zq_min >= qmax_q - 16 && zq_max <= 16 : MODE == I8 ? zq_min >= qmax_q - 127 && zq_max <= 128 : 0;
     g.status = device_status_word();
     const void* fn = reinterpret_cast<const void*>(prefill_kernel<MODE, K8, V8>);

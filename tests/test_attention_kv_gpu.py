@@ -179,3 +179,10 @@ def test_many_items_and_wide_heads():
     _check(c, _query(np.random.default_rng(8), 140, 90 * 16), True)
     c = Case(731, H=2, hd=256, gh=1, Tq=130, Tk=140, bits=(4, 8, 8))
     _check(c, _query(np.random.default_rng(9), 130, 512), True)
+
+
+@pytest.mark.parametrize("hd,Tq", [(36, 140), (20, 129), (8, 256), (136, 140)])
+def test_query_rows_of_any_width(hd, Tq):
+    """Heads whose rows are whole pieces of 16 bytes are staged and permuted in place, others are gathered channel by channel."""
+    c = Case(740 + hd, H=2, hd=hd, gh=2, Tq=Tq, Tk=Tq + 61)
+    _check(c, _query(np.random.default_rng(hd), Tq, 2 * hd), True)
