@@ -38,6 +38,7 @@
 #include <cuda_fp16.h>
 
 #include <mutex>
+#include <type_traits>
 
 #include "pack.cuh"
 #include "rptq_internal.h"
@@ -98,7 +99,8 @@ __host__ __device__ constexpr SmemLayout smem_layout(int ncta, int bits, bool a8
 
 struct Params {
     int M, N, n_kb, n_seg, g;
-    int tiles_m, n_tiles;
+    int tiles_m, n_items;        // work items: the first n_full are whole tiles, every further tile is cut into 1 << split strips of columns
+    int n_full, split;
     const uint8_t* a_codes;      // [M][a_row_bytes]
     int64_t a_row_bytes;
     const uint8_t* w_codes;      // tile-major: n_wtiles * n_kb tiles of 8 KiB
@@ -319,7 +321,7 @@ cluster_gemm_kernel(const Params p)
     constexpr SmemLayout SL = smem_layout(NCTA, BITS, A8, ASYM);
     constexpr int W_ROWS = w_rows(NCTA);                 // weight rows this CTA stages and unpacks
     constexpr int N_P = n_p_stages(NCTA, BITS), N_U = n_u_stages(NCTA, A8);
-    constexpr uint32_t kInstrDesc = DEQ ? instr_desc_bf16(NCTA) : instr_desc(NCTA);
+    constexpr uint32_t kInstrDesc = DEQ ? instr_desc_bf16(NCTA) : instr_desc(NCTA);      // (of a whole tile)
     // dynamic shared memory is only guaranteed 16-byte alignment: round up to the swizzle span
     // (the offset is the same in both CTAs of a pair, as cta_group::2 descriptors require)
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
@@ -346,6 +348,14 @@ cluster_gemm_kernel(const Params p)
     const int n_steps = p.n_kb * 4;
     const uint32_t cta_rank = NCTA == 2 ? cluster_ctarank() : 0u;       // rank 0 issues the MMAs
     const int pair_id = (int)blockIdx.x / NCTA, n_pairs = (int)gridDim.x / NCTA;
+    // Work item -> token tile, first column, and how many times its 256 columns are halved
+    auto item_of = [&](int w, int& mt, int& n0) {
+        const int sh = w < p.n_full ? 0 : p.split, x = w - p.n_full;
+        const int t = sh ? p.n_full + (x >> sh) : w, nt = t / p.tiles_m;
+        mt = t - nt * p.tiles_m;
+        n0 = nt * TILE_N + (sh ? (x & ((1 << sh) - 1)) * (TILE_N >> sh) : 0);
+        return sh;
+    };
     // arrive on a barrier that lives in the issuing CTA of the pair
     auto arrive_leader = [&](uint32_t b) { if constexpr (NCTA == 1) mbar_arrive(b); else mbar_arrive_remote(b, 0); };
 
@@ -393,21 +403,24 @@ cluster_gemm_kernel(const Params p)
         if (lane == 0) {
             uint32_t n_issued = 0;
             bool ok = true;
-            for (int t = pair_id; t < p.n_tiles && ok; t += n_pairs) {
-                // 128-row weight tiles this CTA stages; tiles past the end of the buffer are skipped
-                // (their columns are never stored)
-                const int wt0 = ((t / p.tiles_m) * TILE_N + (int)cta_rank * W_ROWS) >> 7;
-                int n_valid = p.n_wtiles - wt0;
-                n_valid = n_valid < 0 ? 0 : (n_valid > W_ROWS / 128 ? W_ROWS / 128 : n_valid);
+            for (int t = pair_id; t < p.n_items && ok; t += n_pairs) {
+                // weight rows this CTA stages: whole 128-row tiles, or part of one; tiles past the end of the buffer are
+                // skipped (their columns are never stored)
+                int mt, n0;
+                const int sh = item_of(t, mt, n0), rows = W_ROWS >> sh, row0 = n0 + (int)cta_rank * rows;
+                const uint32_t bytes = rows < 128 ? (uint32_t)rows * 64 : (uint32_t)WTILE_BYTES;
+                int n_valid = p.n_wtiles - (row0 >> 7);
+                const int n_copies = rows < 128 ? 1 : rows >> 7;
+                n_valid = n_valid < 0 ? 0 : (n_valid > n_copies ? n_copies : n_valid);
+                const uint8_t* src = p.w_codes + (int64_t)(row0 >> 7) * p.n_kb * WTILE_BYTES + (row0 & 127) * 64;
                 for (int kb = 0; kb < p.n_kb; ++kb, ++n_issued) {
                     const int s = n_issued % N_P;
                     const uint32_t ph = (n_issued / N_P) & 1;
                     if (!mbar_wait(bar(B_PEMPTY + s), ph ^ 1, s_abort)) { ok = false; break; }
                     const uint32_t dst = smem_base + SL.off_p + s * SL.p_stage;
-                    mbar_arrive_expect_tx(bar(B_PFULL + s), (uint32_t)(n_valid * WTILE_BYTES));
+                    mbar_arrive_expect_tx(bar(B_PFULL + s), (uint32_t)n_valid * bytes);
                     for (int j = 0; j < n_valid; ++j)
-                        bulk_load(dst + j * WTILE_BYTES, p.w_codes + ((int64_t)(wt0 + j) * p.n_kb + kb) * WTILE_BYTES,
-                                  (uint32_t)WTILE_BYTES, bar(B_PFULL + s));
+                        bulk_load(dst + j * WTILE_BYTES, src + ((int64_t)j * p.n_kb + kb) * WTILE_BYTES, bytes, bar(B_PFULL + s));
                 }
             }
             if (!ok) {
@@ -431,7 +444,11 @@ cluster_gemm_kernel(const Params p)
             const uint64_t a_desc0 = smem_desc_sw128(smem_base);
             const uint32_t* flags4 = reinterpret_cast<const uint32_t*>(s_flags);
             uint32_t f4 = flags4[0];
-            const uint32_t total_kb = (uint32_t)(((p.n_tiles - pair_id + n_pairs - 1) / n_pairs) * p.n_kb);
+            const uint32_t total_kb = (uint32_t)(((p.n_items - pair_id + n_pairs - 1) / n_pairs) * p.n_kb);
+            // (a pair has at most one strip, its last item; n_full is a multiple of the pairs)
+            const uint32_t full_kb = p.split ? (uint32_t)(p.n_full / n_pairs * p.n_kb) : total_kb;
+            const uint32_t strip_desc = (kInstrDesc & ~(0x3Fu << 17)) | ((uint32_t)(TILE_N >> p.split >> 3) << 17);
+            uint32_t idesc = kInstrDesc;
             int kb = 0;
             if constexpr (DEQ) {
                 // One accumulator per tile, the two buffers alternate from tile to tile; every operand
@@ -440,6 +457,7 @@ cluster_gemm_kernel(const Params p)
                 uint32_t in_tile = 0, b = 0;
                 for (uint32_t n = 0; n < total_steps; ++n) {
                     const int st = n % N_U;
+                    if (n == 2u * full_kb) idesc = strip_desc;
                     if (in_tile == 0) {
                         if (!mbar_wait_warp(bar(B_ACCEMPTY + b), ((par >> b) & 1u) ^ 1u, s_abort)) { ok = false; break; }
                         tc_fence_after();
@@ -448,10 +466,10 @@ cluster_gemm_kernel(const Params p)
                     tc_fence_after();
                     const uint64_t ad = a_desc0 + (uint64_t)(st * (SL.u_stage >> 4)), wd = ad + (uint64_t)(A8_BYTES >> 4);
                     const uint32_t d_tmem = tmem_base + b * TILE_N;
-                    tc_mma_bf16<NCTA>(d_tmem, ad, wd, kInstrDesc, in_tile);
-                    tc_mma_bf16<NCTA>(d_tmem, ad + 2, wd + 2, kInstrDesc, 1u);
-                    tc_mma_bf16<NCTA>(d_tmem, ad + 4, wd + 4, kInstrDesc, 1u);
-                    tc_mma_bf16<NCTA>(d_tmem, ad + 6, wd + 6, kInstrDesc, 1u);
+                    tc_mma_bf16<NCTA>(d_tmem, ad, wd, idesc, in_tile);
+                    tc_mma_bf16<NCTA>(d_tmem, ad + 2, wd + 2, idesc, 1u);
+                    tc_mma_bf16<NCTA>(d_tmem, ad + 4, wd + 4, idesc, 1u);
+                    tc_mma_bf16<NCTA>(d_tmem, ad + 6, wd + 6, idesc, 1u);
                     tc_commit<NCTA>(bar(B_UEMPTY + st));
                     if (++in_tile == steps_per_tile) {
                         tc_commit<NCTA>(bar(B_ACCFULL + b));
@@ -463,6 +481,7 @@ cluster_gemm_kernel(const Params p)
             } else
             for (uint32_t n_kb_done = 0; n_kb_done < total_kb; ++n_kb_done) {
                     const int s = n_kb_done % N_U;
+                    if (n_kb_done == full_kb) idesc = strip_desc;
                     kb = kb + 1 == p.n_kb ? 0 : kb + 1;
                     const uint32_t f4_next = flags4[kb];                              // read while waiting
                     if (!mbar_wait_warp(bar(B_UFULL + s), (n_kb_done / N_U) & 1, s_abort)) { ok = false; break; }
@@ -473,10 +492,10 @@ cluster_gemm_kernel(const Params p)
                     if (f4 == 0u || f4 == 0x01010101u * STEP_BUF) {
                         // four steps inside one cluster
                         const uint32_t d_tmem = tmem_base + (f4 ? TILE_N : 0);
-                        tc_mma_i8<NCTA>(d_tmem, ad, wd, kInstrDesc, 1u);
-                        tc_mma_i8<NCTA>(d_tmem, ad + 2, wd + 2, kInstrDesc, 1u);
-                        tc_mma_i8<NCTA>(d_tmem, ad + 4, wd + 4, kInstrDesc, 1u);
-                        tc_mma_i8<NCTA>(d_tmem, ad + 6, wd + 6, kInstrDesc, 1u);
+                        tc_mma_i8<NCTA>(d_tmem, ad, wd, idesc, 1u);
+                        tc_mma_i8<NCTA>(d_tmem, ad + 2, wd + 2, idesc, 1u);
+                        tc_mma_i8<NCTA>(d_tmem, ad + 4, wd + 4, idesc, 1u);
+                        tc_mma_i8<NCTA>(d_tmem, ad + 6, wd + 6, idesc, 1u);
                     } else {
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
@@ -484,7 +503,7 @@ cluster_gemm_kernel(const Params p)
                             const uint32_t b = (f / STEP_BUF) & 1u;
                             const uint32_t d_tmem = tmem_base + b * TILE_N;
                             if ((f & (STEP_FIRST | STEP_LAST | STEP_SKIP)) == 0) {       // inside a cluster
-                                tc_mma_i8<NCTA>(d_tmem, ad + 2 * j, wd + 2 * j, kInstrDesc, 1u);
+                                tc_mma_i8<NCTA>(d_tmem, ad + 2 * j, wd + 2 * j, idesc, 1u);
                                 continue;
                             }
                             if (f & STEP_SKIP) continue;
@@ -493,7 +512,7 @@ cluster_gemm_kernel(const Params p)
                                 if (!mbar_wait_warp(bar(B_ACCEMPTY + b), ((par >> b) & 1u) ^ 1u, s_abort)) { ok = false; break; }
                                 tc_fence_after();
                             }
-                            tc_mma_i8<NCTA>(d_tmem, ad + 2 * j, wd + 2 * j, kInstrDesc, (f & STEP_FIRST) ? 0u : 1u);
+                            tc_mma_i8<NCTA>(d_tmem, ad + 2 * j, wd + 2 * j, idesc, (f & STEP_FIRST) ? 0u : 1u);
                             if (f & STEP_LAST) {
                                 tc_commit<NCTA>(bar(B_ACCFULL + b));
                                 par ^= 1u << b;
@@ -517,8 +536,10 @@ cluster_gemm_kernel(const Params p)
         const int tt = tid - TABLE_WARP0 * 32;
         uint32_t n_tile = 0, n_seg_done = 0;
         bool ok = true;
-        for (int t = pair_id; t < p.n_tiles && ok; t += n_pairs, ++n_tile) {
-            const int n = (t / p.tiles_m) * TILE_N + 4 * tt;
+        for (int t = pair_id; t < p.n_items && ok; t += n_pairs, ++n_tile) {
+            int mt, n0;
+            item_of(t, mt, n0);
+            const int n = n0 + 4 * tt;                     // (of a strip, the lanes past its columns work for nothing)
             const bool vec = (p.ld_w & 3) == 0 && n + 4 <= p.ld_w;
             float corr[4] = {0.f, 0.f, 0.f, 0.f};
             if constexpr (ASYM) {
@@ -587,7 +608,8 @@ cluster_gemm_kernel(const Params p)
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_UNPACK));
         const int ut = tid - UNPACK_WARP0 * 32;      // 0..127
         uint32_t n_done = 0;
-        const int total_kb = ((p.n_tiles - pair_id + n_pairs - 1) / n_pairs) * p.n_kb;
+        const int total_kb = ((p.n_items - pair_id + n_pairs - 1) / n_pairs) * p.n_kb;
+        const int full_kb = p.split ? p.n_full / n_pairs * p.n_kb : total_kb;      // K blocks of whole tiles; those of a strip follow
         // Weight item i of this thread is row (ut >> 2) + 32 i, unit ut & 3, so its two chunk positions in
         // the swizzled row (16-byte chunk j of row r lives at position j ^ (r & 7)) are the same for every i.
         const int row0 = ut >> 2, unit = ut & 3, sw = row0 & 7;
@@ -610,7 +632,9 @@ cluster_gemm_kernel(const Params p)
             const int64_t step4 = 4 * p.a_row_bytes;
             int n_rows_ok = 0;                               // how many of my 8 rows exist
             auto a8_tile = [&]() {
-                const int row = (t_f % p.tiles_m) * (TILE_M * NCTA) + (int)cta_rank * TILE_M + wrow;
+                int mt, n0;
+                item_of(t_f, mt, n0);
+                const int row = mt * (TILE_M * NCTA) + (int)cta_rank * TILE_M + wrow;
                 const int left = p.M - row;
                 n_rows_ok = left <= 0 ? 0 : (left + 3) >> 2;
                 a_src = p.a_codes + (int64_t)(left > 0 ? row : 0) * p.a_row_bytes + 16 * ch;
@@ -647,11 +671,13 @@ cluster_gemm_kernel(const Params p)
                 uint32_t pw_w[W_ITEMS][4];
 #pragma unroll
                 for (int i = 0; i < W_ITEMS; ++i) {
+                    if (i == W_ITEMS / 2 && it >= full_kb) break;
                     const uint4 v = lds128(pw + (ut + i * 128) * 16);
                     pw_w[i][0] = v.x; pw_w[i][1] = v.y; pw_w[i][2] = v.z; pw_w[i][3] = v.w;
                 }
 #pragma unroll
                 for (int i = 0; i < W_ITEMS; ++i) {
+                    if (i == W_ITEMS / 2 && it >= full_kb) break;
                     uint32_t o[8];
                     unpack_w32_x16(pw_w[i], o);
                     sts128(w_tile + off0 + i * 4096, o[0], o[1], o[2], o[3]);
@@ -686,7 +712,9 @@ cluster_gemm_kernel(const Params p)
         }
         int rows_left = 0;                               // rows of the tile being fetched that exist
         auto fetch_tile_row = [&]() {
-            const int row0 = (t_f % p.tiles_m) * (TILE_M * NCTA) + (int)cta_rank * TILE_M;
+            int mt, n0;
+            item_of(t_f, mt, n0);
+            const int row0 = mt * (TILE_M * NCTA) + (int)cta_rank * TILE_M;
             rows_left = p.M - row0;
             a_src = p.a_codes + (int64_t)(rows_left > 0 ? row0 : 0) * p.a_row_bytes;
         };
@@ -762,6 +790,7 @@ cluster_gemm_kernel(const Params p)
 #pragma unroll
                     for (int i = 0; i < W_ROWS / 64; ++i) {
                         const int r = (ut >> 1) + 64 * i;
+                        if (it >= full_kb && r >= (W_ROWS >> p.split)) break;
                         const uint4 v = lds128(pw + r * 64 + (2 * h + (ut & 1)) * 16);
                         const uint32_t pk[4] = {v.x, v.y, v.z, v.w};
                         uint32_t o[8];
@@ -787,27 +816,33 @@ cluster_gemm_kernel(const Params p)
             tc_fence_after();
             const uint32_t pw = smem_base + SL.off_p + sp * SL.p_stage;
             const uint32_t a_tile = smem_base + su * SL.u_stage, w_tile = a_tile + A8_BYTES;
-            // all packed weight words of my items first (independent loads), then unpack and store
-            uint32_t pw_w[W_ITEMS][4];
+            // n_w: my weight items. Of a strip half of them (its rows, or as many more that no product reads). In code of its own for
+            // each: a test inside costs the whole tiles 2 to 5 %.
+            auto convert = [&](auto n_w) {
+                constexpr int NW = decltype(n_w)::value;
+                // all packed weight words of my items first (independent loads), then unpack and store
+                uint32_t pw_w[NW][4];
 #pragma unroll
-            for (int i = 0; i < W_ITEMS; ++i) {
-                const uint4 v = lds128(pw + (ut + i * 128) * 16);
-                pw_w[i][0] = v.x; pw_w[i][1] = v.y; pw_w[i][2] = v.z; pw_w[i][3] = v.w;
-            }
+                for (int i = 0; i < NW; ++i) {
+                    const uint4 v = lds128(pw + (ut + i * 128) * 16);
+                    pw_w[i][0] = v.x; pw_w[i][1] = v.y; pw_w[i][2] = v.z; pw_w[i][3] = v.w;
+                }
 #pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                uint32_t o[8];
-                unpack_act32<BITS>(pa_w[u], o);
-                sts128(a_tile + a_off + (((2 * u) ^ a_sw) << 4), o[0], o[1], o[2], o[3]);
-                sts128(a_tile + a_off + (((2 * u + 1) ^ a_sw) << 4), o[4], o[5], o[6], o[7]);
-            }
+                for (int u = 0; u < 4; ++u) {
+                    uint32_t o[8];
+                    unpack_act32<BITS>(pa_w[u], o);
+                    sts128(a_tile + a_off + (((2 * u) ^ a_sw) << 4), o[0], o[1], o[2], o[3]);
+                    sts128(a_tile + a_off + (((2 * u + 1) ^ a_sw) << 4), o[4], o[5], o[6], o[7]);
+                }
 #pragma unroll
-            for (int i = 0; i < W_ITEMS; ++i) {
-                uint32_t o[8];
-                unpack_w32_x16(pw_w[i], o);
-                sts128(w_tile + off0 + i * 4096, o[0], o[1], o[2], o[3]);
-                sts128(w_tile + off1 + i * 4096, o[4], o[5], o[6], o[7]);
-            }
+                for (int i = 0; i < NW; ++i) {
+                    uint32_t o[8];
+                    unpack_w32_x16(pw_w[i], o);
+                    sts128(w_tile + off0 + i * 4096, o[0], o[1], o[2], o[3]);
+                    sts128(w_tile + off1 + i * 4096, o[4], o[5], o[6], o[7]);
+                }
+            };
+            if (it < full_kb) convert(std::integral_constant<int, W_ITEMS>()); else convert(std::integral_constant<int, W_ITEMS / 2>());
             fence_proxy_async();          // make the generic-proxy stores visible to the tensor core
             __syncwarp();
             if (lane == 0) { arrive_leader(bar(B_UFULL + su)); mbar_arrive(bar(B_PEMPTY + sp)); }
@@ -824,8 +859,10 @@ cluster_gemm_kernel(const Params p)
         bool ok = true;
         uint32_t n_seg_done = 0;                     // ASYM: clusters drained so far, over all tiles
         float2 R[64];                                // running sums of columns 2 i, 2 i + 1
-        for (int t = pair_id; t < p.n_tiles && ok; t += n_pairs, ++n_tile_done) {
-            const int m0 = (t % p.tiles_m) * (TILE_M * NCTA) + (int)cta_rank * TILE_M, n0 = (t / p.tiles_m) * TILE_N;
+        for (int t = pair_id; t < p.n_items && ok; t += n_pairs, ++n_tile_done) {
+            int mt, n0;
+            const int sh = item_of(t, mt, n0), half_cols = 128 >> sh;      // columns of my half
+            const int m0 = mt * (TILE_M * NCTA) + (int)cta_rank * TILE_M;
             float* tab = s_tab + (n_tile_done & 1) * 3 * TILE_N;
             // a warp whose 32 accumulator lanes all lie beyond the last token row keeps the barriers'
             // protocol but reads and accumulates nothing (few-token calls: most of the tile is empty)
@@ -846,7 +883,7 @@ cluster_gemm_kernel(const Params p)
                 const float sc = ASYM ? 0.f : s_seg_scale[sgi];
                 const float2 sc2 = make_float2(sc, sc);
                 const uint32_t seg_slot = n_seg_done % SEG_SLOTS;
-                const float4* seg_tab = s_seg_tab + seg_slot * (TILE_N / 2) + h * 64;
+                const float4* seg_tab = s_seg_tab + seg_slot * (TILE_N / 2) + (h * half_cols >> 1);
                 float2 xs2 = make_float2(0.f, 0.f);
                 if constexpr (ASYM) {
                     if (!mbar_wait(bar(B_SEGFULL + seg_slot), (n_seg_done / SEG_SLOTS) & 1, s_abort)) { ok = false; break; }
@@ -855,7 +892,7 @@ cluster_gemm_kernel(const Params p)
                     xs2 = make_float2(x, x);
                     if (xs_row && sgi + 1 < p.n_seg) xs_next = __ldg(xs_row + s_seg_cl[sgi + 1]);
                 }
-                const uint32_t taddr = tmem_base + ((uint32_t)(32 * q) << 16) + buf * TILE_N + h * 128;
+                const uint32_t taddr = tmem_base + ((uint32_t)(32 * q) << 16) + buf * TILE_N + h * half_cols;
                 if (live) {
                 uint32_t va[16], vb[16];
                 tc_ld16(taddr, va);
@@ -884,8 +921,10 @@ cluster_gemm_kernel(const Params p)
                     tc_ld16(taddr + (ch + 1) * 16, vb);
                     accumulate(va, ch * 8);
                     tc_wait_ld();
-                    if (ch + 2 < 8) tc_ld16(taddr + (ch + 2) * 16, va);
+                    const bool more = ch + 2 < 8 && 16 * (ch + 2) < half_cols;
+                    if (more) tc_ld16(taddr + (ch + 2) * 16, va);
                     accumulate(vb, (ch + 1) * 8);
+                    if (!more) break;
                 }
                 }
                 tc_fence_before();
@@ -902,8 +941,8 @@ cluster_gemm_kernel(const Params p)
             // exchanged through a small buffer of the warp instead, and leave as whole sectors of 16 rows
             // (1999 x 2048 x 6144, 8 bits, fp32 out: 70.5 -> 59.4 us with the LayerNorm; 4096 x 9216 x 36864, fp16 out: 1455 -> 1435).
             if (live) {
-                const int mw = m0 + 32 * q, nb = n0 + h * 128;                 // my warp's first row, my first column
-                const float4* t_corr = reinterpret_cast<const float4*>(tab + h * 128);
+                const int mw = m0 + 32 * q, nb = n0 + h * half_cols;           // my warp's first row, my first column
+                const float4* t_corr = reinterpret_cast<const float4*>(tab + h * half_cols);
                 const float4* t_sw = t_corr + TILE_N / 4;
                 const float4* t_bs = t_sw + TILE_N / 4;
                 const bool relu = p.act == RPTQ_ACT_RELU;
@@ -940,6 +979,7 @@ cluster_gemm_kernel(const Params p)
                     uint8_t* dst = static_cast<uint8_t*>(p.y) + ((int64_t)mw * p.ldy + nb) * 2;
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {                              // 16 columns
+                        if (16 * c >= half_cols) break;
                         float2 v[8];
 #pragma unroll
                         for (int i = 0; i < 4; ++i) finish(4 * c + i, v[2 * i], v[2 * i + 1]);
@@ -950,6 +990,7 @@ cluster_gemm_kernel(const Params p)
                     uint8_t* dst = static_cast<uint8_t*>(p.y) + ((int64_t)mw * p.ldy + nb) * 4;
 #pragma unroll
                     for (int c = 0; c < 16; ++c) {                             // 8 columns
+                        if (8 * c >= half_cols) break;
                         float2 v[4];
                         finish(2 * c, v[0], v[1]);
                         finish(2 * c + 1, v[2], v[3]);
@@ -964,7 +1005,7 @@ cluster_gemm_kernel(const Params p)
 #pragma unroll
                     for (int uu = 0; uu < 4; ++uu) {
                         const int unit = (nb >> 5) + uu;
-                        if (nb + 32 * uu >= p.N) break;                        // (N is a multiple of 128)
+                        if (32 * uu >= half_cols || nb + 32 * uu >= p.N) break;    // (N is a multiple of 128)
                         const uint4 t4 = __ldg(reinterpret_cast<const uint4*>(p.out_unit + unit));
                         const float inv_s = __uint_as_float(t4.x);
                         const int zc = (int)t4.y, nvalid = (int)t4.w;
@@ -1036,7 +1077,7 @@ static int launch(const Params& p, int dev, int n_sm, cudaStream_t st)
     }
     if (allow_smem(fn, dev, smem, done) != RPTQ_OK) return RPTQ_ERR_CUDA;
     const int slots = n_sm / NCTA;
-    const int groups = p.n_tiles < slots ? p.n_tiles : slots;
+    const int groups = p.n_items < slots ? p.n_items : slots;
     return launch_kernel(cluster_gemm_kernel<BITS, NCTA, A8, MODE>, dim3((unsigned)(groups * NCTA)), THREADS, (size_t)smem, NCTA, st, p);
 }
 
@@ -1084,7 +1125,7 @@ static int launch_gemm(const rptq_layout_t* Lin, const void* a_codes, int M, con
     // CTA pairs share a 256-row tile; one token tile or less gains nothing from pairing
     const int ncta = M > gemm::TILE_M ? 2 : 1;
     p.tiles_m = (M + gemm::TILE_M * ncta - 1) / (gemm::TILE_M * ncta);
-    p.n_tiles = p.tiles_m * ((N + gemm::TILE_N - 1) / gemm::TILE_N);
+    const int n_tiles = p.tiles_m * ((N + gemm::TILE_N - 1) / gemm::TILE_N);
     p.a_codes = static_cast<const uint8_t*>(a_codes); p.a_row_bytes = Lin->row_bytes;
     p.w_codes = static_cast<const uint8_t*>(w_codes); p.n_wtiles = (int)((ld_w + 127) / 128);
     p.step_flags = Lin->d_step_flags; p.seg_scale = Lin->d_seg_scale; p.seg_buf = Lin->d_seg_buf; p.cl_sz = Lin->d_cl_sz;
@@ -1099,6 +1140,15 @@ static int launch_gemm(const rptq_layout_t* Lin, const void* a_codes, int M, con
 
     const int n_sm = sm_count(dev);
     if (n_sm == 0) return RPTQ_ERR_CUDA;
+    // The tiles of the last round, when they are at most half (a quarter) as many as there are blocks (pairs) to work on them, are
+    // cut into two (four) strips of columns: the round then takes the time of a strip, about two thirds (half) of a tile's (a
+    // strip's token codes are unpacked all the same). 200 x 9216 x 27648: 90 -> 86 us; 1024 x 4096 x 16384 with clustered weights
+    // 136 -> 129; calls with fewer tiles than blocks up to 1.4 times as fast. With more tiles left than half the blocks a cut
+    // would only add a round. Not four for re-quantised outputs (a warp writes its columns in pieces of 64).
+    const int slots = n_sm / ncta, rest = n_tiles % slots;
+    p.split = rest == 0 ? 0 : 4 * rest <= slots && y_dtype != RPTQ_OUT_CODES ? 2 : 2 * rest <= slots ? 1 : 0;
+    p.n_full = p.split ? n_tiles - rest : n_tiles;
+    p.n_items = p.n_full + ((n_tiles - p.n_full) << p.split);
     auto st = static_cast<cudaStream_t>(stream);
     // a few tokens (decoding): the kernel that streams the weights through mma.sync with the channels as its M dimension
     if (!deq && !sw_c && y_dtype != RPTQ_OUT_CODES && smallm::fits(M, Lin->bits, Lin->K_pad)) {

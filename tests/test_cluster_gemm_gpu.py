@@ -364,3 +364,21 @@ def test_few_tokens_take_the_direct_kernel_and_give_the_same_bits(bits, order):
     # no bias, no activation, an output pitch wider than N
     y = _gemm(dict(case, M=5), d, ldy=320)[:, :N]
     assert np.max(np.abs(y - _oracle_y(case)[:5])) <= TOL * np.abs(want).max()
+
+
+@pytest.mark.parametrize("bits", [4, 3, 8])
+@pytest.mark.parametrize("M,rest", [(100, 2), (100, 70), (200, 1), (200, 30)])
+def test_last_round_in_strips(M, rest, bits):
+    """One whole round of tiles on every block (pair), then `rest` tiles more: a few are cut into quarters, more into halves."""
+    import torch
+    from paper_2304_01089_b200 import binding
+    slots = torch.cuda.get_device_properties(0).multi_processor_count // (2 if M > 128 else 1)
+    rng = np.random.default_rng(2000 * bits + M + rest)
+    N = (slots + rest) * 256 - 56
+    case = _case(rng, M, N, 256, 3, bits)
+    d = _dev(case)
+    want = _oracle_y(case)
+    y32 = _gemm(case, d, ldy=N + 8)[:, :N]
+    assert np.max(np.abs(y32 - want)) <= TOL * np.abs(want).max()
+    y16 = _gemm(case, d, y_dtype=binding.OUT_F16, ldy=N + 8)[:, :N]
+    assert np.array_equal(y16, y32.astype(np.float16))
