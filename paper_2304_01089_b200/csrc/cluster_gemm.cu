@@ -51,41 +51,48 @@ namespace gemm {
 using namespace tc;
 
 constexpr int TILE_M = 128, TILE_N = 256, KBLK = 128;   // TILE_M is per CTA
-constexpr int THREADS = 512;
+enum { MODE_INT = 0, MODE_ASYM = 1, MODE_DEQ = 2 };      // see cluster_gemm_kernel
+// MODE_DEQ: two groups of unpack warps (its conversions take three times as long), and an epilogue without running sums
+constexpr int threads_of(int mode) { return mode == MODE_DEQ ? 640 : 512; }
 constexpr int TABLE_WARP0 = 2, N_TABLE_WARPS = 2;
-constexpr int UNPACK_WARP0 = 4, N_UNPACK_WARPS = 4;
-constexpr int EPI_WARP0 = 8, N_EPI_WARPS = 8;
-// registers per thread after the in-kernel re-partition (the block is launched with 128 each): the
-// producer / MMA-issuer group, the unpack group, the two epilogue groups (128 running sums per thread)
-constexpr int REGS_WG0 = 40, REGS_UNPACK = 88, REGS_EPI = 192;
-static_assert(128 * (REGS_WG0 + REGS_UNPACK + 2 * REGS_EPI) <= 128 * THREADS, "register pool");
+constexpr int UNPACK_WARP0 = 4, GROUP_WARPS = 4;          // warps of an unpack group
+constexpr int n_unpack_warps(int mode) { return mode == MODE_DEQ ? 2 * GROUP_WARPS : GROUP_WARPS; }
+constexpr int N_EPI_WARPS = 8;
+// registers per thread after the in-kernel re-partition (the block is launched with 128, MODE_DEQ 96 each): the
+// producer / MMA-issuer group, the unpack groups, the two epilogue groups (128 running sums per thread, none in MODE_DEQ)
+constexpr int REGS_WG0 = 40;
+constexpr int regs_unpack(int mode) { return mode == MODE_DEQ ? 104 : 88; }
+constexpr int regs_epi(int mode) { return mode == MODE_DEQ ? 112 : 192; }
+constexpr int regs_all(int mode) { return 128 * REGS_WG0 + 32 * n_unpack_warps(mode) * regs_unpack(mode) + 256 * regs_epi(mode); }
+static_assert(regs_all(MODE_INT) <= 128 * 512 && regs_all(MODE_DEQ) <= 96 * 640, "register pool");
 constexpr int A8_BYTES = TILE_M * KBLK;                  // 16 KiB of 8-bit activation operands per stage
 constexpr int WTILE_BYTES = 8192;                        // one packed weight tile: 128 rows x 64 bytes
 
 __host__ __device__ constexpr int w_rows(int ncta) { return TILE_N / ncta; }           // weight rows staged per CTA
 // packed weight stages; the single-CTA variant (at most 128 tokens) is a weight stream and takes what shared memory is left
-__host__ __device__ constexpr int n_p_stages(int ncta, int bits) { return ncta == 2 ? 4 : (bits == 3 ? 5 : 4); }
+__host__ __device__ constexpr int n_p_stages(int ncta, int bits, int mode) { return ncta == 2 ? 4 : mode == MODE_DEQ ? 3 : (bits == 3 ? 5 : 4); }
 __host__ __device__ constexpr int n_u_stages(int ncta, bool a8) { return ncta == 2 ? (a8 ? 5 : 4) : 2; }   // operand stages
 // ring of packed activation K blocks fetched ahead by the unpack threads: one slot per token row
 // per K block; the pitch is an odd number of 16-byte units so that the threads' vector reads of
 // their own slots do not collide in the banks
-__host__ __device__ constexpr int a_slot_pitch(int bits) { return bits == 3 ? 48 : 16 * bits + 16; }
-__host__ __device__ constexpr int n_a_stages(int bits) { return bits == 8 ? 2 : 4; }
+__host__ __device__ constexpr int a_slot_pitch(int bits, int mode) { return mode == MODE_DEQ ? (bits == 8 ? 80 : 48) : bits == 3 ? 48 : 16 * bits + 16; }
+__host__ __device__ constexpr int n_a_stages(int bits, int mode) { return bits == 8 ? 2 : mode == MODE_DEQ ? 3 : 4; }
 
 struct SmemLayout {
     int u_stage, p_stage, a_stage, off_p, off_a, off_flags, off_seg_scale, off_seg_buf, off_tab, off_seg_tab, off_seg_cl, off_stage, off_bar, total;
 };
 constexpr int STAGE_OUT = 1024;                          // bytes of the output staging buffer of an epilogue warp
 constexpr int SEG_SLOTS = 2;                             // ASYM: clusters whose column tables are held at a time
-__host__ __device__ constexpr SmemLayout smem_layout(int ncta, int bits, bool a8, bool asym)
+__host__ __device__ constexpr SmemLayout smem_layout(int ncta, int bits, bool a8, int mode)
 {
+    const bool asym = mode == MODE_ASYM;
     SmemLayout s{};
     s.u_stage = A8_BYTES + w_rows(ncta) * KBLK;
     s.p_stage = w_rows(ncta) * KBLK / 2;
-    s.a_stage = a8 ? 0 : TILE_M * a_slot_pitch(bits);      // 8-bit activations go straight to the operand stage
+    s.a_stage = a8 ? 0 : n_unpack_warps(mode) / GROUP_WARPS * TILE_M * a_slot_pitch(bits, mode);      // 8-bit activations go straight to the operand stage
     s.off_p = n_u_stages(ncta, a8) * s.u_stage;
-    s.off_a = s.off_p + n_p_stages(ncta, bits) * s.p_stage;
-    s.off_flags = s.off_a + n_a_stages(bits) * s.a_stage;
+    s.off_a = s.off_p + n_p_stages(ncta, bits, mode) * s.p_stage;
+    s.off_flags = s.off_a + n_a_stages(bits, mode) * s.a_stage;
     s.off_seg_scale = s.off_flags + 2048;
     s.off_seg_buf = s.off_seg_scale + (asym ? 0 : kMaxGemmSegments * 4);
     s.off_tab = s.off_seg_buf + kMaxGemmSegments;
@@ -262,15 +269,22 @@ __device__ __forceinline__ float byte_as_magic(uint32_t w)
 {
     return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7650u | (uint32_t)I));
 }
-// Four 8-bit values of one word -> four bfloat16 (two words): v = (byte - c1) * s with c1 = 2^23 + z.
-// byte - c1 is exact, the product is rounded once to fp32 and once more to bfloat16.
-__device__ __forceinline__ void bytes_to_bf16(uint32_t w, float2 neg_c1, float2 s2, bool scale, uint32_t& out_lo, uint32_t& out_hi)
+// Four 8-bit values of one word -> four bfloat16, bytes 0 and 2 in one word, 1 and 3 in the other: v = (byte - c1) * s with
+// c1 = 2^23 + z. byte - c1 is exact, the product is rounded once to fp32 and once more to bfloat16.
+__device__ __forceinline__ void bytes_to_bf16(uint32_t w, float2 neg_c1, float2 s2, uint32_t& out_02, uint32_t& out_13)
 {
-    float2 a = add2(make_float2(byte_as_magic<0>(w), byte_as_magic<1>(w)), neg_c1);
-    float2 b = add2(make_float2(byte_as_magic<2>(w), byte_as_magic<3>(w)), neg_c1);
-    if (scale) { a = mul2(a, s2); b = mul2(b, s2); }
-    out_lo = pack_bf16(a.x, a.y);
-    out_hi = pack_bf16(b.x, b.y);
+    const float2 a = mul2(add2(make_float2(byte_as_magic<0>(w), byte_as_magic<2>(w)), neg_c1), s2);
+    const float2 b = mul2(add2(make_float2(byte_as_magic<1>(w), byte_as_magic<3>(w)), neg_c1), s2);
+    out_02 = pack_bf16(a.x, a.y);
+    out_13 = pack_bf16(b.x, b.y);
+}
+// The two's complement nibbles in bits 0-3 and 16-19 as bfloat16: n with its sign bit flipped, dropped into the mantissa of
+// 128, is 136 + w.
+__device__ __forceinline__ uint32_t nibbles_to_bf16(uint32_t w)
+{
+    uint32_t d;
+    asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"((w & 0x000F000Fu) ^ 0x43084308u), "r"(0x43084308u));
+    return d;
 }
 
 // packed fp32 pairs: one instruction, two independent IEEE results
@@ -306,21 +320,20 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr)
 // the first two are applied per element while a cluster's accumulator is drained, the last two are a
 // constant of the output column.
 // MODE_DEQ: the first computation method of the Appendix (de-quantise, then one floating-point product):
-// the unpack warps write X^ = s_c (X_q - z_c) as bfloat16 and the weight codes as bfloat16 integers
-// (16 w, exact), the MMAs are kind::f16 into ONE fp32 accumulator per tile -- no per-cluster
+// the unpack warps write X^ = s_c (X_q - z_c) as bfloat16 and the weight codes as bfloat16 integers, the MMAs are kind::f16 into ONE fp32 accumulator per tile -- no per-cluster
 // accumulators, no drains at cluster boundaries -- and s_w[n] multiplies the finished sum. A bfloat16
 // operand row of 128 bytes holds 64 positions, so a K block of 128 positions is two operand stages.
-enum { MODE_INT = 0, MODE_ASYM = 1, MODE_DEQ = 2 };
 template <int BITS, int NCTA, bool A8, int MODE>
-__global__ void __launch_bounds__(THREADS, 1)
+__global__ void __launch_bounds__(threads_of(MODE), 1)
 cluster_gemm_kernel(const Params p)
 {
     constexpr bool ASYM = MODE == MODE_ASYM, DEQ = MODE == MODE_DEQ;
     static_assert(!(DEQ && A8), "the de-quantising variant unpacks every bit width");
     extern __shared__ __align__(1024) uint8_t smem_raw[];
-    constexpr SmemLayout SL = smem_layout(NCTA, BITS, A8, ASYM);
+    constexpr SmemLayout SL = smem_layout(NCTA, BITS, A8, MODE);
+    constexpr int THREADS = threads_of(MODE), EPI_WARP0 = UNPACK_WARP0 + n_unpack_warps(MODE);
     constexpr int W_ROWS = w_rows(NCTA);                 // weight rows this CTA stages and unpacks
-    constexpr int N_P = n_p_stages(NCTA, BITS), N_U = n_u_stages(NCTA, A8);
+    constexpr int N_P = n_p_stages(NCTA, BITS, MODE), N_U = n_u_stages(NCTA, A8);
     constexpr uint32_t kInstrDesc = DEQ ? instr_desc_bf16(NCTA) : instr_desc(NCTA);      // (of a whole tile)
     // dynamic shared memory is only guaranteed 16-byte alignment: round up to the swizzle span
     // (the offset is the same in both CTAs of a pair, as cta_group::2 descriptors require)
@@ -360,8 +373,8 @@ cluster_gemm_kernel(const Params p)
     auto arrive_leader = [&](uint32_t b) { if constexpr (NCTA == 1) mbar_arrive(b); else mbar_arrive_remote(b, 0); };
 
     if (tid == 0) {
-        for (int i = 0; i < N_P; ++i) { mbar_init(bar(B_PFULL + i), 1); mbar_init(bar(B_PEMPTY + i), N_UNPACK_WARPS); }
-        for (int i = 0; i < N_U; ++i) { mbar_init(bar(B_UFULL + i), N_UNPACK_WARPS * NCTA); mbar_init(bar(B_UEMPTY + i), 1); }
+        for (int i = 0; i < N_P; ++i) { mbar_init(bar(B_PFULL + i), 1); mbar_init(bar(B_PEMPTY + i), n_unpack_warps(MODE)); }
+        for (int i = 0; i < N_U; ++i) { mbar_init(bar(B_UFULL + i), GROUP_WARPS * NCTA); mbar_init(bar(B_UEMPTY + i), 1); }
         for (int i = 0; i < 2; ++i) {
             mbar_init(bar(B_ACCFULL + i), 1); mbar_init(bar(B_ACCEMPTY + i), N_EPI_WARPS * NCTA); mbar_init(bar(B_TAB + i), N_TABLE_WARPS);
             mbar_init(bar(B_TABEMPTY + i), N_EPI_WARPS);
@@ -595,8 +608,8 @@ cluster_gemm_kernel(const Params p)
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const bool in = n + e < p.N;
-                // ASYM: the column's scale is applied per cluster; DEQ: the weight operands were 16 w, zero points are in X^
-                const float sw = !in ? 0.f : ASYM ? 1.f : DEQ ? __ldg(p.s_w + n + e) * 0.0625f : __ldg(p.s_w + n + e);
+                // ASYM: the column's scale is applied per cluster
+                const float sw = !in ? 0.f : ASYM ? 1.f : __ldg(p.s_w + n + e);
                 tab[e] = corr[e]; tab[TILE_N + e] = sw; tab[2 * TILE_N + e] = in && p.bias ? __ldg(p.bias + n + e) : 0.f;
             }
             __syncwarp();
@@ -605,8 +618,9 @@ cluster_gemm_kernel(const Params p)
       }
     } else if (warp < EPI_WARP0) {
         // ------------------------------------------------------------ unpack warps
-        asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_UNPACK));
-        const int ut = tid - UNPACK_WARP0 * 32;      // 0..127
+        if constexpr (DEQ) asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(regs_unpack(MODE)));
+        else asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(regs_unpack(MODE)));
+        const int ut = (tid - UNPACK_WARP0 * 32) & 127;        // within my group
         uint32_t n_done = 0;
         const int total_kb = ((p.n_items - pair_id + n_pairs - 1) / n_pairs) * p.n_kb;
         const int full_kb = p.split ? p.n_full / n_pairs * p.n_kb : total_kb;      // K blocks of whole tiles; those of a strip follow
@@ -689,6 +703,119 @@ cluster_gemm_kernel(const Params p)
                 if (lane == 0) { arrive_leader(bar(B_UFULL + su)); mbar_arrive(bar(B_PEMPTY + sp)); }
             }
             cp_async_wait<0>();
+        } else if constexpr (DEQ) {
+            // Two operand stages per K block, 64 positions each; group `grp` fills every other stage. A thread de-quantises units
+            // 2 grp and 2 grp + 1 of its token row with their (s_c, z_c), and converts unit 2 grp + (ut & 1) of weight rows
+            // (ut >> 1) + 64 i. Positions of every eight are stored in the order 0 2, 1 3, 4 6, 5 7 in both operands: the order in
+            // which nibbles come out of a word in pairs (weights: three instructions for two codes).
+            // One group of four warps, fp32 arithmetic for the weights too: 2800 clocks per K block, of which the products need 1070
+            // (2048 x 4096 x 16384, 4 bits, LayerNorm included: 380 us). Two groups 306; all loads of a block before its first
+            // store 287. Half of what is left is still the conversion (tensor pipe 55 % busy, ALU pipe 50 %).
+            const int grp = warp >= UNPACK_WARP0 + GROUP_WARPS ? 1 : 0;
+            constexpr int CH = BITS == 8 ? 4 : 2;            // 16-byte pieces of a row's K block that hold the two units
+            constexpr int N_A = n_a_stages(BITS, MODE), PITCH = a_slot_pitch(BITS, MODE);
+            static_assert(PITCH == 16 * CH + 16, "slot");
+            const uint32_t a_ring0 = smem_base + SL.off_a + grp * TILE_M * PITCH, a_ring = a_ring0 + ut * PITCH;
+            uint32_t d_off[CH], s_off[CH];
+            int r_of[CH];
+#pragma unroll
+            for (int i = 0; i < CH; ++i) {
+                const int c = 32 * i + lane;
+                r_of[i] = (ut & ~31) + c / CH;
+                d_off[i] = (uint32_t)r_of[i] * PITCH + 16u * (uint32_t)(c % CH);
+                s_off[i] = (uint32_t)r_of[i] * (uint32_t)p.a_row_bytes + (uint32_t)((8 * BITS * grp) & ~15) + 16u * (uint32_t)(c % CH);
+            }
+            int rows_left = 0;
+            auto fetch_tile_row = [&]() {
+                int mt, n0;
+                item_of(t_f, mt, n0);
+                const int row0 = mt * (TILE_M * NCTA) + (int)cta_rank * TILE_M;
+                rows_left = p.M - row0;
+                a_src = p.a_codes + (int64_t)(rows_left > 0 ? row0 : 0) * p.a_row_bytes;
+            };
+            fetch_tile_row();
+            auto fetch_next = [&]() {
+                if (n_fetched < total_kb) {
+                    const uint32_t dst = a_ring0 + (n_fetched % N_A) * SL.a_stage;
+#pragma unroll
+                    for (int i = 0; i < CH; ++i) {
+                        const bool v = r_of[i] < rows_left;
+                        cp_async16(dst + d_off[i], v ? a_src + s_off[i] : p.a_codes, v);
+                    }
+                    a_src += 16 * BITS;
+                    if (++kb_f == p.n_kb) { kb_f = 0; t_f += n_pairs; fetch_tile_row(); }
+                }
+                ++n_fetched;
+                cp_async_commit();
+            };
+#pragma unroll 1
+            for (int i = 0; i < N_A - 1; ++i) fetch_next();
+            int kb_next = 0;
+            const float2* unit_sz = p.unit_sz + 2 * grp;
+            float2 sz_next[2] = {__ldg(unit_sz), __ldg(unit_sz + 1)};
+            for (int it = 0; it < total_kb; ++it, ++n_done) {
+                const int sp = n_done % N_P;
+                const float2 sz[2] = {sz_next[0], sz_next[1]};
+                kb_next = kb_next + 1 == p.n_kb ? 0 : kb_next + 1;
+                sz_next[0] = __ldg(unit_sz + 4 * kb_next); sz_next[1] = __ldg(unit_sz + 4 * kb_next + 1);
+                fetch_next();
+                cp_async_wait<N_A - 1>();
+                __syncwarp();
+                uint32_t pa_w[2][BITS];
+                {
+                    uint32_t raw[4 * CH];
+                    const uint32_t slot = a_ring + (it % N_A) * SL.a_stage;
+#pragma unroll
+                    for (int j = 0; j < CH; ++j) {
+                        const uint4 v = lds128(slot + 16 * j);
+                        raw[4 * j] = v.x; raw[4 * j + 1] = v.y; raw[4 * j + 2] = v.z; raw[4 * j + 3] = v.w;
+                    }
+#pragma unroll
+                    for (int u = 0; u < 2; ++u)
+#pragma unroll
+                        for (int j = 0; j < BITS; ++j) pa_w[u][j] = BITS == 3 && grp ? raw[2 + 3 * u + j] : raw[BITS * u + j];
+                }
+                const uint32_t n_step = 2u * n_done + (uint32_t)grp;
+                const int st = n_step % N_U;
+                if (!mbar_wait(bar(B_PFULL + sp), (n_done / N_P) & 1, s_abort)) break;
+                // (all loads before the first store: they are not reordered)
+                const uint32_t pw = smem_base + SL.off_p + sp * SL.p_stage, a_tile = smem_base + st * SL.u_stage, w_tile = a_tile + A8_BYTES;
+                uint32_t pk[W_ROWS / 64][4];
+#pragma unroll
+                for (int i = 0; i < W_ROWS / 64; ++i) {
+                    const uint4 v = lds128(pw + ((ut >> 1) + 64 * i) * 64 + (2 * grp + (ut & 1)) * 16);
+                    pk[i][0] = v.x; pk[i][1] = v.y; pk[i][2] = v.z; pk[i][3] = v.w;
+                }
+                if (!mbar_wait(bar(B_UEMPTY + st), ((n_step / N_U) & 1) ^ 1, s_abort)) break;
+                tc_fence_after();
+#pragma unroll
+                for (int uu = 0; uu < 2; ++uu) {
+                    const float c1 = -(8388608.0f + sz[uu].y);
+                    const float2 neg_c1 = make_float2(c1, c1), s2 = make_float2(sz[uu].x, sz[uu].x);
+                    uint32_t o[8];
+                    unpack_act32<BITS>(pa_w[uu], o);
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) {
+                        uint32_t b0, b1, b2, b3;
+                        bytes_to_bf16(o[2 * c], neg_c1, s2, b0, b1);
+                        bytes_to_bf16(o[2 * c + 1], neg_c1, s2, b2, b3);
+                        sts128(a_tile + a_off + (((4 * uu + c) ^ a_sw) << 4), b0, b1, b2, b3);
+                    }
+                }
+#pragma unroll
+                for (int i = 0; i < W_ROWS / 64; ++i) {
+                    const int r = (ut >> 1) + 64 * i;
+                    if (it >= full_kb && r >= (W_ROWS >> p.split)) break;
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+                        sts128(w_tile + r * 128 + (((4 * (ut & 1) + c) ^ (r & 7)) << 4), nibbles_to_bf16(pk[i][c]), nibbles_to_bf16(pk[i][c] >> 8),
+                               nibbles_to_bf16(pk[i][c] >> 4), nibbles_to_bf16(pk[i][c] >> 12));
+                }
+                fence_proxy_async();
+                __syncwarp();
+                if (lane == 0) { arrive_leader(bar(B_UFULL + st)); mbar_arrive(bar(B_PEMPTY + sp)); }
+            }
+            cp_async_wait<0>();
         } else {
         // Activation codes: this thread owns token row `ut` of the tile and unpacks it. A K block of a
         // row is 16 BITS contiguous bytes; the rows' K blocks are fetched N_A - 1 K blocks ahead with
@@ -698,7 +825,7 @@ cluster_gemm_kernel(const Params p)
         // 32 / BITS rows, not 32: the load path looks up one cache line per row touched, and with one
         // row per lane those look-ups, not the bytes, set the pace. A row's chunks are copied by
         // lanes of the row owner's own warp, so a __syncwarp after the wait is all the hand-over needs.
-        constexpr int N_A = n_a_stages(BITS), PITCH = a_slot_pitch(BITS);
+        constexpr int N_A = n_a_stages(BITS, MODE), PITCH = a_slot_pitch(BITS, MODE);
         const uint32_t a_ring0 = smem_base + SL.off_a;
         const uint32_t a_ring = a_ring0 + ut * PITCH;
         uint32_t d_off[BITS], s_off[BITS];               // where my chunks go in a ring stage / come from in the tile's rows
@@ -755,63 +882,6 @@ cluster_gemm_kernel(const Params p)
                     for (int j = 0; j < BITS; ++j) pa_w[u][j] = raw[BITS * u + j];
             }
             if (!mbar_wait(bar(B_PFULL + sp), (n_done / N_P) & 1, s_abort)) break;
-            if constexpr (DEQ) {
-                // Two operand stages per K block, 64 positions each. My token row: units 2 h and 2 h + 1,
-                // de-quantised to bfloat16 with the unit's (s_c, z_c). Weights: for half h this thread
-                // converts unit 2 h + (ut & 1) of rows (ut >> 1) + 64 i.
-                const uint32_t pw = smem_base + SL.off_p + sp * SL.p_stage;
-                const int kb_now = it % p.n_kb;
-                bool ok = true;
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    const uint32_t n_step = 2u * n_done + (uint32_t)h;
-                    const int st = n_step % N_U;
-                    if (!mbar_wait(bar(B_UEMPTY + st), ((n_step / N_U) & 1) ^ 1, s_abort)) { ok = false; break; }
-                    tc_fence_after();
-                    const uint32_t a_tile = smem_base + st * SL.u_stage, w_tile = a_tile + A8_BYTES;
-#pragma unroll
-                    for (int uu = 0; uu < 2; ++uu) {
-                        const int u = 2 * h + uu;
-                        const float2 sz = __ldg(p.unit_sz + 4 * kb_now + u);
-                        const float c1 = -(8388608.0f + sz.y);
-                        const float2 neg_c1 = make_float2(c1, c1), s2 = make_float2(sz.x, sz.x);
-                        uint32_t o[8];
-                        unpack_act32<BITS>(pa_w[u], o);
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            uint32_t b0, b1, b2, b3;
-                            bytes_to_bf16(o[2 * c], neg_c1, s2, true, b0, b1);
-                            bytes_to_bf16(o[2 * c + 1], neg_c1, s2, true, b2, b3);
-                            sts128(a_tile + a_off + (((4 * uu + c) ^ a_sw) << 4), b0, b1, b2, b3);
-                        }
-                    }
-                    const float cw = -(8388608.0f + 128.0f);
-                    const float2 neg_cw = make_float2(cw, cw);
-#pragma unroll
-                    for (int i = 0; i < W_ROWS / 64; ++i) {
-                        const int r = (ut >> 1) + 64 * i;
-                        if (it >= full_kb && r >= (W_ROWS >> p.split)) break;
-                        const uint4 v = lds128(pw + r * 64 + (2 * h + (ut & 1)) * 16);
-                        const uint32_t pk[4] = {v.x, v.y, v.z, v.w};
-                        uint32_t o[8];
-                        unpack_w32_x16(pk, o);
-#pragma unroll
-                        for (int c = 0; c < 4; ++c) {
-                            uint32_t b0, b1, b2, b3;       // 16 w as bfloat16: the byte, sign bit flipped, minus 128
-                            bytes_to_bf16(o[2 * c] ^ 0x80808080u, neg_cw, neg_cw, false, b0, b1);
-                            bytes_to_bf16(o[2 * c + 1] ^ 0x80808080u, neg_cw, neg_cw, false, b2, b3);
-                            sts128(w_tile + r * 128 + (((4 * (ut & 1) + c) ^ (r & 7)) << 4), b0, b1, b2, b3);
-                        }
-                    }
-                    fence_proxy_async();
-                    __syncwarp();
-                    if (lane == 0) arrive_leader(bar(B_UFULL + st));
-                }
-                if (!ok) break;
-                __syncwarp();
-                if (lane == 0) mbar_arrive(bar(B_PEMPTY + sp));
-                continue;
-            }
             if (!mbar_wait(bar(B_UEMPTY + su), ((n_done / N_U) & 1) ^ 1, s_abort)) break;
             tc_fence_after();
             const uint32_t pw = smem_base + SL.off_p + sp * SL.p_stage;
@@ -851,7 +921,7 @@ cluster_gemm_kernel(const Params p)
         }
     } else {
         // ------------------------------------------------------------ epilogue warps
-        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_EPI));
+        asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(regs_epi(MODE)));
         const int ew = warp - EPI_WARP0;
         const int q = ew & 3, h = ew >> 2;           // TMEM lane quarter (= warp % 4), column half
         uint32_t n_tile_done = 0;
@@ -893,7 +963,7 @@ cluster_gemm_kernel(const Params p)
                     if (xs_row && sgi + 1 < p.n_seg) xs_next = __ldg(xs_row + s_seg_cl[sgi + 1]);
                 }
                 const uint32_t taddr = tmem_base + ((uint32_t)(32 * q) << 16) + buf * TILE_N + h * half_cols;
-                if (live) {
+                if (live && !DEQ) {
                 uint32_t va[16], vb[16];
                 tc_ld16(taddr, va);
                 // R += s_c * acc, two columns per packed fused multiply-add
@@ -906,9 +976,6 @@ cluster_gemm_kernel(const Params p)
                             const float2 t = fma2(make_float2(k.z, k.w), xs2, make_float2((float)(int)v[2 * i], (float)(int)v[2 * i + 1]));
                             R[c0 + i] = fma2(make_float2(k.x, k.y), t, R[c0 + i]);
                         }
-                    } else if constexpr (DEQ) {
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) R[c0 + i] = make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));   // the fp32 sums themselves
                     } else {
 #pragma unroll
                         for (int i = 0; i < 8; ++i)
@@ -927,6 +994,7 @@ cluster_gemm_kernel(const Params p)
                     if (!more) break;
                 }
                 }
+                if constexpr (DEQ) break;                    // (the sums are read as the outputs are formed)
                 tc_fence_before();
                 __syncwarp();
                 if (lane == 0) {
@@ -974,12 +1042,22 @@ cluster_gemm_kernel(const Params p)
                     hi = fma2(make_float2(w.z, w.w), add2(R[2 * i4 + 1], make_float2(-c.z, -c.w)), make_float2(b.z, b.w));
                     if (relu) { lo.x = fmaxf(lo.x, 0.f); lo.y = fmaxf(lo.y, 0.f); hi.x = fmaxf(hi.x, 0.f); hi.y = fmaxf(hi.y, 0.f); }
                 };
+                // DEQ: columns 16 c .. 16 c + 15 are the finished fp32 sums in tensor memory
+                const uint32_t t_acc = tmem_base + ((uint32_t)(32 * q) << 16) + (n_tile_done & 1u) * TILE_N + h * half_cols;
+                auto read_sums = [&](int c) {
+                    uint32_t v[16];
+                    tc_ld16(t_acc + 16 * c, v);
+                    tc_wait_ld();
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) R[8 * c + i] = make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+                };
                 auto h2 = [](float2 v) { const __half2 x = __floats2half2_rn(v.x, v.y); return *reinterpret_cast<const uint32_t*>(&x); };
                 if (p.y_dtype == RPTQ_OUT_F16) {
                     uint8_t* dst = static_cast<uint8_t*>(p.y) + ((int64_t)mw * p.ldy + nb) * 2;
 #pragma unroll
                     for (int c = 0; c < 8; ++c) {                              // 16 columns
                         if (16 * c >= half_cols) break;
+                        if constexpr (DEQ) read_sums(c);
                         float2 v[8];
 #pragma unroll
                         for (int i = 0; i < 4; ++i) finish(4 * c + i, v[2 * i], v[2 * i + 1]);
@@ -991,6 +1069,7 @@ cluster_gemm_kernel(const Params p)
 #pragma unroll
                     for (int c = 0; c < 16; ++c) {                             // 8 columns
                         if (8 * c >= half_cols) break;
+                        if constexpr (DEQ) if (c % 2 == 0) read_sums(c / 2);
                         float2 v[4];
                         finish(2 * c, v[0], v[1]);
                         finish(2 * c + 1, v[2], v[3]);
@@ -1043,8 +1122,12 @@ cluster_gemm_kernel(const Params p)
                     }
                 }
             }
+            if constexpr (DEQ) tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar(B_TABEMPTY + (n_tile_done & 1)));
+            if (lane == 0) {
+                mbar_arrive(bar(B_TABEMPTY + (n_tile_done & 1)));
+                if constexpr (DEQ) arrive_leader(bar(B_ACCEMPTY + (n_tile_done & 1)));
+            }
         }
     }
 
@@ -1064,15 +1147,17 @@ cluster_gemm_kernel(const Params p)
 template <int BITS, int NCTA, bool A8, int MODE>
 static int launch(const Params& p, int dev, int n_sm, cudaStream_t st)
 {
-    constexpr SmemLayout SL = smem_layout(NCTA, BITS, A8, MODE == MODE_ASYM);
+    constexpr SmemLayout SL = smem_layout(NCTA, BITS, A8, MODE);
+    constexpr int THREADS = threads_of(MODE);
     const int smem = SL.total + 1024;     // slack for the in-kernel 1024-byte alignment
     const void* fn = reinterpret_cast<const void*>(cluster_gemm_kernel<BITS, NCTA, A8, MODE>);
+    static_assert(SL.total + 1024 <= 227 * 1024, "shared memory");
     static std::atomic<uint64_t> done{0}, pool_ok{0};
     if (!(pool_ok.load(std::memory_order_acquire) >> (dev & 63) & 1u)) {
         cudaFuncAttributes attr;
         if (cudaFuncGetAttributes(&attr, fn) != cudaSuccess) return RPTQ_ERR_CUDA;
         // the register re-partition inside the kernel (setmaxnreg) assumes this pool; refuse to launch otherwise
-        if (attr.numRegs * THREADS < 128 * (REGS_WG0 + REGS_UNPACK + 2 * REGS_EPI)) return RPTQ_ERR_UNSUPPORTED;
+        if (attr.numRegs * THREADS < regs_all(MODE)) return RPTQ_ERR_UNSUPPORTED;
         if (dev >= 0 && dev < 64) pool_ok.fetch_or(uint64_t(1) << dev, std::memory_order_release);
     }
     if (allow_smem(fn, dev, smem, done) != RPTQ_OK) return RPTQ_ERR_CUDA;
