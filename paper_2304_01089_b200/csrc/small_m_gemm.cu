@@ -16,13 +16,18 @@
 //     multiplies with mma.sync m16n8k32: the weight rows are the instruction's M dimension (signed
 //     8-bit operands = 16 w, as in the large kernel, three logic instructions per operand pair), the
 //     tokens its N dimension (unsigned 8-bit), so the per-channel constants of the epilogue are
-//     per-thread scalars. Lane (g, t) reads the 16 bytes of unit t of rows g and g + 8 of the K
-//     block; instruction j of the block's four takes word j of every lane, i.e. positions 8j..8j+7
-//     of all four units.
-//   - an instruction therefore mixes the block's four units. Where they belong to one cluster (most
-//     blocks) that is the cluster's sum; where a block holds several clusters, it is multiplied once
-//     per cluster with the other clusters' lanes zeroed ("passes", prepared per K block when the
-//     kernel starts, in the order in which the clusters end).
+//     per-thread scalars. An instruction multiplies one unit of 32 positions: ldmatrix hands lane (g, t)
+//     word t of every unit of rows g and g + 8 (a matrix = eight rows' 16 bytes of one unit), and the tokens' words are stored
+//     so that one 16-byte load has the lane's word of all four units of a K block. So a unit's products go to its own
+//     cluster's accumulator, and a cluster is drained where its last unit was multiplied.
+//     (An instruction over one word of all four units needs no ldmatrix, but a K block
+//     whose units belong to several clusters is then multiplied once per cluster with the others' lanes zeroed: twice the
+//     instructions. 16 x 9216 x 36864, 3 bits, with the LayerNorm: 58.1 -> 51.4 us; the copies' 64-byte swizzle, which keeps
+//     ldmatrix free of bank conflicts, 49.6.)
+//   - the zero-point corrections (a sum over the clusters per channel) are formed by two warps of their own while the weights
+//     stream, not at the end, and a consumer warp unpacks whole token rows, four units' loads at a time: 46.0 us (one token
+//     44.7 -> 39.1; with the consumers' arithmetic left out 38.7: the weight stream bounds that, at 4.9 TB/s).
+#include <cuda.h>
 #include <cuda_fp16.h>
 
 #include "rptq_internal.h"
@@ -32,7 +37,9 @@ namespace rptq {
 namespace smallm {
 
 constexpr int CONSUMER_WARPS = 16;
-constexpr int THREADS = 32 * (CONSUMER_WARPS + 1);
+constexpr int TABLE_WARPS = 2;
+constexpr int THREADS = 32 * (CONSUMER_WARPS + 1 + TABLE_WARPS);      // consumers, producer, column tables
+constexpr int SMEM_LIMIT = 223 * 1024;      // dynamic (3.2 KB more are static)
 constexpr int STAGES = 8;
 constexpr int STAGE_BYTES = 16384;          // two 8 KiB weight tiles: K block kb of both 128-row tiles
 constexpr long long WAIT_BUDGET_CYCLES = 4000000000ll;   // about two seconds
@@ -71,25 +78,27 @@ __device__ __forceinline__ void mma_s8u8(int (&d)[4], uint32_t a0, uint32_t a1, 
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// One pass of a K block: which of its four units take part (bits 0..3), the accumulator (bit 4), whether the
-// cluster ends in this block (bit 5), and the cluster's s_c / 16.
-struct Pass { uint32_t ctrl; float sc; };
-constexpr uint32_t PASS_BUF = 16u, PASS_LAST = 32u;
+__device__ __forceinline__ void ldmatrix4(uint32_t (&x)[4], uint32_t addr)
+{
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];" : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]) : "r"(addr) : "memory");
+}
 
 template <int BITS, int NT>
 __global__ void __launch_bounds__(THREADS, 1)
-small_m_kernel(const SmallMParams p)
+small_m_kernel(const SmallMParams p, const __grid_constant__ CUtensorMap w_map)
 {
     extern __shared__ __align__(128) uint8_t smem_raw[];
-    const uint32_t base = (smem_u32(smem_raw) + 127u) & ~127u;
+    const uint32_t base = (smem_u32(smem_raw) + 511u) & ~511u;         // (the ring's swizzle repeats every 512 bytes)
     uint8_t* smem = smem_raw + (base - smem_u32(smem_raw));
-    // ring | token codes (nibbles) | passes | barriers
+    // ring | token codes (nibbles) | per unit: s_c / 16, step flags | barriers
     const int a_pitch = p.K_pad / 2 + (((p.K_pad / 2) & 127) ? 0 : 64);      // odd multiple of 64: two token rows fill the 32 banks
     uint8_t* ring = smem;
     uint8_t* act = ring + STAGES * STAGE_BYTES;
-    Pass* passes = reinterpret_cast<Pass*>(act + 8 * NT * a_pitch);          // [n_kb][4]
-    uint64_t* bars = reinterpret_cast<uint64_t*>(passes + 4 * p.n_kb);       // full[STAGES], empty[STAGES]
+    float* unit_scale = reinterpret_cast<float*>(act + 8 * NT * a_pitch);    // [4 n_kb]
+    uint8_t* unit_flags = reinterpret_cast<uint8_t*>(unit_scale + 4 * p.n_kb);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(unit_flags + (4 * p.n_kb + 7) / 8 * 8);       // full[STAGES], empty[STAGES]
     __shared__ int s_abort_flag;
+    __shared__ float s_col[3][256];              // zero-point correction, s_w and bias of the block's channels
     volatile int* s_abort = &s_abort_flag;
 
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, g8 = lane >> 2, t4 = lane & 3;
@@ -103,12 +112,13 @@ small_m_kernel(const SmallMParams p)
         }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    // (the layout's own tables)
+    for (int u = tid; u < 4 * p.n_kb; u += THREADS) { unit_scale[u] = __ldg(&p.unit_sz[u].x) * 0.0625f; unit_flags[u] = __ldg(p.step_flags + u); }
+    const int tileA = p.tiles_per_block * (int)blockIdx.x;
+    const bool haveB = p.tiles_per_block == 2 && tileA + 1 < p.n_wtiles;
     __syncthreads();
     pdl_trigger();
     pdl_wait();
-
-    const int tileA = 2 * (int)blockIdx.x;
-    const bool haveB = tileA + 1 < p.n_wtiles;
 
     float R[NT][4];
 #pragma unroll
@@ -119,9 +129,9 @@ small_m_kernel(const SmallMParams p)
     if (warp == CONSUMER_WARPS) {
         // ------------------------------------------------------------ producer
         if (lane == 0) {
-            const uint8_t* srcA = p.w + (int64_t)tileA * p.n_kb * 8192;
-            const uint8_t* srcB = srcA + (int64_t)p.n_kb * 8192;
-            const uint32_t bytes = haveB ? STAGE_BYTES : STAGE_BYTES / 2;
+            // the weights as rows of 64 bytes: K block kb of tile t is rows 128 (t n_kb + kb) ..
+            const int rowA = tileA * p.n_kb * 128, rowB = rowA + p.n_kb * 128;
+            const uint32_t bytes = haveB ? STAGE_BYTES : STAGE_BYTES / 2;      // (the second tile's half of a stage stays empty)
             int issued = 0;
             for (int kb = 0; kb < p.n_kb; ++kb) {
                 const int s = kb % STAGES;
@@ -129,11 +139,12 @@ small_m_kernel(const SmallMParams p)
                 if (*s_abort) break;
                 const uint32_t dst = smem_u32(ring + s * STAGE_BYTES), bar = full0 + 8 * s;
                 asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-                asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                             ::"r"(dst), "l"(srcA + (int64_t)kb * 8192), "r"(8192), "r"(bar) : "memory");
-                if (haveB)
-                    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                                 ::"r"(dst + 8192), "l"(srcB + (int64_t)kb * 8192), "r"(8192), "r"(bar) : "memory");
+                auto load = [&](uint32_t to, int row) {
+                    asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+                                 ::"r"(to), "l"(&w_map), "r"(0), "r"(row), "r"(bar) : "memory");
+                };
+                load(dst, rowA + 128 * kb);
+                if (haveB) load(dst + 8192, rowB + 128 * kb);
                 issued = kb + 1;
             }
             // After a give-up the consumers no longer wait for the copies still in flight: they must have
@@ -144,133 +155,131 @@ small_m_kernel(const SmallMParams p)
                     while (!mbar_try_wait_for(full0 + 8 * (kb % STAGES), (uint32_t)(kb / STAGES) & 1u, 2000u) && clock64() - t0 <= WAIT_BUDGET_CYCLES) {}
             }
         }
+    } else if (warp > CONSUMER_WARPS) {
+        // ------------------------------------------------------------ column tables: two warps, four channels a lane (in the consumers'
+        // own code the loads of the g clusters took 3 us at the end of the kernel)
+        const int at = 128 * (warp - CONSUMER_WARPS - 1) + lane, n = tileA * 128 + at;      // my channels: n + 32 e
+        float corr[4] = {0.f, 0.f, 0.f, 0.f};
+        if (p.corr) {
+#pragma unroll
+            for (int e = 0; e < 4; ++e) if (n + 32 * e < p.N) corr[e] = __ldg(p.corr + n + 32 * e);
+        } else {
+#pragma unroll 4
+            for (int c = 0; c < p.g; ++c) {
+                const float sz = __ldg(p.cl_sz + c);
+#pragma unroll
+                for (int e = 0; e < 4; ++e) corr[e] = __fmaf_rn(sz, n + 32 * e < p.N ? (float)__ldg(p.wsum + (int64_t)c * p.ld_w + n + 32 * e) : 0.f, corr[e]);
+            }
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const bool in = n + 32 * e < p.N;
+            s_col[0][at + 32 * e] = corr[e];
+            s_col[1][at + 32 * e] = in ? __ldg(p.s_w + n + 32 * e) : 0.f;
+            s_col[2][at + 32 * e] = in && p.bias ? __ldg(p.bias + n + 32 * e) : 0.f;
+        }
+        asm volatile("bar.arrive 2, %0;" ::"n"(32 * (CONSUMER_WARPS + TABLE_WARPS)) : "memory");
     } else {
         // ------------------------------------------------------------ consumers
         // (the producer is already streaming weights while the consumers prepare their tables)
-        // the tokens' codes as nibbles: word i of a unit holds positions 8i..8i+3 in the low and 8i+4..8i+7
-        // in the high nibbles of its bytes (the packed format of 4-bit codes); rows >= M are zero
-        for (int it = tid; it < 8 * NT * p.n_units; it += 32 * CONSUMER_WARPS) {
-            const int r = it / p.n_units, u = it - r * p.n_units;
-            uint4 v = make_uint4(0, 0, 0, 0);
-            if (r < p.M) {
-                const uint8_t* row = p.a + (int64_t)r * p.a_row_bytes;
-                if constexpr (BITS == 4) {
-                    v = __ldg(reinterpret_cast<const uint4*>(row) + u);
-                } else {
-                    const uint32_t* w = reinterpret_cast<const uint32_t*>(row) + u * 3;
-                    const uint32_t q[3] = {__ldg(w), __ldg(w + 1), __ldg(w + 2)};
-                    uint32_t o[8];
-                    unpack_act32<3>(q, o);
-                    v = make_uint4(o[0] | (o[1] << 4), o[2] | (o[3] << 4), o[4] | (o[5] << 4), o[6] | (o[7] << 4));
-                }
-            }
-            *reinterpret_cast<uint4*>(act + r * a_pitch + 16 * u) = v;
-        }
-        // the passes of every K block
-        for (int kb = tid; kb < p.n_kb; kb += 32 * CONSUMER_WARPS) {
-            int cl[4]; uint32_t ctrl[4]; float sc[4]; int lastpos[4]; int n = 0;
-            for (int ul = 0; ul < 4; ++ul) {
-                const int u = 4 * kb + ul;
-                const int fl = __ldg(p.step_flags + u);
-                if (fl & STEP_SKIP) continue;
-                const int c = __ldg(p.unit_cluster + u);
-                int k = 0;
-                while (k < n && cl[k] != c) ++k;
-                if (k == n) { cl[n] = c; ctrl[n] = (fl & STEP_BUF) ? PASS_BUF : 0u; sc[n] = __ldg(&p.unit_sz[u].x) * 0.0625f; lastpos[n] = 9; ++n; }
-                ctrl[k] |= 1u << ul;
-                if (fl & STEP_LAST) { ctrl[k] |= PASS_LAST; lastpos[k] = ul; }
-            }
-            for (int i = 1; i < n; ++i)                      // clusters that end here first, in the order they end
-                for (int j = i; j > 0 && lastpos[j] < lastpos[j - 1]; --j) {
-                    const int tc = cl[j]; cl[j] = cl[j - 1]; cl[j - 1] = tc;
-                    const uint32_t tt = ctrl[j]; ctrl[j] = ctrl[j - 1]; ctrl[j - 1] = tt;
-                    const float ts = sc[j]; sc[j] = sc[j - 1]; sc[j - 1] = ts;
-                    const int tl = lastpos[j]; lastpos[j] = lastpos[j - 1]; lastpos[j - 1] = tl;
-                }
-            for (int i = 0; i < 4; ++i) passes[4 * kb + i] = Pass{i < n ? ctrl[i] : 0u, i < n ? sc[i] : 0.f};
-        }
-        asm volatile("bar.sync 1, %0;" ::"n"(32 * CONSUMER_WARPS) : "memory");
         const int tile_sel = warp >> 3;                       // which of the block's two tiles
         const bool active = tile_sel == 0 || haveB;
-        const uint8_t* wrow = ring + tile_sel * 8192 + (16 * (warp & 7) + g8) * 64 + 16 * t4;
+        const int n0 = (tileA + tile_sel) * 128 + 16 * (warp & 7);
+        // The tokens' codes as nibbles: word j of a unit holds positions 8j..8j+3 in the low and 8j+4..8j+7 in the high nibbles
+        // of its bytes (the packed format of 4-bit codes). Word j of the four units of a K block are stored side by side. Rows >= M
+        // are zero. Four units a thread at a time, their loads first.
+        {
+            constexpr int SPLIT = 2 / NT;                     // warps of a row
+            const int r = warp / SPLIT;
+            const uint32_t* row = reinterpret_cast<const uint32_t*>(p.a + (int64_t)(r < p.M ? r : 0) * p.a_row_bytes);
+#pragma unroll 1
+            for (int u0 = lane + 32 * (warp % SPLIT); u0 < p.n_units; u0 += 4 * 32 * SPLIT) {
+                uint32_t q[4][BITS];
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int u = u0 + k * 32 * SPLIT;
+                    const bool in = r < p.M && u < p.n_units;
+#pragma unroll
+                    for (int e = 0; e < BITS; ++e) q[k][e] = in ? __ldg(row + u * BITS + e) : 0u;
+                }
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const int u = u0 + k * 32 * SPLIT;
+                    if (u >= p.n_units) break;
+                    uint32_t o[8];
+                    unpack_act32<BITS>(q[k], o);
+                    uint32_t* d = reinterpret_cast<uint32_t*>(act + r * a_pitch + 64 * (u >> 2) + 4 * (u & 3));
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) d[4 * e] = o[2 * e] | (o[2 * e + 1] << 4);
+                }
+            }
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * CONSUMER_WARPS) : "memory");
+        // lane i hands ldmatrix row i % 8 of matrix (unit) i / 8; piece c of row r lies at c ^ ((r / 2) & 3)
+        const uint32_t w_at = smem_u32(ring) + tile_sel * 8192 + (16 * (warp & 7) + (lane & 7)) * 64 + 16 * ((lane >> 3) ^ ((lane >> 1) & 3));
         const uint8_t* arow = act + g8 * a_pitch + 16 * t4;
-        int acc0[2][NT][4], acc1[2][NT][4];                   // [instruction parity][token tile]: two accumulators per buffer
+        int acc0[NT][4], acc1[NT][4];                         // the two accumulators (as in the large kernel, the layout says which)
 #pragma unroll
-        for (int h = 0; h < 2; ++h)
+        for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                for (int e = 0; e < 4; ++e) { acc0[h][nt][e] = 0; acc1[h][nt][e] = 0; }
+            for (int e = 0; e < 4; ++e) { acc0[nt][e] = 0; acc1[nt][e] = 0; }
 
         for (int kb = 0; kb < p.n_kb; ++kb) {
             const int s = kb % STAGES;
-            if (!mbar_wait(full0 + 8 * s, (uint32_t)(kb / STAGES) & 1u, s_abort)) break;
-            uint4 X0 = make_uint4(0, 0, 0, 0), X1 = X0;
-            if (active) {
-                X0 = *reinterpret_cast<const uint4*>(wrow + s * STAGE_BYTES);
-                X1 = *reinterpret_cast<const uint4*>(wrow + s * STAGE_BYTES + 512);
-            }
+            const uint32_t f4 = __shfl_sync(0xffffffffu, *reinterpret_cast<const uint32_t*>(unit_flags + 4 * kb), 0);
             uint4 B[NT];
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) B[nt] = *reinterpret_cast<const uint4*>(arow + 8 * nt * a_pitch + 64 * kb);
-            const uint4 ps01 = *reinterpret_cast<const uint4*>(passes + 4 * kb);
-            const uint4 ps23 = *reinterpret_cast<const uint4*>(passes + 4 * kb + 2);
+            if (!mbar_wait(full0 + 8 * s, (uint32_t)(kb / STAGES) & 1u, s_abort)) break;
+            __syncwarp();
+            if (!active) {
+                if (lane == 0) mbar_arrive(empty0 + 8 * s);
+                continue;
+            }
+            uint32_t x0[4], x1[4];                            // rows g8, g8 + 8: word t4 of the four units
+            ldmatrix4(x0, w_at + s * STAGE_BYTES);
+            ldmatrix4(x1, w_at + s * STAGE_BYTES + 512);
             __syncwarp();
             if (lane == 0) mbar_arrive(empty0 + 8 * s);       // the stage's bytes are in registers
-            const uint32_t xw0[4] = {X0.x, X0.y, X0.z, X0.w}, xw1[4] = {X1.x, X1.y, X1.z, X1.w};
-            const uint32_t ctrls[4] = {ps01.x, ps01.z, ps23.x, ps23.z};
-            const float scs[4] = {__uint_as_float(ps01.y), __uint_as_float(ps01.w), __uint_as_float(ps23.y), __uint_as_float(ps23.w)};
-            uint32_t bw[NT][4][2];                            // the tokens' bytes for instruction j: positions 8j..8j+3, 8j+4..8j+7
+            auto multiply = [&](int j, int (&acc)[NT][4]) {   // unit j
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) {
-                const uint32_t w[4] = {B[nt].x, B[nt].y, B[nt].z, B[nt].w};
+                for (int nt = 0; nt < NT; ++nt) {
+                    const uint32_t b = j == 0 ? B[nt].x : j == 1 ? B[nt].y : j == 2 ? B[nt].z : B[nt].w;
+                    mma_s8u8(acc[nt], (x0[j] << 4) & 0xF0F0F0F0u, (x1[j] << 4) & 0xF0F0F0F0u, x0[j] & 0xF0F0F0F0u, x1[j] & 0xF0F0F0F0u,
+                             b & 0x0F0F0F0Fu, (b >> 4) & 0x0F0F0F0Fu);
+                }
+            };
+            constexpr uint32_t ALL = 0x01010101u;
+            if ((f4 & (ALL * (STEP_LAST | STEP_SKIP | STEP_BUF))) == 0u) {
 #pragma unroll
-                for (int j = 0; j < 4; ++j) { bw[nt][j][0] = w[j] & 0x0F0F0F0Fu; bw[nt][j][1] = (w[j] >> 4) & 0x0F0F0F0Fu; }
-            }
+                for (int j = 0; j < 4; ++j) multiply(j, acc0);
+            } else if ((f4 & (ALL * (STEP_LAST | STEP_SKIP | STEP_BUF))) == ALL * STEP_BUF) {
 #pragma unroll
-            for (int ps = 0; ps < 4; ++ps) {
-                const uint32_t ctrl = ctrls[ps];
-                if ((ctrl & 15u) == 0u) break;
-                const uint32_t keep = 0u - ((ctrl >> t4) & 1u);            // all ones where my unit belongs to the pass's cluster
-                const uint32_t m_lo = 0xF0F0F0F0u & keep;
-                uint32_t aw[4][4];                                         // the four instructions' weight operands
+                for (int j = 0; j < 4; ++j) multiply(j, acc1);
+            } else {
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
-                    aw[j][0] = (xw0[j] << 4) & m_lo; aw[j][2] = xw0[j] & m_lo;
-                    aw[j][1] = (xw1[j] << 4) & m_lo; aw[j][3] = xw1[j] & m_lo;
+                    const uint32_t f = f4 >> (8 * j);
+                    if (f & STEP_SKIP) continue;
+                    auto unit = [&](int (&acc)[NT][4]) {
+                        multiply(j, acc);
+                        if (f & STEP_LAST) {
+                            const float sc = unit_scale[4 * kb + j];
+#pragma unroll
+                            for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+                                for (int e = 0; e < 4; ++e) { R[nt][e] = __fmaf_rn(sc, (float)acc[nt][e], R[nt][e]); acc[nt][e] = 0; }
+                        }
+                    };
+                    if (f & STEP_BUF) unit(acc1); else unit(acc0);
                 }
-                const float sc = scs[ps];
-                auto run = [&](int (&acc)[2][NT][4]) {
-#pragma unroll
-                    for (int j = 0; j < 4; ++j)
-#pragma unroll
-                        for (int nt = 0; nt < NT; ++nt)
-                            mma_s8u8(acc[j & 1][nt], aw[j][0], aw[j][1], aw[j][2], aw[j][3], bw[nt][j][0], bw[nt][j][1]);
-                    if (ctrl & PASS_LAST) {
-#pragma unroll
-                        for (int nt = 0; nt < NT; ++nt)
-#pragma unroll
-                            for (int e = 0; e < 4; ++e) {
-                                R[nt][e] = __fmaf_rn(sc, (float)(acc[0][nt][e] + acc[1][nt][e]), R[nt][e]);
-                                acc[0][nt][e] = 0; acc[1][nt][e] = 0;
-                            }
-                    }
-                };
-                if (ctrl & PASS_BUF) run(acc1); else run(acc0);
             }
         }
 
         // -------------------------------------------------------- epilogue: y = s_w (R - corr) + bias
-        const int n0 = (tileA + tile_sel) * 128 + 16 * (warp & 7);
+        asm volatile("bar.sync 2, %0;" ::"n"(32 * (CONSUMER_WARPS + TABLE_WARPS)) : "memory");
         if (active && n0 < p.N && !*s_abort) {
-            float corr = 0.f, sw = 0.f, bs = 0.f;      // lanes 0..15 each take one of the warp's channels
-            const int nl = n0 + (lane & 15);
-            if (lane < 16 && nl < p.N) {
-                if (p.corr) corr = __ldg(p.corr + nl);
-                else for (int c = 0; c < p.g; ++c) corr = __fmaf_rn(__ldg(p.cl_sz + c), (float)__ldg(p.wsum + (int64_t)c * p.ld_w + nl), corr);
-                sw = __ldg(p.s_w + nl);
-                bs = p.bias ? __ldg(p.bias + nl) : 0.f;
-            }
+            const float corr = s_col[0][n0 - 128 * tileA + (lane & 15)], sw = s_col[1][n0 - 128 * tileA + (lane & 15)], bs = s_col[2][n0 - 128 * tileA + (lane & 15)];
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {             // rows g (accumulator entries 0, 1) and g + 8 (entries 2, 3)
                 const int src = g8 + 8 * hh, n = n0 + src;
@@ -297,22 +306,48 @@ small_m_kernel(const SmallMParams p)
 static int smem_bytes(int nt, int K_pad)
 {
     const int a_pitch = K_pad / 2 + (((K_pad / 2) & 127) ? 0 : 64);
-    return 128 + STAGES * STAGE_BYTES + 8 * nt * a_pitch + (K_pad / 128) * 4 * (int)sizeof(Pass) + 2 * STAGES * 8;
+    return 512 + STAGES * STAGE_BYTES + 8 * nt * a_pitch + (K_pad / 32) * 4 + (K_pad / 32 + 7) / 8 * 8 + 2 * STAGES * 8;
+}
+
+// The packed weights as a matrix of 64-byte rows, copied 128 rows (one tile's K block) at a time with the 64-byte swizzle, so
+// that ldmatrix reads eight rows without a bank conflict.
+static int weight_map(const SmallMParams& p, CUtensorMap* map)
+{
+    using Encode = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
+                                const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
+    static const Encode encode = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) fn = nullptr;
+        return reinterpret_cast<Encode>(fn);
+    }();
+    if (!encode) return RPTQ_ERR_CUDA;
+    const cuuint64_t dims[2] = {64, (cuuint64_t)p.n_wtiles * p.n_kb * 128}, strides[1] = {64};
+    const cuuint32_t box[2] = {64, 128}, step[2] = {1, 1};
+    return encode(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t*>(p.w), dims, strides, box, step, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS ? RPTQ_OK : RPTQ_ERR_CUDA;
 }
 
 template <int BITS, int NT>
-static int launch_one(const SmallMParams& p, int device, cudaStream_t st)
+static int launch_one(SmallMParams p, int device, cudaStream_t st)
 {
     const int smem = smem_bytes(NT, p.K_pad);
     static std::atomic<uint64_t> done{0};
-    if (allow_smem(reinterpret_cast<const void*>(small_m_kernel<BITS, NT>), device, 226 * 1024, done) != RPTQ_OK) return RPTQ_ERR_CUDA;
-    const int blocks = (p.n_wtiles + 1) / 2;
-    return launch_kernel(small_m_kernel<BITS, NT>, dim3((unsigned)blocks), THREADS, (size_t)smem, 0, st, p);
+    if (allow_smem(reinterpret_cast<const void*>(small_m_kernel<BITS, NT>), device, SMEM_LIMIT, done) != RPTQ_OK) return RPTQ_ERR_CUDA;
+    // a block per 128 channels where the SMs suffice: the call then takes as long as one tile's stream
+    const int n_sm = sm_count(device);
+    if (n_sm == 0) return RPTQ_ERR_CUDA;
+    p.tiles_per_block = p.n_wtiles <= n_sm ? 1 : 2;
+    const int blocks = (p.n_wtiles + p.tiles_per_block - 1) / p.tiles_per_block;
+    CUtensorMap map;
+    if (weight_map(p, &map) != RPTQ_OK) return RPTQ_ERR_CUDA;
+    return launch_kernel(small_m_kernel<BITS, NT>, dim3((unsigned)blocks), THREADS, (size_t)smem, 0, st, p, map);
 }
 
 bool fits(int M, int bits, int K_pad)
 {
-    return M <= 16 && (bits == 3 || bits == 4) && smem_bytes(M <= 8 ? 1 : 2, K_pad) <= 226 * 1024;
+    return M <= 16 && (bits == 3 || bits == 4) && smem_bytes(M <= 8 ? 1 : 2, K_pad) <= SMEM_LIMIT;
 }
 
 int launch(const SmallMParams& p, int bits, int device, cudaStream_t st)
