@@ -200,6 +200,12 @@ __device__ __forceinline__ uint4 nibbles(uint32_t row, int u, int bits)
 __device__ __forceinline__ int units_seen(int nu) { return nu > 0 ? nu : 1; }
 
 // One block's walk over its work: item = (query tile, head, sequence), the tiles with the most visible keys first.
+// Every other round of items is dealt out backwards, so that no block gets the dearer one of every round (37 heads, 2048 tokens, causal:
+// items of 16, 12, 8 and 4 tiles on one block, of 13, 9, 5 and 1 on another).
+__device__ __forceinline__ int item_index(uint32_t n)
+{
+    return (int)(n * gridDim.x + ((n & 1u) ? gridDim.x - 1u - blockIdx.x : blockIdx.x));
+}
 struct Item { int qt, h, seq, n_kt; };
 __device__ __forceinline__ Item item_of(const AttnParams& p, const Plan& g, int idx, int keys)
 {
@@ -286,7 +292,7 @@ prefill_kernel(const AttnParams p, const Plan g)
             const uint32_t id = MODE == I8 && g.folded ? ID | (1u << 7) : ID;                // (signed bytes)
             const uint32_t b_full0 = bar(B_SFULL + stream * N_SLOTS), b_empty0 = bar(B_SEMPTY + stream * N_SLOTS);
             uint32_t n_k = 0, slot = 0, par = 1, n_item = 0;                    // n_k: my tiles so far
-            for (int idx = blockIdx.x; idx < g.n_items && ok; idx += gridDim.x, ++n_item) {
+            for (int idx; ok && (idx = item_index(n_item)) < g.n_items; ++n_item) {
                 const Item it = item_of(p, g, idx, KEYS);
                 const int uk0 = __ldg(p.cl_unit0_k + it.h * p.gh_k), nuk = __ldg(p.cl_unit0_k + (it.h + 1) * p.gh_k) - uk0, nu = units_seen(nuk);
                 // bit u: unit u is the last of its cluster
@@ -335,7 +341,7 @@ prefill_kernel(const AttnParams p, const Plan g)
             constexpr uint32_t ID = (MODE == KV ? (1u << 4) : (2u << 4)) | (8u << 24);
             const uint32_t dv = desc(g.off_v), dp = desc(g.off_p), v_step = (uint32_t)(g.v_stage >> 4);
             uint32_t n_v = 0, n_item = 0, n_p0 = 0, n_p1 = 0;                  // (KV: tiles of each stream so far)
-            for (int idx = blockIdx.x; idx < g.n_items && ok; idx += gridDim.x, ++n_item) {
+            for (int idx; ok && (idx = item_index(n_item)) < g.n_items; ++n_item) {
                 const Item it = item_of(p, g, idx, KEYS);
                 const int nuv = __ldg(p.cl_unit0_v + (it.h + 1) * p.gh_v) - __ldg(p.cl_unit0_v + it.h * p.gh_v);
                 const uint32_t id = ID | ((uint32_t)(4 * nuv) << 17);
@@ -387,18 +393,18 @@ prefill_kernel(const AttnParams p, const Plan g)
         const int r0 = ROWS_W * lw + (lane >> 3), c0 = lane & 7;               // eight lanes per row; my rows are r0 + 4 i
         bool ok = true;
         // The tile that is being fetched (`nx`) and the one that is being worked on (`cu`), one tile behind
-        struct Tile { int idx, t, n_t, kt; Item it; int u0, nu; };
+        struct Tile { uint32_t n; int t, n_t, kt; Item it; int u0, nu; };       // (n: the block's n-th item)
         const bool is_k = warp < V_WARP0;
         Tile nx, cu;
-        nx.idx = (int)blockIdx.x - (int)gridDim.x; nx.t = 0; nx.n_t = 1; nx.kt = 0;
+        nx.n = 0xFFFFFFFFu; nx.t = 0; nx.n_t = 1; nx.kt = 0;
         // keys: every item's tiles twice; values: once
         auto advance = [&]() {
             ++nx.kt;
             if (++nx.t == nx.n_t) {
-                nx.idx += gridDim.x;
+                const int idx = item_index(++nx.n);
                 nx.t = 0;
-                if (nx.idx >= g.n_items) return false;
-                nx.it = item_of(p, g, nx.idx, KEYS);
+                if (idx >= g.n_items) return false;
+                nx.it = item_of(p, g, idx, KEYS);
                 nx.n_t = is_k ? 2 * nx.it.n_kt : nx.it.n_kt;
                 const int32_t* u = is_k ? p.cl_unit0_k + nx.it.h * p.gh_k : p.cl_unit0_v + nx.it.h * p.gh_v;
                 nx.u0 = __ldg(u);
@@ -882,7 +888,7 @@ prefill_kernel(const AttnParams p, const Plan g)
         const uint32_t b_full0 = bar(B_SFULL + stream * N_SLOTS), b_empty0 = bar(B_SEMPTY + stream * N_SLOTS);
         uint32_t n_k0 = 0, slot = 0, par = 0, n_s = 0, n_item = 0;   // n_s: my stream's tiles of pass 2 so far
         bool ok = true;
-        for (int idx = blockIdx.x; idx < g.n_items && ok; idx += gridDim.x, ++n_item) {
+        for (int idx; ok && (idx = item_index(n_item)) < g.n_items; ++n_item) {
             const Item it = item_of(p, g, idx, KEYS);
             const int i0 = it.qt * BM, i = i0 + row, off = p.Tk - p.Tq;
             const bool live = i0 + 32 * q4 < p.Tq;                             // some row of my warp exists
