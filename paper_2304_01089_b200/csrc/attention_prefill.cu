@@ -789,6 +789,13 @@ prefill_kernel(const AttnParams p, const Plan g)
                 }
                 if (n > 0 && cu.t == cu.n_t - 1) {
                 // ---- the item's output rows: warp = lane quarter of the accumulator, thread = row
+                // channel of position `lane` of every unit, asked for before the wait
+                int chs[MAX_UNITS];
+#pragma unroll
+                for (int u = 0; u < MAX_UNITS; ++u) {
+                    const int pos = 32 * (uv0 + u) + lane;
+                    chs[u] = u < nuv && __ldg(p.jidx_v + pos) >= 0 ? (int)__ldg(p.src_v + pos) : -1;
+                }
                 if (!mbar_sleep(bar(B_SUM), n_item & 1, s_abort) || !mbar_sleep(bar(B_OFULL), n_item & 1, s_abort)) { ok = false; break; }
                 __syncwarp();
                 tc::tc_fence_after();
@@ -811,8 +818,9 @@ prefill_kernel(const AttnParams p, const Plan g)
 #pragma unroll 1
                     for (int u = 0; u < nuv; ++u) {
                         // channel of position `lane` of the unit
-                        const int pos = 32 * (uv0 + u) + lane;
-                        int ch = __ldg(p.jidx_v + pos) >= 0 ? (int)__ldg(p.src_v + pos) : -1;
+                        int ch = chs[0];
+#pragma unroll
+                        for (int v = 0; v + 1 < MAX_UNITS; ++v) chs[v] = chs[v + 1];      // (a queue: the loop is not unrolled)
                         const float2 sz = __ldg(p.unit_sz_v + uv0 + u);
                         const float sc = MODE == KV ? sz.x * inv_l : p.s_P * sz.x, zf = sz.x * (sz.y - (V8 ? 128.0f : 8.0f));
                         const int zi = (int)sz.y * rs;
