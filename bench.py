@@ -180,11 +180,11 @@ def _attention_leg(w, M, torch, binding):
     ev[n_rep].record()
     torch.cuda.synchronize()
     us_kv = float(np.median([ev[i].elapsed_time(ev[i + 1]) for i in range(n_rep)])) * 1e3
-    return {"kernel": "attention_kernel", "heads": H, "head_dim": 128, "clusters_per_head": 4, "sequences": n_seq, "tokens": T, "causal": True,
+    return {"kernel": "attn_prefill::prefill_kernel", "heads": H, "head_dim": 128, "clusters_per_head": 4, "sequences": n_seq, "tokens": T, "causal": True,
             "bits": w.bits, "us": us, "TOPS": ops / us / 1e6,
-            "kv_only": {"kernel": "attention_kv_kernel", "us": us_kv, "TFLOPS": ops / us_kv / 1e6,
-                        "note": "16-bit query and probabilities, quantised key / value cache; fp16 mma.sync m16n8k16"},
-            "note": "integer products on mma.sync m16n8k32 (the scores are computed twice: the softmax codes need the finished row sums)"}
+            "kv_only": {"kernel": "attn_prefill::prefill_kernel (cache only)", "us": us_kv, "TFLOPS": ops / us_kv / 1e6,
+                        "note": "16-bit query and probabilities, quantised key / value cache; tcgen05 kind::f16"},
+            "note": "exact integer products on tcgen05, one accumulator per cluster (the scores are computed twice: the softmax codes need the finished row sums)"}
 
 
 def _e2e_leg(sites, binding, M, n_steps, torch):
