@@ -32,11 +32,12 @@
 // 4 b + 2 y + {0, 1}. It lets the V loader read and write shared memory without bank conflicts.
 //
 // Measured, us, against a mma.sync kernel with 64 (KV: 128) queries per block (72 heads of 128 channels, four clusters each,
-// causal, two sequences of 2048 tokens): 3 bits 2321 -> 772; KV, 32 heads, three sequences, 1100 queries on 1337 keys, 4 bits
-// 945 -> 369. What bounds it is the instruction cache before any pipe: five roles run side by side, and a warp on its own executes
+// causal, two sequences of 2048 tokens): 3 bits 2321 -> 735; KV, 32 heads, three sequences, 1100 queries on 1337 keys, 4 bits
+// 945 -> 342. What bounds it is the instruction cache before any pipe: five roles run side by side, and a warp on its own executes
 // one instruction per 6 to 10 clocks (scheduler slots 48 % busy). Whatever shortens the code that runs at the same time helps
 // more than shortening a chain: the compiler told that the warp index is uniform 916 -> 790 (93 -> 83 KB of code), the output
 // rows' store loops not unrolled 790 -> 772; a first cluster's drain of its own (two copies of the loop) 790 -> 830.
+// The order in which items are dealt out: see item_index (767 -> 730).
 #include <type_traits>
 
 #include "attn_common.cuh"
@@ -54,7 +55,7 @@ using tc::mbar_sleep_warp;
 
 enum { I8 = 0, F8 = 1, KV = 2 };
 // Softmax warps that share a stream's piece of work (and a lane quarter). 2 (sixteen warps of 32 keys a thread) measured the same
-// within 3 % with small code, KV 35 % slower: the loaders then have 56 registers and spill.
+// (773 and 770 us), KV 3 % slower: the loaders then have 56 registers.
 constexpr int SUB = 1;
 constexpr int BM = 128, THREADS = 384 + 256 * SUB;
 constexpr int K_WARP0 = 4, V_WARP0 = 8, S_WARP0 = 12;

@@ -12,7 +12,7 @@
 // Warp roles (per CTA):
 //   warp 0      bulk-copy producer: one contiguous 8 KiB cp.async.bulk per 128 weight rows per K
 //               block (the packed weights are stored tile-major for this) into a ring of stages
-//   warps 4-7   unpack: packed codes -> 8-bit operands, written in the K-major 128-byte-swizzled
+//   warps 4-7   (MODE_DEQ: 4-11, two groups) unpack: packed codes -> 8-bit operands, written in the K-major 128-byte-swizzled
 //               layout that the tensor core reads (weights become 16 * w, see unpack.cuh). The
 //               activation codes of a K block are 48/64/128 bytes per token row, too narrow for the
 //               copy engine to move at speed (measured: ~10 clk per row), so each unpack thread
@@ -29,8 +29,8 @@
 //   warps 2-3   column tables: zero-point correction, s_w and bias of the columns of the tile to come, and
 //               with per-cluster weight parameters the coefficients of each cluster's drain (they are
 //               the same for every token row: formed once per block instead of in every epilogue thread.
-//               1024 x 4096 x 16384, 16 clusters, LayerNorm included: 428 -> 147 us)
-//   warps 8-15  epilogue: drain a finished cluster's accumulator (tcgen05.ld), add s_c * acc into
+//               1024 x 4096 x 16384, 16 clusters, LayerNorm included: 428 -> 147 us, 129 with all that follows)
+//   warps 8-15  (MODE_DEQ: 12-19) epilogue: drain a finished cluster's accumulator (tcgen05.ld), add s_c * acc into
 //               fp32 running sums held in registers while the next cluster's MMAs run; after the
 //               last cluster apply the zero-point correction, s_w, bias, activation, and store
 // Every wait is bounded: a wait that runs out sets RPTQ_ERR_DEVICE_TIMEOUT in the status word and

@@ -39,7 +39,7 @@ namespace smallm {
 constexpr int CONSUMER_WARPS = 16;
 constexpr int TABLE_WARPS = 2;
 constexpr int THREADS = 32 * (CONSUMER_WARPS + 1 + TABLE_WARPS);      // consumers, producer, column tables
-constexpr int SMEM_LIMIT = 223 * 1024;      // dynamic (3.2 KB more are static)
+constexpr int SMEM_LIMIT = 227 * 1024 - 3328;           // dynamic; the static arrays take 3200 bytes
 constexpr int STAGES = 8;
 constexpr int STAGE_BYTES = 16384;          // two 8 KiB weight tiles: K block kb of both 128-row tiles
 constexpr long long WAIT_BUDGET_CYCLES = 4000000000ll;   // about two seconds
