@@ -46,6 +46,7 @@ constexpr int TILE = 32;                       // keys per tile of a warp
 constexpr int STAGES = 3;
 constexpr int MAX_Q = 8;                       // columns of operand B
 constexpr int LIMB_Q = 2;                      // queries of the LIMB mode (columns 4 q + limb)
+constexpr float P_UNITS = 16776192.0f;         // LIMB: 2^24 - 2^10, so that P = 1 stays below 2^24 by more than ex2's error (2^-22)
 constexpr int MAX_CLUSTER = 8;
 constexpr int SCORE_BYTES_MAX = 96 * 1024;     // of the block's keys
 // shared memory of a block besides the dynamic part: the kernel's static arrays and the system's 1 KiB, rounded up
@@ -463,7 +464,6 @@ decode_kernel(const AttnParams p, int keys_block, int units_k_max, int units_v_m
             fq = p.inv_sP / l;
         }
     }
-    if constexpr (MODE == LIMB) mq -= 23.9999f;
 
     // ---------------------------------------------------------------- outputs: V^T times the probabilities
     // Lane (g8, t4) reads word g8 of a pair of units (8 codes: positions 8 g8 .. 8 g8 + 7 of the 64) of keys
@@ -490,12 +490,14 @@ decode_kernel(const AttnParams p, int keys_block, int units_k_max, int units_v_m
         for (int half = 0; half < 2; ++half) {
             const float2 x = *reinterpret_cast<const float2*>(Sq + jt + 16 * half + 2 * t4), y = *reinterpret_cast<const float2*>(Sq + jt + 16 * half + 8 + 2 * t4);
             if constexpr (MODE == LIMB) {
-                // 24-bit integers: P in units of 2^-23.9999 (the row sum counts in the same unit)
+                // 24-bit integers: P in units of 1 / P_UNITS (the row sum counts in the same unit). The maximum is subtracted before the
+                // scaling: folded into the exponent, the shift would be rounded to the maximum's own grid, and from 2^11 on P = 1 would
+                // need a 25th bit
                 uint32_t X[4];
                 const float v[4] = {x.x, x.y, y.x, y.y};
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
-                    const float f = ex2(v[e] - mq);
+                    const float f = ex2(v[e] - mq) * P_UNITS;
                     lsum += f;
                     X[e] = on ? __float2uint_rn(f) : 0u;
                 }
@@ -607,7 +609,7 @@ decode_kernel(const AttnParams p, int keys_block, int units_k_max, int units_v_m
                 const int q = MODE == LIMB ? t4 >> 1 : 2 * t4 + (e & 1), pos = 64 * a + 8 * g8 + b + 4 * (e >> 1);
                 if constexpr (MODE == LIMB) {
                     if (e & 1) continue;
-                    // the three digits' sums (each below 2^31: a block's keys are bounded) as one number, P counted in 2^-24
+                    // the three digits' sums (each below 2^31: a block's keys are bounded) as one number, P counted in 1 / P_UNITS
                     float v = (t4 & 1) ? 65536.0f * (float)O[a][b][e] : __fmaf_rn(256.0f, (float)O[a][b][e + 1], (float)O[a][b][e]);
                     v += __shfl_xor_sync(0xffffffffu, v, 1);
                     if (q < p.Tq && pos < n_pos && (t4 & 1) == 0) red[warp * part + q * n_pos + pos] = __float_as_uint(v);

@@ -186,3 +186,31 @@ def test_query_rows_of_any_width(hd, Tq):
     """Heads whose rows are whole pieces of 16 bytes are staged and permuted in place, others are gathered channel by channel."""
     c = Case(740 + hd, H=2, hd=hd, gh=2, Tq=Tq, Tk=Tq + 61)
     _check(c, _query(np.random.default_rng(hd), Tq, 2 * hd), True)
+
+
+def _rebuild_keys(c, bits):
+    import torch
+    c.dk = torch.from_numpy(oracle.pack(np.ascontiguousarray(c.k[:, c.LK.contiguous_position()]), bits)).cuda()
+
+
+@pytest.mark.parametrize("Tq", [1, 2, 3])
+@pytest.mark.parametrize("q_offset", [300.0, -300.0, 700.0])
+def test_scores_far_from_zero(Tq, q_offset):
+    """An offset of the query that is the same for every key: the scores as the kernel forms them lie near +-2600 (6000) in units
+    of log2 (the row-constant zero-point term is left out), their differences are ordinary. Key positions 2 i and 2 i + 1 hold
+    codes that add up to 15."""
+    c = Case(60, H=2, hd=64, gh=1, Tq=Tq, Tk=300)
+    c.sK[:] = 0.1
+    from paper_2304_01089_b200 import binding
+    c.LK = binding.Layout(c.perm_qk, c.size_qk, c.sK, c.zK, 4)
+    c.k[:, 1::2] = 15 - c.k[:, 0::2]
+    _rebuild_keys(c, 4)
+    q = q_offset + np.round(4 * np.random.default_rng(11).normal(size=(Tq, 128))) / 4
+    _check(c, q.astype(np.float16), True)
+
+
+@pytest.mark.parametrize("Tq", [1, 2])
+def test_scores_far_apart(Tq):
+    """Row maxima of a few thousand (in units of log2): one key has all the weight."""
+    c = Case(61, H=2, hd=64, gh=1, Tq=Tq, Tk=300)
+    _check(c, _query(np.random.default_rng(12), Tq, 128, 1000.0), True)
