@@ -16,10 +16,12 @@
 //             product gives the per-key code sums of the zero-point term;
 //       LIMB  fp16 query, at most two of them: the kernel is bound by the instructions that turn codes into
 //             operands (1.5 per code for fp16 operands, 0.4 for bytes), and a query fills one column of
-//             eight. So the QUERY becomes three signed bytes in three columns: q = X 2^-k, X an integer of
-//             23 bits (exact unless |q| is below 2^-11 of the head's largest), and the sums are exact
-//             integers. The probabilities become three unsigned bytes (24 bits, at least fp16's precision
-//             everywhere);
+//             eight. So the QUERY becomes four signed bytes in four columns: q = X 2^-k, X an integer of 31 bits, with
+//             one k per cluster (exact unless |q| is below 2^-19 of the cluster's largest: then it is off by 2^-32 of
+//             that at most, less than fp32 sums lose), and the sums are exact integers. (Three bytes and one k per
+//             head took the same time, but where a head's clusters differ by 10^4 in the query's magnitude and the keys'
+//             scale undoes that, the small queries kept four bits.) The probabilities become three unsigned bytes (24
+//             bits, at least fp16's precision everywhere);
 //       HALF  fp16 query, three to eight: fp16 operands, m16n8k16. A nibble n moved to mantissa bits 6-9 of
 //             16.0 is 16 + n, one packed addition makes it n - 8 (bytes: 1024 + n, n - 128). The centre is a
 //             constant of the query row in the scores (it cancels in the softmax) and part of the zero
@@ -149,12 +151,13 @@ decode_kernel(const AttnParams p, int keys_block, int units_k_max, int units_v_m
 {
     constexpr bool KV = MODE != INT;
     extern __shared__ __align__(16) uint8_t smem[];
-    __shared__ float s_coef[MAX_UNITS], s_czq[MAX_UNITS];
+    __shared__ float s_coef[MODE == LIMB ? LIMB_Q : 1][MAX_UNITS], s_czq[MAX_UNITS];      // (LIMB: times the 2^-k of the query's cluster)
+    __shared__ uint32_t s_top[LIMB_Q][MAX_UNITS];             // LIMB: the largest |q| of a unit, as fp16 bits
     __shared__ uint8_t s_last[MAX_UNITS];
     __shared__ float s_wm[WARPS][MAX_Q], s_wl[WARPS][MAX_Q];
     __shared__ float s_m[MAX_Q], s_l[MAX_Q];                  // this block's row maxima and sums (read by its peers)
     __shared__ int s_wrs[WARPS][MAX_Q], s_rs[MAX_Q];
-    // the queries in K's position order: fp16 (HALF) or 23-bit integers (LIMB)
+    // the queries in K's position order: fp16 (HALF) or 31-bit integers (LIMB)
     __shared__ __align__(16) uint32_t s_q[MODE == HALF ? MAX_Q * 16 * MAX_UNITS : MODE == LIMB ? LIMB_Q * 32 * MAX_UNITS : 4];
     __shared__ __align__(16) uint32_t s_qb[32 * MAX_UNITS][MODE == HALF ? 4 : 2];
 
@@ -219,17 +222,16 @@ decode_kernel(const AttnParams p, int keys_block, int units_k_max, int units_v_m
     // ---------------------------------------------------------------- the queries, as operand B of every unit
     if (tid < nuk) {
         const float2 k = __ldg(p.unit_sz_k + uk0 + tid);
-        if constexpr (KV) {
-            s_coef[tid] = k.x * p.qk_scale_log2e;
-        } else {
+        if constexpr (MODE == HALF) {
+            s_coef[0][tid] = k.x * p.qk_scale_log2e;
+        } else if constexpr (MODE == INT) {
             const float2 q = __ldg(p.unit_sz_q + uk0 + tid);
             const float c = q.x * k.x * p.qk_scale_log2e;
-            s_coef[tid] = c;
+            s_coef[0][tid] = c;
             s_czq[tid] = -c * q.y;
         }
         s_last[tid] = (tid == nuk - 1) || (__ldg(p.unit_cluster_k + uk0 + tid + 1) != __ldg(p.unit_cluster_k + uk0 + tid));
     }
-    float q_unit[LIMB_Q] = {};                                 // LIMB: 2^-k of each query
     if constexpr (MODE == HALF) {
         __half* sq = reinterpret_cast<__half*>(s_q);
         for (int it = tid; it < p.Tq * 32 * nuk; it += THREADS) {
@@ -237,28 +239,44 @@ decode_kernel(const AttnParams p, int keys_block, int units_k_max, int units_v_m
             sq[q * 32 * MAX_UNITS + pp] = __ldg(p.jidx_k + pos) >= 0 ? p.q_f16[(q_row0 + q) * p.ldq + __ldg(p.src_k + pos)] : __ushort_as_half(0);
         }
     } else if constexpr (MODE == LIMB) {
+        // my positions of the queries: lane of unit warp + 4 k
+        uint32_t raw[LIMB_Q][MAX_UNITS / WARPS];
+#pragma unroll
+        for (int k = 0; k < MAX_UNITS / WARPS; ++k) {
+            const int u = warp + WARPS * k, pos = 32 * (uk0 + u) + lane;
+            const int ch = u < nuk && __ldg(p.jidx_k + pos) >= 0 ? (int)__ldg(p.src_k + pos) : -1;
+#pragma unroll
+            for (int q = 0; q < LIMB_Q; ++q) {
+                raw[q][k] = ch >= 0 && q < p.Tq ? (uint32_t)__half_as_ushort(p.q_f16[(q_row0 + q) * p.ldq + ch]) : 0u;
+                const uint32_t top = __reduce_max_sync(0xffffffffu, raw[q][k] & 0x7FFFu);
+                if (lane == 0) s_top[q][u] = top;
+            }
+        }
+        __syncthreads();
+        const int cl = lane < nuk ? __ldg(p.unit_cluster_k + uk0 + lane) : -1;
+        const float c = lane < nuk ? __ldg(&p.unit_sz_k[uk0 + lane].x) * p.qk_scale_log2e : 0.f;
 #pragma unroll
         for (int q = 0; q < LIMB_Q; ++q) {
-            if (q >= p.Tq) break;
-            const __half* row = p.q_f16 + (q_row0 + q) * p.ldq;
-            float m = 0.f;
-            bool finite = true;
-            for (int c = lane; c < p.hd; c += 32) {
-                const float v = fabsf(__half2float(row[h * p.hd + c]));
-                finite = finite && v <= 65504.0f;
-                m = fmaxf(m, v);
-            }
+            // lane = unit: the largest |q| of its cluster
+            const uint32_t mine = lane < MAX_UNITS ? s_top[q][lane] : 0u;
+            uint32_t top = mine;
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-            // exponent field e of the largest: |q| < 2^(e - 126), so |q| 2^(148 - e) < 2^22
-            const int e = max((__float_as_int(m) >> 23) & 255, 90);
-            // 2^(e - 148); a query that is not finite makes its scores, and so its outputs, not a number
-            q_unit[q] = __all_sync(0xffffffffu, finite) ? __int_as_float((e - 21) << 23) : __int_as_float(0x7FC00000);
-            const float to_int = __int_as_float((275 - e) << 23);
-            int* x = reinterpret_cast<int*>(s_q) + q * 32 * MAX_UNITS;
-            for (int pp = tid; pp < 32 * nuk; pp += THREADS) {
-                const int pos = 32 * uk0 + pp;
-                x[pp] = __ldg(p.jidx_k + pos) >= 0 ? __float2int_rn(__half2float(row[__ldg(p.src_k + pos)]) * to_int) : 0;
+            for (int i = 0; i < MAX_UNITS; ++i) {
+                const uint32_t t = __shfl_sync(0xffffffffu, mine, i);
+                if (__shfl_sync(0xffffffffu, cl, i) == cl) top = max(top, t);
+            }
+            // its exponent field e: |q| < 2^(e - 126), so |q| 2^(156 - e) < 2^30 (no fp16 number is below 2^-24)
+            const bool finite = top < 0x7C00u;
+            const int e = finite ? max(__float_as_int(__half2float(__ushort_as_half((unsigned short)top))) >> 23, 103) : 103;
+            // a query that is not finite makes its scores, and so its outputs, not a number
+            if (warp == 0 && lane < nuk) s_coef[q][lane] = finite ? c * __int_as_float((e - 29) << 23) : __int_as_float(0x7FC00000);
+            const float to_int = finite ? __int_as_float((283 - e) << 23) : 0.f;
+#pragma unroll
+            for (int k = 0; k < MAX_UNITS / WARPS; ++k) {
+                const int u = warp + WARPS * k;
+                const float f = __shfl_sync(0xffffffffu, to_int, u);
+                // (0 times infinity is converted to 0)
+                reinterpret_cast<int*>(s_q)[q * 32 * MAX_UNITS + 32 * u + lane] = __float2int_rn(__half2float(__ushort_as_half((unsigned short)raw[q][k])) * f);
             }
         }
     }
@@ -277,12 +295,12 @@ decode_kernel(const AttnParams p, int keys_block, int units_k_max, int units_v_m
                 b[2] = __byte_perm(v.z, v.w, 0x5410); b[3] = __byte_perm(v.z, v.w, 0x7632);
             }
         } else if constexpr (MODE == LIMB) {
-            // column 4 q + limb: X = d0 + 2^8 d1 + 2^16 d2 with signed bytes d; adding half of every lower digit's
-            // range turns the arithmetic shift into the balanced digit
+            // column 4 q + limb: X = d0 + 2^8 d1 + 2^16 d2 + 2^24 d3 with signed bytes d; adding half of every lower
+            // digit's range turns the arithmetic shift into the balanced digit
             const int q = col >> 2, limb = col & 3;
-            if (q < p.Tq && limb < 3) {
+            if (q < p.Tq) {
                 const int* x = reinterpret_cast<const int*>(s_q) + q * 32 * MAX_UNITS + 32 * u + 8 * w;
-                const int half = limb == 0 ? 0 : limb == 1 ? 128 : 128 + 32768;
+                const int half = limb == 0 ? 0 : limb == 1 ? 128 : limb == 2 ? 128 + 32768 : 128 + 32768 + 8388608;
 #pragma unroll
                 for (int i = 0; i < 8; ++i) b[i >> 2] |= ((uint32_t)((x[i] + half) >> (8 * limb)) & 255u) << (8 * (i & 3));
             }
@@ -320,9 +338,9 @@ decode_kernel(const AttnParams p, int keys_block, int units_k_max, int units_v_m
     // ---------------------------------------------------------------- scores of my keys
     const int off = p.Tk - p.Tq;
     const int q0 = MODE == LIMB ? t4 >> 1 : 2 * t4, q1 = q0 + 1;               // the queries of my columns of the score fragments
-    // LIMB: my two columns' weights (the two lanes of a query hold digits 0, 1 and digit 2)
-    const float qu = q0 == 0 ? q_unit[0] : q_unit[1];
-    const float w0 = (t4 & 1) ? 65536.0f * qu : qu, w1 = (t4 & 1) ? 0.0f : 256.0f * qu;
+    // LIMB: my two columns' weights (the two lanes of a query hold digits 0, 1 and digits 2, 3)
+    const float w0 = (t4 & 1) ? 65536.0f : 1.0f, w1 = (t4 & 1) ? 16777216.0f : 256.0f;
+    const float* coef = s_coef[MODE == LIMB ? q0 : 0];
     const int vis0 = p.causal ? min(p.Tk - 1, q0 + off) : p.Tk - 1, vis1 = p.causal ? min(p.Tk - 1, q1 + off) : p.Tk - 1;
     float m0 = NEG_BIG, m1 = NEG_BIG;
     uint32_t last_mask = 0u;
@@ -372,7 +390,7 @@ decode_kernel(const AttnParams p, int keys_block, int units_k_max, int units_v_m
                     }
                 }
                 if ((last_mask >> u) & 1u) {
-                    const float c = s_coef[u];
+                    const float c = coef[u];
 #pragma unroll
                     for (int half = 0; half < 2; ++half) {
                         if constexpr (MODE == LIMB) {                          // entries 0 and 2: keys g8 and g8 + 8

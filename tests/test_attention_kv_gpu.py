@@ -214,3 +214,19 @@ def test_scores_far_apart(Tq):
     """Row maxima of a few thousand (in units of log2): one key has all the weight."""
     c = Case(61, H=2, hd=64, gh=1, Tq=Tq, Tk=300)
     _check(c, _query(np.random.default_rng(12), Tq, 128, 1000.0), True)
+
+
+@pytest.mark.parametrize("Tq", [1, 2, 3])
+def test_clusters_of_different_magnitudes(Tq):
+    """A head's clusters differ by 10^4 in the query's magnitude and by as much the other way in the keys' scale: the small
+    queries count as much as the large ones."""
+    from paper_2304_01089_b200 import binding
+    c = Case(62, H=2, hd=64, gh=2, Tq=Tq, Tk=300, allow_empty=False)
+    c.sK = np.tile(np.array([1e-3, 30.0], np.float32), 2)
+    c.LK = binding.Layout(c.perm_qk, c.size_qk, c.sK, c.zK, 4)
+    q = np.random.default_rng(13).normal(size=(Tq, 128))
+    at = 0
+    for cl, n in enumerate(c.size_qk):
+        q[:, c.perm_qk[at:at + n]] *= (200.0, 0.02)[cl % 2]
+        at += n
+    _check(c, q.astype(np.float16), True)
