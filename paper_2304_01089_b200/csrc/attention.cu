@@ -43,6 +43,6 @@ extern "C" int rptq_attention(const rptq_layout_t* LQ, const rptq_layout_t* LK, 
     auto st = static_cast<cudaStream_t>(stream);
     const int n_sm = sm_count(dev);
     if (n_sm == 0) return RPTQ_ERR_CUDA;
-    if (attn_decode::fits(p, false)) return attn_decode::launch(p, false, units_k, units_v, n_seq, dev, n_sm, st);
+    if (attn_decode::fits(p, false, units_k, units_v)) return attn_decode::launch(p, false, units_k, units_v, n_seq, dev, n_sm, st);
     return attn_prefill::launch(p, false, LQ->z_min, LQ->z_max, units_k, units_v, n_seq, heads_own_their_channels(LV, n_heads), dev, n_sm, st);
 }

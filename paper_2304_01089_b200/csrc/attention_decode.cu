@@ -53,6 +53,8 @@ constexpr int MAX_CLUSTER = 8;
 constexpr int SCORE_BYTES_MAX = 96 * 1024;     // of the block's keys
 // shared memory of a block besides the dynamic part: the kernel's static arrays and the system's 1 KiB, rounded up
 constexpr int static_smem(bool half_mode) { return half_mode ? 10 * 1024 : 6 * 1024; }
+constexpr int SM_BYTES = 227 * 1024;                          // shared memory of an SM that blocks can have
+constexpr int dynamic_smem_max(bool half_mode) { return SM_BYTES - static_smem(half_mode); }
 
 __device__ __forceinline__ void mma_u8(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
 {
@@ -697,17 +699,26 @@ decode_kernel(const AttnParams p, int keys_block, int units_k_max, int units_v_m
 // 72 pairs 44 / 25 / 19 / 25, 12 pairs 44 / 25 / 16 / 12, 576 pairs of 300 keys 20 / 27 / 45 / 82; 3 bits (three blocks
 // per SM), 576 pairs of 2011 keys 131 / 109 / 125 / 173.
 constexpr int FIXED_KEYS = 400;
+static int keys_of_split(int Tk, int n_ranks) { return ((Tk + n_ranks - 1) / n_ranks + TILE - 1) / TILE * TILE; }
+// Dynamic shared memory of a block with `keys` keys; 0 where it or the scores are more than a block may have. (The largest, eight
+// units of 8 bits in one tensor and of 3 bits in the other: 104448 bytes of rings, 18432 to expand, 98304 of scores.)
+static int smem_of_split(const AttnParams& p, bool half_mode, int units_k, int units_v, int keys)
+{
+    if ((int64_t)p.Tq * (keys + 8) * 4 > SCORE_BYTES_MAX) return 0;
+    const int bytes = smem_plan(p.bits_k, p.bits_v, units_k, units_v, p.Tq, keys).total;
+    return bytes <= dynamic_smem_max(half_mode) ? bytes : 0;
+}
+static bool half_mode_of(const AttnParams& p, bool kv) { return kv && p.Tq > LIMB_Q; }
 static bool plan(const AttnParams& p, bool half_mode, int units_k, int units_v, int n_seq, int n_sm, int* n_ranks, int* keys_block, int* smem)
 {
     const int64_t pairs = (int64_t)p.H * n_seq;
     int64_t best = -1;
     for (int c = 1; c <= MAX_CLUSTER; c *= 2) {
-        const int keys = ((p.Tk + c - 1) / c + TILE - 1) / TILE * TILE;
-        if ((int64_t)p.Tq * (keys + 8) * 4 > SCORE_BYTES_MAX) continue;
+        const int keys = keys_of_split(p.Tk, c), bytes = smem_of_split(p, half_mode, units_k, units_v, keys);
+        if (bytes == 0) continue;
         if (c > 1 && keys < WARPS * TILE && best >= 0) break;
-        const int bytes = smem_plan(p.bits_k, p.bits_v, units_k, units_v, p.Tq, keys).total;
-        int per_sm = 227 * 1024 / (bytes + static_smem(half_mode));
-        per_sm = per_sm < 1 ? 1 : per_sm > 4 ? 4 : per_sm;
+        int per_sm = SM_BYTES / (bytes + static_smem(half_mode));
+        per_sm = per_sm > 4 ? 4 : per_sm;
         int64_t slots = (int64_t)n_sm * per_sm;
         if (c >= 4) slots -= slots / 8;                          // clusters of this size do not fill every GPC
         const int64_t waves = (pairs * c + slots - 1) / slots;
@@ -717,10 +728,10 @@ static bool plan(const AttnParams& p, bool half_mode, int units_k, int units_v, 
     return best >= 0;
 }
 
-bool fits(const AttnParams& p, bool kv)
+bool fits(const AttnParams& p, bool kv, int units_k, int units_v)
 {
-    // (the scores of a block's keys must fit when eight blocks share them)
-    return p.Tq <= (kv ? MAX_Q : MAX_Q - 1) && (int64_t)p.Tq * ((p.Tk + MAX_CLUSTER - 1) / MAX_CLUSTER + TILE + 8) * 4 <= SCORE_BYTES_MAX;
+    // (what a block needs must fit when eight blocks share the keys)
+    return p.Tq <= (kv ? MAX_Q : MAX_Q - 1) && smem_of_split(p, half_mode_of(p, kv), units_k, units_v, keys_of_split(p.Tk, MAX_CLUSTER)) > 0;
 }
 
 template <int MODE, int BK, int BV>
@@ -729,7 +740,7 @@ static int launch_one(const AttnParams& p, int units_k, int units_v, int n_seq, 
     int n_ranks = 1, keys_block = 0, smem = 0;
     if (!plan(p, MODE == HALF, units_k, units_v, n_seq, n_sm, &n_ranks, &keys_block, &smem)) return RPTQ_ERR_UNSUPPORTED;
     static std::atomic<uint64_t> done{0};
-    if (allow_smem(reinterpret_cast<const void*>(decode_kernel<MODE, BK, BV>), dev, 212 * 1024, done) != RPTQ_OK) return RPTQ_ERR_CUDA;
+    if (allow_smem(reinterpret_cast<const void*>(decode_kernel<MODE, BK, BV>), dev, dynamic_smem_max(MODE == HALF), done) != RPTQ_OK) return RPTQ_ERR_CUDA;
     return launch_kernel(decode_kernel<MODE, BK, BV>, dim3((unsigned)n_ranks, (unsigned)p.H, (unsigned)n_seq), THREADS, (size_t)smem, (unsigned)n_ranks, st,
                          p, keys_block, units_k, units_v);
 }
@@ -743,7 +754,7 @@ int launch(const AttnParams& p, bool kv, int units_k, int units_v, int n_seq, in
         return v8 ? launch_one<MODE, 4, 8>(p, units_k, units_v, n_seq, dev, n_sm, st) : launch_one<MODE, 4, 4>(p, units_k, units_v, n_seq, dev, n_sm, st);
     };
     if (!kv) return pick(std::integral_constant<int, INT>());
-    return p.Tq <= LIMB_Q ? pick(std::integral_constant<int, LIMB>()) : pick(std::integral_constant<int, HALF>());
+    return half_mode_of(p, true) ? pick(std::integral_constant<int, HALF>()) : pick(std::integral_constant<int, LIMB>());
 }
 
 }  // namespace attn_decode

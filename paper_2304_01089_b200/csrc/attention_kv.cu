@@ -39,6 +39,6 @@ extern "C" int rptq_attention_kv(const rptq_layout_t* LK, const rptq_layout_t* L
     auto st = static_cast<cudaStream_t>(stream);
     const int n_sm = sm_count(dev);
     if (n_sm == 0) return RPTQ_ERR_CUDA;
-    if (attn_decode::fits(p, true)) return attn_decode::launch(p, true, units_k, units_v, n_seq, dev, n_sm, st);
+    if (attn_decode::fits(p, true, units_k, units_v)) return attn_decode::launch(p, true, units_k, units_v, n_seq, dev, n_sm, st);
     return attn_prefill::launch(p, true, 0, 0, units_k, units_v, n_seq, heads_own_their_channels(LV, n_heads), dev, n_sm, st);
 }

@@ -115,7 +115,7 @@ inline bool heads_own_their_channels(const rptq_layout_t* L, int n_heads)
 
 // The decode kernel (attention_decode.cu): few queries per sequence, the keys split over a cluster of blocks.
 namespace attn_decode {
-bool fits(const attn::AttnParams& p, bool kv);     // false: the prefill kernel takes the call
+bool fits(const attn::AttnParams& p, bool kv, int units_k, int units_v);     // false: the prefill kernel takes the call
 int launch(const attn::AttnParams& p, bool kv, int units_k, int units_v, int n_seq, int dev, int n_sm, cudaStream_t st);
 }
 // The kernel for more queries (attention_prefill.cu). zq_min, zq_max: the range of the query's zero points (integer calls);

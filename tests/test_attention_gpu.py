@@ -335,3 +335,28 @@ def test_value_heads_that_own_other_channels():
     c.LV = binding.Layout(c.perm_v, c.size_v, c.sV, c.zV, 4)
     c.dv = torch.from_numpy(oracle.pack(np.ascontiguousarray(c.v[:, c.LV.contiguous_position()]), 4)).cuda()
     c.check(True)
+
+
+@pytest.mark.parametrize("bits,Tq,Tk", [((8, 8, 3), 7, 27700), ((8, 3, 8), 7, 27700)])
+def test_few_queries_of_heads_of_eight_units(bits, Tq, Tk):
+    """The most shared memory that the kernel for few queries can need: rings for one tensor's 8-bit rows, room to expand the other's
+    3-bit rows, and the scores of as many keys as a block may have."""
+    Case(970 + Tq, H=2, hd=256, gh=1, Tq=Tq, Tk=Tk, bits=bits).check(True)
+
+
+def test_few_queries_of_many_heads_of_eight_units():
+    """As many (sequence, head) pairs as keep one block for each, with the longest range of keys for a block."""
+    import torch
+    from paper_2304_01089_b200 import binding
+    H, n_seq, Tk = 2, 128, 23550
+    c = Case(979, H=H, hd=256, gh=1, Tq=1, Tk=Tk, bits=(8, 8, 3))
+    rep = lambda t: t.repeat(n_seq, 1)
+    out = torch.empty((n_seq, H * 256), dtype=torch.float16, device="cuda")
+    binding.attention(c.LQ, c.LK, c.LV, H, rep(c.dq), rep(c.dk), rep(c.dv), out, c.s_P, c.qk_scale, True, n_seq=n_seq)
+    one = torch.empty((1, H * 256), dtype=torch.float16, device="cuda")
+    binding.attention(c.LQ, c.LK, c.LV, H, c.dq, c.dk, c.dv, one, c.s_P, c.qk_scale, True)
+    torch.cuda.synchronize()
+    c.check(True)                                       # one sequence against the oracle
+    # (split over blocks or not, a softmax code may differ by one where it lies near a half)
+    vmax = float(c.sV.max()) * 7
+    assert float((out.float() - one.float()).abs().max()) <= 8 * c.s_P * vmax

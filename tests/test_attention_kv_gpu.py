@@ -230,3 +230,11 @@ def test_clusters_of_different_magnitudes(Tq):
         q[:, c.perm_qk[at:at + n]] *= (200.0, 0.02)[cl % 2]
         at += n
     _check(c, q.astype(np.float16), True)
+
+
+@pytest.mark.parametrize("bits,Tq,Tk", [((4, 8, 3), 8, 24000), ((4, 3, 8), 8, 24000), ((4, 8, 3), 1, 23600)])
+def test_few_queries_of_heads_of_eight_units(bits, Tq, Tk):
+    """The most shared memory that the kernel for few queries can need: rings for one cache tensor's 8-bit rows, room to expand the
+    other's 3-bit rows, and the scores of as many keys as a block may have."""
+    c = Case(970 + Tq, H=2, hd=256, gh=1, Tq=Tq, Tk=Tk, bits=bits)
+    _check(c, _query(np.random.default_rng(14), Tq, 512, 0.2), True)
