@@ -17,8 +17,8 @@
  *     throws, aborts or prints.
  *   - "dev" pointers are device global memory of the device that was current when the layout
  *     was created; "host" pointers are ordinary host memory. The caller owns every buffer. The
- *     library allocates device memory only inside rptq_layout_create (small tables) and for one
- *     lazily created status word per device.
+ *     library allocates device memory only inside rptq_layout_create (small tables, and with a
+ *     device's first layout one status word).
  *   - Kernel launches are asynchronous on `stream` (a cudaStream_t passed as void*; NULL is the
  *     default stream). A layout handle is immutable after creation and may be used from several
  *     streams at once.
@@ -245,9 +245,9 @@ int rptq_cluster_gemm_clustered(const rptq_layout_t* Lin, const void* a_codes, i
  * Who needs it: a process whose device memory is owned wholesale by its own pool -- an inference
  * server that reserves the whole GPU at start-up, or a job running under a fixed memory budget --
  * cannot let a library call cudaMalloc behind its back, and code that is recording work on a
- * stream cannot afford a call that allocates on first use. rptq_cluster_gemm does allocate once,
- * lazily (its status word); this entry point never does: it calls no cudaMalloc, cudaFree or
- * allocating library routine.
+ * stream cannot afford a call that allocates on first use. rptq_cluster_gemm reports through the
+ * status word that a device's first layout allocated; this entry point does without it: it calls no
+ * cudaMalloc, cudaFree or allocating library routine.
  * What it uses instead: a table of one float per output column (the zero-point correction
  * sum_c s_c z_c Wsum_c[n], computed by a small kernel on `stream` just before the GEMM) that lives
  * in a static device array of RPTQ_NOALLOC_MAX_N floats. Every device that loads the library

@@ -1152,6 +1152,7 @@ static int launch_one(const AttnParams& p, int zq_min, int zq_max, int units_k, 
     g.q_staged = MODE == KV && p.hd % 8 == 0 && p.ldq % 8 == 0 && aligned16(p.q_f16);
     g.folded = MODE == F8 ? zq_min >= qmax_q - 16 && zq_max <= 16 : MODE == I8 ? zq_min >= qmax_q - 127 && zq_max <= 128 : 0;
     g.status = device_status_word();
+    if (!g.status) return RPTQ_ERR_ALLOC;
     const void* fn = reinterpret_cast<const void*>(prefill_kernel<MODE, K8, V8>);
     static std::atomic<uint64_t> done{0}, pool_ok{0};
     if (!(pool_ok.load(std::memory_order_acquire) >> (dev & 63) & 1u)) {

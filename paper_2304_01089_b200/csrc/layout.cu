@@ -12,8 +12,9 @@
 
 namespace rptq {
 
-// One status word per device, allocated on first use with that device current: a kernel that gives
-// up a wait writes to the word of the device it runs on.
+// One status word per device, allocated with the first layout that is made with that device current (so no later call
+// allocates, and any of them may be the first one under stream capture): a kernel that gives up a wait writes to the word
+// of the device it runs on.
 constexpr int kMaxDevices = 64;
 static std::mutex g_status_mutex;
 static std::atomic<int*> g_status_word[kMaxDevices] = {};
@@ -334,7 +335,8 @@ int rptq_layout_create(rptq_layout_t** out, int C, int g, int bits, const int32_
     }
 
     if (!have_device) { *out = L; return RPTQ_OK; }
-    int rc = upload(&L->d_src, src.data(), src.size());
+    int rc = device_status_word() ? RPTQ_OK : RPTQ_ERR_ALLOC;
+    if (rc == RPTQ_OK) rc = upload(&L->d_src, src.data(), src.size());
     if (rc == RPTQ_OK) rc = upload(&L->d_jidx, jidx.data(), jidx.size());
     if (rc == RPTQ_OK) rc = upload(&L->d_unit, unit.data(), unit.size());
     if (rc == RPTQ_OK) rc = upload(&L->d_step_flags, flags.data(), flags.size());
