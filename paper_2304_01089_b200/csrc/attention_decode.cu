@@ -739,7 +739,7 @@ static int launch_one(const AttnParams& p, int units_k, int units_v, int n_seq, 
 {
     int n_ranks = 1, keys_block = 0, smem = 0;
     if (!plan(p, MODE == HALF, units_k, units_v, n_seq, n_sm, &n_ranks, &keys_block, &smem)) return RPTQ_ERR_UNSUPPORTED;
-    static std::atomic<uint64_t> done{0};
+    static SmemAllowed done;
     if (allow_smem(reinterpret_cast<const void*>(decode_kernel<MODE, BK, BV>), dev, dynamic_smem_max(MODE == HALF), done) != RPTQ_OK) return RPTQ_ERR_CUDA;
     return launch_kernel(decode_kernel<MODE, BK, BV>, dim3((unsigned)n_ranks, (unsigned)p.H, (unsigned)n_seq), THREADS, (size_t)smem, (unsigned)n_ranks, st,
                          p, keys_block, units_k, units_v);

@@ -1154,7 +1154,8 @@ static int launch_one(const AttnParams& p, int zq_min, int zq_max, int units_k, 
     g.status = device_status_word();
     if (!g.status) return RPTQ_ERR_ALLOC;
     const void* fn = reinterpret_cast<const void*>(prefill_kernel<MODE, K8, V8>);
-    static std::atomic<uint64_t> done{0}, pool_ok{0};
+    static SmemAllowed done;
+    static std::atomic<uint64_t> pool_ok{0};
     if (!(pool_ok.load(std::memory_order_acquire) >> (dev & 63) & 1u)) {
         cudaFuncAttributes attr;
         if (cudaFuncGetAttributes(&attr, fn) != cudaSuccess) return RPTQ_ERR_CUDA;

@@ -1152,7 +1152,8 @@ static int launch(const Params& p, int dev, int n_sm, cudaStream_t st)
     const int smem = SL.total + 1024;     // slack for the in-kernel 1024-byte alignment
     const void* fn = reinterpret_cast<const void*>(cluster_gemm_kernel<BITS, NCTA, A8, MODE>);
     static_assert(SL.total + 1024 <= 227 * 1024, "shared memory");
-    static std::atomic<uint64_t> done{0}, pool_ok{0};
+    static SmemAllowed done;
+    static std::atomic<uint64_t> pool_ok{0};
     if (!(pool_ok.load(std::memory_order_acquire) >> (dev & 63) & 1u)) {
         cudaFuncAttributes attr;
         if (cudaFuncGetAttributes(&attr, fn) != cudaSuccess) return RPTQ_ERR_CUDA;

@@ -1,6 +1,8 @@
 // Host side of librptq.so: the layout handle (reorder index S with per-cluster parameters,
 // Sec. 4.1), the offline weight preparation (Sec. 4.2), the packed-format readers and the
 // device status word.
+#include <cuda.h>
+
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -15,7 +17,6 @@ namespace rptq {
 // One status word per device, allocated with the first layout that is made with that device current (so no later call
 // allocates, and any of them may be the first one under stream capture): a kernel that gives up a wait writes to the word
 // of the device it runs on.
-constexpr int kMaxDevices = 64;
 static std::mutex g_status_mutex;
 static std::atomic<int*> g_status_word[kMaxDevices] = {};
 
@@ -32,6 +33,20 @@ int* device_status_word()
         g_status_word[dev].store(p, std::memory_order_release);
     }
     return p;
+}
+
+uint64_t context_id()
+{
+    using GetId = CUresult (*)(CUcontext, unsigned long long*);
+    static const GetId get = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPointByVersion("cuCtxGetId", &fn, 12000, cudaEnableDefault, &found) != cudaSuccess ||
+            found != cudaDriverEntryPointSuccess) fn = nullptr;
+        return reinterpret_cast<GetId>(fn);
+    }();
+    unsigned long long id = 0;
+    return get && get(nullptr, &id) == CUDA_SUCCESS ? id : 0;
 }
 
 int sm_count(int device)

@@ -426,22 +426,23 @@ static KernelFn pick_selftest_kernel(int bits)
 
 // Launch shape of one kernel instance on one device, computed on first use (the attribute and
 // occupancy queries cost more host time than a small launch).
-struct LaunchPlan { const void* fn; int device, T; size_t smem; int blocks; };
+struct LaunchPlan { const void* fn; int device, T; size_t smem; uint64_t context; int blocks; };
 static std::mutex g_plan_mutex;
 static std::vector<LaunchPlan> g_plans;
 
 static int planned_blocks(const void* fn, int device, int T, size_t smem, int* blocks)
 {
+    const uint64_t context = context_id();
     std::lock_guard<std::mutex> lock(g_plan_mutex);
     for (const LaunchPlan& pl : g_plans)
-        if (pl.fn == fn && pl.device == device && pl.T == T && pl.smem == smem) { *blocks = pl.blocks; return RPTQ_OK; }
+        if (pl.fn == fn && pl.device == device && pl.T == T && pl.smem == smem && pl.context == context && context != 0) { *blocks = pl.blocks; return RPTQ_OK; }
     // the attribute belongs to the kernel, not to this plan: always the largest size any plan may ask
     // for, or a later, smaller plan would take the room away from an earlier one that is cached
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) != cudaSuccess) return RPTQ_ERR_CUDA;
     int n_sm = 0, per_sm = 0;
     if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, device) != cudaSuccess) return RPTQ_ERR_CUDA;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, T, smem) != cudaSuccess || per_sm < 1) return RPTQ_ERR_CUDA;
-    g_plans.push_back({fn, device, T, smem, n_sm * per_sm});
+    if (context != 0) g_plans.push_back({fn, device, T, smem, context, n_sm * per_sm});
     *blocks = n_sm * per_sm;
     return RPTQ_OK;
 }

@@ -102,14 +102,21 @@ inline int launch_kernel(void (*fn)(P...), dim3 grid, unsigned threads, size_t s
     return cudaLaunchKernelEx(&cfg, fn, args...) == cudaSuccess ? RPTQ_OK : RPTQ_ERR_CUDA;
 }
 
-// The dynamic shared memory a kernel may ask for, raised once per kernel and device to the most that any launch of it
-// asks for (the runtime call costs about a microsecond of host time). `done`: one bit per device, a static of the caller.
-inline int allow_smem(const void* fn, int device, int bytes, std::atomic<uint64_t>& done)
+constexpr int kMaxDevices = 64;
+// Names the calling thread's current context; no other context of the process ever has the same number. 0 where there is none yet.
+uint64_t context_id();
+
+// The dynamic shared memory a kernel may ask for, raised once per kernel and context (it is an attribute of the kernel in the
+// context: one made after a reset, or beside the first, starts without it) to the most that any launch of it asks for. The
+// runtime call costs about a microsecond of host time. `done`: a static of the caller.
+struct SmemAllowed { std::atomic<uint64_t> context[kMaxDevices]; };
+inline int allow_smem(const void* fn, int device, int bytes, SmemAllowed& done)
 {
-    const uint64_t bit = uint64_t(1) << (device & 63);
-    if (done.load(std::memory_order_acquire) & bit) return RPTQ_OK;
+    const uint64_t id = context_id();
+    const bool known = id != 0 && device >= 0 && device < kMaxDevices;
+    if (known && done.context[device].load(std::memory_order_acquire) == id) return RPTQ_OK;
     if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) return RPTQ_ERR_CUDA;
-    if (device >= 0 && device < 64) done.fetch_or(bit, std::memory_order_release);
+    if (known) done.context[device].store(id, std::memory_order_release);
     return RPTQ_OK;
 }
 

@@ -333,7 +333,7 @@ template <int BITS, int NT>
 static int launch_one(SmallMParams p, int device, cudaStream_t st)
 {
     const int smem = smem_bytes(NT, p.K_pad);
-    static std::atomic<uint64_t> done{0};
+    static SmemAllowed done;
     if (allow_smem(reinterpret_cast<const void*>(small_m_kernel<BITS, NT>), device, SMEM_LIMIT, done) != RPTQ_OK) return RPTQ_ERR_CUDA;
     // a block per 128 channels where the SMs suffice: the call then takes as long as one tile's stream
     const int n_sm = sm_count(device);
