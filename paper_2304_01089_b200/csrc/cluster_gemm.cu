@@ -1346,22 +1346,23 @@ __global__ void noalloc_corr_kernel(const float* __restrict__ cl_sz, const int32
     corr[n] = acc;
 }
 
-// Device address of the scratch array, looked up once per device. In host code the array's name
-// is only a handle for the runtime; the address a kernel can use comes from cudaGetSymbolAddress
-// with that device current.
+// Device address of the scratch array, looked up once per context (each loads the library's code and arrays anew). In host code
+// the array's name is only a handle for the runtime; the address a kernel can use comes from cudaGetSymbolAddress with that
+// device current. One entry per device: the context that called last.
 static int noalloc_scratch(int dev, float** out)
 {
-    constexpr int kMaxDevices = 64;
+    struct Address { uint64_t context; float* p; };
     static std::mutex mu;
-    static float* ptrs[kMaxDevices] = {};
+    static Address known[kMaxDevices] = {};
     if (dev < 0 || dev >= kMaxDevices) return RPTQ_ERR_UNSUPPORTED;
+    const uint64_t id = context_id();
     std::lock_guard<std::mutex> lock(mu);
-    if (!ptrs[dev]) {
+    if (id == 0 || known[dev].context != id) {
         void* p = nullptr;
         if (cudaGetSymbolAddress(&p, g_noalloc_corr) != cudaSuccess || !p) return RPTQ_ERR_CUDA;
-        ptrs[dev] = static_cast<float*>(p);
+        known[dev] = {id, static_cast<float*>(p)};
     }
-    *out = ptrs[dev];
+    *out = known[dev].p;
     return RPTQ_OK;
 }
 

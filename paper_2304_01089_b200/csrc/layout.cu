@@ -14,25 +14,34 @@
 
 namespace rptq {
 
-// One status word per device, allocated with the first layout that is made with that device current (so no later call
-// allocates, and any of them may be the first one under stream capture): a kernel that gives up a wait writes to the word
-// of the device it runs on.
+// One status word per context (a device has one unless the caller makes more), allocated with the first layout that is made in
+// it (so no later call allocates, and any of them may be the first one under stream capture): a kernel that gives up a wait
+// writes to the word of the context it runs in. Entries are only ever added in front, so that looking one up takes no lock.
+struct StatusWord { uint64_t context; int* word; StatusWord* next; };
 static std::mutex g_status_mutex;
-static std::atomic<int*> g_status_word[kMaxDevices] = {};
+static std::atomic<StatusWord*> g_status_words{nullptr};
 
 int* device_status_word()
 {
-    int dev = -1;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return nullptr;
-    if (int* p = g_status_word[dev].load(std::memory_order_acquire)) return p;
-    std::lock_guard<std::mutex> lock(g_status_mutex);
-    int* p = g_status_word[dev].load(std::memory_order_acquire);
-    if (p == nullptr) {
-        if (cudaMalloc(&p, 256) != cudaSuccess) return nullptr;
-        if (cudaMemset(p, 0, 256) != cudaSuccess) { cudaFree(p); return nullptr; }
-        g_status_word[dev].store(p, std::memory_order_release);
+    uint64_t id = context_id();
+    if (id == 0) {                           // a thread that has not used the device yet: its primary context becomes current
+        int dev = -1;
+        if (cudaGetDevice(&dev) != cudaSuccess || cudaSetDevice(dev) != cudaSuccess || (id = context_id()) == 0) return nullptr;
     }
-    return p;
+    auto find = [id]() -> int* {
+        for (const StatusWord* s = g_status_words.load(std::memory_order_acquire); s; s = s->next)
+            if (s->context == id) return s->word;
+        return nullptr;
+    };
+    if (int* word = find()) return word;
+    std::lock_guard<std::mutex> lock(g_status_mutex);
+    if (int* word = find()) return word;
+    int* word = nullptr;
+    if (cudaMalloc(&word, 256) != cudaSuccess) return nullptr;
+    StatusWord* entry = cudaMemset(word, 0, 256) == cudaSuccess ? new (std::nothrow) StatusWord{id, word, g_status_words.load()} : nullptr;
+    if (!entry) { cudaFree(word); return nullptr; }
+    g_status_words.store(entry, std::memory_order_release);
+    return word;
 }
 
 uint64_t context_id()

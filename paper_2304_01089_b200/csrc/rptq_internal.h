@@ -122,7 +122,7 @@ inline int allow_smem(const void* fn, int device, int bytes, SmemAllowed& done)
 
 int sm_count(int device);    // of the device, asked for once; 0 on failure
 
-int* device_status_word();   // the current device's status word (allocated with its first layout), RPTQ_OK when clear; nullptr on failure
+int* device_status_word();   // the current context's status word (allocated with its first layout), RPTQ_OK when clear; nullptr on failure
 
 inline bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
 

@@ -90,10 +90,15 @@ def once():
     ck(lib.rptq_ln_reorder_quant(L.handle, x, 256, ln, ln, 1e-5, 8, codes8, None, None))
     ck(lib.rptq_cluster_gemm(L.handle, codes, M, dw, ds, dws, wsum.shape[1], None, N, 0, None, y, 0, N, None))
     ck(lib.rptq_cluster_gemm(L.handle, codes8, 8, dw, ds, dws, wsum.shape[1], None, N, 0, None, y8, 0, N, None))
+    y_na = up(np.zeros((M, N), np.float32))
+    ck(lib.rptq_cluster_gemm_noalloc(L.handle, codes, M, dw, ds, dws, wsum.shape[1], None, N, 0, None, y_na, 0, N, None))
+    status = C.c_int(1)
+    ck(lib.rptq_get_device_status(C.byref(status)))
+    assert status.value == 0
     o, o8 = up(np.zeros((M, 256), np.float16)), up(np.zeros((4, 256), np.float16))
     ck(lib.rptq_attention(L.handle, L.handle, L.handle, 2, codes, M, codes, codes, M, 1, 1 / 256, 0, 0.05, 1, o, 256, None, None))
     ck(lib.rptq_attention(L.handle, L.handle, L.handle, 2, codes8, 4, codes, codes, M, 1, 1 / 256, 0, 0.05, 1, o8, 256, None, None))
-    return [down(p) for p in (codes, y, y8, o, o8)]
+    return [down(p) for p in (codes, y, y8, y_na, o, o8)]
 ck(cu.cuInit(0))
 dev, ctx = C.c_int(), C.c_void_p()
 ck(cu.cuDeviceGet(C.byref(dev), 0))
