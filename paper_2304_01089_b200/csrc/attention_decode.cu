@@ -312,14 +312,14 @@ decode_kernel(const AttnParams p, int keys_block, int units_k_max, int units_v_m
             const uint8_t* row = p.q + (q_row0 + col) * p.q_row_bytes;
             const int unit = uk0 + u;
             if (p.bits_q == 8) {
-                const uint2 v = __ldg(reinterpret_cast<const uint2*>(row + 32 * unit) + w);
+                const uint2 v = reinterpret_cast<const uint2*>(row + 32 * unit)[w];
                 b[0] = v.x; b[1] = v.y;
             } else if (p.bits_q == 4) {
-                const uint32_t v = __ldg(reinterpret_cast<const uint32_t*>(row + 16 * unit) + w);
+                const uint32_t v = reinterpret_cast<const uint32_t*>(row + 16 * unit)[w];
                 b[0] = v & 0x0F0F0F0Fu; b[1] = (v >> 4) & 0x0F0F0F0Fu;
             } else {
                 const uint32_t* v = reinterpret_cast<const uint32_t*>(row + 12 * unit);
-                const uint32_t q3[3] = {__ldg(v), __ldg(v + 1), __ldg(v + 2)};
+                const uint32_t q3[3] = {v[0], v[1], v[2]};
                 uint32_t o[8];
                 unpack_act32<3>(q3, o);
                 b[0] = w == 0 ? o[0] : w == 1 ? o[2] : w == 2 ? o[4] : o[6];

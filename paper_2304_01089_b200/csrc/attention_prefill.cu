@@ -479,8 +479,8 @@ prefill_kernel(const AttnParams p, const Plan g)
                             if (cb[k] >= 0) y = lds16(row + cb[k]);
                         } else if (r4 + rr < rows) {          // (layouts whose heads share channels, rows without alignment)
                             const uint16_t* row = reinterpret_cast<const uint16_t*>(q_rows) + (r4 + rr) * p.ldq;
-                            if (ca[k] >= 0) x = __ldg(row + ca[k]);
-                            if (cb[k] >= 0) y = __ldg(row + cb[k]);
+                            if (ca[k] >= 0) x = row[ca[k]];
+                            if (cb[k] >= 0) y = row[cb[k]];
                         }
                         v[rr][k] = x | ((uint32_t)y << 16);
                     }

@@ -51,26 +51,8 @@ __device__ __forceinline__ uint32_t pack_half2(float a, float b)
     return *reinterpret_cast<const uint32_t*>(&h);
 }
 
-// Unit `unit` of a packed row in global memory as 32 bytes.
+// Unit `unit` of a packed row (`row` 4-byte aligned for 3-bit codes, 16-byte aligned otherwise) as 32 bytes.
 __device__ __forceinline__ void load_unit(const uint8_t* row, int unit, int bits, uint32_t (&o)[8])
-{
-    if (bits == 4) {
-        const uint4 t = __ldg(reinterpret_cast<const uint4*>(row) + unit);
-        const uint32_t p[4] = {t.x, t.y, t.z, t.w};
-        unpack_act32<4>(p, o);
-    } else if (bits == 3) {
-        const uint32_t* w = reinterpret_cast<const uint32_t*>(row) + unit * 3;
-        const uint32_t p[3] = {__ldg(w), __ldg(w + 1), __ldg(w + 2)};
-        unpack_act32<3>(p, o);
-    } else {
-        const uint4* w = reinterpret_cast<const uint4*>(row) + unit * 2;
-        const uint4 a = __ldg(w), b = __ldg(w + 1);
-        o[0] = a.x; o[1] = a.y; o[2] = a.z; o[3] = a.w; o[4] = b.x; o[5] = b.y; o[6] = b.z; o[7] = b.w;
-    }
-}
-// The same from a staged copy of the packed row in shared memory (`row` points at the head's first unit;
-// 4-byte aligned for 3-bit codes, 16-byte aligned otherwise).
-__device__ __forceinline__ void load_unit_smem(const uint8_t* row, int unit, int bits, uint32_t (&o)[8])
 {
     if (bits == 4) {
         const uint4 t = *(reinterpret_cast<const uint4*>(row) + unit);

@@ -585,7 +585,7 @@ cluster_gemm_kernel(const Params p)
             } else if constexpr (!DEQ) {
                 if (p.corr) {
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) if (n + e < p.N) corr[e] = __ldg(p.corr + n + e);
+                    for (int e = 0; e < 4; ++e) if (n + e < p.N) corr[e] = p.corr[n + e];
                 } else if (vec) {
 #pragma unroll 4
                     for (int c = 0; c < p.g; ++c) {
@@ -943,7 +943,7 @@ cluster_gemm_kernel(const Params p)
             const int32_t* xs_row = nullptr;
             int xs_next = 0;
             if constexpr (ASYM) {
-                if (m0 + 32 * q + lane < p.M) { xs_row = p.xsum + (int64_t)(m0 + 32 * q + lane) * p.g; xs_next = __ldg(xs_row + s_seg_cl[0]); }
+                if (m0 + 32 * q + lane < p.M) { xs_row = p.xsum + (int64_t)(m0 + 32 * q + lane) * p.g; xs_next = xs_row[s_seg_cl[0]]; }
             }
             for (int sgi = 0; sgi < (DEQ ? 1 : p.n_seg); ++sgi) {
                 const uint32_t buf = DEQ ? (n_tile_done & 1u) : (uint32_t)s_seg_buf[sgi];
@@ -960,7 +960,7 @@ cluster_gemm_kernel(const Params p)
                     ++n_seg_done;
                     const float x = (float)xs_next;
                     xs2 = make_float2(x, x);
-                    if (xs_row && sgi + 1 < p.n_seg) xs_next = __ldg(xs_row + s_seg_cl[sgi + 1]);
+                    if (xs_row && sgi + 1 < p.n_seg) xs_next = xs_row[s_seg_cl[sgi + 1]];
                 }
                 const uint32_t taddr = tmem_base + ((uint32_t)(32 * q) << 16) + buf * TILE_N + h * half_cols;
                 if (live && !DEQ) {

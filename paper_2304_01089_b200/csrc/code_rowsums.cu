@@ -10,7 +10,7 @@ namespace rptq {
 
 template <int BITS>
 __global__ void __launch_bounds__(128)
-code_rowsums_kernel(const uint8_t* __restrict__ codes, int64_t row_bytes, int n_units,
+code_rowsums_kernel(const uint8_t* codes, int64_t row_bytes, int n_units,
                     const int32_t* __restrict__ unit_cluster, int g, int32_t* __restrict__ xsum)
 {
     extern __shared__ int32_t s_sum[];
@@ -24,7 +24,7 @@ code_rowsums_kernel(const uint8_t* __restrict__ codes, int64_t row_bytes, int n_
         if (c < 0) continue;
         uint32_t p[BITS], o[8];
 #pragma unroll
-        for (int i = 0; i < BITS; ++i) p[i] = __ldg(row + u * BITS + i);
+        for (int i = 0; i < BITS; ++i) p[i] = row[u * BITS + i];
         unpack_act32<BITS>(p, o);
         int s = 0;
 #pragma unroll

@@ -79,7 +79,9 @@ int launch(const SmallMParams& p, int bits, int device, cudaStream_t st);
 // Programmatic dependent launch: every kernel of the library is launched so that its blocks may become resident, and
 // run their set-up, while the kernel before it in the stream drains. pdl_wait() returns when that kernel has
 // completed and its writes are visible; nothing but the layout's own tables (uploaded before rptq_layout_create
-// returned) is touched before it. pdl_trigger() lets the next kernel's blocks come in. A LayerNorm + GEMM pair of one token:
+// returned) is touched before it. The kernel before may still be writing while this one is resident, so what a kernel of the
+// library writes (codes, outputs, code sums, the no-alloc correction) is read with ordinary loads: the read-only path (__ldg, const
+// __restrict__ arguments) is for what nothing writes while the kernel lives, the layout's tables and the weights'. pdl_trigger() lets the next kernel's blocks come in. A LayerNorm + GEMM pair of one token:
 // 10.9 -> 10.0 us on the device, a LayerNorm launch 3.8 -> 2.7 us.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }

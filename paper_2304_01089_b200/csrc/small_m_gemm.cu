@@ -162,7 +162,7 @@ small_m_kernel(const SmallMParams p, const __grid_constant__ CUtensorMap w_map)
         float corr[4] = {0.f, 0.f, 0.f, 0.f};
         if (p.corr) {
 #pragma unroll
-            for (int e = 0; e < 4; ++e) if (n + 32 * e < p.N) corr[e] = __ldg(p.corr + n + 32 * e);
+            for (int e = 0; e < 4; ++e) if (n + 32 * e < p.N) corr[e] = p.corr[n + 32 * e];
         } else {
 #pragma unroll 4
             for (int c = 0; c < p.g; ++c) {
@@ -200,7 +200,7 @@ small_m_kernel(const SmallMParams p, const __grid_constant__ CUtensorMap w_map)
                     const int u = u0 + k * 32 * SPLIT;
                     const bool in = r < p.M && u < p.n_units;
 #pragma unroll
-                    for (int e = 0; e < BITS; ++e) q[k][e] = in ? __ldg(row + u * BITS + e) : 0u;
+                    for (int e = 0; e < BITS; ++e) q[k][e] = in ? row[u * BITS + e] : 0u;
                 }
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {

@@ -278,3 +278,32 @@ def test_the_layernorm_kernels_hot_instances_do_not_spill(tmp_path):
     # the plain instances (no debug output, no self-test): 3- and 8-bit spill nothing, 4-bit at most one register
     assert spills[(3, False, False)] == (0, 0) and spills[(8, False, False)] == (0, 0)
     assert spills[(4, False, False)][0] <= 8 and spills[(4, False, False)][1] <= 8
+
+
+CSRC = os.path.join(ROOT, "paper_2304_01089_b200", "csrc")
+
+
+def test_only_tables_and_weights_are_read_through_the_read_only_path():
+    """A kernel of the library may be resident while the one before it in the stream still writes (programmatic dependent launch). Loads
+    through the read-only path (ld.global.nc: __ldg, or any load from a const __restrict__ argument) are only defined for memory
+    that nothing writes during the kernel, so they are kept to the layout's tables and the weights' tables."""
+    tables = {"cl_unit0_k", "cl_unit0_v", "unit_sz_q", "unit_sz_k", "unit_sz_v", "unit_cluster_k", "unit_cluster", "jidx_k", "jidx_v", "src_k", "src_v",
+              "unit_sz", "step_flags", "out_unit", "unit_tab", "ch_tab", "jidx_tab", "seg_scale", "cl_sz", "cl_n",
+              "sw_c", "zw_c", "s_w", "wsum", "bias", "gamma", "beta"}
+    aliases = {"u": "cl_unit0_k", "sp": "ch_tab"}                        # locals that point into a table
+    seen = 0
+    for name in sorted(os.listdir(CSRC)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+        for m in re.finditer(r"__ldg\(", text):
+            depth, end = 1, m.end()
+            while depth:
+                depth += {"(": 1, ")": -1}.get(text[end], 0)
+                end += 1
+            arg = text[m.end():end - 1]
+            first = [w for w in re.findall(r"[A-Za-z_]\w*", re.sub(r"reinterpret_cast<[^>]*>", "", arg)) if w != "p"][0]
+            assert aliases.get(first, first) in tables, (name, arg)
+            seen += 1
+        if "launch_kernel(" in text:                                     # kernels that are launched as dependents
+            for m in re.finditer(r"const\s+\w+\s*\*\s*__restrict__\s+(\w+)", text):
+                assert m.group(1) in tables, (name, m.group(0))
+    assert seen > 30
