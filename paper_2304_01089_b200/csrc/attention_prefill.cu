@@ -50,7 +50,6 @@ namespace attn_prefill {
 using namespace attn;
 using tc::mbar_arrive;
 using tc::mbar_init;
-using tc::mbar_sleep;
 using tc::mbar_sleep_warp;
 
 enum { I8 = 0, F8 = 1, KV = 2 };
@@ -453,7 +452,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                 ca[k] = place(pos);
                 cb[k] = place(pos + 2);
             }
-            if (!mbar_sleep(bar(B_QEMPTY), (n_item & 1) ^ 1, s_abort)) return false;
+            if (!mbar_sleep_warp(bar(B_QEMPTY), (n_item & 1) ^ 1, s_abort)) return false;
             if (g.q_staged) {
                 const int per_row = p.hd / 8;                 // 16-byte chunks
 #pragma unroll 1
@@ -512,7 +511,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                 if (ahead ? have : n > 0) {
                     if constexpr (direct) {
                         // (copied into the operand tile itself: its products must have read it)
-                        if (!mbar_sleep(bar(B_KEMPTY + (n & 1)), ((n >> 1) & 1) ^ 1, s_abort)) { ok = false; break; }
+                        if (!mbar_sleep_warp(bar(B_KEMPTY + (n & 1)), ((n >> 1) & 1) ^ 1, s_abort)) { ok = false; break; }
                         const uint32_t to = base + g.off_k + (n & 1) * g.k_stage;
                         copy_rows(nx, [&](int r, int c) { return to + (c >> 3) * K_ATOM + r * 128 + (((c & 7) ^ (r & 7)) << 4); });
                     } else {
@@ -537,7 +536,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                                 const float2 q = __ldg(p.unit_sz_q + cu.u0 + lane), k = __ldg(p.unit_sz_k + cu.u0 + lane);
                                 czq = -(q.x * k.x * p.qk_scale_log2e) * q.y;
                             }
-                            if (!mbar_sleep(bar(B_QEMPTY), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
+                            if (!mbar_sleep_warp(bar(B_QEMPTY), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
 #pragma unroll 2
                             for (int u = 0; u < nu; ++u) {
                                 uint32_t o[8] = {0, 0, 0, 0, 0, 0, 0, 0};
@@ -571,7 +570,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                     }
                     if (ahead && have) cp_async_wait<1>(); else cp_async_wait<0>();
                     __syncwarp();                                              // (a warp unpacks the rows that it copied)
-                    if (!direct && !mbar_sleep(bar(B_KEMPTY + st), (ph & 1) ^ 1, s_abort)) { ok = false; break; }
+                    if (!direct && !mbar_sleep_warp(bar(B_KEMPTY + st), (ph & 1) ^ 1, s_abort)) { ok = false; break; }
                     const uint32_t raw0 = base + g.off_rawk + (ahead ? (m & 1) * g.rawk_stage : 0) + ((4 * p.bits_k * cu.u0) & 15);
                     if constexpr (MODE == KV) {
                         // thread = (row, parity of the unit)
@@ -653,7 +652,7 @@ prefill_kernel(const AttnParams p, const Plan g)
             auto group_sync = [&]() {
                 __syncwarp();
                 if (lane == 0) mbar_arrive(bar(B_XV));
-                const bool done = mbar_sleep(bar(B_XV), n_x & 1, s_abort);
+                const bool done = mbar_sleep_warp(bar(B_XV), n_x & 1, s_abort);
                 ++n_x;
                 return done;
             };
@@ -667,7 +666,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                     const uint32_t st = g.v_stages == 2 ? n_v & 1 : 0u, ph = g.v_stages == 2 ? (n_v >> 1) & 1 : n_v & 1;
                     cp_async_wait<0>();
                     if (!group_sync()) { ok = false; break; }                  // everyone's copies of the tile have landed
-                    if (!mbar_sleep(bar(B_VEMPTY + st), ph ^ 1, s_abort)) { ok = false; break; }
+                    if (!mbar_sleep_warp(bar(B_VEMPTY + st), ph ^ 1, s_abort)) { ok = false; break; }
                     const uint32_t tile = base + g.off_v + st * g.v_stage;
                     if constexpr (MODE == KV) {
                         // lane = (chunk c8 of the 64 slots, word j of the unit). Chunk c8 = 2 blk + y holds the pairs b = 0..3 of keys
@@ -797,8 +796,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                     const int pos = 32 * (uv0 + u) + lane;
                     chs[u] = u < nuv && __ldg(p.jidx_v + pos) >= 0 ? (int)__ldg(p.src_v + pos) : -1;
                 }
-                if (!mbar_sleep(bar(B_SUM), n_item & 1, s_abort) || !mbar_sleep(bar(B_OFULL), n_item & 1, s_abort)) { ok = false; break; }
-                __syncwarp();
+                if (!mbar_sleep_warp(bar(B_SUM), n_item & 1, s_abort) || !mbar_sleep_warp(bar(B_OFULL), n_item & 1, s_abort)) { ok = false; break; }
                 tc::tc_fence_after();
                 const int row = 32 * lw + lane, i0 = it.qt * BM, i = i0 + row;
                 const bool live = i0 + 32 * lw < p.Tq;                         // some row of my warp exists
@@ -928,7 +926,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                     ml[part * BM] = make_float2(m, l);
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(B_XS));
-                    if (!mbar_sleep(bar(B_XS), n_item & 1, s_abort)) { ok = false; break; }
+                    if (!mbar_sleep_warp(bar(B_XS), n_item & 1, s_abort)) { ok = false; break; }
 #pragma unroll
                     for (int q = 0; q < PARTS; ++q) m = fmaxf(m, ml[q * BM].x);
                     if constexpr (MODE != KV) {
@@ -947,8 +945,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                     uint32_t left = last;                                      // (at least one bit)
                     do {
                         const float c = __shfl_sync(0xffffffffu, coef, __ffs(left) - 1);
-                        if (!mbar_sleep(b_full0 + 8 * slot, par, s_abort)) { ok = false; break; }
-                        __syncwarp();
+                        if (!mbar_sleep_warp(b_full0 + 8 * slot, par, s_abort)) { ok = false; break; }
                         tc::tc_fence_after();
                         if (live) {
                             uint32_t v[32];
@@ -1022,11 +1019,11 @@ prefill_kernel(const AttnParams p, const Plan g)
                         continue;
                     }
                     // ---- pass 2: probabilities. P's region also stages the previous item's output
-                    if (kt < 2 && !mbar_sleep(bar(B_OUT), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
+                    if (kt < 2 && !mbar_sleep_warp(bar(B_OUT), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
                     // the buffer's previous tile has been multiplied
                     // (one buffer for both streams: stream 1's first tile waits for stream 0's)
                     const uint32_t behind = ALT && g.p_tiles == 1 && stream == 1 ? 0u : 1u;
-                    if (!mbar_sleep(bar(B_PEMPTY + stream), (n_s & 1) ^ behind, s_abort)) { ok = false; break; }
+                    if (!mbar_sleep_warp(bar(B_PEMPTY + stream), (n_s & 1) ^ behind, s_abort)) { ok = false; break; }
                     ++n_s;
                     if (live) {
                         const float2 nm = make_float2(-m, -m);
@@ -1090,7 +1087,7 @@ prefill_kernel(const AttnParams p, const Plan g)
             }
             if (!ok) break;
             // (a stream without a tile of its own has not waited for the previous item's sums to be read)
-            if (ALT && it.n_kt == 1 && !mbar_sleep(bar(B_OUT), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
+            if (ALT && it.n_kt == 1 && !mbar_sleep_warp(bar(B_OUT), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
             s_sum[part * BM + row] = MODE == KV ? __float_as_uint(lsum) : rsum;
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(B_SUM));

@@ -41,35 +41,32 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity)
         : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
     return ok != 0;
 }
-// Bounded wait for kernels with many waiting warps: sleeps in the barrier instruction instead of polling it. The limit is a
-// number of wake-ups (each at most about a microsecond: two seconds in all). One block of PTX, because a call site then takes
-// half a dozen instructions: kernels with many roles are short of instruction cache.
-__device__ __forceinline__ bool mbar_sleep(uint32_t bar, uint32_t parity, volatile int* abort_flag)
+// Bounded wait of a whole warp, for kernels with many waiting warps: sleeps in the barrier instruction instead of polling it. The
+// limit is a number of wake-ups (each at most about a microsecond: two seconds in all). Every lane leaves with the same answer, or
+// the lanes for which the barrier completed would wait for ever, at the next instruction that the whole warp takes part in, for
+// those that gave up. One block of PTX, because a call site then takes half a dozen instructions: kernels with many roles
+// are short of instruction cache.
+__device__ __forceinline__ bool mbar_sleep_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag)
 {
     uint32_t ok;
     asm volatile(
-        "{\n\t.reg .pred p;\n\t.reg .b32 n, f;\n\t"
-        "mov.b32 %0, 1;\n\tmov.b32 n, 0;\n\t"
+        "{\n\t.reg .pred p, q;\n\t.reg .b32 n, f;\n\t"
+        "mov.b32 n, 0;\n\t"
         "again:\n\t"
         "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, 1000;\n\t"
         "@p bra done;\n\t"
         "ld.volatile.shared.b32 f, [%3];\n\t"
-        "setp.ne.b32 p, f, 0;\n\t"
-        "@p bra failed;\n\t"
+        "setp.ne.b32 q, f, 0;\n\t"
+        "@q bra done;\n\t"
         "add.u32 n, n, 1;\n\t"
-        "setp.lt.u32 p, n, 2097152;\n\t"
-        "@p bra again;\n\t"
+        "setp.lt.u32 q, n, 2097152;\n\t"
+        "@q bra again;\n\t"
         "st.volatile.shared.b32 [%3], 1;\n\t"
-        "failed:\n\t"
-        "mov.b32 %0, 0;\n\t"
-        "done:\n\t}"
-        : "=&r"(ok) : "r"(bar), "r"(parity), "r"(smem_u32(const_cast<const int*>(abort_flag))) : "memory");
+        "done:\n\t"
+        "vote.sync.all.pred p, p, 0xffffffff;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok) : "r"(bar), "r"(parity), "r"(smem_u32(const_cast<const int*>(abort_flag))) : "memory");
     return ok != 0;
-}
-// For a whole warp that must stay converged: every lane leaves with the same answer.
-__device__ __forceinline__ bool mbar_sleep_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag)
-{
-    return __all_sync(0xffffffffu, mbar_sleep(bar, parity, abort_flag));
 }
 // Bounded wait. Returns false when the budget ran out or another role already gave up. The common
 // case (the phase has already completed, or completes within a few polls) touches no timer; the

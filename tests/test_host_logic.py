@@ -307,3 +307,31 @@ def test_only_tables_and_weights_are_read_through_the_read_only_path():
             for m in re.finditer(r"const\s+\w+\s*\*\s*__restrict__\s+(\w+)", text):
                 assert m.group(1) in tables, (name, m.group(0))
     assert seen > 30
+
+
+def _block_end(text, start):
+    """Index behind the brace that closes the block that opens at or behind `start`."""
+    depth, i = 0, text.index("{", start)
+    while True:
+        depth += {"{": 1, "}": -1}.get(text[i], 0)
+        i += 1
+        if depth == 0:
+            return i
+
+
+@pytest.mark.parametrize("name", ["attention_prefill.cu"])
+def test_waits_of_whole_warps_are_voted(name):
+    """A bounded wait that gives up in some lanes of a warp while its barrier completes for the others must not part them: those that
+    go on would wait for ever at the next instruction that the whole warp takes part in. So warps wait through the voting forms
+    (mbar_*_warp); the per-lane forms are for blocks that one lane executes, and for the last wait of a role that has given up
+    already, whose answer nobody asks for."""
+    text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
+    one_lane = [(m.start(), _block_end(text, m.end())) for m in re.finditer(r"if \(lane == 0\)(?=\s*\{)", text)]
+    voted = 0
+    for m in re.finditer(r"\bmbar_(sleep|wait)(_warp)?\(", text):
+        if m.group(2):
+            voted += 1
+            continue
+        line = text[text.rfind("\n", 0, m.start()):text.index("\n", m.start())]
+        assert any(a < m.start() < b for a, b in one_lane) or "B_DRAIN" in line, line
+    assert voted > 0
