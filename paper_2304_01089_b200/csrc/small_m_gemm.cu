@@ -31,6 +31,7 @@
 #include <cuda_fp16.h>
 
 #include "rptq_internal.h"
+#include "tc.cuh"
 #include "unpack.cuh"
 
 namespace rptq {
@@ -42,34 +43,8 @@ constexpr int THREADS = 32 * (CONSUMER_WARPS + 1 + TABLE_WARPS);      // consume
 constexpr int SMEM_LIMIT = 227 * 1024 - 3328;           // dynamic; the static arrays take 3200 bytes
 constexpr int STAGES = 8;
 constexpr int STAGE_BYTES = 16384;          // two 8 KiB weight tiles: K block kb of both 128-row tiles
-constexpr long long WAIT_BUDGET_CYCLES = 4000000000ll;   // about two seconds
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-__device__ __forceinline__ bool mbar_try_wait_for(uint32_t bar, uint32_t parity, uint32_t ns)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity), "r"(ns) : "memory");
-    return ok != 0;
-}
-// Bounded wait: false when the budget ran out or another wait of the block already gave up.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag)
-{
-    if (mbar_try_wait_for(bar, parity, 0u)) return true;
-    const long long t0 = clock64();
-    while (true) {
-        if (mbar_try_wait_for(bar, parity, 2000u)) return true;
-        if (*abort_flag) return false;
-        if (clock64() - t0 > WAIT_BUDGET_CYCLES) { *abort_flag = 1; return false; }
-    }
-}
-__device__ __forceinline__ void mbar_arrive(uint32_t bar)
-{
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
-}
+using namespace tc;
 
 __device__ __forceinline__ void mma_s8u8(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3, uint32_t b0, uint32_t b1)
 {
@@ -150,9 +125,7 @@ small_m_kernel(const SmallMParams p, const __grid_constant__ CUtensorMap w_map)
             // After a give-up the consumers no longer wait for the copies still in flight: they must have
             // landed before the block's shared memory goes away (bounded like every other wait).
             if (*s_abort) {
-                const long long t0 = clock64();
-                for (int kb = issued > STAGES ? issued - STAGES : 0; kb < issued; ++kb)
-                    while (!mbar_try_wait_for(full0 + 8 * (kb % STAGES), (uint32_t)(kb / STAGES) & 1u, 2000u) && clock64() - t0 <= WAIT_BUDGET_CYCLES) {}
+                for (int kb = issued > STAGES ? issued - STAGES : 0; kb < issued; ++kb) mbar_wait(full0 + 8 * (kb % STAGES), (uint32_t)(kb / STAGES) & 1u, s_abort, false);
             }
         }
     } else if (warp > CONSUMER_WARPS) {
@@ -230,7 +203,8 @@ small_m_kernel(const SmallMParams p, const __grid_constant__ CUtensorMap w_map)
             uint4 B[NT];
 #pragma unroll
             for (int nt = 0; nt < NT; ++nt) B[nt] = *reinterpret_cast<const uint4*>(arow + 8 * nt * a_pitch + 64 * kb);
-            if (!mbar_wait(full0 + 8 * s, (uint32_t)(kb / STAGES) & 1u, s_abort)) break;
+            // (when a wait has given up, the remaining K blocks multiply what lies in the ring, and nothing is written out)
+            mbar_sleep_or_abort(full0 + 8 * s, (uint32_t)(kb / STAGES) & 1u, s_abort);
             __syncwarp();
             if (!active) {
                 if (lane == 0) mbar_arrive(empty0 + 8 * s);
@@ -278,7 +252,7 @@ small_m_kernel(const SmallMParams p, const __grid_constant__ CUtensorMap w_map)
 
         // -------------------------------------------------------- epilogue: y = s_w (R - corr) + bias
         asm volatile("bar.sync 2, %0;" ::"n"(32 * (CONSUMER_WARPS + TABLE_WARPS)) : "memory");
-        if (active && n0 < p.N && !*s_abort) {
+        if (active && n0 < p.N && !__any_sync(0xffffffffu, *s_abort)) {
             const float corr = s_col[0][n0 - 128 * tileA + (lane & 15)], sw = s_col[1][n0 - 128 * tileA + (lane & 15)], bs = s_col[2][n0 - 128 * tileA + (lane & 15)];
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {             // rows g (accumulator entries 0, 1) and g + 8 (entries 2, 3)
