@@ -33,8 +33,9 @@
 //   warps 8-15  (MODE_DEQ: 12-19) epilogue: drain a finished cluster's accumulator (tcgen05.ld), add s_c * acc into
 //               fp32 running sums held in registers while the next cluster's MMAs run; after the
 //               last cluster apply the zero-point correction, s_w, bias, activation, and store
-// Every wait is bounded: a wait that runs out sets RPTQ_ERR_DEVICE_TIMEOUT in the status word and
-// all roles drain and return.
+// Every wait is bounded: a wait that runs out sets RPTQ_ERR_DEVICE_TIMEOUT in the status word, every later one returns at once, the
+// producer and the MMA issuer drain and stop, and the other roles run their loops to the end (whole warps that would
+// leave them lane by lane could part).
 #include <cuda_fp16.h>
 
 #include <mutex>
@@ -548,8 +549,7 @@ cluster_gemm_kernel(const Params p)
         // coefficients its drain needs per column.
         const int tt = tid - TABLE_WARP0 * 32;
         uint32_t n_tile = 0, n_seg_done = 0;
-        bool ok = true;
-        for (int t = pair_id; t < p.n_items && ok; t += n_pairs, ++n_tile) {
+        for (int t = pair_id; t < p.n_items; t += n_pairs, ++n_tile) {
             int mt, n0;
             item_of(t, mt, n0);
             const int n = n0 + 4 * tt;                     // (of a strip, the lanes past its columns work for nothing)
@@ -574,14 +574,13 @@ cluster_gemm_kernel(const Params p)
                     corr[2] = __fmaf_rn(sz * sw4.z, (float)ws4.z - nc * (float)zw4.z, corr[2]);
                     corr[3] = __fmaf_rn(sz * sw4.w, (float)ws4.w - nc * (float)zw4.w, corr[3]);
                     const uint32_t sl = n_seg_done % SEG_SLOTS;
-                    if (!mbar_wait(bar(B_SEGEMPTY + sl), ((n_seg_done / SEG_SLOTS) & 1) ^ 1, s_abort)) { ok = false; break; }
+                    mbar_wait(bar(B_SEGEMPTY + sl), ((n_seg_done / SEG_SLOTS) & 1) ^ 1, s_abort);
                     float4* d = s_seg_tab + sl * (TILE_N / 2) + 2 * tt;
                     d[0] = make_float4(sc * sw4.x, sc * sw4.y, (float)(128 - 16 * zw4.x), (float)(128 - 16 * zw4.y));
                     d[1] = make_float4(sc * sw4.z, sc * sw4.w, (float)(128 - 16 * zw4.z), (float)(128 - 16 * zw4.w));
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(B_SEGFULL + sl));
                 }
-                if (!ok) break;
             } else if constexpr (!DEQ) {
                 if (p.corr) {
 #pragma unroll
@@ -603,7 +602,7 @@ cluster_gemm_kernel(const Params p)
                 }
             }
             const uint32_t b = n_tile & 1;
-            if (!mbar_wait(bar(B_TABEMPTY + b), ((n_tile >> 1) & 1) ^ 1, s_abort)) break;
+            mbar_wait(bar(B_TABEMPTY + b), ((n_tile >> 1) & 1) ^ 1, s_abort);
             float* tab = s_tab + b * 3 * TILE_N + 4 * tt;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
@@ -639,7 +638,6 @@ cluster_gemm_kernel(const Params p)
             // operand stage; a warp covers its 32 rows in eight such instructions, PF K blocks
             // ahead of the weights. The stage is waited for (its previous MMAs have read it) first.
             constexpr int PF = N_U - 2;
-            bool ok = true;
             const int wrow = (warp - UNPACK_WARP0) * 32 + (lane >> 3), ch = lane & 7;   // rows wrow + 4 i, chunk ch
             const uint32_t d_even = (uint32_t)wrow * 128 + ((ch ^ (lane >> 3)) << 4);
             const uint32_t d_odd = (uint32_t)wrow * 128 + ((ch ^ ((lane >> 3) + 4)) << 4);
@@ -655,31 +653,28 @@ cluster_gemm_kernel(const Params p)
             };
             a8_tile();
             auto fetch_next = [&]() {
-                if (n_fetched < total_kb && ok) {
+                if (n_fetched < total_kb) {
                     const int s2 = n_fetched % N_U;
-                    if (!mbar_wait(bar(B_UEMPTY + s2), ((n_fetched / N_U) & 1) ^ 1, s_abort)) { ok = false; }
-                    else {
-                        tc_fence_after();
-                        const uint32_t dst = smem_base + s2 * SL.u_stage;
+                    mbar_wait(bar(B_UEMPTY + s2), ((n_fetched / N_U) & 1) ^ 1, s_abort);
+                    tc_fence_after();
+                    const uint32_t dst = smem_base + s2 * SL.u_stage;
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const bool v = i < n_rows_ok;
-                            cp_async16(dst + ((i & 1) ? d_odd : d_even) + i * 512, v ? a_src + i * step4 : p.a_codes, v);
-                        }
-                        a_src += KBLK;
-                        if (++kb_f == p.n_kb) { kb_f = 0; t_f += n_pairs; a8_tile(); }
+                    for (int i = 0; i < 8; ++i) {
+                        const bool v = i < n_rows_ok;
+                        cp_async16(dst + ((i & 1) ? d_odd : d_even) + i * 512, v ? a_src + i * step4 : p.a_codes, v);
                     }
+                    a_src += KBLK;
+                    if (++kb_f == p.n_kb) { kb_f = 0; t_f += n_pairs; a8_tile(); }
                 }
                 ++n_fetched;
                 cp_async_commit();                           // one group per K block, empty past the end
             };
 #pragma unroll 1
             for (int i = 0; i < PF; ++i) fetch_next();
-            for (int it = 0; it < total_kb && ok; ++it, ++n_done) {
+            for (int it = 0; it < total_kb; ++it, ++n_done) {
                 const int sp = n_done % N_P, su = n_done % N_U;
                 fetch_next();
-                if (!ok) break;
-                if (!mbar_wait(bar(B_PFULL + sp), (n_done / N_P) & 1, s_abort)) break;
+                mbar_wait(bar(B_PFULL + sp), (n_done / N_P) & 1, s_abort);
                 const uint32_t pw = smem_base + SL.off_p + sp * SL.p_stage;
                 const uint32_t w_tile = smem_base + su * SL.u_stage + A8_BYTES;
                 uint32_t pw_w[W_ITEMS][4];
@@ -777,7 +772,7 @@ cluster_gemm_kernel(const Params p)
                 }
                 const uint32_t n_step = 2u * n_done + (uint32_t)grp;
                 const int st = n_step % N_U;
-                if (!mbar_wait(bar(B_PFULL + sp), (n_done / N_P) & 1, s_abort)) break;
+                mbar_wait(bar(B_PFULL + sp), (n_done / N_P) & 1, s_abort);
                 // (all loads before the first store: they are not reordered)
                 const uint32_t pw = smem_base + SL.off_p + sp * SL.p_stage, a_tile = smem_base + st * SL.u_stage, w_tile = a_tile + A8_BYTES;
                 uint32_t pk[W_ROWS / 64][4];
@@ -786,7 +781,7 @@ cluster_gemm_kernel(const Params p)
                     const uint4 v = lds128(pw + ((ut >> 1) + 64 * i) * 64 + (2 * grp + (ut & 1)) * 16);
                     pk[i][0] = v.x; pk[i][1] = v.y; pk[i][2] = v.z; pk[i][3] = v.w;
                 }
-                if (!mbar_wait(bar(B_UEMPTY + st), ((n_step / N_U) & 1) ^ 1, s_abort)) break;
+                mbar_wait(bar(B_UEMPTY + st), ((n_step / N_U) & 1) ^ 1, s_abort);
                 tc_fence_after();
 #pragma unroll
                 for (int uu = 0; uu < 2; ++uu) {
@@ -881,8 +876,8 @@ cluster_gemm_kernel(const Params p)
 #pragma unroll
                     for (int j = 0; j < BITS; ++j) pa_w[u][j] = raw[BITS * u + j];
             }
-            if (!mbar_wait(bar(B_PFULL + sp), (n_done / N_P) & 1, s_abort)) break;
-            if (!mbar_wait(bar(B_UEMPTY + su), ((n_done / N_U) & 1) ^ 1, s_abort)) break;
+            mbar_wait(bar(B_PFULL + sp), (n_done / N_P) & 1, s_abort);
+            mbar_wait(bar(B_UEMPTY + su), ((n_done / N_U) & 1) ^ 1, s_abort);
             tc_fence_after();
             const uint32_t pw = smem_base + SL.off_p + sp * SL.p_stage;
             const uint32_t a_tile = smem_base + su * SL.u_stage, w_tile = a_tile + A8_BYTES;
@@ -926,10 +921,9 @@ cluster_gemm_kernel(const Params p)
         const int q = ew & 3, h = ew >> 2;           // TMEM lane quarter (= warp % 4), column half
         uint32_t n_tile_done = 0;
         uint32_t par = 0;                    // bit b: parity of how many clusters of accumulator b I have drained
-        bool ok = true;
         uint32_t n_seg_done = 0;                     // ASYM: clusters drained so far, over all tiles
         float2 R[64];                                // running sums of columns 2 i, 2 i + 1
-        for (int t = pair_id; t < p.n_items && ok; t += n_pairs, ++n_tile_done) {
+        for (int t = pair_id; t < p.n_items; t += n_pairs, ++n_tile_done) {
             int mt, n0;
             const int sh = item_of(t, mt, n0), half_cols = 128 >> sh;      // columns of my half
             const int m0 = mt * (TILE_M * NCTA) + (int)cta_rank * TILE_M;
@@ -947,7 +941,7 @@ cluster_gemm_kernel(const Params p)
             }
             for (int sgi = 0; sgi < (DEQ ? 1 : p.n_seg); ++sgi) {
                 const uint32_t buf = DEQ ? (n_tile_done & 1u) : (uint32_t)s_seg_buf[sgi];
-                if (!mbar_wait(bar(B_ACCFULL + buf), (par >> buf) & 1u, s_abort)) { ok = false; break; }
+                mbar_wait(bar(B_ACCFULL + buf), (par >> buf) & 1u, s_abort);
                 par ^= 1u << buf;
                 tc_fence_after();
                 const float sc = ASYM ? 0.f : s_seg_scale[sgi];
@@ -956,7 +950,7 @@ cluster_gemm_kernel(const Params p)
                 const float4* seg_tab = s_seg_tab + seg_slot * (TILE_N / 2) + (h * half_cols >> 1);
                 float2 xs2 = make_float2(0.f, 0.f);
                 if constexpr (ASYM) {
-                    if (!mbar_wait(bar(B_SEGFULL + seg_slot), (n_seg_done / SEG_SLOTS) & 1, s_abort)) { ok = false; break; }
+                    mbar_wait(bar(B_SEGFULL + seg_slot), (n_seg_done / SEG_SLOTS) & 1, s_abort);
                     ++n_seg_done;
                     const float x = (float)xs_next;
                     xs2 = make_float2(x, x);
@@ -1002,8 +996,7 @@ cluster_gemm_kernel(const Params p)
                     arrive_leader(bar(B_ACCEMPTY + buf));
                 }
             }
-            if (!ok) break;
-            if (!mbar_wait(bar(B_TAB + (n_tile_done & 1)), (n_tile_done >> 1) & 1, s_abort)) { ok = false; break; }
+            mbar_wait(bar(B_TAB + (n_tile_done & 1)), (n_tile_done >> 1) & 1, s_abort);
             // y = s_w * (R - corr) + bias, activation, store. A thread holds 128 columns of one row: stored from there, every
             // instruction of a warp touches 32 rows with 16 bytes each. Pieces of 32 bytes per row (one memory sector) are
             // exchanged through a small buffer of the warp instead, and leave as whole sectors of 16 rows

@@ -90,7 +90,8 @@ __device__ __forceinline__ void mbar_sleep_or_abort(uint32_t bar, uint32_t parit
 }
 // Bounded wait. Returns false when the budget ran out or another role already gave up. The common
 // case (the phase has already completed, or completes within a few polls) touches no timer; the
-// budget is counted on the SM's cycle counter, read once per batch of polls.
+// budget is counted on the SM's cycle counter, read once per batch of polls. Each lane has its own answer: for blocks that one
+// lane executes, and for loops of a fixed trip count that go on whatever came of it.
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort_flag, bool heed_abort = true)
 {
     auto poll = [&]() { return mbar_try_wait(bar, parity); };
@@ -100,7 +101,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 #pragma unroll 1
     while (true) {
 #pragma unroll 1
-        for (int i = 0; i < 1024; ++i)
+        for (int i = 0; i < 16; ++i)
             if (poll()) return true;
         if (heed_abort && *abort_flag) return false;
         if (clock64() - t0 > WAIT_BUDGET_CYCLES) { *abort_flag = 1; return false; }

@@ -319,19 +319,18 @@ def _block_end(text, start):
             return i
 
 
-@pytest.mark.parametrize("name", ["attention_prefill.cu", "small_m_gemm.cu"])
+@pytest.mark.parametrize("name", ["attention_prefill.cu", "small_m_gemm.cu", "cluster_gemm.cu"])
 def test_waits_of_whole_warps_are_voted(name):
     """A bounded wait that gives up in some lanes of a warp while its barrier completes for the others must not part them: those that
-    go on would wait for ever at the next instruction that the whole warp takes part in. So warps wait through the voting forms
-    (mbar_*_warp) or go on without an answer (mbar_sleep_or_abort); the per-lane forms are for blocks that one lane executes, and
-    for the last wait of a role that has given up already, whose answer nobody asks for."""
+    go on would wait for ever at the next instruction that the whole warp takes part in. So a whole warp waits through the voting
+    forms, or does not ask for the answer; answers of its own a lane only has in blocks that one lane executes."""
     text = re.sub(r"//[^\n]*", "", open(os.path.join(CSRC, name)).read())
     one_lane = [(m.start(), _block_end(text, m.end())) for m in re.finditer(r"if \(lane == 0\)(?=\s*\{)", text)]
     voted = 0
     for m in re.finditer(r"\bmbar_(?:sleep|wait)(_warp|_or_abort)?\(", text):
-        if m.group(1):
+        before = text[max(text.rfind(c, 0, m.start()) for c in ";{}") + 1:m.start()]
+        if m.group(1) or not before.replace("tc::", "").strip():
             voted += 1
-            continue
-        line = text[text.rfind("\n", 0, m.start()):text.index("\n", m.start())]
-        assert any(a < m.start() < b for a, b in one_lane) or "B_DRAIN" in line, line
+        else:
+            assert any(a < m.start() < b for a, b in one_lane), text[m.start() - 60:m.end() + 60]
     assert voted > 0
