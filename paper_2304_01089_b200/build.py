@@ -21,12 +21,16 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
+def dependencies():
+    headers = [os.path.join(CSRC, "*.h"), os.path.join(CSRC, "*.cuh"), os.path.join(ROOT, "include", "*.h")]
+    return sources() + [f for pattern in headers for f in sorted(glob.glob(pattern))]
+
+
 def needs_build() -> bool:
     if not os.path.exists(LIB):
         return True
     t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.h")) + glob.glob(os.path.join(ROOT, "include", "*.h"))
-    return any(os.path.getmtime(d) > t for d in deps)
+    return any(os.path.getmtime(d) > t for d in dependencies())
 
 
 def build(force: bool = False, verbose: bool = False) -> str:

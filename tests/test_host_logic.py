@@ -283,6 +283,10 @@ def test_the_layernorm_kernels_hot_instances_do_not_spill(tmp_path):
 CSRC = os.path.join(ROOT, "paper_2304_01089_b200", "csrc")
 
 
+def test_every_source_file_takes_part_in_the_check_for_a_stale_library():
+    assert {os.path.join(CSRC, f) for f in os.listdir(CSRC)} <= set(lib_build.dependencies())
+
+
 def test_only_tables_and_weights_are_read_through_the_read_only_path():
     """A kernel of the library may be resident while the one before it in the stream still writes (programmatic dependent launch). Loads
     through the read-only path (ld.global.nc: __ldg, or any load from a const __restrict__ argument) are only defined for memory
