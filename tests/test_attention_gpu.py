@@ -291,16 +291,26 @@ def test_empty_and_oversized_calls():
 
 
 # The kernel for at most seven queries splits the keys over warps (tiles of 32 keys) and a cluster of blocks: sizes around a
-# tile, around four warps' tiles, an empty last block, eight blocks per head, every pair of code widths.
+# tile, around four warps' tiles, eight blocks per head, every pair of code widths.
 @pytest.mark.parametrize("bits", [(4, 4, 4), (3, 3, 3), (8, 8, 8), (4, 8, 3), (8, 3, 8)])
 @pytest.mark.parametrize("Tq,Tk,causal", [(1, 31, True), (7, 33, True), (2, 128, False), (7, 1000, True), (1, 2500, True)])
 def test_few_queries(Tq, Tk, causal, bits):
     Case(900 + Tk + 10 * bits[0] + bits[1], H=2, hd=72, gh=4, Tq=Tq, Tk=Tk, bits=bits).check(causal)
 
 
+# With two heads on 148 SMs: two blocks per head of 160 keys, four of 160, eight of 160 of which the last one has none.
+@pytest.mark.parametrize("bits", [(4, 4, 4), (8, 3, 8)])
+@pytest.mark.parametrize("Tk", [300, 600, 1030])
+@pytest.mark.parametrize("Tq", [1, 2, 3, 7])
+def test_few_queries_splits(Tq, Tk, bits):
+    Case(930 + Tk + Tq, H=2, hd=72, gh=4, Tq=Tq, Tk=Tk, bits=bits).check(True)
+
+
 def test_few_queries_of_many_heads_take_one_block_per_head():
-    """300 heads: no split of the keys."""
+    """300 heads of 40 keys, too few to split, and of 700: a split would need a second round of blocks, so each of a block's warps
+    walks five or six tiles through its ring of three."""
     Case(950, H=300, hd=16, gh=4, Tq=3, Tk=40, bits=(4, 4, 4)).check(True)
+    Case(951, H=300, hd=16, gh=4, Tq=3, Tk=700, bits=(4, 4, 4)).check(True)
 
 
 # The kernel for more queries: tiles of 128 queries and 128 keys (two streams of 64), query zero points folded into the operand where

@@ -166,6 +166,21 @@ def test_few_queries(Tq, Tk, n_seq, causal, bits):
     _check(c, _query(np.random.default_rng(3), Tq * n_seq, 144), causal, n_seq=n_seq)
 
 
+# See test_attention_gpu.py::test_few_queries_splits; one or two queries and three or more take different operand types.
+@pytest.mark.parametrize("bits", [(4, 4, 4), (4, 3, 8)])
+@pytest.mark.parametrize("Tk", [300, 600, 1030])
+@pytest.mark.parametrize("Tq", [1, 2, 3, 7])
+def test_few_queries_splits(Tq, Tk, bits):
+    c = Case(930 + Tk + Tq, H=2, hd=72, gh=4, Tq=Tq, Tk=Tk, bits=bits)
+    _check(c, _query(np.random.default_rng(15), Tq, 144), True)
+
+
+@pytest.mark.parametrize("Tq", [1, 3])
+def test_few_queries_of_many_heads_take_one_block_per_head(Tq):
+    c = Case(951 + Tq, H=300, hd=16, gh=4, Tq=Tq, Tk=700)
+    _check(c, _query(np.random.default_rng(16), Tq, 300 * 16), True)
+
+
 # The kernel for more queries: see test_attention_gpu.py::test_tile_edges; tiles of 64 keys that two streams take by turns.
 @pytest.mark.parametrize("Tq,Tk,n_seq,causal", [(9, 9, 1, True), (64, 65, 1, True), (128, 128, 2, False), (129, 257, 1, True), (200, 400, 1, True)])
 @pytest.mark.parametrize("bits", [(4, 4, 4), (4, 3, 8), (4, 8, 3)])
