@@ -557,22 +557,28 @@ cluster_gemm_kernel(const Params p)
             float corr[4] = {0.f, 0.f, 0.f, 0.f};
             if constexpr (ASYM) {
                 // y += s^X_c s^W_c[n] / 16 * (acc' + Z xsum), Z = -16 (z^W_c[n] - 8); the tile constant is
-                // sum_c s^X_c z^X_c s^W_c[n] (Wsum_c[n] - n_c z^W_c[n])
-                for (int sgi = 0; sgi < p.n_seg; ++sgi, ++n_seg_done) {
-                    const int cid = s_seg_cl[sgi];
-                    const int64_t i = (int64_t)cid * p.ld_w + n;
-                    float4 sw4 = make_float4(0.f, 0.f, 0.f, 0.f);
-                    int4 zw4 = make_int4(8, 8, 8, 8), ws4 = make_int4(0, 0, 0, 0);
-                    if (vec) {
-                        sw4 = __ldg(reinterpret_cast<const float4*>(p.sw_c + i));
-                        zw4 = __ldg(reinterpret_cast<const int4*>(p.zw_c + i));
-                        ws4 = __ldg(reinterpret_cast<const int4*>(p.wsum + i));
-                    }
-                    const float sz = __ldg(p.cl_sz + cid), nc = __ldg(p.cl_n + cid), sc = __ldg(p.seg_scale + sgi) * 0.0625f;
+                // sum_c s^X_c z^X_c s^W_c[n] (Wsum_c[n] - n_c z^W_c[n]), summed over the clusters in their own order, not in the order in which
+                // they end (2 to 5 % further from 64 bits): step sgi prepares segment sgi and adds cluster sgi
+                auto add = [&](int c) {
+                    if (!vec) return;
+                    const int64_t i = (int64_t)c * p.ld_w + n;
+                    const float4 sw4 = __ldg(reinterpret_cast<const float4*>(p.sw_c + i));
+                    const int4 zw4 = __ldg(reinterpret_cast<const int4*>(p.zw_c + i)), ws4 = __ldg(reinterpret_cast<const int4*>(p.wsum + i));
+                    const float sz = __ldg(p.cl_sz + c), nc = __ldg(p.cl_n + c);
                     corr[0] = __fmaf_rn(sz * sw4.x, (float)ws4.x - nc * (float)zw4.x, corr[0]);
                     corr[1] = __fmaf_rn(sz * sw4.y, (float)ws4.y - nc * (float)zw4.y, corr[1]);
                     corr[2] = __fmaf_rn(sz * sw4.z, (float)ws4.z - nc * (float)zw4.z, corr[2]);
                     corr[3] = __fmaf_rn(sz * sw4.w, (float)ws4.w - nc * (float)zw4.w, corr[3]);
+                };
+                for (int sgi = 0; sgi < p.n_seg; ++sgi, ++n_seg_done) {
+                    const int64_t i = (int64_t)s_seg_cl[sgi] * p.ld_w + n;
+                    float4 sw4 = make_float4(0.f, 0.f, 0.f, 0.f);
+                    int4 zw4 = make_int4(8, 8, 8, 8);
+                    if (vec) {
+                        sw4 = __ldg(reinterpret_cast<const float4*>(p.sw_c + i));
+                        zw4 = __ldg(reinterpret_cast<const int4*>(p.zw_c + i));
+                    }
+                    const float sc = __ldg(p.seg_scale + sgi) * 0.0625f;
                     const uint32_t sl = n_seg_done % SEG_SLOTS;
                     mbar_wait(bar(B_SEGEMPTY + sl), ((n_seg_done / SEG_SLOTS) & 1) ^ 1, s_abort);
                     float4* d = s_seg_tab + sl * (TILE_N / 2) + 2 * tt;
@@ -580,7 +586,9 @@ cluster_gemm_kernel(const Params p)
                     d[1] = make_float4(sc * sw4.z, sc * sw4.w, (float)(128 - 16 * zw4.z), (float)(128 - 16 * zw4.w));
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(B_SEGFULL + sl));
+                    add(sgi);
                 }
+                for (int c = p.n_seg; c < p.g; ++c) add(c);          // (where some clusters are empty)
             } else if constexpr (!DEQ) {
                 if (p.corr) {
 #pragma unroll

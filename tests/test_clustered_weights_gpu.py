@@ -178,3 +178,26 @@ def test_opt66b_fc1_sampled_rows_full_launch_shape():
     print(f"opt-66b FC1 clustered weights: max|dy|/max|y| = {err:.2e} on {len(rows)} rows x {len(cols)} columns")
     assert err <= TOL
     assert np.array_equal(xsum[ridx].cpu().numpy(), oracle.code_rowsums(a, site.cal.size))
+
+
+def test_the_tile_constant_does_not_depend_on_the_unit_order():
+    """The zero-point terms of a column are summed over the clusters in their own order, whatever order the units end in: with codes of
+    zero nothing else is left, and both unit orders give the same bits."""
+    import torch
+    from paper_2304_01089_b200 import binding
+    rng = np.random.default_rng(7300)
+    M, N, C, g = 130, 512, 1536, 40
+    perm, size, scale, zero = random_layout_params(rng, C, g, 4)
+    W = (rng.normal(size=(N, C)) * rng.lognormal(0, 0.7, size=C) * 0.02).astype(np.float32)
+    out = []
+    for order in (binding.ORDER_CONTIGUOUS, binding.ORDER_INTERLEAVED):
+        L = binding.Layout(perm, size, scale, zero, 4, order=order)
+        last = [np.flatnonzero(L.unit_cluster == c).max() for c in range(g) if size[c]]
+        assert (np.diff(last) > 0).all() == (order == binding.ORDER_CONTIGUOUS)
+        packed, s_w, z_w, wsum = binding.weight_pack_clustered(L, W)
+        y = torch.empty((M, N), dtype=torch.float32, device="cuda")
+        binding.cluster_gemm_clustered(L, torch.zeros((M, L.row_bytes), dtype=torch.uint8, device="cuda"), M,
+                                       torch.zeros((M, g), dtype=torch.int32, device="cuda"), torch.from_numpy(packed).cuda(),
+                                       torch.from_numpy(s_w).cuda(), torch.from_numpy(z_w).cuda(), torch.from_numpy(wsum).cuda(), N, y)
+        out.append(y)
+    assert torch.equal(out[0], out[1]) and bool((out[0] != 0).any())
