@@ -74,22 +74,6 @@ __device__ __forceinline__ void mma_f16(float (&d)[4], uint32_t a0, uint32_t a1,
                  : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                  : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
-// The nibbles at bit B of the two halves of w as a pair of fp16 numbers n - 8 (B = 0, 4, 8, 12).
-template <int B>
-__device__ __forceinline__ uint32_t nib_half(uint32_t w)
-{
-    const uint32_t t = ((B <= 6 ? w << (6 - B) : w >> (B - 6)) & 0x03C003C0u) | 0x4C004C00u;      // 16 + n
-    const __half2 r = __hadd2(*reinterpret_cast<const __half2*>(&t), __float2half2_rn(-24.0f));
-    return *reinterpret_cast<const uint32_t*>(&r);
-}
-// The bytes at bit B of the two halves of w as a pair of fp16 numbers n - 128 (B = 0, 8).
-template <int B>
-__device__ __forceinline__ uint32_t byte_half(uint32_t w)
-{
-    const uint32_t t = ((w >> B) & 0x00FF00FFu) | 0x64006400u;                                    // 1024 + n
-    const __half2 r = __hadd2(*reinterpret_cast<const __half2*>(&t), __float2half2_rn(-1152.0f));
-    return *reinterpret_cast<const uint32_t*>(&r);
-}
 __device__ __forceinline__ uint32_t cluster_rank()
 {
     uint32_t r;
@@ -116,15 +100,6 @@ __device__ __forceinline__ uint32_t ld_peer(uint32_t addr, uint32_t rank)
     return v;
 }
 
-// Bytes per key row of a warp's ring for `units` units of `bits` bits: the row's 16-byte chunks (one more where
-// the head's first unit need not start on a boundary), rounded up to an odd number of chunks so that the eight
-// rows (or four pairs of rows) a warp reads at once lie in different banks.
-__host__ __device__ inline int raw_pitch(int bits, int units)
-{
-    int c = (4 * bits * units + 15) / 16 + (bits == 3 ? 1 : 0);
-    c |= 1;
-    return 16 * c;
-}
 __host__ __device__ inline int nibble_pitch(int units) { return 16 * (units | 1); }
 
 struct SmemPlan { int ring_stage, ring, expand, expand_all, scores, score_pitch, total; };
@@ -190,11 +165,10 @@ decode_kernel(const AttnParams p, int keys_block, int units_k_max, int units_v_m
 #pragma unroll
             for (int rg = 0; rg < TILE / 8; ++rg) {
                 const bool ok = r0 + 8 * rg < n_rows;
-                const uint8_t* from = ok ? src : base;             // (size 0 reads nothing)
-                const int n = ok ? 16 : 0;
+                const uint8_t* from = ok ? src : base;             // (an address that is not read)
 #pragma unroll
                 for (int c = 0; c < 4; ++c) {                      // at most 16 chunks per row
-                    if (c0 + 4 * c < n16) cp_async16(dst + 64 * c, ok ? from + 64 * c : from, n);
+                    if (c0 + 4 * c < n16) cp_async16(dst + 64 * c, ok ? from + 64 * c : from, ok);
                     if (4 * c + 4 >= n16) break;
                 }
                 src += 8 * row_bytes; dst += 8 * pitch;

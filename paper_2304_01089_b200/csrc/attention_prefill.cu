@@ -42,30 +42,24 @@
 
 #include "attn_common.cuh"
 #include "pack.cuh"
-#include "tc.cuh"
 
 namespace rptq {
 namespace attn_prefill {
 
 using namespace attn;
-using tc::mbar_arrive;
-using tc::mbar_init;
-using tc::mbar_sleep_warp;
 
 enum { I8 = 0, F8 = 1, KV = 2 };
-// Softmax warps that share a stream's piece of work (and a lane quarter). 2 (sixteen warps of 32 keys a thread) measured the same
-// (773 and 770 us), KV 3 % slower: the loaders then have 56 registers.
-constexpr int SUB = 1;
-constexpr int BM = 128, THREADS = 384 + 256 * SUB;
+// Eight softmax warps, four for each stream. Sixteen of 32 keys a thread measured the same (773 and 770 us), KV 3 % slower: the loaders
+// then have 56 registers.
+constexpr int BM = 128, THREADS = 640, STREAMS = 2;
 constexpr int K_WARP0 = 4, V_WARP0 = 8, S_WARP0 = 12;
 constexpr int COLS = 64;                                  // keys of a stream's piece of work = columns of a score slot
-constexpr int CT = COLS / SUB;                            // keys of a thread
 constexpr int N_SLOTS = 2;                                // score slots of each stream
-constexpr int S_WARPS = 8 * SUB, PARTS = 2 * SUB;         // softmax warps; threads that share a row
-// registers per thread of the warpgroups: MMA issuers, two of loaders, 2 SUB of softmax (the block is launched with 72 or 96 each)
-constexpr int REGS_MMA = SUB == 2 ? 40 : 48, REGS_LOAD = SUB == 2 ? 56 : 72, REGS_SOFTMAX = SUB == 2 ? 88 : 144;
-constexpr int REGS_ALL = REGS_MMA + 2 * REGS_LOAD + 2 * SUB * REGS_SOFTMAX;
-static_assert(REGS_ALL <= (SUB == 2 ? 7 * 72 : 5 * 96), "register pool");
+constexpr int S_WARPS = 4 * STREAMS;                      // softmax warps
+// registers per thread of the warpgroups: MMA issuers, two of loaders, two of softmax (the block is launched with 96 each)
+constexpr int REGS_MMA = 48, REGS_LOAD = 72, REGS_SOFTMAX = 144;
+constexpr int REGS_ALL = REGS_MMA + 2 * REGS_LOAD + STREAMS * REGS_SOFTMAX;
+static_assert(REGS_ALL <= 5 * 96, "register pool");
 constexpr int O_COLS = 32 * MAX_UNITS;                    // tensor memory: the output accumulator, then the score slots
 constexpr int ATOM_Q = BM * 128;                          // 128 rows of 128 bytes
 
@@ -83,14 +77,6 @@ struct Plan {
     int* status;
 };
 
-// Row pitch of a staged packed tile: an odd number of 16-byte chunks, so that eight rows read at one column lie in
-// different banks.
-static int raw_pitch_of(int bits, int units)
-{
-    const int c = (4 * bits * units + 15) / 16 + (bits == 3 ? 1 : 0);
-    return 16 * (c | 1);
-}
-
 __device__ __forceinline__ void ld32(uint32_t taddr, uint32_t (&v)[32])
 {
     asm volatile(
@@ -101,27 +87,6 @@ __device__ __forceinline__ void ld32(uint32_t taddr, uint32_t (&v)[32])
           "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
           "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
         : "r"(taddr) : "memory");
-}
-__device__ __forceinline__ float2 add2(float2 a, float2 b)
-{
-    float2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(reinterpret_cast<uint64_t&>(d))
-        : "l"(reinterpret_cast<uint64_t&>(a)), "l"(reinterpret_cast<uint64_t&>(b)));
-    return d;
-}
-__device__ __forceinline__ float2 mul2(float2 a, float2 b)
-{
-    float2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(reinterpret_cast<uint64_t&>(d))
-        : "l"(reinterpret_cast<uint64_t&>(a)), "l"(reinterpret_cast<uint64_t&>(b)));
-    return d;
-}
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
-{
-    float2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(reinterpret_cast<uint64_t&>(d))
-        : "l"(reinterpret_cast<uint64_t&>(a)), "l"(reinterpret_cast<uint64_t&>(b)), "l"(reinterpret_cast<uint64_t&>(c)));
-    return d;
 }
 // The whole warp executes these in converged control flow; one elected lane issues. a, b: the low words of the operands'
 // descriptors (the high words are the same for every tile).
@@ -144,47 +109,9 @@ __device__ __forceinline__ void commit(uint32_t bar)
     asm volatile("{\n\t.reg .pred q;\n\telect.sync _|q, 0xffffffff;\n\t"
                  "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}" ::"r"(bar) : "memory");
 }
-// The nibbles (bytes) at bit B of the two halves of w as fp16 numbers n - 8 (n - 128).
-template <int B>
-__device__ __forceinline__ uint32_t nib_half(uint32_t w)
-{
-    const uint32_t t = ((B <= 6 ? w << (6 - B) : w >> (B - 6)) & 0x03C003C0u) | 0x4C004C00u;      // 16 + n
-    const __half2 r = __hadd2(*reinterpret_cast<const __half2*>(&t), __float2half2_rn(-24.0f));
-    return *reinterpret_cast<const uint32_t*>(&r);
-}
-template <int B>
-__device__ __forceinline__ uint32_t byte_half(uint32_t w)
-{
-    const uint32_t t = ((w >> B) & 0x00FF00FFu) | 0x64006400u;                                    // 1024 + n
-    const __half2 r = __hadd2(*reinterpret_cast<const __half2*>(&t), __float2half2_rn(-1152.0f));
-    return *reinterpret_cast<const uint32_t*>(&r);
-}
-__device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
-{
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-__device__ __forceinline__ void sts32(uint32_t addr, uint32_t a) { asm volatile("st.shared.b32 [%0], %1;" ::"r"(addr), "r"(a) : "memory"); }
 __device__ __forceinline__ void sts16_if(bool p, uint32_t addr, uint16_t a)
 {
     asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.b32 q, %2, 0;\n\t@q st.shared.b16 [%0], %1;\n\t}" ::"r"(addr), "h"(a), "r"((int)p) : "memory");
-}
-__device__ __forceinline__ uint4 lds128(uint32_t addr)
-{
-    uint4 v;
-    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ uint32_t lds32(uint32_t addr)
-{
-    uint32_t v;
-    asm volatile("ld.shared.b32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ uint16_t lds16(uint32_t addr)
-{
-    uint16_t v;
-    asm volatile("ld.shared.b16 %0, [%1];" : "=h"(v) : "r"(addr) : "memory");
-    return v;
 }
 // Unit u of a staged packed row of 3- or 4-bit codes as nibble words (the 4-bit format).
 __device__ __forceinline__ uint4 nibbles(uint32_t row, int u, int bits)
@@ -255,9 +182,9 @@ prefill_kernel(const AttnParams p, const Plan g)
         mbar_init(bar(B_QFULL), Q_LOADERS); mbar_init(bar(B_QEMPTY), 2);
         for (int i = 0; i < 2; ++i) {
             mbar_init(bar(B_KFULL + i), 4); mbar_init(bar(B_KEMPTY + i), ALT ? 1 : 2); mbar_init(bar(B_VFULL + i), 4); mbar_init(bar(B_VEMPTY + i), 1);
-            mbar_init(bar(B_PFULL + i), 4 * SUB); mbar_init(bar(B_PEMPTY + i), 1);
+            mbar_init(bar(B_PFULL + i), 4); mbar_init(bar(B_PEMPTY + i), 1);
         }
-        for (int i = 0; i < 2 * N_SLOTS; ++i) { mbar_init(bar(B_SFULL + i), 1); mbar_init(bar(B_SEMPTY + i), 4 * SUB); }
+        for (int i = 0; i < 2 * N_SLOTS; ++i) { mbar_init(bar(B_SFULL + i), 1); mbar_init(bar(B_SEMPTY + i), 4); }
         mbar_init(bar(B_OFULL), 1); mbar_init(bar(B_OEMPTY), 4); mbar_init(bar(B_OUT), 4);
         mbar_init(bar(B_SUM), S_WARPS); mbar_init(bar(B_XS), S_WARPS); mbar_init(bar(B_XV), 4);
         for (int i = 0; i < 3; ++i) mbar_init(bar(B_DRAIN + i), 1);
@@ -268,15 +195,15 @@ prefill_kernel(const AttnParams p, const Plan g)
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(s_tmem)) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    tc::tc_fence_before();
+    tc_fence_before();
     pdl_trigger();
     pdl_wait();
     __syncthreads();
-    tc::tc_fence_after();
+    tc_fence_after();
     const uint32_t tmem = *s_tmem;
     float* s_col = reinterpret_cast<float*>(smem + g.off_col);            // [4][KEYS]
-    float2* s_ml = reinterpret_cast<float2*>(smem + g.off_ml);            // [2][PARTS][BM]: row maxima and sums of the parts
-    uint32_t* s_sum = reinterpret_cast<uint32_t*>(smem + g.off_sum);      // [PARTS][BM]: sums of probabilities (codes)
+    float2* s_ml = reinterpret_cast<float2*>(smem + g.off_ml);            // [2][STREAMS][BM]: row maxima and sums over a stream's keys
+    uint32_t* s_sum = reinterpret_cast<uint32_t*>(smem + g.off_sum);      // [STREAMS][BM]: sums of probabilities (codes)
 
     if (warp < K_WARP0) {
         asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_MMA));
@@ -306,14 +233,14 @@ prefill_kernel(const AttnParams p, const Plan g)
                     for (int kt = ALT ? stream : 0; kt < it.n_kt && ok; kt += ALT ? 2 : 1, ++n_k) {
                         const uint32_t st = ALT ? stream : n_k & 1;            // (KV: a stage belongs to a stream, which so sees all its phases)
                         if (!mbar_sleep_warp(bar(B_KFULL + st), (ALT ? n_k : n_k >> 1) & 1, s_abort)) { ok = false; break; }
-                        tc::tc_fence_after();
+                        tc_fence_after();
                         const uint32_t kb = dk + st * k_step;
                         uint32_t acc = 0u;
 #pragma unroll 1
                         for (uint32_t u = 0; u < (uint32_t)nu; ++u) {
                             if (acc == 0u) {
                                 if (!mbar_sleep_warp(b_empty0 + 8 * slot, par, s_abort)) { ok = false; break; }
-                                tc::tc_fence_after();
+                                tc_fence_after();
                             }
                             const uint32_t d = d0 + slot * COLS, in = (u & ((1u << LOG_ATOM) - 1u)) * STEP;
                             const uint32_t a = dq + (u >> LOG_ATOM) * (ATOM_Q >> 4) + in, b = kb + (u >> LOG_ATOM) * (K_ATOM >> 4) + in;
@@ -355,7 +282,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                     if constexpr (ALT) {
                         const uint32_t stream = kt & 1, n_p = stream ? n_p1 : n_p0;
                         if (!mbar_sleep_warp(bar(B_PFULL + stream), n_p & 1, s_abort)) { ok = false; break; }
-                        tc::tc_fence_after();
+                        tc_fence_after();
                         const uint32_t a0 = dp + (g.p_tiles == 2 ? stream * (BM * 128 >> 4) : 0u);
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
@@ -367,7 +294,7 @@ prefill_kernel(const AttnParams p, const Plan g)
 #pragma unroll
                         for (int half = 0; half < 2; ++half) {
                             if (!mbar_sleep_warp(bar(B_PFULL + half), n_v & 1, s_abort)) { ok = false; break; }
-                            tc::tc_fence_after();
+                            tc_fence_after();
                             if (nuv > 0) {
                                 mma<0>(tmem, dp + 4 * half, b0 + 4 * half, id, half == 0 ? acc : 1u);
                                 mma<0>(tmem, dp + 4 * half + 2, b0 + 4 * half + 2, id, 1u);
@@ -383,7 +310,7 @@ prefill_kernel(const AttnParams p, const Plan g)
         }
         if (warp < 3 && !ok) {
             commit(bar(B_DRAIN + warp));
-            tc::mbar_wait(bar(B_DRAIN + warp), 0, s_abort, false);
+            mbar_wait(bar(B_DRAIN + warp), 0, s_abort, false);
         }
     } else if (warp < S_WARP0) {
         // ---------------------------------------------------------------- loaders: keys and queries (warps 4-7), values and outputs (8-11)
@@ -427,7 +354,7 @@ prefill_kernel(const AttnParams p, const Plan g)
 #pragma unroll
                 for (int i = 0; i < ROWS_W / 4; ++i) {
                     const bool in = r0 + 4 * i < rows;
-                    cp_async16(dst(r0 + 4 * i, c), in ? from + (uint64_t)(4 * i) * rb : codes, in ? 16 : 0);       // (size 0 reads nothing)
+                    cp_async16(dst(r0 + 4 * i, c), in ? from + (uint64_t)(4 * i) * rb : codes, in);
                 }
             }
         };
@@ -458,7 +385,7 @@ prefill_kernel(const AttnParams p, const Plan g)
 #pragma unroll 1
                 for (int i = lane; i < 16 * per_row; i += 32) {
                     const int r = i / per_row, c = i - r * per_row;
-                    cp_async16(base + (c >> 3) * ATOM_Q + (r0 + r) * 128 + 16 * (c & 7), r < rows ? q_rows + r * p.ldq + it.h * p.hd + 8 * c : p.q_f16, r < rows ? 16 : 0);
+                    cp_async16(base + (c >> 3) * ATOM_Q + (r0 + r) * 128 + 16 * (c & 7), r < rows ? q_rows + r * p.ldq + it.h * p.hd + 8 * c : p.q_f16, r < rows);
                 }
                 cp_async_commit();
                 cp_async_wait<0>();
@@ -491,7 +418,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                         if (lane + 32 * k < 16 * nu)
                             sts32(base + k * ATOM_Q + (r0 + r4 + rr) * 128 + (((lane >> 2) ^ ((r4 + rr) & 7)) << 4) + 4 * (lane & 3), v[rr][k]);
             }
-            tc::fence_proxy_async();
+            fence_proxy_async();
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(B_QFULL));
             return true;
@@ -562,7 +489,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                                 sts128(d + ((c ^ sw) << 4), o[0], o[1], o[2], o[3]);
                                 sts128(d + (((c + 1) ^ sw) << 4), o[4], o[5], o[6], o[7]);
                             }
-                            tc::fence_proxy_async();
+                            fence_proxy_async();
                             __syncwarp();
                             if (lane == 0) mbar_arrive(bar(B_QFULL));
                         }
@@ -635,7 +562,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                             s_col[(m & 3) * KEYS + r] = col;
                         }
                     }
-                    tc::fence_proxy_async();
+                    fence_proxy_async();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(B_KFULL + st));
                 }
@@ -777,7 +704,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                             }
                         }
                     }
-                    tc::fence_proxy_async();
+                    fence_proxy_async();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(B_VFULL + st));
                     if (!group_sync()) { ok = false; break; }                  // the raw rows have been read
@@ -797,7 +724,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                     chs[u] = u < nuv && __ldg(p.jidx_v + pos) >= 0 ? (int)__ldg(p.src_v + pos) : -1;
                 }
                 if (!mbar_sleep_warp(bar(B_SUM), n_item & 1, s_abort) || !mbar_sleep_warp(bar(B_OFULL), n_item & 1, s_abort)) { ok = false; break; }
-                tc::tc_fence_after();
+                tc_fence_after();
                 const int row = 32 * lw + lane, i0 = it.qt * BM, i = i0 + row;
                 const bool live = i0 + 32 * lw < p.Tq;                         // some row of my warp exists
                 if (live) {
@@ -806,11 +733,11 @@ prefill_kernel(const AttnParams p, const Plan g)
                     if constexpr (MODE == KV) {
                         float l = 0.f;
 #pragma unroll
-                        for (int q = 0; q < PARTS; ++q) l += __uint_as_float(s_sum[q * BM + row]);
+                        for (int q = 0; q < STREAMS; ++q) l += __uint_as_float(s_sum[q * BM + row]);
                         inv_l = 1.0f / l;
                     } else {
 #pragma unroll
-                        for (int q = 0; q < PARTS; ++q) rs += (int)s_sum[q * BM + row];
+                        for (int q = 0; q < STREAMS; ++q) rs += (int)s_sum[q * BM + row];
                     }
                     const uint32_t stage = base + g.off_v, o_row = stage + row * g.out_pitch;
                     __half* out_row = p.out + ((int64_t)it.seq * p.Tq + i) * p.ldo;
@@ -835,7 +762,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                                 const int c = __shfl_sync(0xffffffffu, ch, e);
                                 uint32_t v;
                                 asm volatile("tcgen05.ld.sync.aligned.32x32b.x1.b32 {%0}, [%1];" : "=r"(v) : "r"(t_unit + e) : "memory");
-                                tc::tc_wait_ld();
+                                tc_wait_ld();
                                 if (c >= 0 && i < p.Tq) out_row[c] = __ushort_as_half(value(v));
                             }
                             continue;
@@ -843,8 +770,8 @@ prefill_kernel(const AttnParams p, const Plan g)
 #pragma unroll 1
                         for (int h = 0; h < 2; ++h) {
                             uint32_t v[16];
-                            tc::tc_ld16(t_unit + 16 * h, v);
-                            tc::tc_wait_ld();
+                            tc_ld16(t_unit + 16 * h, v);
+                            tc_wait_ld();
                             // (the staged words of row r are exchanged by r & 31: no bank conflicts)
 #pragma unroll
                             for (int e = 0; e < 16; ++e) {
@@ -853,7 +780,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                             }
                         }
                     }
-                    tc::tc_fence_before();
+                    tc_fence_before();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(B_OEMPTY));
                     if (g.local_v) {
@@ -889,9 +816,9 @@ prefill_kernel(const AttnParams p, const Plan g)
     } else {
         // ---------------------------------------------------------------- softmax
         asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(REGS_SOFTMAX));
-        const int q4 = warp & 3, part = (warp - S_WARP0) >> 2, stream = part / SUB, sub = part % SUB;      // q4: lane quarter of the accumulators
+        const int q4 = warp & 3, stream = (warp - S_WARP0) >> 2;              // q4: lane quarter of the accumulators
         const int row = 32 * q4 + lane;                                        // query row within the tile
-        const uint32_t t_col = tmem + ((uint32_t)(32 * q4) << 16) + O_COLS + stream * (N_SLOTS * COLS) + sub * CT;
+        const uint32_t t_col = tmem + ((uint32_t)(32 * q4) << 16) + O_COLS + stream * (N_SLOTS * COLS);
         const uint32_t b_full0 = bar(B_SFULL + stream * N_SLOTS), b_empty0 = bar(B_SEMPTY + stream * N_SLOTS);
         uint32_t n_k0 = 0, slot = 0, par = 0, n_s = 0, n_item = 0;   // n_s: my stream's tiles of pass 2 so far
         bool ok = true;
@@ -921,41 +848,41 @@ prefill_kernel(const AttnParams p, const Plan g)
 #pragma unroll 1
             for (int pass = 0; pass < 2 && ok; ++pass, n_k0 += it.n_kt) {
                 if (pass == 1) {
-                    // the parts' statistics meet (two sets by turns: a warp may be an item ahead of another)
-                    float2* ml = s_ml + (n_item & 1) * PARTS * BM + row;
-                    ml[part * BM] = make_float2(m, l);
+                    // the streams' statistics meet (two sets by turns: a warp may be an item ahead of another)
+                    float2* ml = s_ml + (n_item & 1) * STREAMS * BM + row;
+                    ml[stream * BM] = make_float2(m, l);
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(B_XS));
                     if (!mbar_sleep_warp(bar(B_XS), n_item & 1, s_abort)) { ok = false; break; }
 #pragma unroll
-                    for (int q = 0; q < PARTS; ++q) m = fmaxf(m, ml[q * BM].x);
+                    for (int q = 0; q < STREAMS; ++q) m = fmaxf(m, ml[q * BM].x);
                     if constexpr (MODE != KV) {
                         l = 0.f;
 #pragma unroll
-                        for (int q = 0; q < PARTS; ++q) l = __fmaf_rn(ml[q * BM].y, ex2(ml[q * BM].x - m), l);     // (a part without a visible key weighs 0)
+                        for (int q = 0; q < STREAMS; ++q) l = __fmaf_rn(ml[q * BM].y, ex2(ml[q * BM].x - m), l);     // (a stream without a visible key weighs 0)
                         f = p.inv_sP / l * 1.7763568394002505e-15f;            // times 2^-49: see below
                     }
                 }
 #pragma unroll 1
                 for (int kt = ALT ? stream : 0; kt < it.n_kt; kt += ALT ? 2 : 1) {
                     // ---- scores of my row against my keys of the tile, times log2(e); hidden keys at NEG_BIG
-                    float2 S[CT / 2];
-                    const float* col = s_col + ((n_k0 + kt) & 3) * KEYS + stream * COLS + sub * CT;
+                    float2 S[COLS / 2];
+                    const float* col = s_col + ((n_k0 + kt) & 3) * KEYS + stream * COLS;
                     bool first = true;
                     uint32_t left = last;                                      // (at least one bit)
                     do {
                         const float c = __shfl_sync(0xffffffffu, coef, __ffs(left) - 1);
                         if (!mbar_sleep_warp(b_full0 + 8 * slot, par, s_abort)) { ok = false; break; }
-                        tc::tc_fence_after();
+                        tc_fence_after();
                         if (live) {
                             uint32_t v[32];
                             ld32(t_col + slot * COLS, v);
                             if (first) {
 #pragma unroll
-                                for (int e = 0; e < CT / 2; ++e) S[e] = make_float2(0.f, 0.f);
+                                for (int e = 0; e < COLS / 2; ++e) S[e] = make_float2(0.f, 0.f);
                                 if (MODE != KV && !g.folded) {
 #pragma unroll
-                                    for (int e = 0; e < CT / 2; e += 2) {
+                                    for (int e = 0; e < COLS / 2; e += 2) {
                                         const float4 x = *reinterpret_cast<const float4*>(col + 2 * e);
                                         S[e] = make_float2(x.x, x.y); S[e + 1] = make_float2(x.z, x.w);
                                     }
@@ -963,8 +890,8 @@ prefill_kernel(const AttnParams p, const Plan g)
                             }
                             const float2 c2 = make_float2(c, c);
 #pragma unroll
-                            for (int h = 0; h < CT / 32; ++h) {
-                                tc::tc_wait_ld();
+                            for (int h = 0; h < COLS / 32; ++h) {
+                                tc_wait_ld();
 #pragma unroll
                                 for (int e = 0; e < 16; ++e) {
                                     float2 x;
@@ -972,11 +899,11 @@ prefill_kernel(const AttnParams p, const Plan g)
                                     else x = make_float2(__uint_as_float(v[2 * e]), __uint_as_float(v[2 * e + 1]));
                                     S[16 * h + e] = fma2(c2, x, S[16 * h + e]);
                                 }
-                                if (h + 1 < CT / 32) ld32(t_col + slot * COLS + 32, v);
+                                if (h + 1 < COLS / 32) ld32(t_col + slot * COLS + 32, v);
                             }
                         }
                         first = false;
-                        tc::tc_fence_before();
+                        tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive(b_empty0 + 8 * slot);
                         slot ^= 1u;
@@ -984,11 +911,11 @@ prefill_kernel(const AttnParams p, const Plan g)
                         left &= left - 1;
                     } while (left);
                     if (!ok) break;
-                    const int j0 = kt * KEYS + (ALT ? 0 : stream * COLS) + sub * CT;
-                    if (live && j0 + CT - 1 > vis_all) {
+                    const int j0 = kt * KEYS + (ALT ? 0 : stream * COLS);
+                    if (live && j0 + COLS - 1 > vis_all) {
                         const int n_vis = vis - j0;                            // my last visible column
 #pragma unroll
-                        for (int e = 0; e < CT / 2; ++e) {
+                        for (int e = 0; e < COLS / 2; ++e) {
                             if (2 * e > n_vis) S[e].x = NEG_BIG;
                             if (2 * e + 1 > n_vis) S[e].y = NEG_BIG;
                         }
@@ -998,7 +925,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                         if (live) {
                             float x0 = NEG_BIG, x1 = NEG_BIG;
 #pragma unroll
-                            for (int e = 0; e < CT / 2; e += 2) {
+                            for (int e = 0; e < COLS / 2; e += 2) {
                                 x0 = fmaxf(x0, fmaxf(S[e].x, S[e].y));
                                 x1 = fmaxf(x1, fmaxf(S[e + 1].x, S[e + 1].y));
                             }
@@ -1007,7 +934,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                                 const float2 nn = make_float2(-n, -n);
                                 float2 a0 = make_float2(0.f, 0.f), a1 = a0;
 #pragma unroll
-                                for (int e = 0; e < CT / 2; e += 2) {
+                                for (int e = 0; e < COLS / 2; e += 2) {
                                     const float2 y = add2(S[e], nn), z = add2(S[e + 1], nn);
                                     a0 = add2(a0, make_float2(ex2(y.x), ex2(y.y)));
                                     a1 = add2(a1, make_float2(ex2(z.x), ex2(z.y)));
@@ -1030,7 +957,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                         if constexpr (MODE == KV) {
                             const uint32_t p_row = base + g.off_p + (g.p_tiles == 2 ? stream * (BM * 128) : 0) + row * 128;
 #pragma unroll
-                            for (int blk = 0; blk < CT / 16; ++blk)
+                            for (int blk = 0; blk < COLS / 16; ++blk)
 #pragma unroll
                                 for (int y = 0; y < 2; ++y) {                  // chunk 2 blk + y: keys 16 blk + 4 b + 2 y + {0, 1}
                                     uint32_t w[4];
@@ -1041,7 +968,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                                         const float2 r = __half22float2(*reinterpret_cast<const __half2*>(&w[b]));
                                         lsum += r.x + r.y;   // the rounded values: the division normalises what was multiplied
                                     }
-                                    sts128(p_row + (((CT / 8 * sub + 2 * blk + y) ^ (row & 7)) << 4), w[0], w[1], w[2], w[3]);
+                                    sts128(p_row + (((2 * blk + y) ^ (row & 7)) << 4), w[0], w[1], w[2], w[3]);
                                 }
                         } else {
                             // code = min(rne(2^(S - m) / (s_P l)), 255): the product scaled by 2^-149 is rounded once, half to even, to the
@@ -1049,7 +976,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                             const float2 f2 = make_float2(f, f), k100 = make_float2(7.888609052210118e-31f, 7.888609052210118e-31f);   // 2^-100
                             const uint32_t p_row = base + g.off_p + row * 128;
 #pragma unroll
-                            for (int blk = 0; blk < CT / 32; ++blk) {          // 32 keys: word x has keys x + 8 b
+                            for (int blk = 0; blk < COLS / 32; ++blk) {          // 32 keys: word x has keys x + 8 b
                                 uint32_t w[8];
 #pragma unroll
                                 for (int e = 0; e < 4; ++e) {
@@ -1066,21 +993,21 @@ prefill_kernel(const AttnParams p, const Plan g)
                                         rsum = __dp4a(w[2 * e + k], 0x01010101u, rsum);
                                     }
                                 }
-                                const int c = 4 * stream + CT / 16 * sub + 2 * blk;
+                                const int c = 4 * stream + 2 * blk;
                                 sts128(p_row + ((c ^ (row & 7)) << 4), w[0], w[1], w[2], w[3]);
                                 sts128(p_row + (((c + 1) ^ (row & 7)) << 4), w[4], w[5], w[6], w[7]);
                             }
                             if (p.p_dbg && i < p.Tq) {                         // key k of the stream: byte (k & 31) / 8 of word k & 7 of block k / 32
                                 uint8_t* dst = p.p_dbg + (((int64_t)it.seq * p.H + it.h) * p.Tq + i) * p.Tk;
 #pragma unroll 1
-                                for (int k = 0; k < CT && j0 + k < p.Tk; ++k) {
-                                    const int c = 4 * stream + CT / 16 * sub + 2 * (k >> 5) + ((k & 7) >> 2);
+                                for (int k = 0; k < COLS && j0 + k < p.Tk; ++k) {
+                                    const int c = 4 * stream + 2 * (k >> 5) + ((k & 7) >> 2);
                                     dst[j0 + k] = (uint8_t)(lds32(p_row + ((c ^ (row & 7)) << 4) + 4 * (k & 3)) >> (8 * ((k & 31) >> 3)));
                                 }
                             }
                         }
                     }
-                    tc::fence_proxy_async();
+                    fence_proxy_async();
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(B_PFULL + stream));
                 }
@@ -1088,16 +1015,16 @@ prefill_kernel(const AttnParams p, const Plan g)
             if (!ok) break;
             // (a stream without a tile of its own has not waited for the previous item's sums to be read)
             if (ALT && it.n_kt == 1 && !mbar_sleep_warp(bar(B_OUT), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
-            s_sum[part * BM + row] = MODE == KV ? __float_as_uint(lsum) : rsum;
+            s_sum[stream * BM + row] = MODE == KV ? __float_as_uint(lsum) : rsum;
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(B_SUM));
         }
     }
 
     // ---------------------------------------------------------------- teardown
-    tc::tc_fence_before();
+    tc_fence_before();
     __syncthreads();
-    tc::tc_fence_after();
+    tc_fence_after();
     if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tmem) : "memory");
     if (tid == 0 && *s_abort && g.status) atomicExch(g.status, RPTQ_ERR_DEVICE_TIMEOUT);
 }
@@ -1121,10 +1048,10 @@ static int launch_one(const AttnParams& p, int zq_min, int zq_max, int units_k, 
     g.k_stage = atoms * KEYS * 128;
     g.off_v = g.off_k + 2 * g.k_stage;
     g.v_stage = units_v * 32 * 128;
-    g.pitch_k = raw_pitch_of(p.bits_k, units_k);
-    g.pitch_v = raw_pitch_of(p.bits_v, units_v);
+    g.pitch_k = raw_pitch(p.bits_k, units_k);
+    g.pitch_v = raw_pitch(p.bits_v, units_v);
     g.rawk_stage = MODE != KV && p.bits_k == 8 ? 0 : KEYS * g.pitch_k;
-    const int rest = BM * 128 + KEYS * g.pitch_v + 4 * KEYS * 4 + 2 * PARTS * BM * 8 + PARTS * BM * 4 + 512;
+    const int rest = BM * 128 + KEYS * g.pitch_v + 4 * KEYS * 4 + 2 * STREAMS * BM * 8 + STREAMS * BM * 4 + 512;
     constexpr int LIMIT = 226 * 1024;                     // (with 1 KiB for the alignment: the most a block may have)
     // a second packed key tile first (the copies of a tile then have a whole tile's time), then (KV) a probability tile for each
     // stream, then a second value tile
@@ -1139,8 +1066,8 @@ static int launch_one(const AttnParams& p, int zq_min, int zq_max, int units_k, 
     g.off_rawv = g.off_rawk + g.rawk_stages * g.rawk_stage;
     g.off_col = g.off_rawv + KEYS * g.pitch_v;
     g.off_ml = g.off_col + 4 * KEYS * 4;
-    g.off_sum = g.off_ml + 2 * PARTS * BM * 8;
-    g.off_bar = g.off_sum + PARTS * BM * 4;
+    g.off_sum = g.off_ml + 2 * STREAMS * BM * 8;
+    g.off_bar = g.off_sum + STREAMS * BM * 4;
     g.total = g.off_bar + 512;
     if (g.total > LIMIT) return RPTQ_ERR_UNSUPPORTED;
     // the output tile is staged in the V and P region (rows of a multiple of 128 bytes: see the staging stores)

@@ -1,13 +1,16 @@
-// Shared by the attention kernels: launch parameters, packed-row readers, small PTX wrappers, and the
-// host-side checks of per-head layouts.
+// Shared by the attention kernels: launch parameters, packed-row readers and conversions of codes, and the host-side checks of
+// per-head layouts.
 #pragma once
 #include <cuda_fp16.h>
 
 #include "rptq_internal.h"
+#include "tc.cuh"
 #include "unpack.cuh"
 
 namespace rptq {
 namespace attn {
+
+using namespace tc;
 
 constexpr int MAX_UNITS = 8;                 // units of 32 positions per head
 constexpr float NEG_BIG = -1.0e30f;
@@ -30,15 +33,6 @@ struct AttnParams {
     uint8_t* p_dbg;
 };
 
-__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
-// 16 bytes global -> shared without passing through registers; src_bytes = 0 writes zeros
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, int src_bytes)
-{
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(src_bytes) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 __device__ __forceinline__ float ex2(float x)
 {
     float y;
@@ -49,6 +43,32 @@ __device__ __forceinline__ uint32_t pack_half2(float a, float b)
 {
     const __half2 h = __floats2half2_rn(a, b);
     return *reinterpret_cast<const uint32_t*>(&h);
+}
+
+// The nibbles at bit B of the two halves of w as a pair of fp16 numbers n - 8 (B = 0, 4, 8, 12).
+template <int B>
+__device__ __forceinline__ uint32_t nib_half(uint32_t w)
+{
+    const uint32_t t = ((B <= 6 ? w << (6 - B) : w >> (B - 6)) & 0x03C003C0u) | 0x4C004C00u;      // 16 + n
+    const __half2 r = __hadd2(*reinterpret_cast<const __half2*>(&t), __float2half2_rn(-24.0f));
+    return *reinterpret_cast<const uint32_t*>(&r);
+}
+// The bytes at bit B of the two halves of w as a pair of fp16 numbers n - 128 (B = 0, 8).
+template <int B>
+__device__ __forceinline__ uint32_t byte_half(uint32_t w)
+{
+    const uint32_t t = ((w >> B) & 0x00FF00FFu) | 0x64006400u;                                    // 1024 + n
+    const __half2 r = __hadd2(*reinterpret_cast<const __half2*>(&t), __float2half2_rn(-1152.0f));
+    return *reinterpret_cast<const uint32_t*>(&r);
+}
+
+// Bytes per key row of a staged packed tile: the 16-byte chunks of a head's units (one more where the head's first unit need not start
+// on a boundary), rounded up to an odd number of chunks so that the eight rows (or four pairs of rows) a warp reads at once
+// lie in different banks.
+__host__ __device__ inline int raw_pitch(int bits, int units)
+{
+    const int c = (4 * bits * units + 15) / 16 + (bits == 3 ? 1 : 0);
+    return 16 * (c | 1);
 }
 
 // Unit `unit` of a packed row (`row` 4-byte aligned for 3-bit codes, 16-byte aligned otherwise) as 32 bytes.

@@ -159,16 +159,6 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
         ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
-// Asynchronous 16-byte global -> shared copy issued by an ordinary thread; `valid` false writes
-// zeros and reads nothing.
-__device__ __forceinline__ void cp_async16(uint32_t dst, const void* src, bool valid)
-{
-    const uint32_t n = valid ? 16u : 0u;
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(src), "r"(n) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 // The two tensor-core instructions below are executed by the WHOLE issuing warp in converged
 // control flow; elect.sync picks the one lane that issues. Measured on an operand-resident loop: a
 // tcgen05.mma issued from a branch that a single lane took costs the issuing thread ~120 clocks,
@@ -243,20 +233,6 @@ __host__ __device__ constexpr uint32_t instr_desc_bf16(int ncta)
 {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TILE_N >> 3) << 17) | ((uint32_t)((TILE_M * ncta) >> 4) << 24);
 }
-__device__ __forceinline__ float2 add2(float2 a, float2 b)
-{
-    float2 d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(reinterpret_cast<uint64_t&>(d))
-        : "l"(reinterpret_cast<uint64_t&>(a)), "l"(reinterpret_cast<uint64_t&>(b)));
-    return d;
-}
-__device__ __forceinline__ float2 mul2(float2 a, float2 b)
-{
-    float2 d;
-    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(reinterpret_cast<uint64_t&>(d))
-        : "l"(reinterpret_cast<uint64_t&>(a)), "l"(reinterpret_cast<uint64_t&>(b)));
-    return d;
-}
 // two fp32 values rounded to bfloat16 (nearest even): lo in bits 0-15, hi in bits 16-31
 __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi)
 {
@@ -286,32 +262,6 @@ __device__ __forceinline__ uint32_t nibbles_to_bf16(uint32_t w)
     uint32_t d;
     asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(d) : "r"((w & 0x000F000Fu) ^ 0x43084308u), "r"(0x43084308u));
     return d;
-}
-
-// packed fp32 pairs: one instruction, two independent IEEE results
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
-{
-    float2 d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(reinterpret_cast<uint64_t&>(d))
-        : "l"(reinterpret_cast<uint64_t&>(a)), "l"(reinterpret_cast<uint64_t&>(b)), "l"(reinterpret_cast<uint64_t&>(c)));
-    return d;
-}
-
-__device__ __forceinline__ void sts128(uint32_t addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
-{
-    asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-__device__ __forceinline__ uint16_t lds16(uint32_t addr)
-{
-    uint16_t v;
-    asm volatile("ld.shared.b16 %0, [%1];" : "=h"(v) : "r"(addr) : "memory");
-    return v;
-}
-__device__ __forceinline__ uint4 lds128(uint32_t addr)
-{
-    uint4 v;
-    asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
-    return v;
 }
 
 // ASYM: the weights carry one scale and one zero point per (cluster, output channel) (Appendix,
@@ -1242,7 +1192,7 @@ static int launch_gemm(const rptq_layout_t* Lin, const void* a_codes, int M, con
         SmallMParams q{};
         q.a = p.a_codes; q.a_row_bytes = p.a_row_bytes; q.M = M; q.K_pad = Lin->K_pad; q.n_units = Lin->n_units; q.n_kb = p.n_kb;
         q.w = p.w_codes; q.n_wtiles = p.n_wtiles;
-        q.step_flags = Lin->d_step_flags; q.unit_cluster = Lin->d_unit_cluster; q.unit_sz = Lin->d_unit_sz; q.cl_sz = Lin->d_cl_sz; q.g = Lin->g;
+        q.step_flags = Lin->d_step_flags; q.unit_sz = Lin->d_unit_sz; q.cl_sz = Lin->d_cl_sz; q.g = Lin->g;
         q.corr = corr; q.s_w = s_w; q.wsum = wsum; q.ld_w = ld_w; q.bias = p.bias;
         q.N = N; q.act = act; q.y_dtype = y_dtype; q.y = y; q.ldy = ldy; q.status = status;
         return smallm::launch(q, Lin->bits, dev, st);

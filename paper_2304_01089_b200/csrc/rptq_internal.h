@@ -66,7 +66,7 @@ namespace rptq {
 struct SmallMParams {
     const uint8_t* a; int64_t a_row_bytes; int M, K_pad, n_units, n_kb;
     const uint8_t* w; int n_wtiles;
-    const uint8_t* step_flags; const int32_t* unit_cluster; const float2* unit_sz; const float* cl_sz; int g;
+    const uint8_t* step_flags; const float2* unit_sz; const float* cl_sz; int g;
     const float* corr; const float* s_w; const int32_t* wsum; int64_t ld_w; const float* bias;
     int N, act, y_dtype; void* y; int64_t ldy; int* status;
     int tiles_per_block;                     // weight tiles of 128 channels a block takes (set by the launch)
