@@ -136,7 +136,7 @@ def _step(sites, binding, M, events=None):
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum of one FC1 launch, from the 512-token ncu capture of the
-# current kernel (profiles/cluster_gemm_opt66b_fc1_tokens512.txt: 191.5 MB read, 23.4 MB written, part of
+# current kernel (profiles/cluster_gemm_512x9216x36864.txt: 191.3 MB read, 22.2 MB written, part of
 # the output still in L2) scaled to 4096 tokens: weights, Wsum and s_w (191.1 MB) are read once whatever
 # the token count; codes (1.94 MB per 512 tokens) and the fp16 output (37.75 MB per 512 tokens) grow with it.
 FC1_DRAM_BYTES_PER_LAUNCH = int(191.1e6 + 8 * (1.94e6 + 37.75e6))
@@ -383,7 +383,7 @@ def run_ours(args):
                          "peak_int8_measured": int8_peak,
                          "frac_of_int8_measured": None if int8_peak is None else achieved / int8_peak,
                          "frac_of_int8_vendor_4500": achieved / 4500.0,
-                         "pipe_cycles_source": "sm__pipe_tensor_cycles_active in profiles/cluster_gemm_opt66b_fc1_tokens512.txt"},
+                         "pipe_cycles_source": "sm__pipe_tensor_cycles_active in profiles/cluster_gemm_512x9216x36864.txt"},
             "ln": {"bound": "hbm", "kernel": "ln_reorder_quant_kernel<3> 4096x9216", "achieved": ln_gbs, "peak": peaks["hbm"], "unit": "GB/s",
                    "frac": ln_gbs / peaks["hbm"], "frac_of_8TBps": ln_gbs / 8000.0, "bytes": ln_bytes,
                    "us": float(np.mean(ln_ms[1])) * 1e3},

@@ -286,8 +286,8 @@ int64_t rptq_weight_codes_bytes(int K_pad, int64_t N_pad);
 /*
  * Kernels never spin without a limit: a wait that runs out records RPTQ_ERR_DEVICE_TIMEOUT in a
  * device status word, lets the block drain and return, and leaves the output undefined. This call
- * synchronises the current device, returns that device's word in *status (RPTQ_OK if nothing
- * happened) and clears it. Each device has its own word.
+ * synchronises the current device, returns the current context's word in *status (RPTQ_OK if
+ * nothing happened) and clears it. Each device has its own word, and each further context of it.
  */
 int rptq_get_device_status(int* status);
 

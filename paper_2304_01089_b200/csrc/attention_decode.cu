@@ -33,7 +33,7 @@
 //   - outputs: V^T is operand A (positions x keys; pairs or quads of keys are brought together with byte
 //     permutes on the packed words), the probabilities operand B.
 // Measured (72 heads of 128 channels, eight sequences, one query, 2011 keys, 4-bit cache, KV-only):
-// 1072 us before (prefill kernel), 69 us here.
+// 1072 us before (prefill kernel), 65 to 67 us here.
 #include <type_traits>
 
 #include "attn_common.cuh"

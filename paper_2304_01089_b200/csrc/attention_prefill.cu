@@ -33,11 +33,12 @@
 //
 // Measured, us, against a mma.sync kernel with 64 (KV: 128) queries per block (72 heads of 128 channels, four clusters each,
 // causal, two sequences of 2048 tokens): 3 bits 2321 -> 735; KV, 32 heads, three sequences, 1100 queries on 1337 keys, 4 bits
-// 945 -> 342. What bounds it is the instruction cache before any pipe: five roles run side by side, and a warp on its own executes
-// one instruction per 6 to 10 clocks (scheduler slots 48 % busy). Whatever shortens the code that runs at the same time helps
-// more than shortening a chain: the compiler told that the warp index is uniform 916 -> 790 (93 -> 83 KB of code), the output
-// rows' store loops not unrolled 790 -> 772; a first cluster's drain of its own (two copies of the loop) 790 -> 830.
-// The order in which items are dealt out: see item_index (767 -> 730).
+// 945 -> 344. What bounds it is the latency of the hand-overs between the roles: of the 9.7 warp cycles an issue (37 heads, 2048
+// tokens), 3.7 are long scoreboards (tensor-memory loads, barrier waits), 1.7 fixed latencies, 0.4 instruction fetch (cache-only
+// 4.0, 1.5, 0.9); issue slots are 52 % busy, the tensor pipe 11 %. Code that runs at the same time is worth keeping short all the
+// same: the compiler told that the warp index is uniform 916 -> 790 (93 -> 83 KB of code), the output rows' store loops not
+// unrolled 790 -> 772; a first cluster's drain of its own (two copies of the loop) 790 -> 830. The order in which items are dealt
+// out: see item_index (767 -> 735).
 #include <type_traits>
 
 #include "attn_common.cuh"

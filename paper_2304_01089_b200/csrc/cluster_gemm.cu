@@ -29,7 +29,7 @@
 //   warps 2-3   column tables: zero-point correction, s_w and bias of the columns of the tile to come, and
 //               with per-cluster weight parameters the coefficients of each cluster's drain (they are
 //               the same for every token row: formed once per block instead of in every epilogue thread.
-//               1024 x 4096 x 16384, 16 clusters, LayerNorm included: 428 -> 147 us, 129 with all that follows)
+//               1024 x 4096 x 16384, 16 clusters, LayerNorm included: 428 -> 147 us, 130 with all that follows)
 //   warps 8-15  (MODE_DEQ: 12-19) epilogue: drain a finished cluster's accumulator (tcgen05.ld), add s_c * acc into
 //               fp32 running sums held in registers while the next cluster's MMAs run; after the
 //               last cluster apply the zero-point correction, s_w, bias, activation, and store
@@ -1180,7 +1180,7 @@ static int launch_gemm(const rptq_layout_t* Lin, const void* a_codes, int M, con
     // The tiles of the last round, when they are at most half (a quarter) as many as there are blocks (pairs) to work on them, are
     // cut into two (four) strips of columns: the round then takes the time of a strip, about two thirds (half) of a tile's (a
     // strip's token codes are unpacked all the same). 200 x 9216 x 27648: 90 -> 86 us; 1024 x 4096 x 16384 with clustered weights
-    // 136 -> 129; calls with fewer tiles than blocks up to 1.4 times as fast. With more tiles left than half the blocks a cut
+    // 136 -> 130; calls with fewer tiles than blocks up to 1.4 times as fast. With more tiles left than half the blocks a cut
     // would only add a round. Not four for re-quantised outputs (a warp writes its columns in pieces of 64).
     const int slots = n_sm / ncta, rest = n_tiles % slots;
     p.split = rest == 0 ? 0 : 4 * rest <= slots && y_dtype != RPTQ_OUT_CODES ? 2 : 2 * rest <= slots ? 1 : 0;

@@ -6,9 +6,9 @@
 // With so few tokens the product is bound by reading the packed weights once (N * K_pad / 2 bytes);
 // the 128 x 256 tensor-memory tile of the large kernel would be almost empty and its unpacking of
 // the weights to bytes in shared memory costs more than the reading. Here:
-//   - a block owns 256 output channels (two 128-row weight tiles). A producer warp streams their
-//     8 KiB tiles, K block after K block, into an eight-stage shared-memory ring with cp.async.bulk
-//     (ordinary loads keep too few bytes in flight per SM to fill the memory pipe with a read-only
+//   - a block owns 256 output channels (two 128-row weight tiles), 128 where there are no more tiles than SMs. A producer
+//     warp streams their 8 KiB tiles, K block after K block, into an eight-stage shared-memory ring by tensor-map copies of
+//     64-byte rows (ordinary loads keep too few bytes in flight per SM to fill the memory pipe with a read-only
 //     stream);
 //   - the tokens' codes sit in shared memory as 4-bit nibbles in the packed format of the 4-bit
 //     codes (16 x K_pad / 2 bytes), written once per block;
