@@ -29,7 +29,7 @@
 //   warps 2-3   column tables: zero-point correction, s_w and bias of the columns of the tile to come, and
 //               with per-cluster weight parameters the coefficients of each cluster's drain (they are
 //               the same for every token row: formed once per block instead of in every epilogue thread.
-//               1024 x 4096 x 16384, 16 clusters, LayerNorm included: 428 -> 147 us, 130 with all that follows)
+//               1024 x 4096 x 16384, 16 clusters, LayerNorm included: 428 -> 147 us, 113 with all that follows)
 //   warps 8-15  (MODE_DEQ: 12-19) epilogue: drain a finished cluster's accumulator (tcgen05.ld), add s_c * acc into
 //               fp32 running sums held in registers while the next cluster's MMAs run; after the
 //               last cluster apply the zero-point correction, s_w, bias, activation, and store
@@ -71,18 +71,21 @@ constexpr int WTILE_BYTES = 8192;                        // one packed weight ti
 
 __host__ __device__ constexpr int w_rows(int ncta) { return TILE_N / ncta; }           // weight rows staged per CTA
 // packed weight stages; the single-CTA variant (at most 128 tokens) is a weight stream and takes what shared memory is left
-__host__ __device__ constexpr int n_p_stages(int ncta, int bits, int mode) { return ncta == 2 ? 4 : mode == MODE_DEQ ? 3 : (bits == 3 ? 5 : 4); }
+__host__ __device__ constexpr int n_p_stages(int ncta, int bits, int mode) 
+{
+    if (ncta == 2) return mode == MODE_DEQ && bits == 8 ? 3 : 4;
+    return mode == MODE_DEQ || (mode == MODE_ASYM && bits == 8) ? 3 : bits == 3 ? 5 : 4;
+}
 __host__ __device__ constexpr int n_u_stages(int ncta, bool a8) { return ncta == 2 ? (a8 ? 5 : 4) : 2; }   // operand stages
 // ring of packed activation K blocks fetched ahead by the unpack threads: one slot per token row
-// per K block; the pitch is an odd number of 16-byte units so that the threads' vector reads of
-// their own slots do not collide in the banks
-__host__ __device__ constexpr int a_slot_pitch(int bits, int mode) { return mode == MODE_DEQ ? (bits == 8 ? 80 : 48) : bits == 3 ? 48 : 16 * bits + 16; }
-__host__ __device__ constexpr int n_a_stages(int bits, int mode) { return bits == 8 ? 2 : mode == MODE_DEQ ? 3 : 4; }
+// per K block; the pitch is an odd number of 16-byte units (4 bits: four, and the pieces of a slot exchanged) so that the threads'
+// vector reads of their own slots do not collide in the banks
+__host__ __device__ constexpr int a_slot_pitch(int bits, int mode) { return mode == MODE_DEQ ? (bits == 8 ? 80 : 48) : bits == 3 ? 48 : bits == 4 ? 64 : 16 * bits + 16; }
+__host__ __device__ constexpr int n_a_stages(int ncta, int bits, int mode) { return bits == 8 || (ncta == 1 && bits == 3 && mode != MODE_DEQ) ? 2 : mode == MODE_DEQ ? 3 : 4; }
 
 struct SmemLayout {
-    int u_stage, p_stage, a_stage, off_p, off_a, off_flags, off_seg_scale, off_seg_buf, off_tab, off_seg_tab, off_seg_cl, off_stage, off_bar, total;
+    int u_stage, p_stage, a_stage, out_row, off_p, off_a, off_flags, off_seg_scale, off_seg_buf, off_tab, off_seg_tab, off_seg_cl, off_stage, off_bar, total;
 };
-constexpr int STAGE_OUT = 1024;                          // bytes of the output staging buffer of an epilogue warp
 constexpr int SEG_SLOTS = 2;                             // ASYM: clusters whose column tables are held at a time
 __host__ __device__ constexpr SmemLayout smem_layout(int ncta, int bits, bool a8, int mode)
 {
@@ -93,14 +96,16 @@ __host__ __device__ constexpr SmemLayout smem_layout(int ncta, int bits, bool a8
     s.a_stage = a8 ? 0 : n_unpack_warps(mode) / GROUP_WARPS * TILE_M * a_slot_pitch(bits, mode);      // 8-bit activations go straight to the operand stage
     s.off_p = n_u_stages(ncta, a8) * s.u_stage;
     s.off_a = s.off_p + n_p_stages(ncta, bits, mode) * s.p_stage;
-    s.off_flags = s.off_a + n_a_stages(bits, mode) * s.a_stage;
+    s.off_flags = s.off_a + n_a_stages(ncta, bits, mode) * s.a_stage;
     s.off_seg_scale = s.off_flags + 2048;
     s.off_seg_buf = s.off_seg_scale + (asym ? 0 : kMaxGemmSegments * 4);
     s.off_tab = s.off_seg_buf + kMaxGemmSegments;
     s.off_seg_tab = s.off_tab + 2 * 3 * TILE_N * 4;
     s.off_seg_cl = s.off_seg_tab + (asym ? SEG_SLOTS * 2 * TILE_N * 4 : 0);
     s.off_stage = s.off_seg_cl + (asym ? kMaxGemmSegments * 2 : 0);
-    s.off_bar = s.off_stage + N_EPI_WARPS * STAGE_OUT;
+    // output staging buffer of an epilogue warp: 32 rows of 64 or 128 bytes, as there is room for
+    s.out_row = s.off_stage + N_EPI_WARPS * 32 * 128 + 320 + 1024 <= 227 * 1024 ? 128 : 64;
+    s.off_bar = s.off_stage + N_EPI_WARPS * 32 * s.out_row;
     s.total = s.off_bar + 320;
     return s;
 }
@@ -201,6 +206,30 @@ __device__ __forceinline__ void tc_mma_i8(uint32_t d_tmem, uint64_t a_desc, uint
             ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
     }
 }
+// The four products of a K block inside one cluster, and the commit that frees its operand stage, with one election: a0, b0 the low words of
+// the first step's descriptors (the high words are the same for every tile; the start address counts 16-byte units, 32 bytes a step)
+constexpr uint32_t DESC_HI = (uint32_t)(1024 >> 4) | (1u << 14) | (2u << 29);       // of smem_desc_sw128
+template <int NCTA>
+__device__ __forceinline__ void tc_block_i8(uint32_t d_tmem, uint32_t a0, uint32_t b0, uint32_t idesc, uint32_t bar)
+{
+#define RPTQ_BLOCK(GROUP, COMMIT)                                                                                    \
+    "{\n\t.reg .pred q, t;\n\t.reg .b64 da, db;\n\t.reg .b32 a, b;\n\t"                                               \
+    "elect.sync _|q, 0xffffffff;\n\tsetp.eq.u32 t, 0, 0;\n\t"                                                         \
+    "mov.b64 da, {%1, %4};\n\tmov.b64 db, {%2, %4};\n\t"                                                              \
+    "@q tcgen05.mma.cta_group::" GROUP ".kind::i8 [%0], da, db, %3, t;\n\t"                                           \
+    "add.u32 a, %1, 2;\n\tadd.u32 b, %2, 2;\n\tmov.b64 da, {a, %4};\n\tmov.b64 db, {b, %4};\n\t"                      \
+    "@q tcgen05.mma.cta_group::" GROUP ".kind::i8 [%0], da, db, %3, t;\n\t"                                           \
+    "add.u32 a, %1, 4;\n\tadd.u32 b, %2, 4;\n\tmov.b64 da, {a, %4};\n\tmov.b64 db, {b, %4};\n\t"                      \
+    "@q tcgen05.mma.cta_group::" GROUP ".kind::i8 [%0], da, db, %3, t;\n\t"                                           \
+    "add.u32 a, %1, 6;\n\tadd.u32 b, %2, 6;\n\tmov.b64 da, {a, %4};\n\tmov.b64 db, {b, %4};\n\t"                      \
+    "@q tcgen05.mma.cta_group::" GROUP ".kind::i8 [%0], da, db, %3, t;\n\t"                                           \
+    "@q tcgen05.commit.cta_group::" GROUP ".mbarrier::arrive::one.shared::cluster" COMMIT "\n\t}"
+    if constexpr (NCTA == 1)
+        asm volatile(RPTQ_BLOCK("1", ".b64 [%5];") ::"r"(d_tmem), "r"(a0), "r"(b0), "r"(idesc), "r"(DESC_HI), "r"(bar) : "memory");
+    else
+        asm volatile(RPTQ_BLOCK("2", ".multicast::cluster.b64 [%5], %6;") ::"r"(d_tmem), "r"(a0), "r"(b0), "r"(idesc), "r"(DESC_HI), "r"(bar), "h"((uint16_t)3) : "memory");
+#undef RPTQ_BLOCK
+}
 // bf16 x bf16 -> fp32, same operand layout and issue pattern as tc_mma_i8 (K = 16 elements = 32 bytes)
 template <int NCTA>
 __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc, uint32_t accumulate)
@@ -220,6 +249,24 @@ __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, ui
             "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}"
             ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
     }
+}
+// 16 lanes x 32 columns: v[4 j + 2 r + c] is row lane / 4 + 8 r, column 8 j + 2 (lane % 4) + c
+__device__ __forceinline__ void tc_ld16x4(uint32_t taddr, uint32_t (&v)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+        : "r"(taddr) : "memory");
+}
+// four 8 x 8 matrices of 16-bit values, matrix j's rows at the addresses that lanes 8 j .. 8 j + 7 name
+__device__ __forceinline__ void stmatrix4(uint32_t addr, const uint32_t (&f)[4])
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(f[0]), "r"(f[1]), "r"(f[2]), "r"(f[3]) : "memory");
+}
+__device__ __forceinline__ void sts64(uint32_t addr, float2 v)
+{
+    asm volatile("st.shared.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(v.x), "f"(v.y) : "memory");
 }
 // kind::i8, D = s32, A = unsigned 8-bit (activation codes), B = signed 8-bit (weights), both
 // K-major, M = 128 per CTA, N = 256.
@@ -456,10 +503,7 @@ cluster_gemm_kernel(const Params p)
                     if (f4 == 0u || f4 == 0x01010101u * STEP_BUF) {
                         // four steps inside one cluster
                         const uint32_t d_tmem = tmem_base + (f4 ? TILE_N : 0);
-                        tc_mma_i8<NCTA>(d_tmem, ad, wd, idesc, 1u);
-                        tc_mma_i8<NCTA>(d_tmem, ad + 2, wd + 2, idesc, 1u);
-                        tc_mma_i8<NCTA>(d_tmem, ad + 4, wd + 4, idesc, 1u);
-                        tc_mma_i8<NCTA>(d_tmem, ad + 6, wd + 6, idesc, 1u);
+                        tc_block_i8<NCTA>(d_tmem, (uint32_t)ad, (uint32_t)wd, idesc, bar(B_UEMPTY + s));
                     } else {
 #pragma unroll
                         for (int j = 0; j < 4; ++j) {
@@ -483,8 +527,8 @@ cluster_gemm_kernel(const Params p)
                             }
                         }
                         if (!ok) break;
+                        tc_commit<NCTA>(bar(B_UEMPTY + s));  // the stage may be overwritten once these MMAs have read it
                     }
-                    tc_commit<NCTA>(bar(B_UEMPTY + s));      // the stage may be overwritten once these MMAs have read it
                     f4 = f4_next;
             }
             if (!ok) {
@@ -666,7 +710,7 @@ cluster_gemm_kernel(const Params p)
             // store 287. Half of what is left is still the conversion (tensor pipe 55 % busy, ALU pipe 50 %).
             const int grp = warp >= UNPACK_WARP0 + GROUP_WARPS ? 1 : 0;
             constexpr int CH = BITS == 8 ? 4 : 2;            // 16-byte pieces of a row's K block that hold the two units
-            constexpr int N_A = n_a_stages(BITS, MODE), PITCH = a_slot_pitch(BITS, MODE);
+            constexpr int N_A = n_a_stages(NCTA, BITS, MODE), PITCH = a_slot_pitch(BITS, MODE);
             static_assert(PITCH == 16 * CH + 16, "slot");
             const uint32_t a_ring0 = smem_base + SL.off_a + grp * TILE_M * PITCH, a_ring = a_ring0 + ut * PITCH;
             uint32_t d_off[CH], s_off[CH];
@@ -778,16 +822,17 @@ cluster_gemm_kernel(const Params p)
         // 32 / BITS rows, not 32: the load path looks up one cache line per row touched, and with one
         // row per lane those look-ups, not the bytes, set the pace. A row's chunks are copied by
         // lanes of the row owner's own warp, so a __syncwarp after the wait is all the hand-over needs.
-        constexpr int N_A = n_a_stages(BITS, MODE), PITCH = a_slot_pitch(BITS, MODE);
+        constexpr int N_A = n_a_stages(NCTA, BITS, MODE), PITCH = a_slot_pitch(BITS, MODE);
         const uint32_t a_ring0 = smem_base + SL.off_a;
         const uint32_t a_ring = a_ring0 + ut * PITCH;
+        auto slot_sw = [](int r) { return BITS == 4 ? (r >> 1) & 3 : 0; };      // (four pieces a row: exchanged in place of a pad)
         uint32_t d_off[BITS], s_off[BITS];               // where my chunks go in a ring stage / come from in the tile's rows
         int r_of[BITS];                                  // their rows within the tile
 #pragma unroll
         for (int i = 0; i < BITS; ++i) {
             const int c = 32 * i + lane;
             r_of[i] = (ut & ~31) + c / BITS;
-            d_off[i] = (uint32_t)r_of[i] * PITCH + 16u * (uint32_t)(c % BITS);
+            d_off[i] = (uint32_t)r_of[i] * PITCH + 16u * (uint32_t)((c % BITS) ^ slot_sw(r_of[i]));
             s_off[i] = (uint32_t)r_of[i] * (uint32_t)p.a_row_bytes + 16u * (uint32_t)(c % BITS);
         }
         int rows_left = 0;                               // rows of the tile being fetched that exist
@@ -826,7 +871,7 @@ cluster_gemm_kernel(const Params p)
                 uint32_t raw[4 * BITS];
 #pragma unroll
                 for (int j = 0; j < BITS; ++j) {
-                    const uint4 v = lds128(slot + 16 * j);
+                    const uint4 v = lds128(slot + 16 * (j ^ slot_sw(ut)));
                     raw[4 * j] = v.x; raw[4 * j + 1] = v.y; raw[4 * j + 2] = v.z; raw[4 * j + 3] = v.w;
                 }
 #pragma unroll
@@ -880,7 +925,12 @@ cluster_gemm_kernel(const Params p)
         uint32_t n_tile_done = 0;
         uint32_t par = 0;                    // bit b: parity of how many clusters of accumulator b I have drained
         uint32_t n_seg_done = 0;                     // ASYM: clusters drained so far, over all tiles
-        float2 R[64];                                // running sums of columns 2 i, 2 i + 1
+        // Running sums, in the layout of the 16-lane tensor-memory loads: my rows of the warp's 32 are 16 h + lane / 4 + 8 r, my
+        // columns 8 i + 2 (lane % 4) + {0, 1}, R[(i / 4 * 2 + h) * 8 + i % 4 * 2 + r]. With a thread per row and all 128 columns instead,
+        // what belongs to a column is read by every thread, and a warp-wide load of 16 bytes takes four clocks of the SM's shared-memory
+        // port even where all lanes read the same: 64 a drain of clustered weights (2048 of its 2125 clocks), 96 a tile for the
+        // tables of the outputs. Here a load serves four rows.
+        float2 R[64];
         for (int t = pair_id; t < p.n_items; t += n_pairs, ++n_tile_done) {
             int mt, n0;
             const int sh = item_of(t, mt, n0), half_cols = 128 >> sh;      // columns of my half
@@ -891,11 +941,15 @@ cluster_gemm_kernel(const Params p)
             const bool live = m0 + 32 * q < p.M;
 #pragma unroll
             for (int i = 0; i < 64; ++i) R[i] = make_float2(0.f, 0.f);
-            // ASYM: my token's code sum of the cluster to come
-            const int32_t* xs_row = nullptr;
-            int xs_next = 0;
+            // ASYM: my tokens' code sums of the cluster to come (rows past the last token read the last one's)
+            const int32_t* xs_row[4] = {nullptr, nullptr, nullptr, nullptr};
+            int xs_next[4] = {0, 0, 0, 0};
             if constexpr (ASYM) {
-                if (m0 + 32 * q + lane < p.M) { xs_row = p.xsum + (int64_t)(m0 + 32 * q + lane) * p.g; xs_next = xs_row[s_seg_cl[0]]; }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    xs_row[i] = p.xsum + (int64_t)min(m0 + 32 * q + (lane >> 2) + 8 * i, p.M - 1) * p.g;
+                    xs_next[i] = xs_row[i][s_seg_cl[0]];
+                }
             }
             for (int sgi = 0; sgi < (DEQ ? 1 : p.n_seg); ++sgi) {
                 const uint32_t buf = DEQ ? (n_tile_done & 1u) : (uint32_t)s_seg_buf[sgi];
@@ -905,169 +959,219 @@ cluster_gemm_kernel(const Params p)
                 const float sc = ASYM ? 0.f : s_seg_scale[sgi];
                 const float2 sc2 = make_float2(sc, sc);
                 const uint32_t seg_slot = n_seg_done % SEG_SLOTS;
-                const float4* seg_tab = s_seg_tab + seg_slot * (TILE_N / 2) + (h * half_cols >> 1);
-                float2 xs2 = make_float2(0.f, 0.f);
+                const float4* seg_tab = s_seg_tab + seg_slot * (TILE_N / 2) + (h * half_cols >> 1) + (lane & 3);
+                float xs[4] = {0.f, 0.f, 0.f, 0.f};
                 if constexpr (ASYM) {
                     mbar_wait(bar(B_SEGFULL + seg_slot), (n_seg_done / SEG_SLOTS) & 1, s_abort);
                     ++n_seg_done;
-                    const float x = (float)xs_next;
-                    xs2 = make_float2(x, x);
-                    if (xs_row && sgi + 1 < p.n_seg) xs_next = xs_row[s_seg_cl[sgi + 1]];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        xs[i] = (float)xs_next[i];
+                        if (sgi + 1 < p.n_seg) xs_next[i] = xs_row[i][s_seg_cl[sgi + 1]];
+                    }
                 }
                 const uint32_t taddr = tmem_base + ((uint32_t)(32 * q) << 16) + buf * TILE_N + h * half_cols;
                 if (live && !DEQ) {
-                uint32_t va[16], vb[16];
-                tc_ld16(taddr, va);
-                // R += s_c * acc, two columns per packed fused multiply-add
-                auto accumulate = [&](const uint32_t (&v)[16], int c0) {
-                    if constexpr (ASYM) {
-                        // R += s^X_c s^W_c[n] / 16 (acc' - 16 (z^W_c[n] - 8) xsum), coefficients of two columns per load
+                // R += s_c * acc, two columns per packed fused multiply-add: 32 columns of 16 rows (half hh of the warp's). Both halves are asked
+                // for at once and, with clustered weights, their coefficients before the wait for them: a wait in the middle has the next
+                // load's latency behind it (1024 x 4096 x 16384, 16 clusters: 125 -> 112 us).
+                auto accumulate = [&](const uint32_t (&v)[16], const float4 (&k)[4], int jc, int hh) {
 #pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            const float4 k = seg_tab[c0 + i];
-                            const float2 t = fma2(make_float2(k.z, k.w), xs2, make_float2((float)(int)v[2 * i], (float)(int)v[2 * i + 1]));
-                            R[c0 + i] = fma2(make_float2(k.x, k.y), t, R[c0 + i]);
+                    for (int j = 0; j < 4; ++j) {
+                        float2* r = R + (jc * 2 + hh) * 8 + 2 * j;
+                        const float2 a0 = make_float2((float)(int)v[4 * j], (float)(int)v[4 * j + 1]), a1 = make_float2((float)(int)v[4 * j + 2], (float)(int)v[4 * j + 3]);
+                        if constexpr (ASYM) {
+                            // R += s^X_c s^W_c[n] / 16 (acc' - 16 (z^W_c[n] - 8) xsum)
+                            const float2 kz = make_float2(k[j].z, k[j].w), ks = make_float2(k[j].x, k[j].y);
+                            r[0] = fma2(ks, fma2(kz, make_float2(xs[2 * hh], xs[2 * hh]), a0), r[0]);
+                            r[1] = fma2(ks, fma2(kz, make_float2(xs[2 * hh + 1], xs[2 * hh + 1]), a1), r[1]);
+                        } else {
+                            r[0] = fma2(sc2, a0, r[0]);
+                            r[1] = fma2(sc2, a1, r[1]);
                         }
-                    } else {
-#pragma unroll
-                        for (int i = 0; i < 8; ++i)
-                            R[c0 + i] = fma2(sc2, make_float2((float)(int)v[2 * i], (float)(int)v[2 * i + 1]), R[c0 + i]);
                     }
                 };
 #pragma unroll
-                for (int ch = 0; ch < 8; ch += 2) {
+                for (int jc = 0; jc < 4; ++jc) {
+                    uint32_t va[16], vb[16];
+                    float4 k[4];
+                    tc_ld16x4(taddr + 32 * jc, va);
+                    tc_ld16x4(taddr + (16u << 16) + 32 * jc, vb);
+                    if constexpr (ASYM) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) k[j] = seg_tab[(jc * 4 + j) * 4];
+                    }
                     tc_wait_ld();
-                    tc_ld16(taddr + (ch + 1) * 16, vb);
-                    accumulate(va, ch * 8);
-                    tc_wait_ld();
-                    const bool more = ch + 2 < 8 && 16 * (ch + 2) < half_cols;
-                    if (more) tc_ld16(taddr + (ch + 2) * 16, va);
-                    accumulate(vb, (ch + 1) * 8);
+                    const bool more = jc < 3 && 32 * (jc + 1) < half_cols;
+                    if (!more) {
+                        // all of it has been read: the accumulator goes back before the last sums are formed
+                        tc_fence_before();
+                        __syncwarp();
+                        if (lane == 0) arrive_leader(bar(B_ACCEMPTY + buf));
+                    }
+                    accumulate(va, k, jc, 0);
+                    accumulate(vb, k, jc, 1);
                     if (!more) break;
                 }
                 }
                 if constexpr (DEQ) break;                    // (the sums are read as the outputs are formed)
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) {
-                    if constexpr (ASYM) mbar_arrive(bar(B_SEGEMPTY + seg_slot));
-                    arrive_leader(bar(B_ACCEMPTY + buf));
+                if (ASYM || !live) {
+                    __syncwarp();
+                    if (lane == 0) {
+                        if constexpr (ASYM) mbar_arrive(bar(B_SEGEMPTY + seg_slot));
+                        if (!live) arrive_leader(bar(B_ACCEMPTY + buf));
+                    }
                 }
             }
             mbar_wait(bar(B_TAB + (n_tile_done & 1)), (n_tile_done >> 1) & 1, s_abort);
-            // y = s_w * (R - corr) + bias, activation, store. A thread holds 128 columns of one row: stored from there, every
-            // instruction of a warp touches 32 rows with 16 bytes each. Pieces of 32 bytes per row (one memory sector) are
-            // exchanged through a small buffer of the warp instead, and leave as whole sectors of 16 rows
-            // (1999 x 2048 x 6144, 8 bits, fp32 out: 70.5 -> 59.4 us with the LayerNorm; 4096 x 9216 x 36864, fp16 out: 1455 -> 1435).
+            // y = s_w * (R - corr) + bias, activation, store. Rows leave through a buffer of the warp, in pieces of 64 or 128 bytes a row: whole
+            // memory sectors, and few hand-overs between lanes (1999 x 2048 x 6144, 8 bits, fp32 out, with the LayerNorm: stores of a lane's
+            // own 16 bytes 70 us, pieces of 32 bytes 55, these 50.5)
             if (live) {
                 const int mw = m0 + 32 * q, nb = n0 + h * half_cols;           // my warp's first row, my first column
-                const float4* t_corr = reinterpret_cast<const float4*>(tab + h * half_cols);
-                const float4* t_sw = t_corr + TILE_N / 4;
-                const float4* t_bs = t_sw + TILE_N / 4;
+                const float2* t_corr = reinterpret_cast<const float2*>(tab + h * half_cols) + (lane & 3);
+                const float2* t_sw = t_corr + TILE_N / 2;
+                const float2* t_bs = t_sw + TILE_N / 2;
                 const bool relu = p.act == RPTQ_ACT_RELU;
-                const uint32_t stage = smem_base + SL.off_stage + ew * STAGE_OUT;
-                // my row's two 16-byte pieces, and the piece that I store: row lane / 2 (+ 16), piece lane & 1. Rows 4 to 7 of every eight
-                // have their pieces exchanged (no bank conflicts)
-                const uint32_t put0 = stage + lane * 32 + ((lane & 4) << 2), put1 = put0 ^ 16u;
-                const uint32_t get = stage + (lane >> 1) * 32 + ((((lane & 1) ^ ((lane >> 3) & 1))) << 4);
-                auto exchange = [&](uint4 a, uint4 b, uint8_t* dst, int64_t row_bytes, int n_bytes) {   // dst: the warp's first row; n_bytes valid of 32
+                // piece j (16 bytes) of row r lies at j ^ sw(r): neither what a warp puts nor what it reads in one instruction meets in a bank
+                constexpr int OUT_ROW = SL.out_row, PIECES = OUT_ROW / 16, ROWS_I = 32 / PIECES;          // ROWS_I: rows that a warp-wide access covers
+                const uint32_t stage = smem_base + SL.off_stage + ew * 32 * OUT_ROW;
+                auto sw_f16 = [](int r) { return OUT_ROW == 128 ? r & 7 : (r >> 1) & 3; };                  // 16 bytes of eight rows at a time
+                auto sw_f32 = [](int r) { return OUT_ROW == 128 ? (r & 3) << 1 : (r & 2); };                // 32 bytes of four rows at a time
+                auto store = [&](auto sw, uint8_t* dst, int64_t row_bytes, int n_bytes) {   // dst: the warp's first row; n_bytes valid of OUT_ROW
                     __syncwarp();
-                    sts128(put0, a.x, a.y, a.z, a.w);
-                    sts128(put1, b.x, b.y, b.z, b.w);
-                    __syncwarp();
-                    const int piece = 16 * (lane & 1), left = n_bytes - piece;
+                    const int j = lane % PIECES, r0 = lane / PIECES, left = n_bytes - 16 * j, rows = p.M - mw;
+                    uint8_t* d = dst + r0 * row_bytes + 16 * j;
+                    uint4 v[PIECES];
 #pragma unroll
-                    for (int i = 0; i < 2; ++i) {
-                        const int r = (lane >> 1) + 16 * i;
-                        if (mw + r >= p.M || left <= 0) continue;
-                        uint8_t* d = dst + r * row_bytes + piece;
-                        if (left >= 16) { *reinterpret_cast<uint4*>(d) = lds128(get + 512 * i); continue; }
-#pragma unroll 1
-                        for (int k = 0; k < left; k += 2) *reinterpret_cast<uint16_t*>(d + k) = lds16(get + 512 * i + k);     // the end of a ragged row
+                    for (int i = 0; i < PIECES; ++i) v[i] = lds128(stage + (r0 + ROWS_I * i) * OUT_ROW + ((j ^ sw(r0 + ROWS_I * i)) << 4));
+#pragma unroll
+                    for (int i = 0; i < PIECES; ++i, d += ROWS_I * row_bytes) {
+                        if (r0 + ROWS_I * i >= rows || left <= 0) continue;
+                        if (left >= 16) { *reinterpret_cast<uint4*>(d) = v[i]; continue; }
+                        const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};       // the end of a ragged row
+#pragma unroll
+                        for (int k = 0; k < 7; ++k) if (2 * k < left) *reinterpret_cast<uint16_t*>(d + 2 * k) = (uint16_t)(w[k >> 1] >> (16 * (k & 1)));
+                    }
+                    __syncwarp();
+                };
+                // DEQ: the finished fp32 sums are in tensor memory
+                const uint32_t t_acc = tmem_base + ((uint32_t)(32 * q) << 16) + (n_tile_done & 1u) * TILE_N + h * half_cols;
+                // my values of columns 8 i + {0, 1} (i = 4 jc + j), rows 16 hh + 8 r
+                auto finish = [&](int jc, auto use) {
+                    if constexpr (DEQ) {
+#pragma unroll
+                        for (int hh = 0; hh < 2; ++hh) {
+                            uint32_t v[16];
+                            tc_ld16x4(t_acc + ((uint32_t)(16 * hh) << 16) + 32 * jc, v);
+                            tc_wait_ld();
+#pragma unroll
+                            for (int i = 0; i < 8; ++i) R[(jc * 2 + hh) * 8 + i] = make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
+                        }
+                    }
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        const float2 c = t_corr[(jc * 4 + j) * 4], w = t_sw[(jc * 4 + j) * 4], b = t_bs[(jc * 4 + j) * 4];
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {                          // rows lane / 4 + 8 k
+                            float2 v = fma2(w, add2(R[(jc * 2 + (k >> 1)) * 8 + 2 * j + (k & 1)], make_float2(-c.x, -c.y)), b);
+                            if (relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); }
+                            use(j, k, v);
+                        }
                     }
                 };
-                // columns 2 i, 2 i + 1 finished
-                auto finish = [&](int i4, float2& lo, float2& hi) {            // columns 4 i4 .. 4 i4 + 3
-                    const float4 c = t_corr[i4], w = t_sw[i4], b = t_bs[i4];
-                    lo = fma2(make_float2(w.x, w.y), add2(R[2 * i4], make_float2(-c.x, -c.y)), make_float2(b.x, b.y));
-                    hi = fma2(make_float2(w.z, w.w), add2(R[2 * i4 + 1], make_float2(-c.z, -c.w)), make_float2(b.z, b.w));
-                    if (relu) { lo.x = fmaxf(lo.x, 0.f); lo.y = fmaxf(lo.y, 0.f); hi.x = fmaxf(hi.x, 0.f); hi.y = fmaxf(hi.y, 0.f); }
-                };
-                // DEQ: columns 16 c .. 16 c + 15 are the finished fp32 sums in tensor memory
-                const uint32_t t_acc = tmem_base + ((uint32_t)(32 * q) << 16) + (n_tile_done & 1u) * TILE_N + h * half_cols;
-                auto read_sums = [&](int c) {
-                    uint32_t v[16];
-                    tc_ld16(t_acc + 16 * c, v);
-                    tc_wait_ld();
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) R[8 * c + i] = make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
-                };
-                auto h2 = [](float2 v) { const __half2 x = __floats2half2_rn(v.x, v.y); return *reinterpret_cast<const uint32_t*>(&x); };
                 if (p.y_dtype == RPTQ_OUT_F16) {
                     uint8_t* dst = static_cast<uint8_t*>(p.y) + ((int64_t)mw * p.ldy + nb) * 2;
+                    const int n_bytes = 2 * min(p.N - nb, half_cols);
+                    // (my lane names row 8 k + lane % 8, piece lane / 8 of the 32 columns, to stmatrix)
 #pragma unroll
-                    for (int c = 0; c < 8; ++c) {                              // 16 columns
-                        if (16 * c >= half_cols) break;
-                        if constexpr (DEQ) read_sums(c);
-                        float2 v[8];
+                    for (int jc = 0; jc < 4; ++jc) {
+                        if (32 * jc >= half_cols) break;
+                        uint32_t f[4][4];                                      // [k][j]
+                        finish(jc, [&](int j, int k, float2 v) { const __half2 x = __floats2half2_rn(v.x, v.y); f[k][j] = *reinterpret_cast<const uint32_t*>(&x); });
+                        const int j0 = 4 * jc % PIECES;
 #pragma unroll
-                        for (int i = 0; i < 4; ++i) finish(4 * c + i, v[2 * i], v[2 * i + 1]);
-                        exchange(make_uint4(h2(v[0]), h2(v[1]), h2(v[2]), h2(v[3])), make_uint4(h2(v[4]), h2(v[5]), h2(v[6]), h2(v[7])),
-                                 dst + 32 * c, p.ldy * 2, 2 * (p.N - nb - 16 * c));
+                        for (int k = 0; k < 4; ++k) {
+                            const int r = 8 * k + (lane & 7);
+                            stmatrix4(stage + r * OUT_ROW + (((j0 + (lane >> 3)) ^ sw_f16(r)) << 4), f[k]);
+                        }
+                        const int from = 64 * jc / OUT_ROW * OUT_ROW;
+                        if (j0 + 4 == PIECES || 32 * (jc + 1) >= half_cols) store(sw_f16, dst + from, p.ldy * 2, n_bytes - from);
                     }
                 } else if (p.y_dtype == RPTQ_OUT_F32) {
                     uint8_t* dst = static_cast<uint8_t*>(p.y) + ((int64_t)mw * p.ldy + nb) * 4;
+                    const int n_bytes = 4 * min(p.N - nb, half_cols);
+                    const uint32_t put = stage + (lane >> 2) * OUT_ROW + 8 * (lane & 1);
+                    const int piece = (lane & 3) >> 1;
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) {                             // 8 columns
-                        if (8 * c >= half_cols) break;
-                        if constexpr (DEQ) if (c % 2 == 0) read_sums(c / 2);
-                        float2 v[4];
-                        finish(2 * c, v[0], v[1]);
-                        finish(2 * c + 1, v[2], v[3]);
-                        auto u4 = [](float2 a, float2 b) { return make_uint4(__float_as_uint(a.x), __float_as_uint(a.y), __float_as_uint(b.x), __float_as_uint(b.y)); };
-                        exchange(u4(v[0], v[1]), u4(v[2], v[3]), dst + 32 * c, p.ldy * 4, 4 * (p.N - nb - 8 * c));
+                    for (int jc = 0; jc < 4; ++jc) {
+                        if (32 * jc >= half_cols) break;
+                        finish(jc, [&](int j, int k, float2 v) {
+                            const int at = 2 * j % PIECES;
+                            sts64(put + 8 * k * OUT_ROW + (((at + piece) ^ sw_f32(lane >> 2)) << 4), v);      // (8 k changes no swizzle)
+                            if (k == 3 && at + 2 == PIECES) {
+                                const int from = (32 * jc + 8 * (j + 1)) * 4 - OUT_ROW;
+                                store(sw_f32, dst + from, p.ldy * 4, n_bytes - from);
+                            }
+                        });
                     }
                 } else if constexpr (MODE != MODE_DEQ) {
-                    // re-quantise for the next site: column n is padded position n of the output layout
-                    const int m = mw + lane;
-                    uint8_t* row = static_cast<uint8_t*>(p.y) + (int64_t)m * p.out_row_bytes;
-                    uint32_t held[4] = {0u, 0u, 0u, 0u};
+                    // Re-quantise for the next site: column n is padded position n of the output layout. A word of eight nibbles is eight columns of
+                    // a row, which four lanes hold, two codes each: a byte for each of a unit's four words. The bytes change lanes so that lane
+                    // l of the four has word l.
+                    const int n_units = min(half_cols, p.N - nb) >> 5;         // (N is a multiple of 128)
+                    const int l = lane & 3;
 #pragma unroll
-                    for (int uu = 0; uu < 4; ++uu) {
-                        const int unit = (nb >> 5) + uu;
-                        if (32 * uu >= half_cols || nb + 32 * uu >= p.N) break;    // (N is a multiple of 128)
+                    for (int jc = 0; jc < 4; ++jc) {
+                        if (jc >= n_units) break;
+                        const int unit = (nb >> 5) + jc;
                         const uint4 t4 = __ldg(reinterpret_cast<const uint4*>(p.out_unit + unit));
-                        const float inv_s = __uint_as_float(t4.x);
+                        const float2 s2 = make_float2(__uint_as_float(t4.x), __uint_as_float(t4.x)), c2 = make_float2(12582912.0f, 12582912.0f);
                         const int zc = (int)t4.y, nvalid = (int)t4.w;
-                        int qv[32];                                            // not yet clamped: the pack saturates
-#pragma unroll
-                        for (int i = 0; i < 8; ++i) {
-                            float2 lo, hi;
-                            finish(8 * uu + i, lo, hi);
-                            const float2 s2 = make_float2(inv_s, inv_s), k = make_float2(12582912.0f, 12582912.0f);
-                            lo = fma2(lo, s2, k); hi = fma2(hi, s2, k);
-                            qv[4 * i] = quant_int(lo.x, zc); qv[4 * i + 1] = quant_int(lo.y, zc);
-                            qv[4 * i + 2] = quant_int(hi.x, zc); qv[4 * i + 3] = quant_int(hi.y, zc);
-                        }
+                        int qv[4][4][2];                                       // [row k][word j]: not yet clamped, the pack saturates
+                        finish(jc, [&](int j, int k, float2 v) {
+                            v = fma2(v, s2, c2);
+                            qv[k][j][0] = quant_int(v.x, zc); qv[k][j][1] = quant_int(v.y, zc);
+                        });
                         if (nvalid < 32) {
 #pragma unroll
-                            for (int e = 0; e < 32; ++e) qv[e] = e < nvalid ? qv[e] : 0;
-                        }
-                        if (p.out_bits == 4) {
-                            uint32_t w[4]; pack32_sat<4>(qv, w);
-                            if (uu & 1) exchange(make_uint4(held[0], held[1], held[2], held[3]), make_uint4(w[0], w[1], w[2], w[3]),
-                                                 static_cast<uint8_t*>(p.y) + (int64_t)mw * p.out_row_bytes + (unit - 1) * 16, p.out_row_bytes, 32);
+                            for (int j = 0; j < 4; ++j)
 #pragma unroll
-                            for (int e = 0; e < 4; ++e) held[e] = w[e];
-                        } else if (m < p.M) {
-                            if (p.out_bits == 3) {
-                                uint32_t w[3]; pack32_sat<3>(qv, w);
-                                uint32_t* d = reinterpret_cast<uint32_t*>(row + unit * 12);
-                                d[0] = w[0]; d[1] = w[1]; d[2] = w[2];
+                                for (int e = 0; e < 2; ++e)
+#pragma unroll
+                                    for (int k = 0; k < 4; ++k) qv[k][j][e] = 8 * j + 2 * l + e < nvalid ? qv[k][j][e] : 0;
+                        }
+                        uint8_t* row = static_cast<uint8_t*>(p.y) + (int64_t)(mw + (lane >> 2)) * p.out_row_bytes;
+#pragma unroll
+                        for (int k = 0; k < 4; ++k, row += 8 * p.out_row_bytes) {
+                            const bool in = mw + (lane >> 2) + 8 * k < p.M;
+                            if (p.out_bits == 8) {
+                                // word 2 j is lanes 0 and 1, word 2 j + 1 lanes 2 and 3
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) {
+                                    const uint32_t x = sat_pack_u8(qv[k][j][1], qv[k][j][0], 0u), hi = __shfl_down_sync(0xffffffffu, x, 1);
+                                    if (in && (l & 1) == 0) *reinterpret_cast<uint32_t*>(row + unit * 32 + 8 * j + 2 * l) = x | (hi << 16);
+                                }
+                                continue;
+                            }
+                            uint32_t x = 0u;                                   // byte j: codes 2 l (low nibble) and 2 l + 1 of word j
+#pragma unroll
+                            for (int j = 3; j >= 0; --j) x = sat_pack_u4(qv[k][j][1], qv[k][j][0], x);
+                            // bytes 0, 1 of lanes 2, 3 for bytes 2, 3 of lanes 0, 1; then the same with lane ^ 1 and single bytes: lane l has byte l of
+                            // lanes 0, 1, 2, 3
+                            uint32_t o = __shfl_xor_sync(0xffffffffu, x, 2);
+                            x = __byte_perm(x, o, l & 2 ? 0x3276 : 0x5410);    // (words 2 (l / 2), 2 (l / 2) + 1) of lane l & 1, then of lane (l & 1) + 2
+                            o = __shfl_xor_sync(0xffffffffu, x, 1);
+                            x = __byte_perm(x, o, l & 1 ? 0x3715 : 0x6240);
+                            // codes 0 .. 3: the low nibbles of bytes 0 .. 3, codes 4 .. 7: the high ones
+                            const uint32_t lo = __byte_perm(x, x, 0x1100), hi = __byte_perm(x, x, 0x3322);
+                            uint32_t word = (lo & 0x000F000Fu) | ((lo >> 4) & 0x0F000F00u) | ((hi << 4) & 0x00F000F0u) | (hi & 0xF000F000u);
+                            if (p.out_bits == 4) {
+                                if (in) *reinterpret_cast<uint32_t*>(row + unit * 16 + 4 * l) = word;
                             } else {
-                                uint32_t w[8]; pack32_sat<8>(qv, w);
-                                uint4* d = reinterpret_cast<uint4*>(row + unit * 32);
-                                d[0] = make_uint4(w[0], w[1], w[2], w[3]); d[1] = make_uint4(w[4], w[5], w[6], w[7]);
+                                word = (word | (((word >> 3) & 0x11111111u) * 7u)) & 0x77777777u;                  // nibbles above 7 become 7
+                                const uint32_t tail = __shfl_sync(0xffffffffu, word, lane | 3);
+                                if (in && l < 3) *reinterpret_cast<uint32_t*>(row + unit * 12 + 4 * l) = word | (((tail >> l) & 0x11111111u) << 3);
                             }
                         }
                     }
