@@ -1,9 +1,10 @@
 // Attention for more queries than a decode step has: rptq_attention and rptq_attention_kv on the tcgen05 tensor cores.
 //
-// A persistent block works on 128 queries of one head at a time. The softmax output is needed with the row's final maximum
-// (and, where it is quantised at 8 bits, its final sum), so the keys are walked twice: pass 1 finds the row maxima
-// (integer calls: and the row sums), pass 2 forms the probabilities and multiplies them with V. Nothing is
-// rescaled on the way. Scores are computed in both passes; the tensor cores have room for that.
+// A persistent block works on 128 queries of one head at a time. Where the softmax output is quantised at 8 bits it is needed with the
+// row's final maximum and sum, so integer calls walk the keys twice: pass 1 finds the row maxima and sums, pass 2 forms the
+// probabilities and multiplies them with V. Nothing is rescaled on the way. Scores are computed in both passes; the tensor cores
+// have room for that. KV calls walk the keys once: probabilities are relative to a reference that follows the row's maximum, and
+// the output accumulator is brought to a new reference where it moves (two walks: 346 us, one: 316; 3 x 1100 queries on 1337 keys).
 //
 // What bounds it: one exponential per score and pass (the special-function unit gives 16 per clock and SM), then the
 // issue slots of the softmax warps: a score costs one multiply-add per cluster of the head, and five or six
@@ -12,13 +13,13 @@
 //                 of 64 keys): one accumulator per CLUSTER of the head (the scales differ), handed over slot by slot
 //                 through the stream's own ring in tensor memory. The streams run on their own, so that one's drains
 //                 fall under the other's exponentials
-//   warp 2        issues P V (pass 2) into the head's output accumulator, which stays in tensor memory
+//   warp 2        issues P V (integer calls: in pass 2) into the head's output accumulator, which stays in tensor memory
 //   warps 4-7     keys: packed rows arrive by cp.async one tile ahead, are unpacked into the swizzled operand tile; they
 //                 also lay out the queries: integer calls store q - z^Q where that fits the operand type (a byte; 16 in
 //                 magnitude for E4M3), otherwise q, and form the per-key term -sum_c s^Q s^K z^Q sum_p K_q
 //   warps 8-11    values: unpacked and transposed into [position][key] (byte permutes on the packed words); and the
 //                 output of an item, while the next item's pass 1 runs (they have nothing else to do there)
-//   warps 12-19   softmax, four per stream: thread = query row, 64 keys; S = sum_c coef_c acc_c in registers
+//   warps 12-19   softmax, four per stream: thread = query row, 64 keys; S = sum_c coef_c acc_c in registers; KV: rescaling
 // Operand types (MODE):
 //   I8   bytes, kind::i8, int32 sums
 //   F8   both codes of at most four bits: a nibble n as an 8-bit E4M3 pattern IS the number n 2^-9, so the same bytes
@@ -33,7 +34,7 @@
 //
 // Measured, us, against a mma.sync kernel with 64 (KV: 128) queries per block (72 heads of 128 channels, four clusters each,
 // causal, two sequences of 2048 tokens): 3 bits 2321 -> 735; KV, 32 heads, three sequences, 1100 queries on 1337 keys, 4 bits
-// 945 -> 344. What bounds it is the latency of the hand-overs between the roles: of the 9.7 warp cycles an issue (37 heads, 2048
+// 945 -> 316. What bounds it is the latency of the hand-overs between the roles: of the 9.7 warp cycles an issue (37 heads, 2048
 // tokens), 3.7 are long scoreboards (tensor-memory loads, barrier waits), 1.7 fixed latencies, 0.4 instruction fetch (cache-only
 // 4.0, 1.5, 0.9); issue slots are 52 % busy, the tensor pipe 11 %. Code that runs at the same time is worth keeping short all the
 // same: the compiler told that the warp index is uniform 916 -> 790 (93 -> 83 KB of code), the output rows' store loops not
@@ -56,6 +57,11 @@ constexpr int BM = 128, THREADS = 640, STREAMS = 2;
 constexpr int K_WARP0 = 4, V_WARP0 = 8, S_WARP0 = 12;
 constexpr int COLS = 64;                                  // keys of a stream's piece of work = columns of a score slot
 constexpr int N_SLOTS = 2;                                // score slots of each stream
+// KV: how far (log2) a score may lie above its row's reference before the reference moves. Rows whose largest probability is exactly 1
+// are the most accurate ones, and the passes over the accumulator cost next to nothing: error against 64 bits of seven calls
+// (64 to 1337 queries, 500 to 3000 keys), ratio to that of two passes: 8: 1.000 to 1.011, 1: 0.998 to 1.000; 3 x 1100 queries on
+// 1337 keys 313.5 and 315.8 us.
+constexpr float REF_ROOM = 1.0f;
 constexpr int S_WARPS = 4 * STREAMS;                      // softmax warps
 // registers per thread of the warpgroups: MMA issuers, two of loaders, two of softmax (the block is launched with 96 each)
 constexpr int REGS_MMA = 48, REGS_LOAD = 72, REGS_SOFTMAX = 144;
@@ -88,6 +94,13 @@ __device__ __forceinline__ void ld32(uint32_t taddr, uint32_t (&v)[32])
           "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
           "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
         : "r"(taddr) : "memory");
+}
+__device__ __forceinline__ void st16(uint32_t taddr, const uint32_t (&v)[16])
+{
+    asm volatile(
+        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15};"
+        ::"r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
+          "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(taddr) : "memory");
 }
 // The whole warp executes these in converged control flow; one elected lane issues. a, b: the low words of the operands'
 // descriptors (the high words are the same for every tile).
@@ -162,6 +175,7 @@ prefill_kernel(const AttnParams p, const Plan g)
 {
     constexpr int KEYS = keys_of(MODE);
     constexpr bool ALT = MODE == KV;                      // the streams take tiles by turns (otherwise halves of every tile)
+    constexpr int PASSES = MODE == KV ? 1 : 2;            // over the keys
     static_assert(O_COLS + 2 * N_SLOTS * COLS <= 512, "tensor memory");
     constexpr int K_ATOM = KEYS * 128;                    // operand tile of the keys: KEYS rows of 128 bytes per atom
     constexpr int Q_LOADERS = MODE == KV ? 8 : 4;         // warps that lay out the queries
@@ -171,7 +185,7 @@ prefill_kernel(const AttnParams p, const Plan g)
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + g.off_bar);
     constexpr int B_QFULL = 0, B_QEMPTY = 1, B_KFULL = 2, B_KEMPTY = 4, B_SFULL = 6, B_SEMPTY = B_SFULL + 2 * N_SLOTS, B_PFULL = B_SEMPTY + 2 * N_SLOTS,
                   B_PEMPTY = B_PFULL + 2, B_VFULL = B_PEMPTY + 2, B_VEMPTY = B_VFULL + 2, B_OFULL = B_VEMPTY + 2, B_OEMPTY = B_OFULL + 1,
-                  B_OUT = B_OEMPTY + 1, B_SUM = B_OUT + 1, B_XS = B_SUM + 1, B_XV = B_XS + 1, B_DRAIN = B_XV + 1, N_BARS = B_DRAIN + 3;
+                  B_OUT = B_OEMPTY + 1, B_SUM = B_OUT + 1, B_XS = B_SUM + 1, B_XV = B_XS + 1, B_DRAIN = B_XV + 1, B_REF = B_DRAIN + 3, N_BARS = B_REF + (ALT ? 16 : 0);
     static_assert(N_BARS * 8 + 16 <= 512, "barrier block");
     uint32_t* s_tmem = reinterpret_cast<uint32_t*>(bars + N_BARS);
     volatile int* s_abort = reinterpret_cast<volatile int*>(s_tmem + 1);
@@ -189,6 +203,7 @@ prefill_kernel(const AttnParams p, const Plan g)
         mbar_init(bar(B_OFULL), 1); mbar_init(bar(B_OEMPTY), 4); mbar_init(bar(B_OUT), 4);
         mbar_init(bar(B_SUM), S_WARPS); mbar_init(bar(B_XS), S_WARPS); mbar_init(bar(B_XV), 4);
         for (int i = 0; i < 3; ++i) mbar_init(bar(B_DRAIN + i), 1);
+        if constexpr (ALT) for (int i = 0; i < 16; ++i) mbar_init(bar(B_REF + i), 1);
         *s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -203,7 +218,7 @@ prefill_kernel(const AttnParams p, const Plan g)
     tc_fence_after();
     const uint32_t tmem = *s_tmem;
     float* s_col = reinterpret_cast<float*>(smem + g.off_col);            // [4][KEYS]
-    float2* s_ml = reinterpret_cast<float2*>(smem + g.off_ml);            // [2][STREAMS][BM]: row maxima and sums over a stream's keys
+    float2* s_ml = reinterpret_cast<float2*>(smem + g.off_ml);            // [2][STREAMS][BM]: row maxima and sums over a stream's keys; KV: references
     uint32_t* s_sum = reinterpret_cast<uint32_t*>(smem + g.off_sum);      // [STREAMS][BM]: sums of probabilities (codes)
 
     if (warp < K_WARP0) {
@@ -229,7 +244,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                 const uint32_t last = __ballot_sync(0xffffffffu, lane < nu && (lane >= nuk - 1 || cl != cl_next));
                 if (!mbar_sleep_warp(bar(B_QFULL), n_item & 1, s_abort)) { ok = false; break; }
 #pragma unroll 1
-                for (int pass = 0; pass < 2 && ok; ++pass) {
+                for (int pass = 0; pass < PASSES && ok; ++pass) {
 #pragma unroll 1
                     for (int kt = ALT ? stream : 0; kt < it.n_kt && ok; kt += ALT ? 2 : 1, ++n_k) {
                         const uint32_t st = ALT ? stream : n_k & 1;            // (KV: a stage belongs to a stream, which so sees all its phases)
@@ -325,7 +340,7 @@ prefill_kernel(const AttnParams p, const Plan g)
         const bool is_k = warp < V_WARP0;
         Tile nx, cu;
         nx.n = 0xFFFFFFFFu; nx.t = 0; nx.n_t = 1; nx.kt = 0;
-        // keys: every item's tiles twice; values: once
+        // keys: every item's tiles once a pass; values: once
         auto advance = [&]() {
             ++nx.kt;
             if (++nx.t == nx.n_t) {
@@ -333,7 +348,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                 nx.t = 0;
                 if (idx >= g.n_items) return false;
                 nx.it = item_of(p, g, idx, KEYS);
-                nx.n_t = is_k ? 2 * nx.it.n_kt : nx.it.n_kt;
+                nx.n_t = is_k ? PASSES * nx.it.n_kt : nx.it.n_kt;
                 const int32_t* u = is_k ? p.cl_unit0_k + nx.it.h * p.gh_k : p.cl_unit0_v + nx.it.h * p.gh_v;
                 nx.u0 = __ldg(u);
                 nx.nu = __ldg(u + (is_k ? p.gh_k : p.gh_v)) - nx.u0;
@@ -732,9 +747,12 @@ prefill_kernel(const AttnParams p, const Plan g)
                     float inv_l = 0.f;
                     int rs = 0;
                     if constexpr (MODE == KV) {
+                        // (the later reference, in which the accumulator is, is the larger one)
+                        const float2* ml = s_ml + (n_item & 1) * STREAMS * BM + row;
+                        const float ref = fmaxf(ml[0].y, ml[BM].y);
                         float l = 0.f;
 #pragma unroll
-                        for (int q = 0; q < STREAMS; ++q) l += __uint_as_float(s_sum[q * BM + row]);
+                        for (int q = 0; q < STREAMS; ++q) l = __fmaf_rn(__uint_as_float(s_sum[q * BM + row]), ex2(ml[q * BM].y - ref), l);
                         inv_l = 1.0f / l;
                     } else {
 #pragma unroll
@@ -821,7 +839,8 @@ prefill_kernel(const AttnParams p, const Plan g)
         const int row = 32 * q4 + lane;                                        // query row within the tile
         const uint32_t t_col = tmem + ((uint32_t)(32 * q4) << 16) + O_COLS + stream * (N_SLOTS * COLS);
         const uint32_t b_full0 = bar(B_SFULL + stream * N_SLOTS), b_empty0 = bar(B_SEMPTY + stream * N_SLOTS);
-        uint32_t n_k0 = 0, slot = 0, par = 0, n_s = 0, n_item = 0;   // n_s: my stream's tiles of pass 2 so far
+        uint32_t n_k0 = 0, slot = 0, par = 0, n_s = 0, n_item = 0;   // n_s: my tiles multiplied with V so far
+        uint32_t ref_par = 0, n_other = 0;                           // KV: phases of the other stream's references (one bit for each set), its tiles so far
         bool ok = true;
         for (int idx; ok && (idx = item_index(n_item)) < g.n_items; ++n_item) {
             const Item it = item_of(p, g, idx, KEYS);
@@ -847,8 +866,8 @@ prefill_kernel(const AttnParams p, const Plan g)
             float m = NEG_BIG, l = 0.f, f = 0.f, lsum = 0.f;
             uint32_t rsum = 0u;
 #pragma unroll 1
-            for (int pass = 0; pass < 2 && ok; ++pass, n_k0 += it.n_kt) {
-                if (pass == 1) {
+            for (int pass = 2 - PASSES; pass < 2 && ok; ++pass, n_k0 += it.n_kt) {
+                if (PASSES == 2 && pass == 1) {
                     // the streams' statistics meet (two sets by turns: a warp may be an item ahead of another)
                     float2* ml = s_ml + (n_item & 1) * STREAMS * BM + row;
                     ml[stream * BM] = make_float2(m, l);
@@ -946,6 +965,41 @@ prefill_kernel(const AttnParams p, const Plan g)
                         }
                         continue;
                     }
+                    // ---- KV: the reference that the row's probabilities are relative to. It is the first tile's maximum, and moves to a later tile's
+                    // where that one is above it by REF_ROOM. References are handed from tile to tile, and so from stream to stream, in
+                    // two sets by turns, since a stream may be an item ahead of the other (no more: see B_OUT below).
+                    float down = 1.f;                                          // what the sums so far are worth in the new reference
+                    bool moved = false;
+                    if constexpr (MODE == KV) {
+                        if (live) {
+                            const uint32_t set = n_item & 1;
+                            float2* ml = s_ml + set * STREAMS * BM + row;
+                            float x0 = NEG_BIG, x1 = NEG_BIG;
+#pragma unroll
+                            for (int e = 0; e < COLS / 2; e += 2) {
+                                x0 = fmaxf(x0, fmaxf(S[e].x, S[e].y));
+                                x1 = fmaxf(x1, fmaxf(S[e + 1].x, S[e + 1].y));
+                            }
+                            const float top = fmaxf(x0, x1);
+                            float ref = top;
+                            if (kt > 0) {
+                                if (!mbar_sleep_warp(bar(B_REF + 8 * set + 2 * q4 + (stream ^ 1)), (ref_par >> set) & 1, s_abort)) { ok = false; break; }
+                                ref_par ^= 1u << set;
+                                const float before = ml[(stream ^ 1) * BM].x;
+                                // (where one row of the warp has to move, all move to their maxima: the pass over the accumulator is the same)
+                                moved = __any_sync(0xffffffffu, top > before + REF_ROOM) && top > before;
+                                if (!moved) ref = before;
+                                else down = ex2(before - ref);
+                            }
+                            if (kt + 1 < it.n_kt) {
+                                ml[stream * BM].x = ref;
+                                __syncwarp();
+                                if (lane == 0) mbar_arrive(bar(B_REF + 8 * set + 2 * q4 + stream));
+                            }
+                            lsum *= ex2(m - ref);
+                            m = ref;
+                        }
+                    }
                     // ---- pass 2: probabilities. P's region also stages the previous item's output
                     if (kt < 2 && !mbar_sleep_warp(bar(B_OUT), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
                     // the buffer's previous tile has been multiplied
@@ -953,6 +1007,28 @@ prefill_kernel(const AttnParams p, const Plan g)
                     const uint32_t behind = ALT && g.p_tiles == 1 && stream == 1 ? 0u : 1u;
                     if (!mbar_sleep_warp(bar(B_PEMPTY + stream), (n_s & 1) ^ behind, s_abort)) { ok = false; break; }
                     ++n_s;
+                    if constexpr (MODE == KV) {
+                        if (live && __any_sync(0xffffffffu, moved)) {
+                            // the output accumulator of my rows in the new reference, when the tile before has been multiplied (with one buffer for both
+                            // streams that is what has just been waited for) and before mine is
+                            const uint32_t n_before = stream == 0 ? n_other + (kt >> 1) : n_other + ((kt + 1) >> 1);
+                            if (g.p_tiles == 2 && !mbar_sleep_warp(bar(B_PEMPTY + (stream ^ 1)), (n_before - 1) & 1, s_abort)) { ok = false; break; }
+                            tc_fence_after();
+                            const int nuv = __ldg(p.cl_unit0_v + (it.h + 1) * p.gh_v) - __ldg(p.cl_unit0_v + it.h * p.gh_v);
+                            const uint32_t t_out = tmem + ((uint32_t)(32 * q4) << 16);
+#pragma unroll 1
+                            for (int c = 0; c < 2 * nuv; ++c) {
+                                uint32_t v[16];
+                                tc_ld16(t_out + 16 * c, v);
+                                tc_wait_ld();
+#pragma unroll
+                                for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * down);
+                                st16(t_out + 16 * c, v);
+                            }
+                            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                            tc_fence_before();
+                        }
+                    }
                     if (live) {
                         const float2 nm = make_float2(-m, -m);
                         if constexpr (MODE == KV) {
@@ -1016,6 +1092,10 @@ prefill_kernel(const AttnParams p, const Plan g)
             if (!ok) break;
             // (a stream without a tile of its own has not waited for the previous item's sums to be read)
             if (ALT && it.n_kt == 1 && !mbar_sleep_warp(bar(B_OUT), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
+            if constexpr (MODE == KV) {
+                s_ml[((n_item & 1) * STREAMS + stream) * BM + row].y = m;
+                n_other += (uint32_t)(stream == 0 ? it.n_kt / 2 : (it.n_kt + 1) / 2);
+            }
             s_sum[stream * BM + row] = MODE == KV ? __float_as_uint(lsum) : rsum;
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(B_SUM));

@@ -253,3 +253,25 @@ def test_few_queries_of_heads_of_eight_units(bits, Tq, Tk):
     other's 3-bit rows, and the scores of as many keys as a block may have."""
     c = Case(970 + Tq, H=2, hd=256, gh=1, Tq=Tq, Tk=Tk, bits=bits)
     _check(c, _query(np.random.default_rng(14), Tq, 512, 0.2), True)
+
+
+@pytest.mark.parametrize("hd,bits,Tq,Tk,n_seq,causal", [(64, (4, 4, 4), 130, 700, 1, True), (64, (4, 4, 4), 200, 200, 2, False), (72, (4, 3, 8), 9, 129, 3, True),
+                                                        (256, (4, 8, 8), 130, 330, 1, True)])
+def test_scores_that_rise_along_the_keys(hd, bits, Tq, Tk, n_seq, causal):
+    """Row maxima that grow by more than 2^8 from tile to tile for some rows, by less for others, and not at all for the rest (one walk
+    over the keys: the sums so far are brought to a new reference where that happens). Heads of eight units leave room for one
+    tile of probabilities only."""
+    rng = np.random.default_rng(15)
+    top = (1 << bits[1]) - 1
+    c = Case(980 + hd + Tk, H=2, hd=hd, gh=1 if hd == 256 else 2, Tq=Tq * n_seq, Tk=Tk * n_seq, bits=bits)
+    ramp = np.tile(np.arange(Tk) / (Tk - 1.0), n_seq)[:, None] * top
+    real = np.arange(c.k.shape[1])
+    codes = np.clip(np.rint(ramp + 0.05 * top * rng.normal(size=c.k.shape)), 0, top).astype(c.k.dtype)
+    off, _ = oracle.segment_offsets(c.size_qk)
+    for cl, n in enumerate(c.size_qk):
+        at = real[off[cl]:off[cl] + n]
+        c.k[:, at] = codes[:, at]
+    _rebuild_keys(c, bits[1])
+    step = float(np.dot(c.size_qk, c.sK)) / 2 * top * c.qk_scale          # what a query of ones gains from the first key to the last
+    rise = rng.choice([-300.0, -20.0, 0.0, 3.0, 12.0, 60.0, 300.0], size=(Tq * n_seq, 1)) / step
+    _check(c, (rise * (1 + 0.1 * rng.normal(size=(Tq * n_seq, 2 * hd)))).astype(np.float16), causal, n_seq=n_seq)
