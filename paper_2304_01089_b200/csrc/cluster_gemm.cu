@@ -73,7 +73,7 @@ __host__ __device__ constexpr int w_rows(int ncta) { return TILE_N / ncta; }    
 // packed weight stages; the single-CTA variant (at most 128 tokens) is a weight stream and takes what shared memory is left
 __host__ __device__ constexpr int n_p_stages(int ncta, int bits, int mode) 
 {
-    if (ncta == 2) return mode == MODE_DEQ && bits == 8 ? 3 : 4;
+    if (ncta == 2) return 4;
     return mode == MODE_DEQ || (mode == MODE_ASYM && bits == 8) ? 3 : bits == 3 ? 5 : 4;
 }
 __host__ __device__ constexpr int n_u_stages(int ncta, bool a8) { return ncta == 2 ? (a8 ? 5 : 4) : 2; }   // operand stages
@@ -98,8 +98,8 @@ __host__ __device__ constexpr SmemLayout smem_layout(int ncta, int bits, bool a8
     s.off_a = s.off_p + n_p_stages(ncta, bits, mode) * s.p_stage;
     s.off_flags = s.off_a + n_a_stages(ncta, bits, mode) * s.a_stage;
     s.off_seg_scale = s.off_flags + 2048;
-    s.off_seg_buf = s.off_seg_scale + (asym ? 0 : kMaxGemmSegments * 4);
-    s.off_tab = s.off_seg_buf + kMaxGemmSegments;
+    s.off_seg_buf = s.off_seg_scale + (mode == MODE_INT ? kMaxGemmSegments * 4 : 0);
+    s.off_tab = s.off_seg_buf + (mode == MODE_DEQ ? 0 : kMaxGemmSegments);          // (DEQ: one accumulator per tile, no clusters)
     s.off_seg_tab = s.off_tab + 2 * 3 * TILE_N * 4;
     s.off_seg_cl = s.off_seg_tab + (asym ? SEG_SLOTS * 2 * TILE_N * 4 : 0);
     s.off_stage = s.off_seg_cl + (asym ? kMaxGemmSegments * 2 : 0);
@@ -383,7 +383,7 @@ cluster_gemm_kernel(const Params p)
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     for (int i = tid; i < n_steps; i += THREADS) s_flags[i] = p.step_flags[i];
-    for (int i = tid; i < p.n_seg; i += THREADS) {
+    if constexpr (!DEQ) for (int i = tid; i < p.n_seg; i += THREADS) {
         if constexpr (!ASYM) s_seg_scale[i] = p.seg_scale[i] * 0.0625f;        // operands were 16 * w
         s_seg_buf[i] = p.seg_buf[i];
     }
@@ -1033,6 +1033,17 @@ cluster_gemm_kernel(const Params p)
                 const float2* t_sw = t_corr + TILE_N / 2;
                 const float2* t_bs = t_sw + TILE_N / 2;
                 const bool relu = p.act == RPTQ_ACT_RELU;
+                // 32 columns at a time (DEQ: its sums are not in registers, of which it has few: a rolled loop)
+                auto each_jc = [&](auto body) {
+                    if constexpr (DEQ) {
+#pragma unroll 1
+                        for (int jc = 0; 32 * jc < half_cols; ++jc) body(jc);
+                    } else {
+                        body(std::integral_constant<int, 0>());
+                        if (half_cols > 32) body(std::integral_constant<int, 1>());
+                        if (half_cols > 64) { body(std::integral_constant<int, 2>()); body(std::integral_constant<int, 3>()); }
+                    }
+                };
                 // piece j (16 bytes) of row r lies at j ^ sw(r): neither what a warp puts nor what it reads in one instruction meets in a bank
                 constexpr int OUT_ROW = SL.out_row, PIECES = OUT_ROW / 16, ROWS_I = 32 / PIECES;          // ROWS_I: rows that a warp-wide access covers
                 const uint32_t stage = smem_base + SL.off_stage + ew * 32 * OUT_ROW;
@@ -1059,22 +1070,23 @@ cluster_gemm_kernel(const Params p)
                 const uint32_t t_acc = tmem_base + ((uint32_t)(32 * q) << 16) + (n_tile_done & 1u) * TILE_N + h * half_cols;
                 // my values of columns 8 i + {0, 1} (i = 4 jc + j), rows 16 hh + 8 r
                 auto finish = [&](int jc, auto use) {
+                    float2 own[16];
                     if constexpr (DEQ) {
+                        uint32_t v[2][16];
+                        tc_ld16x4(t_acc + 32 * jc, v[0]);
+                        tc_ld16x4(t_acc + (16u << 16) + 32 * jc, v[1]);
+                        tc_wait_ld();
 #pragma unroll
-                        for (int hh = 0; hh < 2; ++hh) {
-                            uint32_t v[16];
-                            tc_ld16x4(t_acc + ((uint32_t)(16 * hh) << 16) + 32 * jc, v);
-                            tc_wait_ld();
-#pragma unroll
-                            for (int i = 0; i < 8; ++i) R[(jc * 2 + hh) * 8 + i] = make_float2(__uint_as_float(v[2 * i]), __uint_as_float(v[2 * i + 1]));
-                        }
+                        for (int i = 0; i < 16; ++i) own[i] = make_float2(__uint_as_float(v[i >> 3][2 * (i & 7)]), __uint_as_float(v[i >> 3][2 * (i & 7) + 1]));
                     }
 #pragma unroll
                     for (int j = 0; j < 4; ++j) {
                         const float2 c = t_corr[(jc * 4 + j) * 4], w = t_sw[(jc * 4 + j) * 4], b = t_bs[(jc * 4 + j) * 4];
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {                          // rows lane / 4 + 8 k
-                            float2 v = fma2(w, add2(R[(jc * 2 + (k >> 1)) * 8 + 2 * j + (k & 1)], make_float2(-c.x, -c.y)), b);
+                            float2 sum;
+                            if constexpr (DEQ) sum = own[(k >> 1) * 8 + 2 * j + (k & 1)]; else sum = R[(jc * 2 + (k >> 1)) * 8 + 2 * j + (k & 1)];
+                            float2 v = fma2(w, add2(sum, make_float2(-c.x, -c.y)), b);
                             if (relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); }
                             use(j, k, v);
                         }
@@ -1084,9 +1096,8 @@ cluster_gemm_kernel(const Params p)
                     uint8_t* dst = static_cast<uint8_t*>(p.y) + ((int64_t)mw * p.ldy + nb) * 2;
                     const int n_bytes = 2 * min(p.N - nb, half_cols);
                     // (my lane names row 8 k + lane % 8, piece lane / 8 of the 32 columns, to stmatrix)
-#pragma unroll
-                    for (int jc = 0; jc < 4; ++jc) {
-                        if (32 * jc >= half_cols) break;
+                    each_jc([&](auto at_jc) {
+                        const int jc = at_jc;
                         uint32_t f[4][4];                                      // [k][j]
                         finish(jc, [&](int j, int k, float2 v) { const __half2 x = __floats2half2_rn(v.x, v.y); f[k][j] = *reinterpret_cast<const uint32_t*>(&x); });
                         const int j0 = 4 * jc % PIECES;
@@ -1097,15 +1108,14 @@ cluster_gemm_kernel(const Params p)
                         }
                         const int from = 64 * jc / OUT_ROW * OUT_ROW;
                         if (j0 + 4 == PIECES || 32 * (jc + 1) >= half_cols) store(sw_f16, dst + from, p.ldy * 2, n_bytes - from);
-                    }
+                    });
                 } else if (p.y_dtype == RPTQ_OUT_F32) {
                     uint8_t* dst = static_cast<uint8_t*>(p.y) + ((int64_t)mw * p.ldy + nb) * 4;
                     const int n_bytes = 4 * min(p.N - nb, half_cols);
                     const uint32_t put = stage + (lane >> 2) * OUT_ROW + 8 * (lane & 1);
                     const int piece = (lane & 3) >> 1;
-#pragma unroll
-                    for (int jc = 0; jc < 4; ++jc) {
-                        if (32 * jc >= half_cols) break;
+                    each_jc([&](auto at_jc) {
+                        const int jc = at_jc;
                         finish(jc, [&](int j, int k, float2 v) {
                             const int at = 2 * j % PIECES;
                             sts64(put + 8 * k * OUT_ROW + (((at + piece) ^ sw_f32(lane >> 2)) << 4), v);      // (8 k changes no swizzle)
@@ -1114,11 +1124,11 @@ cluster_gemm_kernel(const Params p)
                                 store(sw_f32, dst + from, p.ldy * 4, n_bytes - from);
                             }
                         });
-                    }
+                    });
                 } else if constexpr (MODE != MODE_DEQ) {
                     // Re-quantise for the next site: column n is padded position n of the output layout. A word of eight nibbles is eight columns of
-                    // a row, which four lanes hold, two codes each: a byte for each of a unit's four words. The bytes change lanes so that lane
-                    // l of the four has word l.
+                    // a row, which four lanes hold, two codes each. Codes of at most four bits: a byte for each of a unit's four words goes through the
+                    // warp's buffer as the fragment of a 16-bit matrix, which gives every lane the 16 bytes of its own row.
                     const int n_units = min(half_cols, p.N - nb) >> 5;         // (N is a multiple of 128)
                     const int l = lane & 3;
 #pragma unroll
@@ -1141,37 +1151,54 @@ cluster_gemm_kernel(const Params p)
 #pragma unroll
                                     for (int k = 0; k < 4; ++k) qv[k][j][e] = 8 * j + 2 * l + e < nvalid ? qv[k][j][e] : 0;
                         }
-                        uint8_t* row = static_cast<uint8_t*>(p.y) + (int64_t)(mw + (lane >> 2)) * p.out_row_bytes;
+                        if (p.out_bits == 8) {
+                            uint8_t* row = static_cast<uint8_t*>(p.y) + (int64_t)(mw + (lane >> 2)) * p.out_row_bytes;
 #pragma unroll
-                        for (int k = 0; k < 4; ++k, row += 8 * p.out_row_bytes) {
-                            const bool in = mw + (lane >> 2) + 8 * k < p.M;
-                            if (p.out_bits == 8) {
-                                // word 2 j is lanes 0 and 1, word 2 j + 1 lanes 2 and 3
-#pragma unroll
-                                for (int j = 0; j < 4; ++j) {
-                                    const uint32_t x = sat_pack_u8(qv[k][j][1], qv[k][j][0], 0u), hi = __shfl_down_sync(0xffffffffu, x, 1);
-                                    if (in && (l & 1) == 0) *reinterpret_cast<uint32_t*>(row + unit * 32 + 8 * j + 2 * l) = x | (hi << 16);
-                                }
-                                continue;
+                            for (int k = 0; k < 4; ++k, row += 8 * p.out_row_bytes) {
+                                // two codes of each of the unit's four pairs of words: lane l ends with pair l. With lane ^ 2 pairs 0, 1 (of lanes 0, 1) for 2, 3
+                                // (of lanes 2, 3), then with lane ^ 1 the even pair for the odd one
+                                auto two = [&](int j) { return sat_pack_u8(qv[k][j][1], qv[k][j][0], 0u); };
+                                const uint32_t lo = two(0) | (two(1) << 16), hi = two(2) | (two(3) << 16);
+                                const uint32_t own = l & 2 ? hi : lo, o2 = __shfl_xor_sync(0xffffffffu, l & 2 ? lo : hi, 2);
+                                const uint32_t x = l & 2 ? o2 : own, y = l & 2 ? own : o2;           // of lanes l & 1 and (l & 1) + 2
+                                const uint32_t even = __byte_perm(x, y, 0x5410), odd = __byte_perm(x, y, 0x7632);
+                                const uint32_t o1 = __shfl_xor_sync(0xffffffffu, l & 1 ? even : odd, 1);
+                                const uint32_t a = l & 1 ? o1 : even, c = l & 1 ? odd : o1;          // of the lower, the higher lane
+                                if (mw + (lane >> 2) + 8 * k < p.M)
+                                    *reinterpret_cast<uint2*>(row + unit * 32 + 8 * l) = make_uint2(__byte_perm(a, c, 0x5410), __byte_perm(a, c, 0x7632));
                             }
-                            uint32_t x = 0u;                                   // byte j: codes 2 l (low nibble) and 2 l + 1 of word j
+                            continue;
+                        }
+                        uint32_t x[4] = {0u, 0u, 0u, 0u};                      // byte j: codes 2 l (low nibble) and 2 l + 1 of word j
 #pragma unroll
-                            for (int j = 3; j >= 0; --j) x = sat_pack_u4(qv[k][j][1], qv[k][j][0], x);
-                            // bytes 0, 1 of lanes 2, 3 for bytes 2, 3 of lanes 0, 1; then the same with lane ^ 1 and single bytes: lane l has byte l of
-                            // lanes 0, 1, 2, 3
-                            uint32_t o = __shfl_xor_sync(0xffffffffu, x, 2);
-                            x = __byte_perm(x, o, l & 2 ? 0x3276 : 0x5410);    // (words 2 (l / 2), 2 (l / 2) + 1) of lane l & 1, then of lane (l & 1) + 2
-                            o = __shfl_xor_sync(0xffffffffu, x, 1);
-                            x = __byte_perm(x, o, l & 1 ? 0x3715 : 0x6240);
-                            // codes 0 .. 3: the low nibbles of bytes 0 .. 3, codes 4 .. 7: the high ones
-                            const uint32_t lo = __byte_perm(x, x, 0x1100), hi = __byte_perm(x, x, 0x3322);
-                            uint32_t word = (lo & 0x000F000Fu) | ((lo >> 4) & 0x0F000F00u) | ((hi << 4) & 0x00F000F0u) | (hi & 0xF000F000u);
-                            if (p.out_bits == 4) {
-                                if (in) *reinterpret_cast<uint32_t*>(row + unit * 16 + 4 * l) = word;
-                            } else {
-                                word = (word | (((word >> 3) & 0x11111111u) * 7u)) & 0x77777777u;                  // nibbles above 7 become 7
-                                const uint32_t tail = __shfl_sync(0xffffffffu, word, lane | 3);
-                                if (in && l < 3) *reinterpret_cast<uint32_t*>(row + unit * 12 + 4 * l) = word | (((tail >> l) & 0x11111111u) << 3);
+                        for (int k = 0; k < 4; ++k)
+#pragma unroll
+                            for (int j = 3; j >= 0; --j) x[k] = sat_pack_u4(qv[k][j][1], qv[k][j][0], x[k]);
+                        const uint32_t own_row = stage + lane * OUT_ROW + ((jc ^ sw_f16(lane)) << 4);
+                        stmatrix4(own_row, x);
+                        __syncwarp();
+                        const uint4 t = lds128(own_row);                       // word l: byte j is codes 2 l, 2 l + 1 of word j
+                        const uint32_t a01 = __byte_perm(t.x, t.y, 0x5140), a23 = __byte_perm(t.x, t.y, 0x7362);
+                        const uint32_t b01 = __byte_perm(t.z, t.w, 0x5140), b23 = __byte_perm(t.z, t.w, 0x7362);
+                        uint32_t w[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            // codes 0, 1, 2, 3 of word j (bytes 0, 0, 1, 1 of its two) and 4, 5, 6, 7: low nibbles, high nibbles
+                            const uint32_t lo = __byte_perm(j < 2 ? a01 : a23, 0u, j & 1 ? 0x3322 : 0x1100), hi = __byte_perm(j < 2 ? b01 : b23, 0u, j & 1 ? 0x3322 : 0x1100);
+                            w[j] = (lo & 0x000F000Fu) | ((lo >> 4) & 0x0F000F00u) | ((hi << 4) & 0x00F000F0u) | (hi & 0xF000F000u);
+                        }
+                        uint8_t* row = static_cast<uint8_t*>(p.y) + (int64_t)(mw + lane) * p.out_row_bytes + unit * 4 * p.out_bits;
+                        if (p.out_bits == 4) {
+                            // back to the same place, and out in pieces of up to 64 bytes a row
+                            sts128(own_row, w[0], w[1], w[2], w[3]);
+                            if (jc + 1 == n_units)
+                                store(sw_f16, static_cast<uint8_t*>(p.y) + (int64_t)mw * p.out_row_bytes + (nb >> 5) * 16, p.out_row_bytes, 16 * n_units);
+                        } else {
+                            auto clamp7 = [](uint32_t v) { return (v | (((v >> 3) & 0x11111111u) * 7u)) & 0x77777777u; };        // nibbles above 7 become 7
+                            const uint32_t tail = clamp7(w[3]);
+                            if (mw + lane < p.M) {
+#pragma unroll
+                                for (int j = 0; j < 3; ++j) reinterpret_cast<uint32_t*>(row)[j] = clamp7(w[j]) | (((tail >> j) & 0x11111111u) << 3);
                             }
                         }
                     }

@@ -382,3 +382,39 @@ def test_last_round_in_strips(M, rest, bits):
     assert np.max(np.abs(y32 - want)) <= TOL * np.abs(want).max()
     y16 = _gemm(case, d, y_dtype=binding.OUT_F16, ldy=N + 8)[:, :N]
     assert np.array_equal(y16, y32.astype(np.float16))
+
+
+@pytest.mark.parametrize("out", ["f32", "f16", 3, 4, 8])
+def test_whole_tiles_and_strips_give_the_bits_of_small_calls(out):
+    """80 tiles on 74 pairs of blocks: 74 whole ones and 6 that are cut into strips, the last rows and (float outputs) the last columns ragged,
+    against calls of at most 128 tokens, which the tests above hold to the oracle: each output's rows leave the kernel in the
+    same arithmetic whatever the tile."""
+    import torch
+    from paper_2304_01089_b200 import binding
+    codes = isinstance(out, int)
+    M, N, n_pad = 2401, 2048 if codes else 2045, 2048
+    rng = np.random.default_rng(77)
+    size = np.array([70, 5, 181])
+    case = dict(zip(("perm", "size", "scale", "zero"), random_layout_params(rng, 256, 3, 4)))
+    case.update(size=size)
+    W = (rng.normal(size=(N, 256)) * 0.02).astype(np.float32)
+    w_codes, s_w, wsum = oracle.weight_quantize(W, case["perm"], size, None, n_pad)
+    off, k_pad = oracle.segment_offsets(size)
+    a = np.zeros((M, k_pad), np.uint8)
+    for c in range(3):
+        a[:, off[c]:off[c] + size[c]] = rng.integers(0, 16, size=(M, size[c]))
+    case.update(w_codes=w_codes, s_w=s_w, wsum=wsum, a=a, k_pad=k_pad, bits=4, M=M, N=N, n_pad=n_pad)
+    d = _dev(case)
+    kw = dict(y_dtype=binding.OUT_F32 if out == "f32" else binding.OUT_F16, ldy=n_pad)
+    if codes:
+        y = _gemm(case, d)
+        size2 = np.array([1, 31, 32, 33, 64, 500, 700, 500, 59])
+        perm2, g2 = np.arange(size2.sum(), dtype=np.int32), len(size2)
+        L2 = binding.Layout(perm2, size2, np.full(g2, np.abs(y).max() / (1 << out), np.float32), np.full(g2, 1 << (out - 1), np.int32), out)
+        assert L2.K_pad == N
+        kw = dict(y_dtype=binding.OUT_CODES, layout_out=L2)
+    whole = _gemm(case, d, **kw)
+    for lo in range(0, M, 128):
+        n = min(128, M - lo)
+        part = _gemm(dict(case, M=n), dict(d, a=d["a"][lo:lo + n].contiguous()), **kw)
+        np.testing.assert_array_equal(whole[lo:lo + n].view(np.uint8), part.view(np.uint8))
