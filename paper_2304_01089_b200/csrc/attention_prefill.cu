@@ -57,11 +57,6 @@ constexpr int BM = 128, THREADS = 640, STREAMS = 2;
 constexpr int K_WARP0 = 4, V_WARP0 = 8, S_WARP0 = 12;
 constexpr int COLS = 64;                                  // keys of a stream's piece of work = columns of a score slot
 constexpr int N_SLOTS = 2;                                // score slots of each stream
-// KV: how far (log2) a score may lie above its row's reference before the reference moves. Rows whose largest probability is exactly 1
-// are the most accurate ones, and the passes over the accumulator cost next to nothing: error against 64 bits of seven calls
-// (64 to 1337 queries, 500 to 3000 keys), ratio to that of two passes: 8: 1.000 to 1.011, 1: 0.998 to 1.000; 3 x 1100 queries on
-// 1337 keys 313.5 and 315.8 us.
-constexpr float REF_ROOM = 1.0f;
 constexpr int S_WARPS = 4 * STREAMS;                      // softmax warps
 // registers per thread of the warpgroups: MMA issuers, two of loaders, two of softmax (the block is launched with 96 each)
 constexpr int REGS_MMA = 48, REGS_LOAD = 72, REGS_SOFTMAX = 144;
@@ -750,10 +745,10 @@ prefill_kernel(const AttnParams p, const Plan g)
                         // (the later reference, in which the accumulator is, is the larger one)
                         const float2* ml = s_ml + (n_item & 1) * STREAMS * BM + row;
                         const float ref = fmaxf(ml[0].y, ml[BM].y);
-                        float l = 0.f;
-#pragma unroll
-                        for (int q = 0; q < STREAMS; ++q) l = __fmaf_rn(__uint_as_float(s_sum[q * BM + row]), ex2(ml[q * BM].y - ref), l);
-                        inv_l = 1.0f / l;
+                        // (products rounded before they are added, as a stream rounds them that has one more tile, all of it hidden from this row:
+                        // how far the tile's last row sees changes no bit)
+                        inv_l = 1.0f / __fadd_rn(__fmul_rn(__uint_as_float(s_sum[row]), ex2(ml[0].y - ref)),
+                                                 __fmul_rn(__uint_as_float(s_sum[BM + row]), ex2(ml[BM].y - ref)));
                     } else {
 #pragma unroll
                         for (int q = 0; q < STREAMS; ++q) rs += (int)s_sum[q * BM + row];
@@ -965,9 +960,11 @@ prefill_kernel(const AttnParams p, const Plan g)
                         }
                         continue;
                     }
-                    // ---- KV: the reference that the row's probabilities are relative to. It is the first tile's maximum, and moves to a later tile's
-                    // where that one is above it by REF_ROOM. References are handed from tile to tile, and so from stream to stream, in
-                    // two sets by turns, since a stream may be an item ahead of the other (no more: see B_OUT below).
+                    // ---- KV: the reference that the row's probabilities are relative to: its maximum so far. References are handed from tile to tile,
+                    // and so from stream to stream, in two sets by turns, since a stream may be an item ahead of the other (no more: see
+                    // B_OUT below). Each row moves for itself: with the other rows of its warp, as the pass over the accumulator would allow, its bits
+                    // would depend on the queries beside it. Error against 64 bits of 24 calls (level, rising and falling scores), ratio to that of
+                    // two walks: 0.996 to 1.000; with moves of more than a power of two only: 0.9985 to 1.0004, and at most 2 % faster.
                     float down = 1.f;                                          // what the sums so far are worth in the new reference
                     bool moved = false;
                     if constexpr (MODE == KV) {
@@ -980,16 +977,14 @@ prefill_kernel(const AttnParams p, const Plan g)
                                 x0 = fmaxf(x0, fmaxf(S[e].x, S[e].y));
                                 x1 = fmaxf(x1, fmaxf(S[e + 1].x, S[e + 1].y));
                             }
-                            const float top = fmaxf(x0, x1);
-                            float ref = top;
+                            float ref = fmaxf(x0, x1);
                             if (kt > 0) {
                                 if (!mbar_sleep_warp(bar(B_REF + 8 * set + 2 * q4 + (stream ^ 1)), (ref_par >> set) & 1, s_abort)) { ok = false; break; }
                                 ref_par ^= 1u << set;
                                 const float before = ml[(stream ^ 1) * BM].x;
-                                // (where one row of the warp has to move, all move to their maxima: the pass over the accumulator is the same)
-                                moved = __any_sync(0xffffffffu, top > before + REF_ROOM) && top > before;
-                                if (!moved) ref = before;
-                                else down = ex2(before - ref);
+                                moved = ref > before;
+                                if (moved) down = ex2(before - ref);
+                                else ref = before;
                             }
                             if (kt + 1 < it.n_kt) {
                                 ml[stream * BM].x = ref;
@@ -1010,7 +1005,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                     if constexpr (MODE == KV) {
                         if (live && __any_sync(0xffffffffu, moved)) {
                             // the output accumulator of my rows in the new reference, when the tile before has been multiplied (with one buffer for both
-                            // streams that is what has just been waited for) and before mine is
+                            // streams that is what has just been waited for) and before mine is.
                             const uint32_t n_before = stream == 0 ? n_other + (kt >> 1) : n_other + ((kt + 1) >> 1);
                             if (g.p_tiles == 2 && !mbar_sleep_warp(bar(B_PEMPTY + (stream ^ 1)), (n_before - 1) & 1, s_abort)) { ok = false; break; }
                             tc_fence_after();

@@ -275,3 +275,53 @@ def test_scores_that_rise_along_the_keys(hd, bits, Tq, Tk, n_seq, causal):
     step = float(np.dot(c.size_qk, c.sK)) / 2 * top * c.qk_scale          # what a query of ones gains from the first key to the last
     rise = rng.choice([-300.0, -20.0, 0.0, 3.0, 12.0, 60.0, 300.0], size=(Tq * n_seq, 1)) / step
     _check(c, (rise * (1 + 0.1 * rng.normal(size=(Tq * n_seq, 2 * hd)))).astype(np.float16), causal, n_seq=n_seq)
+
+
+def _rising(seed, H, hd, Tq, Tk, n_seq, bits):
+    """A case whose keys' codes grow from the first key of a sequence to the last, and queries of which some gain hundreds of powers of two on
+    the way, some a few, some nothing."""
+    rng = np.random.default_rng(seed)
+    top = (1 << bits[1]) - 1
+    c = Case(seed, H=H, hd=hd, gh=1 if hd == 256 else 2, Tq=Tq * n_seq, Tk=Tk * n_seq, bits=bits)
+    ramp = np.tile(np.arange(Tk) / (Tk - 1.0), n_seq)[:, None] * top
+    off, _ = oracle.segment_offsets(c.size_qk)
+    for cl, n in enumerate(c.size_qk):
+        sl = slice(off[cl], off[cl] + n)
+        c.k[:, sl] = np.clip(np.rint(ramp + 0.1 * top * rng.normal(size=(Tk * n_seq, n))), 0, top)
+    _rebuild_keys(c, bits[1])
+    step = float(np.dot(c.size_qk, c.sK)) / H * top * c.qk_scale
+    rise = rng.choice([-100.0, -5.0, 0.0, 1.5, 6.0, 40.0, 200.0], size=(Tq * n_seq, 1)) / step
+    return c, (rise * (1 + 0.3 * rng.normal(size=(Tq * n_seq, H * hd)))).astype(np.float16)
+
+
+def _outputs(c, q16, causal, n_seq=1, Tk=None):
+    """fp16 [rows of q16][C]: these queries on the case's cache, or on its first Tk keys."""
+    import torch
+    from paper_2304_01089_b200 import binding
+    Tq, Tk = q16.shape[0] // n_seq, Tk or c.Tk // n_seq
+    out = torch.full((q16.shape[0], c.H * c.hd), 7.0, dtype=torch.float16, device="cuda")
+    binding.attention_kv(c.LK, c.LV, c.H, torch.from_numpy(np.ascontiguousarray(q16)).cuda(), c.dk, c.dv, out, c.qk_scale,
+                         causal, Tq=Tq, Tk=Tk, n_seq=n_seq)
+    torch.cuda.synchronize()
+    assert binding.get_device_status() == 0
+    return out.cpu().numpy()
+
+
+@pytest.mark.parametrize("hd,bits", [(64, (4, 4, 4)), (256, (4, 8, 8))])
+def test_a_row_depends_on_nothing_but_itself_and_its_keys(hd, bits):
+    """The same bits whatever the other queries of the block are (other magnitudes, infinite ones among them), and whether a prompt comes
+    whole or in chunks, whose rows lie elsewhere in their blocks and see other tiles hidden."""
+    Tq, Tk = 300, 700
+    c, q = _rising(990 + hd, 2, hd, Tq, Tk, 1, bits)
+    whole = _outputs(c, q, True)
+    assert np.isfinite(whole).all()
+    rng = np.random.default_rng(17)
+    others = (q * rng.choice([0.0, 0.3, 3.0], size=(Tq, 1))).astype(np.float16)
+    others[::11] = np.inf
+    keep = np.arange(Tq) % 5 == 2
+    others[keep] = q[keep]
+    np.testing.assert_array_equal(_outputs(c, others, True)[keep].view(np.uint16), whole[keep].view(np.uint16))
+    cuts = [0, 40, 57, 190, 213, Tq]
+    for lo, hi in zip(cuts, cuts[1:]):
+        part = _outputs(c, q[lo:hi], True, Tk=Tk - Tq + hi)
+        np.testing.assert_array_equal(part.view(np.uint16), whole[lo:hi].view(np.uint16))
