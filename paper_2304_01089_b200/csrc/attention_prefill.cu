@@ -90,12 +90,15 @@ __device__ __forceinline__ void ld32(uint32_t taddr, uint32_t (&v)[32])
           "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
         : "r"(taddr) : "memory");
 }
-__device__ __forceinline__ void st16(uint32_t taddr, const uint32_t (&v)[16])
+__device__ __forceinline__ void st32(uint32_t taddr, const uint32_t (&v)[32])
 {
     asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x16.b32 [%16], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15};"
+        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31};"
         ::"r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]),
-          "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]), "r"(taddr) : "memory");
+          "r"(v[8]), "r"(v[9]), "r"(v[10]), "r"(v[11]), "r"(v[12]), "r"(v[13]), "r"(v[14]), "r"(v[15]),
+          "r"(v[16]), "r"(v[17]), "r"(v[18]), "r"(v[19]), "r"(v[20]), "r"(v[21]), "r"(v[22]), "r"(v[23]),
+          "r"(v[24]), "r"(v[25]), "r"(v[26]), "r"(v[27]), "r"(v[28]), "r"(v[29]), "r"(v[30]), "r"(v[31]), "r"(taddr) : "memory");
 }
 // The whole warp executes these in converged control flow; one elected lane issues. a, b: the low words of the operands'
 // descriptors (the high words are the same for every tile).
@@ -1005,20 +1008,23 @@ prefill_kernel(const AttnParams p, const Plan g)
                     if constexpr (MODE == KV) {
                         if (live && __any_sync(0xffffffffu, moved)) {
                             // the output accumulator of my rows in the new reference, when the tile before has been multiplied (with one buffer for both
-                            // streams that is what has just been waited for) and before mine is.
+                            // streams that is what has just been waited for) and before mine is. What it costs, us, scores that fall along the keys and so
+                            // hardly move, rise, and show no trend: heads of 128 channels (32 heads, 3 x 1100 queries on 1337 keys) 292, 301, 304
+                            // (two walks: 326); of 64 (32 heads, 2 x 2048 tokens) 283, 347, 349 (two walks: 355). 32 columns a wait instead of 16:
+                            // 64 queries on 3000 keys 114 -> 112.
                             const uint32_t n_before = stream == 0 ? n_other + (kt >> 1) : n_other + ((kt + 1) >> 1);
                             if (g.p_tiles == 2 && !mbar_sleep_warp(bar(B_PEMPTY + (stream ^ 1)), (n_before - 1) & 1, s_abort)) { ok = false; break; }
                             tc_fence_after();
                             const int nuv = __ldg(p.cl_unit0_v + (it.h + 1) * p.gh_v) - __ldg(p.cl_unit0_v + it.h * p.gh_v);
                             const uint32_t t_out = tmem + ((uint32_t)(32 * q4) << 16);
 #pragma unroll 1
-                            for (int c = 0; c < 2 * nuv; ++c) {
-                                uint32_t v[16];
-                                tc_ld16(t_out + 16 * c, v);
+                            for (int u = 0; u < nuv; ++u) {
+                                uint32_t v[32];
+                                ld32(t_out + 32 * u, v);
                                 tc_wait_ld();
 #pragma unroll
-                                for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * down);
-                                st16(t_out + 16 * c, v);
+                                for (int e = 0; e < 32; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) * down);
+                                st32(t_out + 32 * u, v);
                             }
                             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
                             tc_fence_before();
