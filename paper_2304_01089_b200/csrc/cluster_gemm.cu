@@ -60,11 +60,12 @@ constexpr int UNPACK_WARP0 = 4, GROUP_WARPS = 4;          // warps of an unpack 
 constexpr int n_unpack_warps(int mode) { return mode == MODE_DEQ ? 2 * GROUP_WARPS : GROUP_WARPS; }
 constexpr int N_EPI_WARPS = 8;
 // registers per thread after the in-kernel re-partition (the block is launched with 128, MODE_DEQ 96 each): the
-// producer / MMA-issuer group, the unpack groups, the two epilogue groups (128 running sums per thread, none in MODE_DEQ)
-constexpr int REGS_WG0 = 40;
+// producer / MMA-issuer group, the unpack groups, the two epilogue groups (128 running sums per thread, none in MODE_DEQ). With 40 for its
+// first group MODE_DEQ spills there, in the loops that feed the tensor core (one block, 8 bits, 128 x 9216 x 9216: 76 us, with 48 67)
+constexpr int regs_wg0(int mode) { return mode == MODE_DEQ ? 48 : 40; }
 constexpr int regs_unpack(int mode) { return mode == MODE_DEQ ? 104 : 88; }
 constexpr int regs_epi(int mode) { return mode == MODE_DEQ ? 112 : 192; }
-constexpr int regs_all(int mode) { return 128 * REGS_WG0 + 32 * n_unpack_warps(mode) * regs_unpack(mode) + 256 * regs_epi(mode); }
+constexpr int regs_all(int mode) { return 128 * regs_wg0(mode) + 32 * n_unpack_warps(mode) * regs_unpack(mode) + 256 * regs_epi(mode); }
 static_assert(regs_all(MODE_INT) <= 128 * 512 && regs_all(MODE_DEQ) <= 96 * 640, "register pool");
 constexpr int A8_BYTES = TILE_M * KBLK;                  // 16 KiB of 8-bit activation operands per stage
 constexpr int WTILE_BYTES = 8192;                        // one packed weight tile: 128 rows x 64 bytes
@@ -84,8 +85,12 @@ __host__ __device__ constexpr int a_slot_pitch(int bits, int mode) { return mode
 __host__ __device__ constexpr int n_a_stages(int ncta, int bits, int mode) { return bits == 8 || (ncta == 1 && bits == 3 && mode != MODE_DEQ) ? 2 : mode == MODE_DEQ ? 3 : 4; }
 
 struct SmemLayout {
-    int u_stage, p_stage, a_stage, out_row, off_p, off_a, off_flags, off_seg_scale, off_seg_buf, off_tab, off_seg_tab, off_seg_cl, off_stage, off_bar, total;
+    int u_stage, p_stage, a_stage, off_p, off_a, off_flags, off_seg_scale, off_seg_buf, off_tab, off_seg_tab, off_seg_cl, off_stage, off_bar, total;
 };
+constexpr int OUT_ROW = 64;                              // output staging buffer of an epilogue warp: 32 rows of so many bytes (128 would fit in
+                                                         // MODE_DEQ's one-block instances only, and is no faster there)
+// rows of the column tables: zero-point correction (none in MODE_DEQ), s_w, bias
+__host__ __device__ constexpr int n_tab_rows(int mode) { return mode == MODE_DEQ ? 2 : 3; }
 constexpr int SEG_SLOTS = 2;                             // ASYM: clusters whose column tables are held at a time
 __host__ __device__ constexpr SmemLayout smem_layout(int ncta, int bits, bool a8, int mode)
 {
@@ -100,12 +105,10 @@ __host__ __device__ constexpr SmemLayout smem_layout(int ncta, int bits, bool a8
     s.off_seg_scale = s.off_flags + 2048;
     s.off_seg_buf = s.off_seg_scale + (mode == MODE_INT ? kMaxGemmSegments * 4 : 0);
     s.off_tab = s.off_seg_buf + (mode == MODE_DEQ ? 0 : kMaxGemmSegments);          // (DEQ: one accumulator per tile, no clusters)
-    s.off_seg_tab = s.off_tab + 2 * 3 * TILE_N * 4;
+    s.off_seg_tab = s.off_tab + 2 * n_tab_rows(mode) * TILE_N * 4;
     s.off_seg_cl = s.off_seg_tab + (asym ? SEG_SLOTS * 2 * TILE_N * 4 : 0);
     s.off_stage = s.off_seg_cl + (asym ? kMaxGemmSegments * 2 : 0);
-    // output staging buffer of an epilogue warp: 32 rows of 64 or 128 bytes, as there is room for
-    s.out_row = s.off_stage + N_EPI_WARPS * 32 * 128 + 320 + 1024 <= 227 * 1024 ? 128 : 64;
-    s.off_bar = s.off_stage + N_EPI_WARPS * 32 * s.out_row;
+    s.off_bar = s.off_stage + N_EPI_WARPS * 32 * OUT_ROW;
     s.total = s.off_bar + 320;
     return s;
 }
@@ -251,7 +254,7 @@ __device__ __forceinline__ void tc_mma_bf16(uint32_t d_tmem, uint64_t a_desc, ui
     }
 }
 // 16 lanes x 32 columns: v[4 j + 2 r + c] is row lane / 4 + 8 r, column 8 j + 2 (lane % 4) + c
-__device__ __forceinline__ void tc_ld16x4(uint32_t taddr, uint32_t (&v)[16])
+__device__ __forceinline__ void tc_ld16xn(uint32_t taddr, uint32_t (&v)[16])
 {
     asm volatile(
         "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
@@ -259,8 +262,20 @@ __device__ __forceinline__ void tc_ld16x4(uint32_t taddr, uint32_t (&v)[16])
           "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
         : "r"(taddr) : "memory");
 }
-// four 8 x 8 matrices of 16-bit values, matrix j's rows at the addresses that lanes 8 j .. 8 j + 7 name
-__device__ __forceinline__ void stmatrix4(uint32_t addr, const uint32_t (&f)[4])
+// 16 lanes x 16 columns in the same manner
+__device__ __forceinline__ void tc_ld16xn(uint32_t taddr, uint32_t (&v)[8])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7])
+        : "r"(taddr) : "memory");
+}
+// four (two) 8 x 8 matrices of 16-bit values, matrix j's rows at the addresses that lanes 8 j .. 8 j + 7 name
+__device__ __forceinline__ void stmatrixn(uint32_t addr, const uint32_t (&f)[2])
+{
+    asm volatile("stmatrix.sync.aligned.m8n8.x2.shared.b16 [%0], {%1, %2};" ::"r"(addr), "r"(f[0]), "r"(f[1]) : "memory");
+}
+__device__ __forceinline__ void stmatrixn(uint32_t addr, const uint32_t (&f)[4])
 {
     asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(f[0]), "r"(f[1]), "r"(f[2]), "r"(f[3]) : "memory");
 }
@@ -330,6 +345,7 @@ cluster_gemm_kernel(const Params p)
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     constexpr SmemLayout SL = smem_layout(NCTA, BITS, A8, MODE);
     constexpr int THREADS = threads_of(MODE), EPI_WARP0 = UNPACK_WARP0 + n_unpack_warps(MODE);
+    constexpr int TAB_ROWS = n_tab_rows(MODE);
     constexpr int W_ROWS = w_rows(NCTA);                 // weight rows this CTA stages and unpacks
     constexpr int N_P = n_p_stages(NCTA, BITS, MODE), N_U = n_u_stages(NCTA, A8);
     constexpr uint32_t kInstrDesc = DEQ ? instr_desc_bf16(NCTA) : instr_desc(NCTA);      // (of a whole tile)
@@ -341,7 +357,7 @@ cluster_gemm_kernel(const Params p)
     uint8_t* s_flags = smem + SL.off_flags;
     float* s_seg_scale = reinterpret_cast<float*>(smem + SL.off_seg_scale);
     uint8_t* s_seg_buf = smem + SL.off_seg_buf;
-    float* s_tab = reinterpret_cast<float*>(smem + SL.off_tab);           // [2][3][TILE_N]
+    float* s_tab = reinterpret_cast<float*>(smem + SL.off_tab);           // [2][TAB_ROWS][TILE_N]
     float4* s_seg_tab = reinterpret_cast<float4*>(smem + SL.off_seg_tab); // ASYM: [SEG_SLOTS][TILE_N / 2]
     uint16_t* s_seg_cl = reinterpret_cast<uint16_t*>(smem + SL.off_seg_cl);   // ASYM: the cluster of each segment
     uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SL.off_bar);
@@ -408,7 +424,7 @@ cluster_gemm_kernel(const Params p)
     // The register file is re-partitioned by warpgroup (the epilogue holds 128 running sums per
     // thread); each setmaxnreg is executed by the four warps of its group at one place.
     if (warp < UNPACK_WARP0) {
-      asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(REGS_WG0));
+      asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(regs_wg0(MODE)));
       if (warp == 0) {
         // ------------------------------------------------------------ bulk-copy producer
         if (lane == 0) {
@@ -605,13 +621,14 @@ cluster_gemm_kernel(const Params p)
             }
             const uint32_t b = n_tile & 1;
             mbar_wait(bar(B_TABEMPTY + b), ((n_tile >> 1) & 1) ^ 1, s_abort);
-            float* tab = s_tab + b * 3 * TILE_N + 4 * tt;
+            float* tab = s_tab + b * TAB_ROWS * TILE_N + 4 * tt;
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 const bool in = n + e < p.N;
+                if constexpr (!DEQ) tab[e] = corr[e];
                 // ASYM: the column's scale is applied per cluster
-                const float sw = !in ? 0.f : ASYM ? 1.f : __ldg(p.s_w + n + e);
-                tab[e] = corr[e]; tab[TILE_N + e] = sw; tab[2 * TILE_N + e] = in && p.bias ? __ldg(p.bias + n + e) : 0.f;
+                tab[(TAB_ROWS - 2) * TILE_N + e] = !in ? 0.f : ASYM ? 1.f : __ldg(p.s_w + n + e);
+                tab[(TAB_ROWS - 1) * TILE_N + e] = in && p.bias ? __ldg(p.bias + n + e) : 0.f;
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(bar(B_TAB + b));
@@ -935,7 +952,7 @@ cluster_gemm_kernel(const Params p)
             int mt, n0;
             const int sh = item_of(t, mt, n0), half_cols = 128 >> sh;      // columns of my half
             const int m0 = mt * (TILE_M * NCTA) + (int)cta_rank * TILE_M;
-            float* tab = s_tab + (n_tile_done & 1) * 3 * TILE_N;
+            float* tab = s_tab + (n_tile_done & 1) * TAB_ROWS * TILE_N;
             // a warp whose 32 accumulator lanes all lie beyond the last token row keeps the barriers'
             // protocol but reads and accumulates nothing (few-token calls: most of the tile is empty)
             const bool live = m0 + 32 * q < p.M;
@@ -995,8 +1012,8 @@ cluster_gemm_kernel(const Params p)
                 for (int jc = 0; jc < 4; ++jc) {
                     uint32_t va[16], vb[16];
                     float4 k[4];
-                    tc_ld16x4(taddr + 32 * jc, va);
-                    tc_ld16x4(taddr + (16u << 16) + 32 * jc, vb);
+                    tc_ld16xn(taddr + 32 * jc, va);
+                    tc_ld16xn(taddr + (16u << 16) + 32 * jc, vb);
                     if constexpr (ASYM) {
 #pragma unroll
                         for (int j = 0; j < 4; ++j) k[j] = seg_tab[(jc * 4 + j) * 4];
@@ -1030,14 +1047,16 @@ cluster_gemm_kernel(const Params p)
             if (live) {
                 const int mw = m0 + 32 * q, nb = n0 + h * half_cols;           // my warp's first row, my first column
                 const float2* t_corr = reinterpret_cast<const float2*>(tab + h * half_cols) + (lane & 3);
-                const float2* t_sw = t_corr + TILE_N / 2;
-                const float2* t_bs = t_sw + TILE_N / 2;
+                const float2* t_sw = t_corr + (TAB_ROWS - 2) * (TILE_N / 2);
+                const float2* t_bs = t_corr + (TAB_ROWS - 1) * (TILE_N / 2);
                 const bool relu = p.act == RPTQ_ACT_RELU;
-                // 32 columns at a time (DEQ: its sums are not in registers, of which it has few: a rolled loop)
-                auto each_jc = [&](auto body) {
+                // J times 8 columns at a time (DEQ: its sums are not in registers, of which it has few: a rolled loop, and with one block, whose output
+                // phase is short, half as many columns: 100 x 4096 x 12288, 3 and 4 bits, 41.5 and 42.5 us -> 40.4 and 41.4)
+                constexpr int J = DEQ && NCTA == 1 ? 2 : 4;
+                auto each_step = [&](auto body) {
                     if constexpr (DEQ) {
 #pragma unroll 1
-                        for (int jc = 0; 32 * jc < half_cols; ++jc) body(jc);
+                        for (int st = 0; 8 * J * st < half_cols; ++st) body(st);
                     } else {
                         body(std::integral_constant<int, 0>());
                         if (half_cols > 32) body(std::integral_constant<int, 1>());
@@ -1045,10 +1064,10 @@ cluster_gemm_kernel(const Params p)
                     }
                 };
                 // piece j (16 bytes) of row r lies at j ^ sw(r): neither what a warp puts nor what it reads in one instruction meets in a bank
-                constexpr int OUT_ROW = SL.out_row, PIECES = OUT_ROW / 16, ROWS_I = 32 / PIECES;          // ROWS_I: rows that a warp-wide access covers
+                constexpr int PIECES = OUT_ROW / 16, ROWS_I = 32 / PIECES;     // ROWS_I: rows that a warp-wide access covers
                 const uint32_t stage = smem_base + SL.off_stage + ew * 32 * OUT_ROW;
-                auto sw_f16 = [](int r) { return OUT_ROW == 128 ? r & 7 : (r >> 1) & 3; };                  // 16 bytes of eight rows at a time
-                auto sw_f32 = [](int r) { return OUT_ROW == 128 ? (r & 3) << 1 : (r & 2); };                // 32 bytes of four rows at a time
+                auto sw_f16 = [](int r) { return (r >> 1) & 3; };              // 16 bytes of eight rows at a time
+                auto sw_f32 = [](int r) { return r & 2; };                     // 32 bytes of four rows at a time
                 auto store = [&](auto sw, uint8_t* dst, int64_t row_bytes, int n_bytes) {   // dst: the warp's first row; n_bytes valid of OUT_ROW
                     __syncwarp();
                     const int j = lane % PIECES, r0 = lane / PIECES, left = n_bytes - 16 * j, rows = p.M - mw;
@@ -1068,25 +1087,28 @@ cluster_gemm_kernel(const Params p)
                 };
                 // DEQ: the finished fp32 sums are in tensor memory
                 const uint32_t t_acc = tmem_base + ((uint32_t)(32 * q) << 16) + (n_tile_done & 1u) * TILE_N + h * half_cols;
-                // my values of columns 8 i + {0, 1} (i = 4 jc + j), rows 16 hh + 8 r
-                auto finish = [&](int jc, auto use) {
-                    float2 own[16];
+                // my values of columns 8 (J st + j) + {0, 1}, rows lane / 4 + 8 k
+                auto finish = [&](int st, auto use) {
+                    float2 own[4 * J];
                     if constexpr (DEQ) {
-                        uint32_t v[2][16];
-                        tc_ld16x4(t_acc + 32 * jc, v[0]);
-                        tc_ld16x4(t_acc + (16u << 16) + 32 * jc, v[1]);
+                        uint32_t v[2][4 * J];
+                        tc_ld16xn(t_acc + 8 * J * st, v[0]);
+                        tc_ld16xn(t_acc + (16u << 16) + 8 * J * st, v[1]);
                         tc_wait_ld();
 #pragma unroll
-                        for (int i = 0; i < 16; ++i) own[i] = make_float2(__uint_as_float(v[i >> 3][2 * (i & 7)]), __uint_as_float(v[i >> 3][2 * (i & 7) + 1]));
+                        for (int i = 0; i < 4 * J; ++i) own[i] = make_float2(__uint_as_float(v[i / (2 * J)][2 * (i % (2 * J))]), __uint_as_float(v[i / (2 * J)][2 * (i % (2 * J)) + 1]));
                     }
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        const float2 c = t_corr[(jc * 4 + j) * 4], w = t_sw[(jc * 4 + j) * 4], b = t_bs[(jc * 4 + j) * 4];
+                    for (int j = 0; j < J; ++j) {
+                        const int at = (J * st + j) * 4;
+                        const float2 w = t_sw[at], b = t_bs[at];
+                        float2 c;
+                        if constexpr (!DEQ) c = t_corr[at];
 #pragma unroll
-                        for (int k = 0; k < 4; ++k) {                          // rows lane / 4 + 8 k
-                            float2 sum;
-                            if constexpr (DEQ) sum = own[(k >> 1) * 8 + 2 * j + (k & 1)]; else sum = R[(jc * 2 + (k >> 1)) * 8 + 2 * j + (k & 1)];
-                            float2 v = fma2(w, add2(sum, make_float2(-c.x, -c.y)), b);
+                        for (int k = 0; k < 4; ++k) {
+                            float2 v;
+                            if constexpr (DEQ) v = own[(k >> 1) * 2 * J + 2 * j + (k & 1)]; else v = add2(R[(st * 2 + (k >> 1)) * 8 + 2 * j + (k & 1)], make_float2(-c.x, -c.y));
+                            v = fma2(w, v, b);
                             if (relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); }
                             use(j, k, v);
                         }
@@ -1095,32 +1117,30 @@ cluster_gemm_kernel(const Params p)
                 if (p.y_dtype == RPTQ_OUT_F16) {
                     uint8_t* dst = static_cast<uint8_t*>(p.y) + ((int64_t)mw * p.ldy + nb) * 2;
                     const int n_bytes = 2 * min(p.N - nb, half_cols);
-                    // (my lane names row 8 k + lane % 8, piece lane / 8 of the 32 columns, to stmatrix)
-                    each_jc([&](auto at_jc) {
-                        const int jc = at_jc;
-                        uint32_t f[4][4];                                      // [k][j]
-                        finish(jc, [&](int j, int k, float2 v) { const __half2 x = __floats2half2_rn(v.x, v.y); f[k][j] = *reinterpret_cast<const uint32_t*>(&x); });
-                        const int j0 = 4 * jc % PIECES;
+                    // (my lane names row 8 k + lane % 8, piece lane / 8 of the step's columns, to stmatrix)
+                    each_step([&](auto at_st) {
+                        const int st = at_st, j0 = J * st % 4;
+                        uint32_t f[4][J];                                      // [k][j]
+                        finish(st, [&](int j, int k, float2 v) { const __half2 x = __floats2half2_rn(v.x, v.y); f[k][j] = *reinterpret_cast<const uint32_t*>(&x); });
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
                             const int r = 8 * k + (lane & 7);
-                            stmatrix4(stage + r * OUT_ROW + (((j0 + (lane >> 3)) ^ sw_f16(r)) << 4), f[k]);
+                            stmatrixn(stage + r * OUT_ROW + (((j0 + (lane >> 3) % J) ^ sw_f16(r)) << 4), f[k]);
                         }
-                        const int from = 64 * jc / OUT_ROW * OUT_ROW;
-                        if (j0 + 4 == PIECES || 32 * (jc + 1) >= half_cols) store(sw_f16, dst + from, p.ldy * 2, n_bytes - from);
+                        const int from = 16 * (J * st - j0);
+                        if (j0 + J == 4) store(sw_f16, dst + from, p.ldy * 2, n_bytes - from);
                     });
                 } else if (p.y_dtype == RPTQ_OUT_F32) {
                     uint8_t* dst = static_cast<uint8_t*>(p.y) + ((int64_t)mw * p.ldy + nb) * 4;
                     const int n_bytes = 4 * min(p.N - nb, half_cols);
                     const uint32_t put = stage + (lane >> 2) * OUT_ROW + 8 * (lane & 1);
                     const int piece = (lane & 3) >> 1;
-                    each_jc([&](auto at_jc) {
-                        const int jc = at_jc;
-                        finish(jc, [&](int j, int k, float2 v) {
-                            const int at = 2 * j % PIECES;
-                            sts64(put + 8 * k * OUT_ROW + (((at + piece) ^ sw_f32(lane >> 2)) << 4), v);      // (8 k changes no swizzle)
-                            if (k == 3 && at + 2 == PIECES) {
-                                const int from = (32 * jc + 8 * (j + 1)) * 4 - OUT_ROW;
+                    each_step([&](auto at_st) {
+                        const int st = at_st;
+                        finish(st, [&](int j, int k, float2 v) {
+                            sts64(put + 8 * k * OUT_ROW + (((2 * (j & 1) + piece) ^ sw_f32(lane >> 2)) << 4), v);      // (8 k changes no swizzle)
+                            if (k == 3 && (j & 1)) {
+                                const int from = 32 * (J * st + j - 1);
                                 store(sw_f32, dst + from, p.ldy * 4, n_bytes - from);
                             }
                         });
@@ -1175,7 +1195,7 @@ cluster_gemm_kernel(const Params p)
 #pragma unroll
                             for (int j = 3; j >= 0; --j) x[k] = sat_pack_u4(qv[k][j][1], qv[k][j][0], x[k]);
                         const uint32_t own_row = stage + lane * OUT_ROW + ((jc ^ sw_f16(lane)) << 4);
-                        stmatrix4(own_row, x);
+                        stmatrixn(own_row, x);
                         __syncwarp();
                         const uint4 t = lds128(own_row);                       // word l: byte j is codes 2 l, 2 l + 1 of word j
                         const uint32_t a01 = __byte_perm(t.x, t.y, 0x5140), a23 = __byte_perm(t.x, t.y, 0x7362);

@@ -98,3 +98,41 @@ def test_workload_sites_sampled_rows(name, li, Ms):
         exact = oracle.dequant_matmul(a, w_o, site.cal.size, site.cal.scale.astype(np.float64), site.cal.zero, s_o)
         print(f"{name} M={M}: max|dy|/max|y| = {err:.2e} vs the bf16 statement, {np.max(np.abs(got - exact)) / np.abs(exact).max():.2e} vs the exact first method")
         assert err <= TOL
+
+
+@pytest.mark.parametrize("bits", [4, 3, 8])
+@pytest.mark.parametrize("f16", [False, True])
+def test_whole_tiles_and_strips_give_the_bits_of_small_calls(f16, bits):
+    """80 tiles on 74 pairs of blocks: 74 whole ones and 6 that are cut into strips, the last rows and columns ragged, against calls of at most
+    128 tokens (other blocks, which read their sums 16 columns at a time instead of 32)."""
+    import torch
+    from paper_2304_01089_b200 import binding
+    M, N, n_pad = 2401, 2045, 2048
+    rng = np.random.default_rng(9300 + bits)
+    perm, size, scale, zero = random_layout_params(rng, 256, 3, bits, allow_empty=False)
+    L = binding.Layout(perm, size, scale, zero, bits)
+    W = (rng.normal(size=(N, 256)) * 0.02).astype(np.float32)
+    w_o, s_w, _ = oracle.weight_quantize(W, perm, size, None, n_pad)
+    m = L.contiguous_position()
+    off, k_pad = oracle.segment_offsets(size)
+    a = np.zeros((M, k_pad), np.uint8)
+    for c in range(3):
+        a[:, off[c]:off[c] + size[c]] = rng.integers(0, 1 << bits, size=(M, size[c]))
+    a_dev = torch.from_numpy(oracle.pack(np.ascontiguousarray(a[:, m]), bits)).cuda()
+    w_dev = torch.from_numpy(oracle.pack_weights(np.ascontiguousarray(w_o[:, m]))).cuda()
+    s_dev = torch.from_numpy(s_w).cuda()
+    bias = torch.from_numpy((rng.normal(size=n_pad) * 0.05).astype(np.float32)).cuda()
+
+    def call(lo, n):
+        y = torch.full((n + 1, n_pad), float("nan"), dtype=torch.float16 if f16 else torch.float32, device="cuda")
+        binding.dequant_gemm(L, a_dev[lo:lo + n].contiguous(), n, w_dev, s_dev, N, y, ld_w=n_pad, bias=bias, act=binding.ACT_RELU,
+                             y_dtype=binding.OUT_F16 if f16 else binding.OUT_F32)
+        torch.cuda.synchronize()
+        assert binding.get_device_status() == 0 and bool(torch.isnan(y[n]).all()) and bool(torch.isnan(y[:, N:]).all())
+        return y.cpu().numpy()[:n, :N]
+
+    whole = call(0, M)
+    assert np.isfinite(whole).all() and whole.max() > 0
+    for lo in range(0, M, 128):
+        n = min(128, M - lo)
+        np.testing.assert_array_equal(whole[lo:lo + n], call(lo, n))
