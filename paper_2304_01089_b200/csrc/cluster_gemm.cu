@@ -75,7 +75,7 @@ __host__ __device__ constexpr int w_rows(int ncta) { return TILE_N / ncta; }    
 __host__ __device__ constexpr int n_p_stages(int ncta, int bits, int mode) 
 {
     if (ncta == 2) return 4;
-    return mode == MODE_DEQ || (mode == MODE_ASYM && bits == 8) ? 3 : bits == 3 ? 5 : 4;
+    return mode == MODE_DEQ ? 3 : bits == 3 ? 5 : 4;
 }
 __host__ __device__ constexpr int n_u_stages(int ncta, bool a8) { return ncta == 2 ? (a8 ? 5 : 4) : 2; }   // operand stages
 // ring of packed activation K blocks fetched ahead by the unpack threads: one slot per token row
@@ -89,8 +89,9 @@ struct SmemLayout {
 };
 constexpr int OUT_ROW = 64;                              // output staging buffer of an epilogue warp: 32 rows of so many bytes (128 would fit in
                                                          // MODE_DEQ's one-block instances only, and is no faster there)
-// rows of the column tables: zero-point correction (none in MODE_DEQ), s_w, bias
-__host__ __device__ constexpr int n_tab_rows(int mode) { return mode == MODE_DEQ ? 2 : 3; }
+// rows of the column tables: zero-point correction (none in MODE_DEQ), s_w (none in MODE_ASYM, which applies it per cluster), bias. Rows that hold
+// one constant cost the 8-bit one-block instance of MODE_ASYM a weight stage (32 x 4096 x 12288: 25.7 us with four, 26.2 with three)
+__host__ __device__ constexpr int n_tab_rows(int mode) { return mode == MODE_INT ? 3 : 2; }
 constexpr int SEG_SLOTS = 2;                             // ASYM: clusters whose column tables are held at a time
 __host__ __device__ constexpr SmemLayout smem_layout(int ncta, int bits, bool a8, int mode)
 {
@@ -626,8 +627,7 @@ cluster_gemm_kernel(const Params p)
             for (int e = 0; e < 4; ++e) {
                 const bool in = n + e < p.N;
                 if constexpr (!DEQ) tab[e] = corr[e];
-                // ASYM: the column's scale is applied per cluster
-                tab[(TAB_ROWS - 2) * TILE_N + e] = !in ? 0.f : ASYM ? 1.f : __ldg(p.s_w + n + e);
+                if constexpr (!ASYM) tab[(TAB_ROWS - 2) * TILE_N + e] = in ? __ldg(p.s_w + n + e) : 0.f;
                 tab[(TAB_ROWS - 1) * TILE_N + e] = in && p.bias ? __ldg(p.bias + n + e) : 0.f;
             }
             __syncwarp();
@@ -1101,14 +1101,15 @@ cluster_gemm_kernel(const Params p)
 #pragma unroll
                     for (int j = 0; j < J; ++j) {
                         const int at = (J * st + j) * 4;
-                        const float2 w = t_sw[at], b = t_bs[at];
-                        float2 c;
+                        float2 c, w;
                         if constexpr (!DEQ) c = t_corr[at];
+                        if constexpr (!ASYM) w = t_sw[at];
+                        const float2 b = t_bs[at];
 #pragma unroll
                         for (int k = 0; k < 4; ++k) {
                             float2 v;
                             if constexpr (DEQ) v = own[(k >> 1) * 2 * J + 2 * j + (k & 1)]; else v = add2(R[(st * 2 + (k >> 1)) * 8 + 2 * j + (k & 1)], make_float2(-c.x, -c.y));
-                            v = fma2(w, v, b);
+                            if constexpr (ASYM) v = add2(v, b); else v = fma2(w, v, b);
                             if (relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); }
                             use(j, k, v);
                         }

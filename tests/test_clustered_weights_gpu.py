@@ -201,3 +201,53 @@ def test_the_tile_constant_does_not_depend_on_the_unit_order():
                                        torch.from_numpy(s_w).cuda(), torch.from_numpy(z_w).cuda(), torch.from_numpy(wsum).cuda(), N, y)
         out.append(y)
     assert torch.equal(out[0], out[1]) and bool((out[0] != 0).any())
+
+
+@pytest.mark.parametrize("out", ["f32", "f16", 3, 4, 8])
+def test_whole_tiles_and_strips_give_the_bits_of_small_calls(out):
+    """80 tiles on 74 pairs of blocks: 74 whole ones and 6 that are cut into strips, the last rows and (float outputs) the last columns ragged,
+    against calls of at most 128 tokens."""
+    import torch
+    from paper_2304_01089_b200 import binding
+    codes = isinstance(out, int)
+    M, N, n_pad = 2401, 2048 if codes else 2041, 2048
+    rng = np.random.default_rng(7300)
+    perm, _, scale, zero = random_layout_params(rng, 256, 3, 4)
+    size = np.array([70, 5, 181])
+    L = binding.Layout(perm, size, scale, zero, 4)
+    packed, s_w, z_w, wsum = (torch.from_numpy(t).cuda() for t in binding.weight_pack_clustered(L, (rng.normal(size=(N, 256)) * 0.02).astype(np.float32), n_pad))
+    off, k_pad = oracle.segment_offsets(size)
+    a = np.zeros((M, k_pad), np.uint8)
+    for c in range(3):
+        a[:, off[c]:off[c] + size[c]] = rng.integers(0, 16, size=(M, size[c]))
+    a_dev = torch.from_numpy(oracle.pack(np.ascontiguousarray(a[:, L.contiguous_position()]), 4)).cuda()
+    xsum = torch.empty((M, 3), dtype=torch.int32, device="cuda")
+    binding.code_rowsums(L, a_dev, M, xsum)
+    bias = torch.from_numpy((rng.normal(size=n_pad) * 0.05).astype(np.float32)).cuda()
+    L2 = None
+    if codes:
+        size2 = np.array([1, 31, 32, 33, 64, 500, 700, 500, 59])
+        y = torch.empty((128, N), dtype=torch.float32, device="cuda")
+        binding.cluster_gemm_clustered(L, a_dev, 128, xsum, packed, s_w, z_w, wsum, N, y)
+        step = float(y.abs().max()) / (1 << out)
+        L2 = binding.Layout(np.arange(size2.sum(), dtype=np.int32), size2, np.full(9, step, np.float32), np.full(9, 1 << (out - 1), np.int32), out)
+        assert L2.K_pad == N
+
+    def call(lo, n):
+        if codes:
+            y = torch.full((n + 1, L2.row_bytes), 0xA5, dtype=torch.uint8, device="cuda")
+        else:
+            y = torch.full((n + 1, n_pad), float("nan"), dtype=torch.float32 if out == "f32" else torch.float16, device="cuda")
+        # (the code sums' rows of three clusters need not begin on a 16-byte boundary: copied)
+        binding.cluster_gemm_clustered(L, a_dev[lo:lo + n].contiguous(), n, xsum[lo:lo + n].clone(), packed, s_w, z_w, wsum, N, y, bias=bias, act=binding.ACT_RELU,
+                                       layout_out=L2, y_dtype=binding.OUT_CODES if codes else binding.OUT_F32 if out == "f32" else binding.OUT_F16)
+        torch.cuda.synchronize()
+        assert binding.get_device_status() == 0
+        return y.cpu().numpy().view(np.uint8)
+
+    whole = call(0, M)
+    for lo in range(0, M, 128):
+        n = min(128, M - lo)
+        np.testing.assert_array_equal(whole[lo:lo + n], call(lo, n)[:n])
+    assert len(np.unique(whole[:M, :64])) > 4
+    np.testing.assert_array_equal(whole[M], call(0, 1)[1])                # nothing past the last row
