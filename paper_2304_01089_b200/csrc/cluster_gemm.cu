@@ -958,6 +958,13 @@ cluster_gemm_kernel(const Params p)
             const bool live = m0 + 32 * q < p.M;
 #pragma unroll
             for (int i = 0; i < 64; ++i) R[i] = make_float2(0.f, 0.f);
+            // outputs as codes: lane l holds the output layout's unit l of my columns, asked for before the sums (700 x 768 x 3072, 8
+            // clusters: 14.4 -> 13.6 us)
+            uint4 unit4 = make_uint4(0u, 0u, 0u, 0u);
+            if constexpr (!DEQ) {
+                const int unit = (n0 + h * half_cols) / 32 + (lane & 3);
+                if (p.y_dtype == RPTQ_OUT_CODES && 32 * unit < p.N) unit4 = __ldg(reinterpret_cast<const uint4*>(p.out_unit + unit));
+            }
             // ASYM: my tokens' code sums of the cluster to come (rows past the last token read the last one's)
             const int32_t* xs_row[4] = {nullptr, nullptr, nullptr, nullptr};
             int xs_next[4] = {0, 0, 0, 0};
@@ -1156,9 +1163,9 @@ cluster_gemm_kernel(const Params p)
                     for (int jc = 0; jc < 4; ++jc) {
                         if (jc >= n_units) break;
                         const int unit = (nb >> 5) + jc;
-                        const uint4 t4 = __ldg(reinterpret_cast<const uint4*>(p.out_unit + unit));
-                        const float2 s2 = make_float2(__uint_as_float(t4.x), __uint_as_float(t4.x)), c2 = make_float2(12582912.0f, 12582912.0f);
-                        const int zc = (int)t4.y, nvalid = (int)t4.w;
+                        const float inv_s = __uint_as_float(__shfl_sync(0xffffffffu, unit4.x, jc));
+                        const int zc = (int)__shfl_sync(0xffffffffu, unit4.y, jc), nvalid = (int)__shfl_sync(0xffffffffu, unit4.w, jc);
+                        const float2 s2 = make_float2(inv_s, inv_s), c2 = make_float2(12582912.0f, 12582912.0f);
                         int qv[4][4][2];                                       // [row k][word j]: not yet clamped, the pack saturates
                         finish(jc, [&](int j, int k, float2 v) {
                             v = fma2(v, s2, c2);
