@@ -337,12 +337,14 @@ __device__ __forceinline__ uint32_t nibbles_to_bf16(uint32_t w)
 // the unpack warps write X^ = s_c (X_q - z_c) as bfloat16 and the weight codes as bfloat16 integers, the MMAs are kind::f16 into ONE fp32 accumulator per tile -- no per-cluster
 // accumulators, no drains at cluster boundaries -- and s_w[n] multiplies the finished sum. A bfloat16
 // operand row of 128 bytes holds 64 positions, so a K block of 128 positions is two operand stages.
-template <int BITS, int NCTA, bool A8, int MODE>
+// ROWS (MODE_INT, CTA pairs): the epilogue holds its sums a token row per thread (see there).
+template <int BITS, int NCTA, bool A8, int MODE, bool ROWS>
 __global__ void __launch_bounds__(threads_of(MODE), 1)
 cluster_gemm_kernel(const Params p)
 {
     constexpr bool ASYM = MODE == MODE_ASYM, DEQ = MODE == MODE_DEQ;
     static_assert(!(DEQ && A8), "the de-quantising variant unpacks every bit width");
+    static_assert(!ROWS || (MODE == MODE_INT && NCTA == 2), "rows");
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     constexpr SmemLayout SL = smem_layout(NCTA, BITS, A8, MODE);
     constexpr int THREADS = threads_of(MODE), EPI_WARP0 = UNPACK_WARP0 + n_unpack_warps(MODE);
@@ -942,11 +944,12 @@ cluster_gemm_kernel(const Params p)
         uint32_t n_tile_done = 0;
         uint32_t par = 0;                    // bit b: parity of how many clusters of accumulator b I have drained
         uint32_t n_seg_done = 0;                     // ASYM: clusters drained so far, over all tiles
-        // Running sums, in the layout of the 16-lane tensor-memory loads: my rows of the warp's 32 are 16 h + lane / 4 + 8 r, my
-        // columns 8 i + 2 (lane % 4) + {0, 1}, R[(i / 4 * 2 + h) * 8 + i % 4 * 2 + r]. With a thread per row and all 128 columns instead,
-        // what belongs to a column is read by every thread, and a warp-wide load of 16 bytes takes four clocks of the SM's shared-memory
-        // port even where all lanes read the same: 64 a drain of clustered weights (2048 of its 2125 clocks), 96 a tile for the
-        // tables of the outputs. Here a load serves four rows.
+        // Running sums. ROWS: columns 2 i, 2 i + 1 of the thread's row in R[i]. Otherwise the layout of the 16-lane tensor-memory loads: my
+        // rows of the warp's 32 are 16 h + lane / 4 + 8 r, my columns 8 i + 2 (lane % 4) + {0, 1}, R[(i / 4 * 2 + h) * 8 + i % 4 * 2 + r].
+        // With a thread per row, what belongs to a column is read by every thread, and a warp-wide load of 16 bytes takes four clocks of
+        // the SM's shared-memory port even where all lanes read the same: 64 a drain of clustered weights (2048 of its 2125 clocks), 96 a tile
+        // for the tables of the outputs; in the other layout a load serves four rows. But its tensor-memory loads take longer (some 66 clocks a
+        // drain more), and a word of codes lies in four lanes. Which of the two is the faster depends on the clusters of a tile: see launch_gemm.
         float2 R[64];
         for (int t = pair_id; t < p.n_items; t += n_pairs, ++n_tile_done) {
             int mt, n0;
@@ -996,7 +999,7 @@ cluster_gemm_kernel(const Params p)
                 }
                 const uint32_t taddr = tmem_base + ((uint32_t)(32 * q) << 16) + buf * TILE_N + h * half_cols;
                 if (live && !DEQ) {
-                // R += s_c * acc, two columns per packed fused multiply-add: 32 columns of 16 rows (half hh of the warp's). Both halves are asked
+                // R += s_c * acc, two columns per packed fused multiply-add: 32 columns of 16 rows (half hh of the warp's; ROWS: 16 columns). Both halves are asked
                 // for at once and, with clustered weights, their coefficients before the wait for them: a wait in the middle has the next
                 // load's latency behind it (1024 x 4096 x 16384, 16 clusters: 125 -> 112 us).
                 auto accumulate = [&](const uint32_t (&v)[16], const float4 (&k)[4], int jc, int hh) {
@@ -1019,8 +1022,13 @@ cluster_gemm_kernel(const Params p)
                 for (int jc = 0; jc < 4; ++jc) {
                     uint32_t va[16], vb[16];
                     float4 k[4];
-                    tc_ld16xn(taddr + 32 * jc, va);
-                    tc_ld16xn(taddr + (16u << 16) + 32 * jc, vb);
+                    if constexpr (ROWS) {
+                        tc_ld16(taddr + 32 * jc, va);
+                        tc_ld16(taddr + 32 * jc + 16, vb);
+                    } else {
+                        tc_ld16xn(taddr + 32 * jc, va);
+                        tc_ld16xn(taddr + (16u << 16) + 32 * jc, vb);
+                    }
                     if constexpr (ASYM) {
 #pragma unroll
                         for (int j = 0; j < 4; ++j) k[j] = seg_tab[(jc * 4 + j) * 4];
@@ -1048,28 +1056,12 @@ cluster_gemm_kernel(const Params p)
                 }
             }
             mbar_wait(bar(B_TAB + (n_tile_done & 1)), (n_tile_done >> 1) & 1, s_abort);
-            // y = s_w * (R - corr) + bias, activation, store. Rows leave through a buffer of the warp, in pieces of 64 or 128 bytes a row: whole
-            // memory sectors, and few hand-overs between lanes (1999 x 2048 x 6144, 8 bits, fp32 out, with the LayerNorm: stores of a lane's
-            // own 16 bytes 70 us, pieces of 32 bytes 55, these 50.5)
+            // y = s_w * (R - corr) + bias, activation, store. Rows leave through a buffer of the warp, in pieces of 64 bytes a row: whole memory
+            // sectors, and few hand-overs between lanes (1999 x 2048 x 6144, 8 bits, fp32 out, with the LayerNorm: stores of a lane's own 16 bytes
+            // 70 us, pieces of 32 bytes 55; 50.5 with these and with sums that are not held by rows)
             if (live) {
                 const int mw = m0 + 32 * q, nb = n0 + h * half_cols;           // my warp's first row, my first column
-                const float2* t_corr = reinterpret_cast<const float2*>(tab + h * half_cols) + (lane & 3);
-                const float2* t_sw = t_corr + (TAB_ROWS - 2) * (TILE_N / 2);
-                const float2* t_bs = t_corr + (TAB_ROWS - 1) * (TILE_N / 2);
                 const bool relu = p.act == RPTQ_ACT_RELU;
-                // J times 8 columns at a time (DEQ: its sums are not in registers, of which it has few: a rolled loop, and with one block, whose output
-                // phase is short, half as many columns: 100 x 4096 x 12288, 3 and 4 bits, 41.5 and 42.5 us -> 40.4 and 41.4)
-                constexpr int J = DEQ && NCTA == 1 ? 2 : 4;
-                auto each_step = [&](auto body) {
-                    if constexpr (DEQ) {
-#pragma unroll 1
-                        for (int st = 0; 8 * J * st < half_cols; ++st) body(st);
-                    } else {
-                        body(std::integral_constant<int, 0>());
-                        if (half_cols > 32) body(std::integral_constant<int, 1>());
-                        if (half_cols > 64) { body(std::integral_constant<int, 2>()); body(std::integral_constant<int, 3>()); }
-                    }
-                };
                 // piece j (16 bytes) of row r lies at j ^ sw(r): neither what a warp puts nor what it reads in one instruction meets in a bank
                 constexpr int PIECES = OUT_ROW / 16, ROWS_I = 32 / PIECES;     // ROWS_I: rows that a warp-wide access covers
                 const uint32_t stage = smem_base + SL.off_stage + ew * 32 * OUT_ROW;
@@ -1092,141 +1084,242 @@ cluster_gemm_kernel(const Params p)
                     }
                     __syncwarp();
                 };
-                // DEQ: the finished fp32 sums are in tensor memory
-                const uint32_t t_acc = tmem_base + ((uint32_t)(32 * q) << 16) + (n_tile_done & 1u) * TILE_N + h * half_cols;
-                // my values of columns 8 (J st + j) + {0, 1}, rows lane / 4 + 8 k
-                auto finish = [&](int st, auto use) {
-                    float2 own[4 * J];
-                    if constexpr (DEQ) {
-                        uint32_t v[2][4 * J];
-                        tc_ld16xn(t_acc + 8 * J * st, v[0]);
-                        tc_ld16xn(t_acc + (16u << 16) + 8 * J * st, v[1]);
-                        tc_wait_ld();
+                // re-quantised outputs: column n is padded position n of the output layout (N is a multiple of 128)
+                const int n_units = min(half_cols, p.N - nb) >> 5;
+                uint8_t* const unit0 = static_cast<uint8_t*>(p.y) + (int64_t)mw * p.out_row_bytes + (nb >> 5) * 4 * p.out_bits;
+                if constexpr (ROWS) {
+                    const float4* t_row = reinterpret_cast<const float4*>(tab + h * half_cols);
+                    auto own = [&](int piece) { return stage + lane * OUT_ROW + ((piece ^ sw_f16(lane)) << 4); };
+                    auto finish = [&](int i, float2& lo, float2& hi) {         // columns 4 i .. 4 i + 3
+                        const float4 c = t_row[i], w = t_row[TILE_N / 4 + i], b = t_row[TILE_N / 2 + i];
+                        lo = fma2(make_float2(w.x, w.y), add2(R[2 * i], make_float2(-c.x, -c.y)), make_float2(b.x, b.y));
+                        hi = fma2(make_float2(w.z, w.w), add2(R[2 * i + 1], make_float2(-c.z, -c.w)), make_float2(b.z, b.w));
+                        if (relu) { lo.x = fmaxf(lo.x, 0.f); lo.y = fmaxf(lo.y, 0.f); hi.x = fmaxf(hi.x, 0.f); hi.y = fmaxf(hi.y, 0.f); }
+                    };
+                    auto h2 = [](float2 v) { const __half2 x = __floats2half2_rn(v.x, v.y); return *reinterpret_cast<const uint32_t*>(&x); };
+                    if (p.y_dtype == RPTQ_OUT_F16) {
+                        uint8_t* dst = static_cast<uint8_t*>(p.y) + ((int64_t)mw * p.ldy + nb) * 2;
+                        const int n_bytes = 2 * min(p.N - nb, half_cols);
 #pragma unroll
-                        for (int i = 0; i < 4 * J; ++i) own[i] = make_float2(__uint_as_float(v[i / (2 * J)][2 * (i % (2 * J))]), __uint_as_float(v[i / (2 * J)][2 * (i % (2 * J)) + 1]));
-                    }
+                        for (int u = 0; u < 4; ++u) {                          // 32 columns
+                            if (32 * u >= half_cols) break;
 #pragma unroll
-                    for (int j = 0; j < J; ++j) {
-                        const int at = (J * st + j) * 4;
-                        float2 c, w;
-                        if constexpr (!DEQ) c = t_corr[at];
-                        if constexpr (!ASYM) w = t_sw[at];
-                        const float2 b = t_bs[at];
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            float2 v;
-                            if constexpr (DEQ) v = own[(k >> 1) * 2 * J + 2 * j + (k & 1)]; else v = add2(R[(st * 2 + (k >> 1)) * 8 + 2 * j + (k & 1)], make_float2(-c.x, -c.y));
-                            if constexpr (ASYM) v = add2(v, b); else v = fma2(w, v, b);
-                            if (relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); }
-                            use(j, k, v);
-                        }
-                    }
-                };
-                if (p.y_dtype == RPTQ_OUT_F16) {
-                    uint8_t* dst = static_cast<uint8_t*>(p.y) + ((int64_t)mw * p.ldy + nb) * 2;
-                    const int n_bytes = 2 * min(p.N - nb, half_cols);
-                    // (my lane names row 8 k + lane % 8, piece lane / 8 of the step's columns, to stmatrix)
-                    each_step([&](auto at_st) {
-                        const int st = at_st, j0 = J * st % 4;
-                        uint32_t f[4][J];                                      // [k][j]
-                        finish(st, [&](int j, int k, float2 v) { const __half2 x = __floats2half2_rn(v.x, v.y); f[k][j] = *reinterpret_cast<const uint32_t*>(&x); });
-#pragma unroll
-                        for (int k = 0; k < 4; ++k) {
-                            const int r = 8 * k + (lane & 7);
-                            stmatrixn(stage + r * OUT_ROW + (((j0 + (lane >> 3) % J) ^ sw_f16(r)) << 4), f[k]);
-                        }
-                        const int from = 16 * (J * st - j0);
-                        if (j0 + J == 4) store(sw_f16, dst + from, p.ldy * 2, n_bytes - from);
-                    });
-                } else if (p.y_dtype == RPTQ_OUT_F32) {
-                    uint8_t* dst = static_cast<uint8_t*>(p.y) + ((int64_t)mw * p.ldy + nb) * 4;
-                    const int n_bytes = 4 * min(p.N - nb, half_cols);
-                    const uint32_t put = stage + (lane >> 2) * OUT_ROW + 8 * (lane & 1);
-                    const int piece = (lane & 3) >> 1;
-                    each_step([&](auto at_st) {
-                        const int st = at_st;
-                        finish(st, [&](int j, int k, float2 v) {
-                            sts64(put + 8 * k * OUT_ROW + (((2 * (j & 1) + piece) ^ sw_f32(lane >> 2)) << 4), v);      // (8 k changes no swizzle)
-                            if (k == 3 && (j & 1)) {
-                                const int from = 32 * (J * st + j - 1);
-                                store(sw_f32, dst + from, p.ldy * 4, n_bytes - from);
+                            for (int j = 0; j < 4; ++j) {
+                                float2 v[4];
+                                finish(8 * u + 2 * j, v[0], v[1]);
+                                finish(8 * u + 2 * j + 1, v[2], v[3]);
+                                sts128(own(j), h2(v[0]), h2(v[1]), h2(v[2]), h2(v[3]));
                             }
-                        });
-                    });
-                } else if constexpr (MODE != MODE_DEQ) {
-                    // Re-quantise for the next site: column n is padded position n of the output layout. A word of eight nibbles is eight columns of
-                    // a row, which four lanes hold, two codes each. Codes of at most four bits: a byte for each of a unit's four words goes through the
-                    // warp's buffer as the fragment of a 16-bit matrix, which gives every lane the 16 bytes of its own row.
-                    const int n_units = min(half_cols, p.N - nb) >> 5;         // (N is a multiple of 128)
-                    const int l = lane & 3;
-#pragma unroll
-                    for (int jc = 0; jc < 4; ++jc) {
-                        if (jc >= n_units) break;
-                        const int unit = (nb >> 5) + jc;
-                        const float inv_s = __uint_as_float(__shfl_sync(0xffffffffu, unit4.x, jc));
-                        const int zc = (int)__shfl_sync(0xffffffffu, unit4.y, jc), nvalid = (int)__shfl_sync(0xffffffffu, unit4.w, jc);
-                        const float2 s2 = make_float2(inv_s, inv_s), c2 = make_float2(12582912.0f, 12582912.0f);
-                        int qv[4][4][2];                                       // [row k][word j]: not yet clamped, the pack saturates
-                        finish(jc, [&](int j, int k, float2 v) {
-                            v = fma2(v, s2, c2);
-                            qv[k][j][0] = quant_int(v.x, zc); qv[k][j][1] = quant_int(v.y, zc);
-                        });
-                        if (nvalid < 32) {
-#pragma unroll
-                            for (int j = 0; j < 4; ++j)
-#pragma unroll
-                                for (int e = 0; e < 2; ++e)
-#pragma unroll
-                                    for (int k = 0; k < 4; ++k) qv[k][j][e] = 8 * j + 2 * l + e < nvalid ? qv[k][j][e] : 0;
+                            store(sw_f16, dst + 64 * u, p.ldy * 2, n_bytes - 64 * u);
                         }
-                        if (p.out_bits == 8) {
-                            uint8_t* row = static_cast<uint8_t*>(p.y) + (int64_t)(mw + (lane >> 2)) * p.out_row_bytes;
+                    } else if (p.y_dtype == RPTQ_OUT_F32) {
+                        uint8_t* dst = static_cast<uint8_t*>(p.y) + ((int64_t)mw * p.ldy + nb) * 4;
+                        const int n_bytes = 4 * min(p.N - nb, half_cols);
 #pragma unroll
-                            for (int k = 0; k < 4; ++k, row += 8 * p.out_row_bytes) {
-                                // two codes of each of the unit's four pairs of words: lane l ends with pair l. With lane ^ 2 pairs 0, 1 (of lanes 0, 1) for 2, 3
-                                // (of lanes 2, 3), then with lane ^ 1 the even pair for the odd one
-                                auto two = [&](int j) { return sat_pack_u8(qv[k][j][1], qv[k][j][0], 0u); };
-                                const uint32_t lo = two(0) | (two(1) << 16), hi = two(2) | (two(3) << 16);
-                                const uint32_t own = l & 2 ? hi : lo, o2 = __shfl_xor_sync(0xffffffffu, l & 2 ? lo : hi, 2);
-                                const uint32_t x = l & 2 ? o2 : own, y = l & 2 ? own : o2;           // of lanes l & 1 and (l & 1) + 2
-                                const uint32_t even = __byte_perm(x, y, 0x5410), odd = __byte_perm(x, y, 0x7632);
-                                const uint32_t o1 = __shfl_xor_sync(0xffffffffu, l & 1 ? even : odd, 1);
-                                const uint32_t a = l & 1 ? o1 : even, c = l & 1 ? odd : o1;          // of the lower, the higher lane
-                                if (mw + (lane >> 2) + 8 * k < p.M)
-                                    *reinterpret_cast<uint2*>(row + unit * 32 + 8 * l) = make_uint2(__byte_perm(a, c, 0x5410), __byte_perm(a, c, 0x7632));
+                        for (int c = 0; c < 8; ++c) {                          // 16 columns
+                            if (16 * c >= half_cols) break;
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                float2 lo, hi;
+                                finish(4 * c + j, lo, hi);
+                                sts128(own(j), __float_as_uint(lo.x), __float_as_uint(lo.y), __float_as_uint(hi.x), __float_as_uint(hi.y));
                             }
-                            continue;
+                            store(sw_f16, dst + 64 * c, p.ldy * 4, n_bytes - 64 * c);
                         }
-                        uint32_t x[4] = {0u, 0u, 0u, 0u};                      // byte j: codes 2 l (low nibble) and 2 l + 1 of word j
+                    } else {
 #pragma unroll
-                        for (int k = 0; k < 4; ++k)
+                        for (int u = 0; u < 4; ++u) {
+                            if (u >= n_units) break;
+                            const float inv_s = __uint_as_float(__shfl_sync(0xffffffffu, unit4.x, u));
+                            const int zc = (int)__shfl_sync(0xffffffffu, unit4.y, u), nvalid = (int)__shfl_sync(0xffffffffu, unit4.w, u);
+                            const float2 s2 = make_float2(inv_s, inv_s), c2 = make_float2(12582912.0f, 12582912.0f);
+                            int qv[32];                                        // not yet clamped, the pack saturates
 #pragma unroll
-                            for (int j = 3; j >= 0; --j) x[k] = sat_pack_u4(qv[k][j][1], qv[k][j][0], x[k]);
-                        const uint32_t own_row = stage + lane * OUT_ROW + ((jc ^ sw_f16(lane)) << 4);
-                        stmatrixn(own_row, x);
-                        __syncwarp();
-                        const uint4 t = lds128(own_row);                       // word l: byte j is codes 2 l, 2 l + 1 of word j
-                        const uint32_t a01 = __byte_perm(t.x, t.y, 0x5140), a23 = __byte_perm(t.x, t.y, 0x7362);
-                        const uint32_t b01 = __byte_perm(t.z, t.w, 0x5140), b23 = __byte_perm(t.z, t.w, 0x7362);
-                        uint32_t w[4];
+                            for (int i = 0; i < 8; ++i) {
+                                float2 lo, hi;
+                                finish(8 * u + i, lo, hi);
+                                lo = fma2(lo, s2, c2); hi = fma2(hi, s2, c2);
+                                qv[4 * i] = quant_int(lo.x, zc); qv[4 * i + 1] = quant_int(lo.y, zc);
+                                qv[4 * i + 2] = quant_int(hi.x, zc); qv[4 * i + 3] = quant_int(hi.y, zc);
+                            }
+                            if (nvalid < 32) {
 #pragma unroll
-                        for (int j = 0; j < 4; ++j) {
-                            // codes 0, 1, 2, 3 of word j (bytes 0, 0, 1, 1 of its two) and 4, 5, 6, 7: low nibbles, high nibbles
-                            const uint32_t lo = __byte_perm(j < 2 ? a01 : a23, 0u, j & 1 ? 0x3322 : 0x1100), hi = __byte_perm(j < 2 ? b01 : b23, 0u, j & 1 ? 0x3322 : 0x1100);
-                            w[j] = (lo & 0x000F000Fu) | ((lo >> 4) & 0x0F000F00u) | ((hi << 4) & 0x00F000F0u) | (hi & 0xF000F000u);
+                                for (int e = 0; e < 32; ++e) qv[e] = e < nvalid ? qv[e] : 0;
+                            }
+                            // rows leave in pieces of up to 64 bytes, 3 bits: 48, those of a strip (which may begin between 16-byte boundaries) unit by unit
+                            if (p.out_bits == 4) {
+                                uint32_t w[4]; pack32_sat<4>(qv, w);
+                                sts128(own(u), w[0], w[1], w[2], w[3]);
+                                if (u + 1 == n_units) store(sw_f16, unit0, p.out_row_bytes, 16 * n_units);
+                            } else if (p.out_bits == 8) {
+                                uint32_t w[8]; pack32_sat<8>(qv, w);
+                                sts128(own(2 * (u & 1)), w[0], w[1], w[2], w[3]);
+                                sts128(own(2 * (u & 1) + 1), w[4], w[5], w[6], w[7]);
+                                if ((u & 1) || u + 1 == n_units) store(sw_f16, unit0 + 32 * (u & 2), p.out_row_bytes, 32 * ((u & 1) + 1));
+                            } else {
+                                uint32_t w[3]; pack32_sat<3>(qv, w);
+                                if (half_cols == 128) {
+#pragma unroll
+                                    for (int j = 0; j < 3; ++j) sts32(own((3 * u + j) >> 2) + 4 * ((3 * u + j) & 3), w[j]);
+                                    if (u == 3) store(sw_f16, unit0, p.out_row_bytes, 48);
+                                } else if (mw + lane < p.M) {
+#pragma unroll
+                                    for (int j = 0; j < 3; ++j) reinterpret_cast<uint32_t*>(unit0 + lane * p.out_row_bytes + 12 * u)[j] = w[j];
+                                }
+                            }
                         }
-                        uint8_t* row = static_cast<uint8_t*>(p.y) + (int64_t)(mw + lane) * p.out_row_bytes + unit * 4 * p.out_bits;
-                        if (p.out_bits == 4) {
-                            // back to the same place, and out in pieces of up to 64 bytes a row
-                            sts128(own_row, w[0], w[1], w[2], w[3]);
-                            if (jc + 1 == n_units)
-                                store(sw_f16, static_cast<uint8_t*>(p.y) + (int64_t)mw * p.out_row_bytes + (nb >> 5) * 16, p.out_row_bytes, 16 * n_units);
+                    }
+                } else {
+                    const float2* t_corr = reinterpret_cast<const float2*>(tab + h * half_cols) + (lane & 3);
+                    const float2* t_sw = t_corr + (TAB_ROWS - 2) * (TILE_N / 2);
+                    const float2* t_bs = t_corr + (TAB_ROWS - 1) * (TILE_N / 2);
+                    // J times 8 columns at a time (DEQ: its sums are not in registers, of which it has few: a rolled loop, and with one block, whose output
+                    // phase is short, half as many columns: 100 x 4096 x 12288, 3 and 4 bits, 41.5 and 42.5 us -> 40.4 and 41.4)
+                    constexpr int J = DEQ && NCTA == 1 ? 2 : 4;
+                    auto each_step = [&](auto body) {
+                        if constexpr (DEQ) {
+#pragma unroll 1
+                            for (int st = 0; 8 * J * st < half_cols; ++st) body(st);
                         } else {
-                            auto clamp7 = [](uint32_t v) { return (v | (((v >> 3) & 0x11111111u) * 7u)) & 0x77777777u; };        // nibbles above 7 become 7
-                            const uint32_t tail = clamp7(w[3]);
-                            if (mw + lane < p.M) {
+                            body(std::integral_constant<int, 0>());
+                            if (half_cols > 32) body(std::integral_constant<int, 1>());
+                            if (half_cols > 64) { body(std::integral_constant<int, 2>()); body(std::integral_constant<int, 3>()); }
+                        }
+                    };
+                    // DEQ: the finished fp32 sums are in tensor memory
+                    const uint32_t t_acc = tmem_base + ((uint32_t)(32 * q) << 16) + (n_tile_done & 1u) * TILE_N + h * half_cols;
+                    // my values of columns 8 (J st + j) + {0, 1}, rows lane / 4 + 8 k
+                    auto finish = [&](int st, auto use) {
+                        float2 own[4 * J];
+                        if constexpr (DEQ) {
+                            uint32_t v[2][4 * J];
+                            tc_ld16xn(t_acc + 8 * J * st, v[0]);
+                            tc_ld16xn(t_acc + (16u << 16) + 8 * J * st, v[1]);
+                            tc_wait_ld();
 #pragma unroll
-                                for (int j = 0; j < 3; ++j) reinterpret_cast<uint32_t*>(row)[j] = clamp7(w[j]) | (((tail >> j) & 0x11111111u) << 3);
+                            for (int i = 0; i < 4 * J; ++i) own[i] = make_float2(__uint_as_float(v[i / (2 * J)][2 * (i % (2 * J))]), __uint_as_float(v[i / (2 * J)][2 * (i % (2 * J)) + 1]));
+                        }
+#pragma unroll
+                        for (int j = 0; j < J; ++j) {
+                            const int at = (J * st + j) * 4;
+                            float2 c, w;
+                            if constexpr (!DEQ) c = t_corr[at];
+                            if constexpr (!ASYM) w = t_sw[at];
+                            const float2 b = t_bs[at];
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                float2 v;
+                                if constexpr (DEQ) v = own[(k >> 1) * 2 * J + 2 * j + (k & 1)]; else v = add2(R[(st * 2 + (k >> 1)) * 8 + 2 * j + (k & 1)], make_float2(-c.x, -c.y));
+                                if constexpr (ASYM) v = add2(v, b); else v = fma2(w, v, b);
+                                if (relu) { v.x = fmaxf(v.x, 0.f); v.y = fmaxf(v.y, 0.f); }
+                                use(j, k, v);
+                            }
+                        }
+                    };
+                    if (p.y_dtype == RPTQ_OUT_F16) {
+                        uint8_t* dst = static_cast<uint8_t*>(p.y) + ((int64_t)mw * p.ldy + nb) * 2;
+                        const int n_bytes = 2 * min(p.N - nb, half_cols);
+                        // (my lane names row 8 k + lane % 8, piece lane / 8 of the step's columns, to stmatrix)
+                        each_step([&](auto at_st) {
+                            const int st = at_st, j0 = J * st % 4;
+                            uint32_t f[4][J];                                      // [k][j]
+                            finish(st, [&](int j, int k, float2 v) { const __half2 x = __floats2half2_rn(v.x, v.y); f[k][j] = *reinterpret_cast<const uint32_t*>(&x); });
+#pragma unroll
+                            for (int k = 0; k < 4; ++k) {
+                                const int r = 8 * k + (lane & 7);
+                                stmatrixn(stage + r * OUT_ROW + (((j0 + (lane >> 3) % J) ^ sw_f16(r)) << 4), f[k]);
+                            }
+                            const int from = 16 * (J * st - j0);
+                            if (j0 + J == 4) store(sw_f16, dst + from, p.ldy * 2, n_bytes - from);
+                        });
+                    } else if (p.y_dtype == RPTQ_OUT_F32) {
+                        uint8_t* dst = static_cast<uint8_t*>(p.y) + ((int64_t)mw * p.ldy + nb) * 4;
+                        const int n_bytes = 4 * min(p.N - nb, half_cols);
+                        const uint32_t put = stage + (lane >> 2) * OUT_ROW + 8 * (lane & 1);
+                        const int piece = (lane & 3) >> 1;
+                        each_step([&](auto at_st) {
+                            const int st = at_st;
+                            finish(st, [&](int j, int k, float2 v) {
+                                sts64(put + 8 * k * OUT_ROW + (((2 * (j & 1) + piece) ^ sw_f32(lane >> 2)) << 4), v);      // (8 k changes no swizzle)
+                                if (k == 3 && (j & 1)) {
+                                    const int from = 32 * (J * st + j - 1);
+                                    store(sw_f32, dst + from, p.ldy * 4, n_bytes - from);
+                                }
+                            });
+                        });
+                    } else if constexpr (!DEQ) {
+                        // A word of eight nibbles is eight columns of a row, which four lanes hold, two codes each. Codes of at most four bits: a byte for
+                        // each of a unit's four words goes through the warp's buffer as the fragment of a 16-bit matrix, which gives every lane the
+                        // 16 bytes of its own row.
+                        const int l = lane & 3;
+#pragma unroll
+                        for (int jc = 0; jc < 4; ++jc) {
+                            if (jc >= n_units) break;
+                            const float inv_s = __uint_as_float(__shfl_sync(0xffffffffu, unit4.x, jc));
+                            const int zc = (int)__shfl_sync(0xffffffffu, unit4.y, jc), nvalid = (int)__shfl_sync(0xffffffffu, unit4.w, jc);
+                            const float2 s2 = make_float2(inv_s, inv_s), c2 = make_float2(12582912.0f, 12582912.0f);
+                            int qv[4][4][2];                                       // [row k][word j]: not yet clamped, the pack saturates
+                            finish(jc, [&](int j, int k, float2 v) {
+                                v = fma2(v, s2, c2);
+                                qv[k][j][0] = quant_int(v.x, zc); qv[k][j][1] = quant_int(v.y, zc);
+                            });
+                            if (nvalid < 32) {
+#pragma unroll
+                                for (int j = 0; j < 4; ++j)
+#pragma unroll
+                                    for (int e = 0; e < 2; ++e)
+#pragma unroll
+                                        for (int k = 0; k < 4; ++k) qv[k][j][e] = 8 * j + 2 * l + e < nvalid ? qv[k][j][e] : 0;
+                            }
+                            if (p.out_bits == 8) {
+                                uint8_t* row = unit0 + (lane >> 2) * p.out_row_bytes + jc * 32 + 8 * l;
+#pragma unroll
+                                for (int k = 0; k < 4; ++k, row += 8 * p.out_row_bytes) {
+                                    // two codes of each of the unit's four pairs of words: lane l ends with pair l. With lane ^ 2 pairs 0, 1 (of lanes 0, 1) for 2, 3
+                                    // (of lanes 2, 3), then with lane ^ 1 the even pair for the odd one
+                                    auto two = [&](int j) { return sat_pack_u8(qv[k][j][1], qv[k][j][0], 0u); };
+                                    const uint32_t lo = two(0) | (two(1) << 16), hi = two(2) | (two(3) << 16);
+                                    const uint32_t own = l & 2 ? hi : lo, o2 = __shfl_xor_sync(0xffffffffu, l & 2 ? lo : hi, 2);
+                                    const uint32_t x = l & 2 ? o2 : own, y = l & 2 ? own : o2;           // of lanes l & 1 and (l & 1) + 2
+                                    const uint32_t even = __byte_perm(x, y, 0x5410), odd = __byte_perm(x, y, 0x7632);
+                                    const uint32_t o1 = __shfl_xor_sync(0xffffffffu, l & 1 ? even : odd, 1);
+                                    const uint32_t a = l & 1 ? o1 : even, c = l & 1 ? odd : o1;          // of the lower, the higher lane
+                                    if (mw + (lane >> 2) + 8 * k < p.M)
+                                        *reinterpret_cast<uint2*>(row) = make_uint2(__byte_perm(a, c, 0x5410), __byte_perm(a, c, 0x7632));
+                                }
+                                continue;
+                            }
+                            uint32_t x[4] = {0u, 0u, 0u, 0u};                      // byte j: codes 2 l (low nibble) and 2 l + 1 of word j
+#pragma unroll
+                            for (int k = 0; k < 4; ++k)
+#pragma unroll
+                                for (int j = 3; j >= 0; --j) x[k] = sat_pack_u4(qv[k][j][1], qv[k][j][0], x[k]);
+                            const uint32_t own_row = stage + lane * OUT_ROW + ((jc ^ sw_f16(lane)) << 4);
+                            stmatrixn(own_row, x);
+                            __syncwarp();
+                            const uint4 t = lds128(own_row);                       // word l: byte j is codes 2 l, 2 l + 1 of word j
+                            const uint32_t a01 = __byte_perm(t.x, t.y, 0x5140), a23 = __byte_perm(t.x, t.y, 0x7362);
+                            const uint32_t b01 = __byte_perm(t.z, t.w, 0x5140), b23 = __byte_perm(t.z, t.w, 0x7362);
+                            uint32_t w[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                // codes 0, 1, 2, 3 of word j (bytes 0, 0, 1, 1 of its two) and 4, 5, 6, 7: low nibbles, high nibbles
+                                const uint32_t lo = __byte_perm(j < 2 ? a01 : a23, 0u, j & 1 ? 0x3322 : 0x1100), hi = __byte_perm(j < 2 ? b01 : b23, 0u, j & 1 ? 0x3322 : 0x1100);
+                                w[j] = (lo & 0x000F000Fu) | ((lo >> 4) & 0x0F000F00u) | ((hi << 4) & 0x00F000F0u) | (hi & 0xF000F000u);
+                            }
+                            uint8_t* row = unit0 + lane * p.out_row_bytes + jc * 4 * p.out_bits;
+                            if (p.out_bits == 4) {
+                                // back to the same place, and out in pieces of up to 64 bytes a row
+                                sts128(own_row, w[0], w[1], w[2], w[3]);
+                                if (jc + 1 == n_units)
+                                    store(sw_f16, unit0, p.out_row_bytes, 16 * n_units);
+                            } else {
+                                auto clamp7 = [](uint32_t v) { return (v | (((v >> 3) & 0x11111111u) * 7u)) & 0x77777777u; };        // nibbles above 7 become 7
+                                const uint32_t tail = clamp7(w[3]);
+                                if (mw + lane < p.M) {
+#pragma unroll
+                                    for (int j = 0; j < 3; ++j) reinterpret_cast<uint32_t*>(row)[j] = clamp7(w[j]) | (((tail >> j) & 0x11111111u) << 3);
+                                }
                             }
                         }
                     }
@@ -1254,13 +1347,13 @@ cluster_gemm_kernel(const Params p)
 }
 
 // ---------------------------------------------------------------- host side
-template <int BITS, int NCTA, bool A8, int MODE>
+template <int BITS, int NCTA, bool A8, int MODE, bool ROWS = false>
 static int launch(const Params& p, int dev, int n_sm, cudaStream_t st)
 {
     constexpr SmemLayout SL = smem_layout(NCTA, BITS, A8, MODE);
     constexpr int THREADS = threads_of(MODE);
     const int smem = SL.total + 1024;     // slack for the in-kernel 1024-byte alignment
-    const void* fn = reinterpret_cast<const void*>(cluster_gemm_kernel<BITS, NCTA, A8, MODE>);
+    const void* fn = reinterpret_cast<const void*>(cluster_gemm_kernel<BITS, NCTA, A8, MODE, ROWS>);
     static_assert(SL.total + 1024 <= 227 * 1024, "shared memory");
     static SmemAllowed done;
     static std::atomic<uint64_t> pool_ok{0};
@@ -1274,7 +1367,7 @@ static int launch(const Params& p, int dev, int n_sm, cudaStream_t st)
     if (allow_smem(fn, dev, smem, done) != RPTQ_OK) return RPTQ_ERR_CUDA;
     const int slots = n_sm / NCTA;
     const int groups = p.n_items < slots ? p.n_items : slots;
-    return launch_kernel(cluster_gemm_kernel<BITS, NCTA, A8, MODE>, dim3((unsigned)(groups * NCTA)), THREADS, (size_t)smem, NCTA, st, p);
+    return launch_kernel(cluster_gemm_kernel<BITS, NCTA, A8, MODE, ROWS>, dim3((unsigned)(groups * NCTA)), THREADS, (size_t)smem, NCTA, st, p);
 }
 
 }  // namespace gemm
@@ -1377,10 +1470,20 @@ static int launch_gemm(const rptq_layout_t* Lin, const void* a_codes, int M, con
         if (Lin->bits == 4) return gemm::launch<4, 1, false, gemm::MODE_ASYM>(p, dev, n_sm, st);
         return gemm::launch<8, 1, false, gemm::MODE_ASYM>(p, dev, n_sm, st);
     }
+    // Sums by rows (see the epilogue) for CTA pairs. Re-quantised outputs: yes (4096 x 2048 x 8192, 3, 4 and 8 bits, 32 clusters 199, 190, 198 -> 182,
+    // 179, 183 us; 4 clusters 84.4, 76.0, 83.4 -> 79.0, 75.5, 82.5; 2048 x 12288 x 12288, 64 clusters, 8 bits 352 -> 343), except for 4 bits after a
+    // long contraction of long clusters, where the tables' loads are in the unpack warps' way (2048 x 8192 x 8192, 32: 142.5 and 144.2; 2048 x
+    // 12288 x 49152, 64: 1169 and 1190). Others: many short clusters over more than one round of tiles, whose drains set the pace (2000 x
+    // 1024 x 4096 to fp16, 4 bits: 64 clusters 87.4 -> 81.5, 32 50.5 -> 47.9; 2048 x 4096 x 16384, 32: 188 -> 184). Not fewer clusters (2000 x
+    // 1024 x 4096 to fp32, 8: 25.5 and 26.0), longer ones, which a drain passes under (1024 x 9216 x 9216, 32: 79.8 and 81.3), a single round, which
+    // ends in the outputs (700 x 768 x 3072, 32: 19.5 and 20.1), or blocks on their own (128 x 2048 x 8192, 64: 26.1 and 26.5; codes the same).
+    const bool short_clusters = Lin->K_pad < 192 * Lin->n_seg;
+    const bool by_rows = Lout ? Lout->bits != 4 || Lin->K_pad <= 8192 || short_clusters : Lin->n_seg >= 20 && short_clusters && n_tiles > slots;
     if (ncta == 2) {
-        if (Lin->bits == 3) return gemm::launch<3, 2, false, gemm::MODE_INT>(p, dev, n_sm, st);
-        if (Lin->bits == 4) return gemm::launch<4, 2, false, gemm::MODE_INT>(p, dev, n_sm, st);
-        return gemm::launch<8, 2, true, gemm::MODE_INT>(p, dev, n_sm, st);      // 8-bit codes need no unpacking
+        if (Lin->bits == 3) return by_rows ? gemm::launch<3, 2, false, gemm::MODE_INT, true>(p, dev, n_sm, st) : gemm::launch<3, 2, false, gemm::MODE_INT>(p, dev, n_sm, st);
+        if (Lin->bits == 4) return by_rows ? gemm::launch<4, 2, false, gemm::MODE_INT, true>(p, dev, n_sm, st) : gemm::launch<4, 2, false, gemm::MODE_INT>(p, dev, n_sm, st);
+        // 8-bit codes need no unpacking
+        return by_rows ? gemm::launch<8, 2, true, gemm::MODE_INT, true>(p, dev, n_sm, st) : gemm::launch<8, 2, true, gemm::MODE_INT>(p, dev, n_sm, st);
     }
     if (Lin->bits == 3) return gemm::launch<3, 1, false, gemm::MODE_INT>(p, dev, n_sm, st);
     if (Lin->bits == 4) return gemm::launch<4, 1, false, gemm::MODE_INT>(p, dev, n_sm, st);

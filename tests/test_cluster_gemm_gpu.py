@@ -418,3 +418,28 @@ def test_whole_tiles_and_strips_give_the_bits_of_small_calls(out):
         n = min(128, M - lo)
         part = _gemm(dict(case, M=n), dict(d, a=d["a"][lo:lo + n].contiguous()), **kw)
         np.testing.assert_array_equal(whole[lo:lo + n].view(np.uint8), part.view(np.uint8))
+
+
+# The epilogue that holds a token row per thread: re-quantised outputs of CTA pairs (above), and many short clusters over more than one round.
+@pytest.mark.parametrize("bits", [4, 3, 8])
+@pytest.mark.parametrize("out", ["f32", "f16"])
+def test_many_short_clusters_give_the_bits_of_small_calls(out, bits):
+    """80 tiles on 74 pairs of blocks, 24 clusters of one or two steps: whole tiles and strips with ragged rows and columns, against calls of at most
+    128 tokens (whose blocks hold their sums in the other layout) and, on some rows, the oracle."""
+    from paper_2304_01089_b200 import binding
+    M, N = 2401, 2045
+    rng = np.random.default_rng(78 + bits)
+    case = _case(rng, M, N, 904, 24, bits, n_pad=2048, allow_empty=False)
+    assert case["k_pad"] < 192 * 24
+    d = _dev(case)
+    bias = (rng.normal(size=N) * 0.05).astype(np.float32)
+    kw = dict(y_dtype=binding.OUT_F32 if out == "f32" else binding.OUT_F16, ldy=2048, bias=bias, act=binding.ACT_RELU)
+    whole = _gemm(case, d, **kw)
+    for lo in range(0, M, 128):
+        n = min(128, M - lo)
+        part = _gemm(dict(case, M=n), dict(d, a=d["a"][lo:lo + n].contiguous()), **kw)
+        np.testing.assert_array_equal(whole[lo:lo + n].view(np.uint8), part.view(np.uint8))
+    if out == "f32":
+        rows = np.r_[0:3, 1200:1203, M - 3:M]
+        want = _oracle_y(dict(case, a=case["a"][rows], M=len(rows)), bias=bias, relu=True)
+        assert np.max(np.abs(whole[rows][:, :N] - want)) <= TOL * np.abs(want).max()
