@@ -443,3 +443,28 @@ def test_many_short_clusters_give_the_bits_of_small_calls(out, bits):
         rows = np.r_[0:3, 1200:1203, M - 3:M]
         want = _oracle_y(dict(case, a=case["a"][rows], M=len(rows)), bias=bias, relu=True)
         assert np.max(np.abs(whole[rows][:, :N] - want)) <= TOL * np.abs(want).max()
+
+
+@pytest.mark.parametrize("out_bits", [3, 4, 8])
+@pytest.mark.parametrize("M,rest", [(100, 2), (100, 70), (200, 1), (200, 30)])
+def test_codes_of_strips_are_those_of_whole_tiles(M, rest, out_bits):
+    """One whole round of tiles and `rest` more, cut into quarters or halves, whose weight rows and output units repeat those of the first ones."""
+    import torch
+    from paper_2304_01089_b200 import binding
+    slots = torch.cuda.get_device_properties(0).multi_processor_count // (2 if M > 128 else 1)
+    rng = np.random.default_rng(79 + rest)
+    case = _case(rng, M, 512, 256, 3, 4)
+    reps = -(-(slots + rest) // 2)
+    N = 512 * reps
+    big = dict(case, N=N, n_pad=N, w_codes=np.tile(case["w_codes"][:512], (reps, 1)), s_w=np.tile(case["s_w"][:512], reps),
+               wsum=np.tile(case["wsum"][:, :512], (1, reps)))
+    y = _gemm(case, _dev(case))
+    size = np.tile([1, 31, 32, 33, 64, 287], reps)                       # 512 padded positions a repetition, pads among them
+    g = len(size)
+    L2 = binding.Layout(np.arange(size.sum(), dtype=np.int32), size, np.full(g, np.abs(y).max() / (1 << out_bits), np.float32),
+                        np.full(g, 1 << (out_bits - 1), np.int32), out_bits)
+    assert L2.K_pad == N
+    codes = _gemm(big, _dev(big), y_dtype=binding.OUT_CODES, layout_out=L2)
+    got = oracle.unpack(codes, N, out_bits).reshape(M, reps, 512)
+    assert len(np.unique(got)) > (1 << out_bits) // 2
+    np.testing.assert_array_equal(got, np.repeat(got[:, :1], reps, axis=1))
