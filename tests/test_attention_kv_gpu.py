@@ -325,3 +325,25 @@ def test_a_row_depends_on_nothing_but_itself_and_its_keys(hd, bits):
     for lo, hi in zip(cuts, cuts[1:]):
         part = _outputs(c, q[lo:hi], True, Tk=Tk - Tq + hi)
         np.testing.assert_array_equal(part.view(np.uint16), whole[lo:hi].view(np.uint16))
+
+
+@pytest.mark.parametrize("H,hd,bits,Tq,Tk,n_seq", [(12, 16, (4, 4, 4), 300, 330, 14), (12, 16, (4, 4, 4), 250, 390, 20), (4, 256, (4, 8, 8), 300, 330, 40),
+                                                   (24, 16, (4, 4, 4), 50, 60, 24)])
+def test_blocks_with_several_items_of_rising_scores(H, hd, bits, Tq, Tk, n_seq):
+    """Three items and more to every block, of which one prompt's have odd and even numbers of key tiles (or one tile each): the state that a block
+    carries from item to item (barrier phases, two sets of references) against calls of one prompt, whose blocks have one item.
+    Heads of 256 channels leave room for one tile of probabilities only."""
+    import torch
+    per_prompt = H * ((Tq + 127) // 128)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    assert per_prompt <= sms and per_prompt * n_seq >= 3 * sms
+    c, q = _rising(1200 + hd + Tk, H, hd, Tq, Tk, n_seq, bits)
+    whole = _outputs(c, q, True, n_seq=n_seq)
+    k, v = c.dk, c.dv
+    for s in range(n_seq):
+        c.dk, c.dv = k[s * Tk:(s + 1) * Tk], v[s * Tk:(s + 1) * Tk]
+        alone = _outputs(c, q[s * Tq:(s + 1) * Tq], True, Tk=Tk)
+        np.testing.assert_array_equal(whole[s * Tq:(s + 1) * Tq].view(np.uint16), alone.view(np.uint16))
+    c.dk, c.dv = k, v
+    if hd == 16:
+        _check(c, q, True, n_seq=n_seq)
