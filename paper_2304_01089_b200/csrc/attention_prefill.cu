@@ -4,7 +4,8 @@
 // row's final maximum and sum, so integer calls walk the keys twice: pass 1 finds the row maxima and sums, pass 2 forms the
 // probabilities and multiplies them with V. Nothing is rescaled on the way. Scores are computed in both passes; the tensor cores
 // have room for that. KV calls walk the keys once: probabilities are relative to a reference that follows the row's maximum, and
-// the output accumulator is brought to a new reference where it moves (two walks: 346 us, one: 316; 3 x 1100 queries on 1337 keys).
+// the output accumulator is brought to a new reference where it moves (3 x 1100 queries on 1337 keys, 32 heads of 128 channels: two walks
+// 347 us, one 314).
 //
 // What bounds it: one exponential per score and pass (the special-function unit gives 16 per clock and SM), then the
 // issue slots of the softmax warps: a score costs one multiply-add per cluster of the head, and five or six
@@ -34,9 +35,9 @@
 //
 // Measured, us, against a mma.sync kernel with 64 (KV: 128) queries per block (72 heads of 128 channels, four clusters each,
 // causal, two sequences of 2048 tokens): 3 bits 2321 -> 735; KV, 32 heads, three sequences, 1100 queries on 1337 keys, 4 bits
-// 945 -> 316. What bounds it is the latency of the hand-overs between the roles: of the 9.7 warp cycles an issue (37 heads, 2048
-// tokens), 3.7 are long scoreboards (tensor-memory loads, barrier waits), 1.7 fixed latencies, 0.4 instruction fetch (cache-only
-// 4.0, 1.5, 0.9); issue slots are 52 % busy, the tensor pipe 11 %. Code that runs at the same time is worth keeping short all the
+// 945 -> 314. What bounds it is the latency of the hand-overs between the roles: of the 9.7 warp cycles an issue (37 heads, 2048
+// tokens), 3.7 are long scoreboards (tensor-memory loads, barrier waits), 1.7 fixed latencies, 0.4 instruction fetch (cache-only, of
+// 11.3: 4.7, 1.5, 1.7); issue slots are 52 % (44 %) busy, the tensor pipe 11 %. Code that runs at the same time is worth keeping short all the
 // same: the compiler told that the warp index is uniform 916 -> 790 (93 -> 83 KB of code), the output rows' store loops not
 // unrolled 790 -> 772; a first cluster's drain of its own (two copies of the loop) 790 -> 830. The order in which items are dealt
 // out: see item_index (767 -> 735).
@@ -199,7 +200,8 @@ prefill_kernel(const AttnParams p, const Plan g)
         }
         for (int i = 0; i < 2 * N_SLOTS; ++i) { mbar_init(bar(B_SFULL + i), 1); mbar_init(bar(B_SEMPTY + i), 4); }
         mbar_init(bar(B_OFULL), 1); mbar_init(bar(B_OEMPTY), 4); mbar_init(bar(B_OUT), 4);
-        mbar_init(bar(B_SUM), S_WARPS); mbar_init(bar(B_XS), S_WARPS); mbar_init(bar(B_XV), 4);
+        mbar_init(bar(B_SUM), S_WARPS); mbar_init(bar(B_XV), 4);
+        if constexpr (PASSES == 2) mbar_init(bar(B_XS), S_WARPS);
         for (int i = 0; i < 3; ++i) mbar_init(bar(B_DRAIN + i), 1);
         if constexpr (ALT) for (int i = 0; i < 16; ++i) mbar_init(bar(B_REF + i), 1);
         *s_abort = 0;
@@ -865,21 +867,19 @@ prefill_kernel(const AttnParams p, const Plan g)
             uint32_t rsum = 0u;
 #pragma unroll 1
             for (int pass = 2 - PASSES; pass < 2 && ok; ++pass, n_k0 += it.n_kt) {
-                if (PASSES == 2 && pass == 1) {
+                if constexpr (PASSES == 2) if (pass == 1) {
                     // the streams' statistics meet (two sets by turns: a warp may be an item ahead of another)
                     float2* ml = s_ml + (n_item & 1) * STREAMS * BM + row;
                     ml[stream * BM] = make_float2(m, l);
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(B_XS));
                     if (!mbar_sleep_warp(bar(B_XS), n_item & 1, s_abort)) { ok = false; break; }
+                    l = 0.f;
 #pragma unroll
                     for (int q = 0; q < STREAMS; ++q) m = fmaxf(m, ml[q * BM].x);
-                    if constexpr (MODE != KV) {
-                        l = 0.f;
 #pragma unroll
-                        for (int q = 0; q < STREAMS; ++q) l = __fmaf_rn(ml[q * BM].y, ex2(ml[q * BM].x - m), l);     // (a stream without a visible key weighs 0)
-                        f = p.inv_sP / l * 1.7763568394002505e-15f;            // times 2^-49: see below
-                    }
+                    for (int q = 0; q < STREAMS; ++q) l = __fmaf_rn(ml[q * BM].y, ex2(ml[q * BM].x - m), l);     // (a stream without a visible key weighs 0)
+                    f = p.inv_sP / l * 1.7763568394002505e-15f;                // times 2^-49: see below
                 }
 #pragma unroll 1
                 for (int kt = ALT ? stream : 0; kt < it.n_kt; kt += ALT ? 2 : 1) {
@@ -938,8 +938,8 @@ prefill_kernel(const AttnParams p, const Plan g)
                             if (2 * e + 1 > n_vis) S[e].y = NEG_BIG;
                         }
                     }
-                    if (pass == 0) {
-                        // ---- pass 1: row maximum (integer calls: and row sum) over my keys
+                    if constexpr (PASSES == 2) if (pass == 0) {
+                        // ---- pass 1: row maximum and sum over my keys
                         if (live) {
                             float x0 = NEG_BIG, x1 = NEG_BIG;
 #pragma unroll
@@ -948,17 +948,15 @@ prefill_kernel(const AttnParams p, const Plan g)
                                 x1 = fmaxf(x1, fmaxf(S[e + 1].x, S[e + 1].y));
                             }
                             const float n = fmaxf(m, fmaxf(x0, x1));
-                            if constexpr (MODE != KV) {
-                                const float2 nn = make_float2(-n, -n);
-                                float2 a0 = make_float2(0.f, 0.f), a1 = a0;
+                            const float2 nn = make_float2(-n, -n);
+                            float2 a0 = make_float2(0.f, 0.f), a1 = a0;
 #pragma unroll
-                                for (int e = 0; e < COLS / 2; e += 2) {
-                                    const float2 y = add2(S[e], nn), z = add2(S[e + 1], nn);
-                                    a0 = add2(a0, make_float2(ex2(y.x), ex2(y.y)));
-                                    a1 = add2(a1, make_float2(ex2(z.x), ex2(z.y)));
-                                }
-                                l = l * ex2(m - n) + ((a0.x + a0.y) + (a1.x + a1.y));
+                            for (int e = 0; e < COLS / 2; e += 2) {
+                                const float2 y = add2(S[e], nn), z = add2(S[e + 1], nn);
+                                a0 = add2(a0, make_float2(ex2(y.x), ex2(y.y)));
+                                a1 = add2(a1, make_float2(ex2(z.x), ex2(z.y)));
                             }
+                            l = l * ex2(m - n) + ((a0.x + a0.y) + (a1.x + a1.y));
                             m = n;
                         }
                         continue;
@@ -998,7 +996,7 @@ prefill_kernel(const AttnParams p, const Plan g)
                             m = ref;
                         }
                     }
-                    // ---- pass 2: probabilities. P's region also stages the previous item's output
+                    // ---- probabilities (integer calls: pass 2). P's region also stages the previous item's output
                     if (kt < 2 && !mbar_sleep_warp(bar(B_OUT), (n_item & 1) ^ 1, s_abort)) { ok = false; break; }
                     // the buffer's previous tile has been multiplied
                     // (one buffer for both streams: stream 1's first tile waits for stream 0's)
