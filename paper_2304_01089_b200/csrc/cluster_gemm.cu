@@ -949,7 +949,7 @@ cluster_gemm_kernel(const Params p)
         // With a thread per row, what belongs to a column is read by every thread, and a warp-wide load of 16 bytes takes four clocks of
         // the SM's shared-memory port even where all lanes read the same: 64 a drain of clustered weights (2048 of its 2125 clocks), 96 a tile
         // for the tables of the outputs; in the other layout a load serves four rows. But its tensor-memory loads take longer (some 66 clocks a
-        // drain more), and a word of codes lies in four lanes. Which of the two is the faster depends on the clusters of a tile: see launch_gemm.
+        // drain more), and a word of codes lies in four lanes. Which of the two is the faster depends on the number of clusters: see launch_gemm.
         float2 R[64];
         for (int t = pair_id; t < p.n_items; t += n_pairs, ++n_tile_done) {
             int mt, n0;
@@ -962,12 +962,14 @@ cluster_gemm_kernel(const Params p)
 #pragma unroll
             for (int i = 0; i < 64; ++i) R[i] = make_float2(0.f, 0.f);
             // outputs as codes: lane l holds the output layout's unit l of my columns, asked for before the sums (700 x 768 x 3072, 8
-            // clusters: 14.4 -> 13.6 us)
+            // clusters: 14.4 -> 13.6 us); LATE: after them, since four registers more cost the drains of float outputs 1 %
             uint4 unit4 = make_uint4(0u, 0u, 0u, 0u);
-            if constexpr (!DEQ) {
+            auto ask_units = [&]() {
                 const int unit = (n0 + h * half_cols) / 32 + (lane & 3);
                 if (p.y_dtype == RPTQ_OUT_CODES && 32 * unit < p.N) unit4 = __ldg(reinterpret_cast<const uint4*>(p.out_unit + unit));
-            }
+            };
+            constexpr bool LATE = MODE == MODE_INT && NCTA == 2 && !ROWS;
+            if constexpr (!DEQ && !LATE) ask_units();
             // ASYM: my tokens' code sums of the cluster to come (rows past the last token read the last one's)
             const int32_t* xs_row[4] = {nullptr, nullptr, nullptr, nullptr};
             int xs_next[4] = {0, 0, 0, 0};
@@ -1055,6 +1057,7 @@ cluster_gemm_kernel(const Params p)
                     }
                 }
             }
+            if constexpr (LATE) ask_units();
             mbar_wait(bar(B_TAB + (n_tile_done & 1)), (n_tile_done >> 1) & 1, s_abort);
             // y = s_w * (R - corr) + bias, activation, store. Rows leave through a buffer of the warp, in pieces of 64 bytes a row: whole memory
             // sectors, and few hand-overs between lanes (1999 x 2048 x 6144, 8 bits, fp32 out, with the LayerNorm: stores of a lane's own 16 bytes
@@ -1470,15 +1473,14 @@ static int launch_gemm(const rptq_layout_t* Lin, const void* a_codes, int M, con
         if (Lin->bits == 4) return gemm::launch<4, 1, false, gemm::MODE_ASYM>(p, dev, n_sm, st);
         return gemm::launch<8, 1, false, gemm::MODE_ASYM>(p, dev, n_sm, st);
     }
-    // Sums by rows (see the epilogue) for CTA pairs. Re-quantised outputs: yes (4096 x 2048 x 8192, 3, 4 and 8 bits, 32 clusters 199, 190, 198 -> 182,
-    // 179, 183 us; 4 clusters 84.4, 76.0, 83.4 -> 79.0, 75.5, 82.5; 2048 x 12288 x 12288, 64 clusters, 8 bits 352 -> 343), except for 4 bits after a
-    // long contraction of long clusters, where the tables' loads are in the unpack warps' way (2048 x 8192 x 8192, 32: 142.5 and 144.2; 2048 x
-    // 12288 x 49152, 64: 1169 and 1190). Others: many short clusters over more than one round of tiles, whose drains set the pace (2000 x
-    // 1024 x 4096 to fp16, 4 bits: 64 clusters 87.4 -> 81.5, 32 50.5 -> 47.9; 2048 x 4096 x 16384, 32: 188 -> 184). Not fewer clusters (2000 x
-    // 1024 x 4096 to fp32, 8: 25.5 and 26.0), longer ones, which a drain passes under (1024 x 9216 x 9216, 32: 79.8 and 81.3), a single round, which
-    // ends in the outputs (700 x 768 x 3072, 32: 19.5 and 20.1), or blocks on their own (128 x 2048 x 8192, 64: 26.1 and 26.5; codes the same).
-    const bool short_clusters = Lin->K_pad < 192 * Lin->n_seg;
-    const bool by_rows = Lout ? Lout->bits != 4 || Lin->K_pad <= 8192 || short_clusters : Lin->n_seg >= 20 && short_clusters && n_tiles > slots;
+    // Sums by rows (see the epilogue) for CTA pairs with many clusters, whose drains set the pace: 4 bits, 16-lane layout -> rows, us: 2000 x 1024 x 4096
+    // to fp16, 64 clusters 87.4 -> 81.5, 32 50.5 -> 47.9; 2048 x 4096 x 16384, 32: 188 -> 184; codes of 4096 x 2048 x 8192, 32: 190 -> 179. With few
+    // the outputs' tables count for more: 2000 x 1024 x 4096 to fp32, 8 clusters: 25.5 and 26.0, 1999 x 2048 x 6144, 8 bits: 50.6 and 52.4
+    // (with the LayerNorm); 16 clusters are even. Long clusters, whose drains pass under the products, would still be up to 1.7 % faster the other way
+    // (1024 x 9216 x 9216, 32: 79.8 and 81.3), and so would be the rows for codes of few clusters (4096 x 768 x 3072, 8: 30.6 and 29.1), but
+    // both linears of an MLP should run the same instance: one whose code the call before did not run costs 2 to 5 us more
+    // (400 x 1328 x 3984 x 1328, 16 clusters: 37.6 with one, 41.2 with both).
+    const bool by_rows = Lin->n_seg >= 20;
     if (ncta == 2) {
         if (Lin->bits == 3) return by_rows ? gemm::launch<3, 2, false, gemm::MODE_INT, true>(p, dev, n_sm, st) : gemm::launch<3, 2, false, gemm::MODE_INT>(p, dev, n_sm, st);
         if (Lin->bits == 4) return by_rows ? gemm::launch<4, 2, false, gemm::MODE_INT, true>(p, dev, n_sm, st) : gemm::launch<4, 2, false, gemm::MODE_INT>(p, dev, n_sm, st);

@@ -420,20 +420,26 @@ def test_whole_tiles_and_strips_give_the_bits_of_small_calls(out):
         np.testing.assert_array_equal(whole[lo:lo + n].view(np.uint8), part.view(np.uint8))
 
 
-# The epilogue that holds a token row per thread: re-quantised outputs of CTA pairs (above), and many short clusters over more than one round.
+# The epilogue that holds a token row per thread: CTA pairs with many clusters.
 @pytest.mark.parametrize("bits", [4, 3, 8])
-@pytest.mark.parametrize("out", ["f32", "f16"])
-def test_many_short_clusters_give_the_bits_of_small_calls(out, bits):
+@pytest.mark.parametrize("out", ["f32", "f16", 3, 4, 8])
+def test_many_clusters_give_the_bits_of_small_calls(out, bits):
     """80 tiles on 74 pairs of blocks, 24 clusters of one or two steps: whole tiles and strips with ragged rows and columns, against calls of at most
     128 tokens (whose blocks hold their sums in the other layout) and, on some rows, the oracle."""
     from paper_2304_01089_b200 import binding
-    M, N = 2401, 2045
+    codes = isinstance(out, int)
+    M, N = 2401, 2048 if codes else 2045
     rng = np.random.default_rng(78 + bits)
     case = _case(rng, M, N, 904, 24, bits, n_pad=2048, allow_empty=False)
-    assert case["k_pad"] < 192 * 24
     d = _dev(case)
     bias = (rng.normal(size=N) * 0.05).astype(np.float32)
     kw = dict(y_dtype=binding.OUT_F32 if out == "f32" else binding.OUT_F16, ldy=2048, bias=bias, act=binding.ACT_RELU)
+    if codes:
+        size2 = np.array([1, 31, 32, 33, 64, 500, 700, 500, 59])
+        step = np.abs(_gemm(dict(case, M=128), dict(d, a=d["a"][:128].contiguous()))).max() / (1 << out)
+        L2 = binding.Layout(np.arange(size2.sum(), dtype=np.int32), size2, np.full(9, step, np.float32), np.full(9, 1 << (out - 1), np.int32), out)
+        assert L2.K_pad == N
+        kw.update(y_dtype=binding.OUT_CODES, layout_out=L2, ldy=None)
     whole = _gemm(case, d, **kw)
     for lo in range(0, M, 128):
         n = min(128, M - lo)
