@@ -136,7 +136,7 @@ def _step(sites, binding, M, events=None):
 
 
 # dram__bytes_read.sum + dram__bytes_write.sum of one FC1 launch, from the 512-token ncu capture of the
-# current kernel (profiles/cluster_gemm_512x9216x36864.txt: 191.3 MB read, 22.2 MB written, part of
+# current kernel (profiles/cluster_gemm_512x9216x36864.txt: 191.6 MB read, 23.0 MB written, part of
 # the output still in L2) scaled to 4096 tokens: weights, Wsum and s_w (191.1 MB) are read once whatever
 # the token count; codes (1.94 MB per 512 tokens) and the fp16 output (37.75 MB per 512 tokens) grow with it.
 FC1_DRAM_BYTES_PER_LAUNCH = int(191.1e6 + 8 * (1.94e6 + 37.75e6))

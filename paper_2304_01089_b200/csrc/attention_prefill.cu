@@ -5,7 +5,7 @@
 // probabilities and multiplies them with V. Nothing is rescaled on the way. Scores are computed in both passes; the tensor cores
 // have room for that. KV calls walk the keys once: probabilities are relative to a reference that follows the row's maximum, and
 // the output accumulator is brought to a new reference where it moves (3 x 1100 queries on 1337 keys, 32 heads of 128 channels: two walks
-// 347 us, one 314).
+// 345 us, one 310).
 //
 // What bounds it: one exponential per score and pass (the special-function unit gives 16 per clock and SM), then the
 // issue slots of the softmax warps: a score costs one multiply-add per cluster of the head, and five or six
@@ -35,7 +35,7 @@
 //
 // Measured, us, against a mma.sync kernel with 64 (KV: 128) queries per block (72 heads of 128 channels, four clusters each,
 // causal, two sequences of 2048 tokens): 3 bits 2321 -> 735; KV, 32 heads, three sequences, 1100 queries on 1337 keys, 4 bits
-// 945 -> 314. What bounds it is the latency of the hand-overs between the roles: of the 9.7 warp cycles an issue (37 heads, 2048
+// 945 -> 310. What bounds it is the latency of the hand-overs between the roles: of the 9.7 warp cycles an issue (37 heads, 2048
 // tokens), 3.7 are long scoreboards (tensor-memory loads, barrier waits), 1.7 fixed latencies, 0.4 instruction fetch (cache-only, of
 // 11.3: 4.7, 1.5, 1.7); issue slots are 52 % (44 %) busy, the tensor pipe 11 %. Code that runs at the same time is worth keeping short all the
 // same: the compiler told that the warp index is uniform 916 -> 790 (93 -> 83 KB of code), the output rows' store loops not
